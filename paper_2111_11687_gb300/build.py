@@ -20,6 +20,9 @@ LIB = os.path.join(HERE, "libnmdose.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
          "--expt-relaxed-constexpr", "-I", INCLUDE, "-I", CSRC]
+# The transport flushes FP32 denormals: its logarithms, divisions and
+# reciprocal roots then need no scaling of denormal operands.
+FILE_FLAGS = {"nm_transport.cu": ["-ftz=true"]}
 
 
 def _nvcc() -> str:
@@ -43,7 +46,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
 
     def compile_one(src):
         obj = os.path.join(BUILD, os.path.basename(src)[:-3] + ".o")
-        cmd = [nv, *ARCH, *FLAGS, *extra_flags, "-c", src, "-o", obj]
+        cmd = [nv, *ARCH, *FLAGS, *FILE_FLAGS.get(os.path.basename(src), []), *extra_flags, "-c", src, "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed for {src}:\n{r.stderr}")

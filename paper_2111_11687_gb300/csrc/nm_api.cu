@@ -591,6 +591,18 @@ static int grid_for_shape(const nm_dose* h, const Shape& sh, bool multi) {
   return per_sm * h->sms;
 }
 
+// Histories per work grab of a launch of n: the handle's chunk, but where it is
+// tuned (on 2^25 decays) at most half of a warp's share, in warps' widths.  A
+// launch of 1e5 in chunks of 256 keeps 391 of 4864 warps busy (point source in
+// water, 1e6 histories in ten batches: 0.85 ms in chunks of 256, 0.50 in chunks
+// of 32, 0.59 in chunks of 16).
+static int launch_chunk(const nm_dose* h, uint64_t n) {
+  if (h->opt.chunk > 0) return h->chunk;
+  const uint64_t warps = (uint64_t)h->grid * (h->block / 32);
+  const uint64_t share = n / (2 * warps) / 32 * 32;
+  return (int)std::min<uint64_t>(h->chunk, std::max<uint64_t>(share, 32));
+}
+
 static void apply_shape(nm_dose* h, const Shape& sh) {
   h->block = sh.block;
   h->chunk = sh.chunk;
@@ -654,8 +666,11 @@ static nm_status autotune(nm_dose* h, Shape sh, bool free_block, bool free_chunk
     if (r == NM_OK && m < best) { best = m; sh = t; }
     return r;
   };
+  // The ring kernel regroups by itself, 32 photons at a time, so it has no lane
+  // count to choose, and regrouping off (the lane kernel) is never faster.
+  const bool ring = !h->opt.history_sigma && !h->nuclide && sh.regroup;
   for (int pass = 0; pass < 2 && st == NM_OK; ++pass) {
-    if (free_regroup || free_lanes) {
+    if ((free_regroup || free_lanes) && !ring) {
       const int lanes[] = {8, 12, 16};
       for (int l : lanes) {
         if (!free_lanes && l != sh.lanes) continue;
@@ -968,6 +983,7 @@ nm_status nm_dose_run(nm_dose* h, uint64_t n, uint64_t seed) {
       TransportParams p = h->params(h->id_next + done, part, seed);
       p.g.tally = tally;
       p.g.work = work;
+      p.chunk = launch_chunk(h, part);
       NM_CUDA(cudaMemsetAsync(work, 0, sizeof(unsigned), bs), "cudaMemsetAsync");
       NM_CUDA(launch_transport(p, h->grid, h->block, h->warp_agg, h->rayleigh, h->regroup, bs, false,
                                h->opt.history_sigma != 0),

@@ -58,15 +58,19 @@ __host__ __device__ inline PhiloxKey philox_key(uint32_t k0, uint32_t k1) {
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const PhiloxKey& k) {
 #pragma unroll
   for (int r = 0; r < 10; ++r) {
-    const uint32_t lo0 = 0xD2511F53u * c.x, hi0 = __umulhi(0xD2511F53u, c.x);
-    const uint32_t lo1 = 0xCD9E8D57u * c.z, hi1 = __umulhi(0xCD9E8D57u, c.z);
-    c = make_uint4(hi1 ^ c.y ^ k.rk[2 * r], lo1, hi0 ^ c.w ^ k.rk[2 * r + 1], lo0);
+    const ull p0 = (ull)0xD2511F53u * c.x, p1 = (ull)0xCD9E8D57u * c.z;
+    c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ k.rk[2 * r], (uint32_t)p1,
+                   (uint32_t)(p0 >> 32) ^ c.w ^ k.rk[2 * r + 1], (uint32_t)p0);
   }
   return c;
 }
 
-// Uniform float in the open interval (0, 1) from 23 random bits.
-__device__ __forceinline__ float u01(uint32_t r) { return ((float)(r >> 9) + 0.5f) * 0x1p-23f; }
+// Uniform float in the open interval (0, 1) from 23 random bits k = r >> 9:
+// (k + 1/2) 2^-23, exactly, as the float 1 + k 2^-23 (one funnel shift puts
+// the exponent before k) less 1 - 2^-24.
+__device__ __forceinline__ float u01(uint32_t r) {
+  return __uint_as_float(__funnelshift_r(r, 0x7fu, 9)) - 0x0.ffffffp0f;
+}
 
 // Random-stream ids inside one history: gamma line j flies on stream
 // kStreamGamma0 + j after the emission draws of kStreamGammaSelect.

@@ -3,18 +3,26 @@
 // grid, Klein-Nishina Compton (Kahn's sampler), photoelectric absorption,
 // optional Rayleigh, 10 keV photon cutoff, int64 fixed-point tally.
 //
-// One persistent launch per batch.  Each lane owns one photon; a lane whose
-// photon ends takes the decay's second photon or, with the rest of its warp,
-// refills from a warp-private pool of history ids that one lane grabs from a
-// global counter in chunks.  Every iteration of the loop is one flight step
-// for every live lane, so lanes stay converged on the flight; the interaction
-// work is regrouped (see the `regroup` variant) so that a warp runs Compton
-// sampling for a batch of lanes at once instead of once per step.
+// One persistent launch per batch, in two kernels.  In transport_ring_kernel
+// (annihilation photons or a point source, one patient: the default) a warp's
+// lanes hand photons on to each other through a ring in shared memory.  In
+// transport_kernel (several patients, history statistics, other decays, or
+// `regroup` off) each lane owns one photon; a lane whose photon ends takes the
+// decay's second photon or, with the rest of its warp, refills from a
+// warp-private pool of history ids that one lane grabs from a global counter
+// in chunks.  Every iteration of the loop is one flight step for every live
+// lane, so lanes stay converged on the flight; the interaction work is
+// regrouped (see the `regroup` variant) so that a warp runs Compton sampling
+// for a batch of lanes at once instead of once per step.  Both give the same
+// bits.
 //
 // A history's random numbers come from Philox4x32-10 keyed by the seed with
 // counter (block index, stream, history id), so which lane or SM simulates it
 // does not matter, and integer atomics make the tally order-independent: a
 // fixed seed gives bit-identical tallies.
+#include <cstddef>
+#include <type_traits>
+
 #include "nm_internal.cuh"
 
 namespace nm {
@@ -22,12 +30,6 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kKahnTrialLimit = 1000;
-// Decay-site queue of the single-patient regrouped variant: per warp a ring
-// of kQueueCap sampled decays in shared memory, structure of arrays with
-// kQueueWords words per decay (site x y z, photon A's direction u v w, the
-// two photons' distances to their region boundary, history id lo and hi,
-// whether the site lies outside the tracking box).
-constexpr int kQueueCap = 64, kQueueWords = 11;
 
 struct Energy {
   float s_c, s_pe, s_r;   // per-unit-density factors: mu/rho = za s_c + zp s_pe + zr s_r
@@ -378,10 +380,10 @@ __device__ __forceinline__ ull warp_sum(ull x) {
 
 // Compton event at energy e: Kahn-sampled angle, new energy and direction, and
 // the local deposit (the electron's energy, or everything below the cutoff).
-template <bool RAYLEIGH>
-// With the tabulated sampler the angle takes the two words (rk, rp) that
-// the flight step which found the event drew but did not use; Kahn's sampler
-// draws its own blocks.
+// With the tabulated sampler (always with TABLE) the angle takes the two words
+// (rk, rp) that the flight step which found the event drew but did not use;
+// Kahn's sampler draws its own blocks.
+template <bool RAYLEIGH, bool TABLE = false>
 __device__ __forceinline__ void compton(const TransportParams& p, const float* s_kn,
                                         const float* s_minv, float& e, int32_t& qe, Energy& f,
                                         float& ux, float& uy, float& uz, uint32_t& ctr,
@@ -391,7 +393,7 @@ __device__ __forceinline__ void compton(const TransportParams& p, const float* s
   uint32_t rphi;
   const float k = e * kInvElectronMassMeV;
   float x;
-  if (p.kn_inv) {
+  if (TABLE || p.kn_inv) {
     x = kn_table_x(p, e, rk);
     rphi = rp;
   } else {
@@ -515,115 +517,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
   uint32_t n_steps = 0, n_compton = 0, n_esc = 0, flags = 0;
   ull escaped = 0;
 
-  // The single-patient regrouped variant samples decays ahead of need: the
-  // whole warp fills its site queue 32 decays at a time, and a lane whose
-  // photons have ended takes the next queued decay at once, so no lane waits
-  // for a refill pass and the sampling runs with every lane busy.
-  constexpr bool SITEQ = REGROUP && !MULTI && !HIST && !BETA;
-  float* const q_base = s_site + 9 * nb + (threadIdx.x >> 5) * (kQueueCap * kQueueWords);
-  uint32_t q_head = 0, q_count = 0;      // warp-uniform ring state
-  bool drained = false;                  // warp-uniform: every history id has been handed out
-
   for (;;) {
-    if constexpr (SITEQ) {
-      // ---- fill the site queue: one new decay per lane -----------------------
-      if (q_count < 32 && !drained) {
-        const uint32_t avail = pool_end - pool_next;
-        uint32_t fresh = 0, fresh_end = 0;
-        if (avail < 32) {
-          if (lane == 0) {
-            const unsigned f0 = atomicAdd(p.g.work, (unsigned)p.chunk);
-            if ((uint64_t)f0 < p.g.n_hist) {
-              fresh = f0;
-              fresh_end = (uint32_t)min((uint64_t)f0 + (uint64_t)p.chunk, p.g.n_hist);
-            }
-          }
-          fresh = __shfl_sync(kFull, fresh, 0);
-          fresh_end = __shfl_sync(kFull, fresh_end, 0);
-        }
-        uint32_t idx = 0;
-        bool got = true;
-        if (lane < avail) {
-          idx = pool_next + lane;
-        } else if (fresh + (lane - avail) < fresh_end) {
-          idx = fresh + (lane - avail);
-        } else {
-          got = false;
-        }
-        if (avail < 32) {
-          pool_next = min(fresh + (32u - avail), fresh_end);
-          pool_end = fresh_end;
-          drained = fresh_end == 0;
-        } else {
-          pool_next += 32;
-        }
-        const uint32_t n_got = __popc(__ballot_sync(kFull, got));   // lanes 0 .. n_got - 1
-        bool has = false;
-        ull* cell = nullptr;
-        if (got) {
-          const uint64_t h = p.g.hist_begin + idx;
-          const uint32_t slo = (uint32_t)h, shi = (uint32_t)(h >> 32);
-          const Site st = sample_site(p.g, p.key, slo, shi);
-          const bool o = outside_box(p.g, st.x, st.y, st.z);
-          float ra, rb;
-          region_distance_pair(p.g, o, st.x, st.y, st.z, st.u, st.v_, st.w, ra, rb);
-          float* qs = q_base + ((q_head + q_count + lane) & (kQueueCap - 1));
-          uint32_t* qw = reinterpret_cast<uint32_t*>(qs);
-          qs[0] = st.x; qs[kQueueCap] = st.y; qs[2 * kQueueCap] = st.z;
-          qs[3 * kQueueCap] = st.u; qs[4 * kQueueCap] = st.v_; qs[5 * kQueueCap] = st.w;
-          qs[6 * kQueueCap] = ra; qs[7 * kQueueCap] = rb;
-          qw[8 * kQueueCap] = slo; qw[9 * kQueueCap] = shi; qw[10 * kQueueCap] = o ? 1u : 0u;
-          if (p.g.source_mode == NM_SOURCE_DECAY) {
-            has = p.g.q_positron > 0;
-            cell = p.g.tally + st.v;
-          }
-        }
-        tally_flush<WARP_AGG>(cell, has, (uint32_t)p.g.q_positron, lane);
-        q_count += n_got;
-        __syncwarp();
-      }
-      // ---- lanes without a photon: the decay's second one, or the next decay -
-      const unsigned want = __ballot_sync(kFull, !alive && !pending_b);
-      const uint32_t n_pop = min((uint32_t)__popc(want), q_count);
-      if (!alive) {
-        if (pending_b) {
-          pending_b = false;
-          alive = true;
-          px = site[0]; py = site[nb]; pz = site[2 * nb];
-          ux = -site[3 * nb]; uy = -site[4 * nb]; uz = -site[5 * nb];
-          e = p.e0; qe = p.q_e0; f = s_f0;
-          stream = kStreamPhotonB; ctr = 0; steps = 0;
-          out = outside_box(p.g, px, py, pz);
-          rem = site[6 * nb];
-          if (out) f.inv_mubar = s_inv0_out;
-        } else {
-          const uint32_t rank = __popc(want & lt_mask);
-          if (rank < n_pop) {
-            const float* qs = q_base + ((q_head + rank) & (kQueueCap - 1));
-            const uint32_t* qw = reinterpret_cast<const uint32_t*>(qs);
-            px = qs[0]; py = qs[kQueueCap]; pz = qs[2 * kQueueCap];
-            ux = qs[3 * kQueueCap]; uy = qs[4 * kQueueCap]; uz = qs[5 * kQueueCap];
-            rem = qs[6 * kQueueCap];
-            hlo = qw[8 * kQueueCap]; hhi = qw[9 * kQueueCap];
-            out = qw[10 * kQueueCap] != 0u;
-            e = p.e0; qe = p.q_e0; f = s_f0;
-            if (out) f.inv_mubar = s_inv0_out;
-            stream = kStreamPhotonA; ctr = 0; steps = 0;
-            alive = true;
-            if (p.g.source_mode == NM_SOURCE_DECAY) {
-              site[0] = px; site[nb] = py; site[2 * nb] = pz;
-              site[3 * nb] = ux; site[4 * nb] = uy; site[5 * nb] = uz;
-              site[6 * nb] = qs[7 * kQueueCap];
-              pending_b = true;
-            }
-          }
-        }
-      }
-      q_head = (q_head + n_pop) & (kQueueCap - 1);
-      q_count -= n_pop;
-      __syncwarp();
-      if (!__any_sync(kFull, alive) && q_count == 0 && drained) break;
-    } else {
     // ---- second photon of the decay: same site, opposite direction ----------
     if (!alive && pending_b) {
       pending_b = false;
@@ -795,7 +689,6 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
       tally_flush<WARP_AGG>(cell, has, (uint32_t)(MULTI ? s_geom[pi].q_positron : p.g.q_positron), lane);
     }
     if (!__any_sync(kFull, alive || !done)) break;
-    }
 
     const PatientGeom& G = MULTI ? s_geom[pi] : p.g;
     bool has = false;
@@ -947,6 +840,540 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
   }
 }
 
+// ---------------------------------------------------------------------------
+// The default transport: photons handed from lane to lane.
+//
+// Bound by instruction issue.  A flight step finds a scatter or ends a photon
+// about every second time, so a warp whose lanes keep their photon through a
+// scatter flies with half its lanes.  Here a lane that finds a Compton event
+// parks its photon in the warp's ring in shared memory and, in the same
+// exchange, takes a photon that is ready to fly; once 32 are parked the whole
+// warp scatters them at once, one per lane, in place.
+//
+// The ring holds kRing photons and is always full: [head - n_parked, head) are
+// parked, the others, from head on, are ready (or empty, energy 0, which hands
+// the lane on to the site queue).  An exchange at the head turns a ready slot
+// into the youngest parked one; a Compton pass over the 32 oldest parked slots
+// makes them the ring's last ready ones.  So the only bookkeeping is head and
+// n_parked (warp-uniform), and all accesses go to consecutive slots (no bank
+// conflicts).  A lane without a photon takes the next of the site queue (32
+// decays sampled at once, two photons each); when every decay has been
+// started, it exchanges an empty slot instead, which turns the ring; and once
+// the lanes can hold all photons left, each scatters its own, so that the last
+// photons of a launch do not wait in the ring (5e6 decays 1.15 -> 1.10 ms, 1e6
+// point-source histories in ten launches 0.76 -> 0.50 ms).
+//
+// Benchmark phantom, 1e9 decays: 234.6 -> 137.3 ms; per decay 238.8 -> 127.2
+// warp instructions at 16.2 -> 24.4 active lanes.  Of that, the ring itself
+// with one word per access 234.6 -> 197.7; slots as 16-byte words, the uniform
+// variates without a conversion and no denormals -> 171.7; branches folded into
+// predicates, both regions' majorants kept with the photon, escapes counted
+// from what is left over -> 150.5; a loop of its own for the end, the region
+// and photon B as signs -> 137.8; shared-memory addresses formed once -> 135.9; the lanes' own scatters at the end -> 137.3.
+// A FIFO that pushes to and pops from different slots (fewer register moves,
+// more bookkeeping) measured 148-160.
+// ---------------------------------------------------------------------------
+constexpr int kRing = 64;       // photons: 31 parked at most before an exchange, 32 lanes more
+constexpr int kSiteQueue = 32;  // decays
+// A ring slot is three 16-byte words and one of eight bytes, each an array
+// over the slots, so that a lane moves its photon with a few wide accesses and
+// the warp's accesses have no bank conflicts:
+//   pos: position (voxel units), energy (0: empty; negative: photon B);
+//   dir: direction, low word of the history id;
+//   mid: ready: s_c, s_pe, 1 / majorant of the photon's region, distance to the
+//        region's boundary; parked: the Compton pass's two Philox words, the
+//        voxel, 1 / majorant;
+//   aux: next Philox counter, 1 / majorant of the other region.
+// A majorant outside the tracking box carries a minus sign, so that the sign
+// tells the region.
+// The site queue: position and history id; photon A's direction and its
+// distance to the region boundary; photon B's distance, and -1 outside the box.
+struct WarpStore {
+  float4 pos[kRing], dir[kRing], mid[kRing];
+  float4 site_pos[kSiteQueue], site_dir[kSiteQueue];
+  uint2 aux[kRing];
+  float2 site_rem[kSiteQueue];
+};
+struct WarpStoreGeneral : WarpStore {
+  uint2 gen[kRing];             // flight steps (the counter also counts other draws), Rayleigh factor
+};
+static_assert(sizeof(WarpStore) % 16 == 0 && sizeof(WarpStoreGeneral) % 16 == 0, "warps' stores stay 16-byte aligned");
+
+template <bool GENERAL>
+struct StoreOf { typedef WarpStore type; };
+template <>
+struct StoreOf<true> { typedef WarpStoreGeneral type; };
+
+// Shared-memory accesses by 32-bit address (the compiler forms the address of
+// a shared array anew at every use).
+__device__ __forceinline__ float4 lds4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ float2 lds2(uint32_t a) {
+  float2 v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ float lds1(uint32_t a) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void sts4(uint32_t a, float x, float y, float z, float w) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
+__device__ __forceinline__ void sts2(uint32_t a, float x, float y) {
+  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(x), "f"(y) : "memory");
+}
+__device__ __forceinline__ void sts1(uint32_t a, float x) {
+  asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(x) : "memory");
+}
+
+// Cross sections at energy e: bins of {kn, next - this, 1 / majorant inside,
+// - 1 / majorant outside the tracking box} (energy_factors, both regions).
+struct RingEnergy {
+  float s_c, s_pe, s_r, maj_in, maj_out;
+};
+template <bool RAYLEIGH>
+__device__ __forceinline__ RingEnergy ring_energy(float e, uint32_t tab, float ln_lo, float inv_dln) {
+  RingEnergy f;
+  float x = (__logf(e) - ln_lo) * inv_dln;
+  x = fminf(fmaxf(x, 0.0f), (float)(kKnTable - 1) - 0x1p-10f);
+  const int i = (int)x;
+  const float4 t = lds4(tab + 16 * i);
+  f.s_c = fmaf(x - (float)i, t.y, t.x);
+  const float ie = __fdividef(1.0f, e);
+  const float ie2 = ie * ie;
+  f.s_pe = ie2 * ie;
+  f.s_r = RAYLEIGH ? ie2 : 0.0f;
+  f.maj_in = t.z;
+  f.maj_out = t.w;
+  return f;
+}
+
+// Tables of a CTA, at the start of its dynamic shared memory; a store per warp
+// follows.
+struct RingTables {
+  float4 tab[kKnTable];
+  float2 mat[NM_MAX_MATERIALS];   // za, zp
+  float zr[NM_MAX_MATERIALS];
+};
+static_assert(sizeof(RingTables) % 16 == 0, "the warps' stores follow");
+
+// GENERAL: Rayleigh scattering and Kahn's sampler, whose trials draw from the
+// photon's counter; otherwise the counter is the number of flight steps.
+template <bool WARP_AGG, bool GENERAL>
+__global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportParams p) {
+  typedef typename StoreOf<GENERAL>::type Store;
+  __shared__ RingEnergy s_f0;                  // at the source energy
+  __shared__ unsigned long long s_cnt[12];     // [0..7]: CounterSlot; photons started, killed; energy deposited
+  extern __shared__ __align__(16) unsigned char s_dyn[];   // tables, then a Store per warp
+  RingTables& tb = *reinterpret_cast<RingTables*>(s_dyn);
+  for (int i = threadIdx.x; i < kKnTable; i += blockDim.x) {
+    const float a = p.kn[i];
+    tb.tab[i] = make_float4(a, p.kn[min(i + 1, kKnTable - 1)] - a, p.minv[i], -p.minv_out[i]);
+  }
+  if (threadIdx.x < NM_MAX_MATERIALS) {
+    const MaterialCoef m = p.mat[threadIdx.x];
+    tb.mat[threadIdx.x] = make_float2(m.za, m.zp);
+    tb.zr[threadIdx.x] = m.zr;
+  }
+  if (threadIdx.x < 12) s_cnt[threadIdx.x] = 0;
+  __syncthreads();
+  uint32_t tables, store;                // volatile: kept, not formed again at every use
+  asm volatile("mov.u32 %0, %1;" : "=r"(tables) : "r"((uint32_t)__cvta_generic_to_shared(s_dyn)));
+  asm volatile("mov.u32 %0, %1;"
+               : "=r"(store)
+               : "r"(tables + (uint32_t)sizeof(RingTables) + (threadIdx.x >> 5) * (uint32_t)sizeof(Store)));
+  const uint32_t tab = tables + offsetof(RingTables, tab), mat = tables + offsetof(RingTables, mat),
+                 zr = tables + offsetof(RingTables, zr);
+  if (threadIdx.x == 0) s_f0 = ring_energy<GENERAL>(p.e0, tab, p.ln_e_lo, p.inv_dln_e);
+  __syncthreads();
+  constexpr int kBorn = 8, kKilled = 9, kDeposit = 10;
+
+  const uint32_t lane = threadIdx.x & 31u;
+  uint32_t lt_mask;                      // volatile: kept, not fetched again at every use
+  asm volatile("mov.u32 %0, %%lanemask_lt;" : "=r"(lt_mask));
+#define RING_AT(word, slot) (store + (uint32_t)offsetof(WarpStore, word) + 16u * (slot))
+#define RING_AT8(word, slot) (store + (uint32_t)offsetof(Store, word) + 8u * (slot))
+  sts1(RING_AT(pos, lane) + 12, 0.0f);   // every slot starts empty
+  sts1(RING_AT(pos, 32 + lane) + 12, 0.0f);
+  __syncwarp();
+
+  // History ids of the launch span less than 2^32: the low word tells the high one.
+  const uint32_t h0 = (uint32_t)p.g.hist_begin, h0_hi = (uint32_t)(p.g.hist_begin >> 32);
+  // warp-uniform state
+  uint32_t head = 0, n_parked = 0;       // ring
+  uint32_t s_next = 0, s_left = 0;       // photons of the site queue
+  uint32_t pool_next = 0, pool_end = 0;  // histories of the launch grabbed and not yet sampled
+  bool drained = false;                  // every history has been handed out
+  uint32_t n_born = 0, n_compton = 0;
+  const bool pairs = p.g.source_mode == NM_SOURCE_DECAY;   // two photons per history
+  // this lane's photon (none while e = 0; photon B while e < 0)
+  float px = 0.f, py = 0.f, pz = 0.f, ux = 0.f, uy = 0.f, uz = 0.f, e = 0.f, rem = 0.f;
+  float s_c = 0.f, s_pe = 0.f, s_r = 0.f, maj = 1.f, maj2 = 1.f;
+  uint32_t hlo = h0, ctr = 0, steps = 0;
+  uint32_t flags = 0;
+  uint32_t n_steps = 0;                  // flight steps of the photons this lane saw end
+  ull deposit = 0;                       // energy of the deposits this lane made
+
+  // The Compton event of a photon of signed energy ce with direction and
+  // history cd, drawn with the flight step's words rk and rp: its deposit dq,
+  // its new direction; returns its new energy, 0 below the cutoff.
+  auto scatter = [&](float ce, float4& cd, uint32_t& cctr, uint32_t rk, uint32_t rp, uint32_t& dq) -> float {
+    const float e1 = fabsf(ce);
+    float x;
+    if (!GENERAL || p.kn_inv) {
+      x = kn_table_x(p, e1, rk);
+    } else {
+      const uint32_t clo = __float_as_uint(cd.w);
+      x = kahn_x(e1 * kInvElectronMassMeV, cctr, ce < 0.0f ? kStreamPhotonB : kStreamPhotonA, clo,
+                 h0_hi + (clo < h0 ? 1u : 0u), p.key, rp, flags);
+    }
+    const float e2 = __fdividef(e1, fmaf(e1 * kInvElectronMassMeV, x, 1.0f));
+    rotate(cd.x, cd.y, cd.z, 1.0f - x, fmaf(kTwoPi, u01(rp), -3.14159265f));
+    const int32_t q1 = q_units(e1);
+    if (e2 < p.cut) {
+      atomicAdd(&s_cnt[kCtrCutoff], 1ull);
+      dq = (uint32_t)q1;
+      deposit += dq;
+      return 0.0f;
+    }
+    dq = (uint32_t)(q1 - q_units(e2));
+    deposit += dq;
+    return copysignf(e2, ce);
+  };
+
+  // ---- Compton pass: the 32 oldest parked photons (all, if fewer), one per
+  // lane; returns the number that fell below the cutoff
+  auto compton_pass = [&]() -> uint32_t {
+    const uint32_t i = (head - n_parked + lane) & (kRing - 1);
+    const float4 cp = lds4(RING_AT(pos, i));
+    uint32_t dq = 0;
+    ull* cell = nullptr;
+    bool gone = false;
+    if (cp.w != 0.0f && lane < n_parked) {
+      float4 cd = lds4(RING_AT(dir, i));
+      const float4 cm = lds4(RING_AT(mid, i));
+      cell = p.g.tally + __float_as_int(cm.z);
+      uint32_t cctr = 0;
+      if constexpr (GENERAL) cctr = __float_as_uint(lds1(RING_AT8(aux, i)));
+      const float ce = scatter(cp.w, cd, cctr, __float_as_uint(cm.x), __float_as_uint(cm.y), dq);
+      sts1(RING_AT(pos, i) + 12, ce);
+      if (ce == 0.0f) {
+        gone = true;
+        if constexpr (GENERAL) n_steps += __float_as_uint(lds1(RING_AT8(gen, i)));
+        else n_steps += __float_as_uint(lds1(RING_AT8(aux, i)));
+      } else {
+        const RingEnergy f = ring_energy<GENERAL>(fabsf(ce), tab, p.ln_e_lo, p.inv_dln_e);
+        const bool cout = cm.w < 0.0f;
+        sts4(RING_AT(dir, i), cd.x, cd.y, cd.z, cd.w);
+        sts4(RING_AT(mid, i), f.s_c, f.s_pe, cout ? f.maj_out : f.maj_in,
+             region_distance(p.g, cout, cp.x, cp.y, cp.z, cd.x, cd.y, cd.z));
+        sts1(RING_AT8(aux, i) + 4, cout ? f.maj_in : f.maj_out);
+        if constexpr (GENERAL) {
+          sts1(RING_AT8(aux, i), __uint_as_float(cctr));
+          sts1(RING_AT8(gen, i) + 4, f.s_r);
+        }
+      }
+    }
+    tally_flush<WARP_AGG>(cell, cell != nullptr, dq, lane);
+    n_parked -= min(n_parked, 32u);
+    const uint32_t n_gone = __popc(__ballot_sync(kFull, gone));
+    __syncwarp();
+    return n_gone;
+  };
+
+  // Takes the ready photon of ring slot i.
+  auto take = [&](uint32_t i) {
+    const float4 np = lds4(RING_AT(pos, i)), nd = lds4(RING_AT(dir, i)), nm = lds4(RING_AT(mid, i));
+    const float2 na = lds2(RING_AT8(aux, i));
+    px = np.x; py = np.y; pz = np.z; e = np.w;
+    ux = nd.x; uy = nd.y; uz = nd.z; hlo = __float_as_uint(nd.w);
+    s_c = nm.x; s_pe = nm.y; maj = nm.z; rem = nm.w;
+    ctr = __float_as_uint(na.x); maj2 = na.y;
+    if constexpr (GENERAL) {
+      const float2 g = lds2(RING_AT8(gen, i));
+      steps = __float_as_uint(g.x);
+      s_r = g.y;
+    }
+  };
+
+  // ---- site queue: 32 new decays, one per lane --------------------------------
+  auto sample_sites = [&]() {
+    const uint32_t avail = pool_end - pool_next;
+    uint32_t fresh = 0, fresh_end = 0;
+    if (avail < 32) {
+      if (lane == 0) {
+        const unsigned f0 = atomicAdd(p.g.work, (unsigned)p.chunk);
+        if ((uint64_t)f0 < p.g.n_hist) {
+          fresh = f0;
+          fresh_end = (uint32_t)min((uint64_t)f0 + (uint64_t)p.chunk, p.g.n_hist);
+        }
+      }
+      fresh = __shfl_sync(kFull, fresh, 0);
+      fresh_end = __shfl_sync(kFull, fresh_end, 0);
+    }
+    uint32_t idx = 0;
+    bool got = true;
+    if (lane < avail) {
+      idx = pool_next + lane;
+    } else if (fresh + (lane - avail) < fresh_end) {
+      idx = fresh + (lane - avail);
+    } else {
+      got = false;
+    }
+    if (avail < 32) {
+      pool_next = min(fresh + (32u - avail), fresh_end);
+      pool_end = fresh_end;
+      drained = fresh_end == 0;
+    } else {
+      pool_next += 32;
+    }
+    bool has = false;
+    ull* cell = nullptr;
+    if (got) {
+      const uint64_t h = p.g.hist_begin + idx;
+      const Site st = sample_site(p.g, p.key, (uint32_t)h, (uint32_t)(h >> 32));
+      const bool o = outside_box(p.g, st.x, st.y, st.z);
+      float ra, rb;
+      region_distance_pair(p.g, o, st.x, st.y, st.z, st.u, st.v_, st.w, ra, rb);
+      sts4(RING_AT(site_pos, lane), st.x, st.y, st.z, __uint_as_float((uint32_t)h));
+      sts4(RING_AT(site_dir, lane), st.u, st.v_, st.w, ra);
+      sts2(RING_AT8(site_rem, lane), rb, o ? -1.0f : 1.0f);
+      if (pairs) {
+        has = p.g.q_positron > 0;
+        cell = p.g.tally + st.v;
+      }
+    }
+    tally_flush<WARP_AGG>(cell, has, (uint32_t)p.g.q_positron, lane);
+    s_next = 0;
+    s_left = (uint32_t)__popc(__ballot_sync(kFull, got)) << (pairs ? 1 : 0);   // lanes 0 .. got - 1
+    n_born += s_left;
+    __syncwarp();
+  };
+
+  // ---- one Woodcock flight step per photon, then the exchanges.  ENDING: the
+  // site queue is empty for good, and lanes without a photon look for one in
+  // the ring, which holds n_ring; returns the new n_ring.  LAST: the ring is
+  // empty for good, and lanes scatter their own photons.
+  auto flight = [&](auto mode, uint32_t n_ring) -> uint32_t {
+    constexpr bool ENDING = decltype(mode)::value == 1, LAST = decltype(mode)::value == 2;
+    const bool fly = e != 0.0f;
+    // words x and y of the step's block; z and w serve the Compton angle if
+    // the step finds a scatter
+    const uint32_t hhi = h0_hi + (hlo < h0 ? 1u : 0u), stream = kStreamPhotonA + (__float_as_uint(e) >> 31);
+    const uint4 rr = draw(ctr, stream, hlo, hhi, p.key);
+    const float imaj = fabsf(maj);
+    float s = -__logf(u01(rr.x)) * imaj;   // cm
+    const bool cross = s >= rem;           // flight cut at the region boundary
+    if (cross) s = rem;
+    rem -= s;
+    px = fmaf(s * p.g.inv_dx, ux, px);
+    py = fmaf(s * p.g.inv_dy, uy, py);
+    pz = fmaf(s * p.g.inv_dz, uz, pz);
+    if (GENERAL) ++steps;
+    // floor once: the same integers test the grid bounds (negative or past
+    // the end, as unsigned) and index the voxel (positions are finite)
+    const int ix = __float2int_rd(px), iy = __float2int_rd(py), iz = __float2int_rd(pz);
+    const bool in_grid = fly && (unsigned)ix < (unsigned)p.g.nx && (unsigned)iy < (unsigned)p.g.ny &&
+                         (unsigned)iz < (unsigned)p.g.nz;
+    const int v = (iz * p.g.ny + iy) * p.g.nx + ix;
+    uint32_t wv = 0;
+    if (in_grid && !cross) wv = __ldg(p.g.vox + v);
+    if (in_grid && cross) {
+      const float t = maj;
+      maj = maj2;
+      maj2 = t;
+      rem = kInf;
+      if (maj > 0.0f) rem = region_distance(p.g, false, px, py, pz, ux, uy, uz);
+    }
+    if (fly && !in_grid) {                 // escapes
+      n_steps += GENERAL ? steps : ctr;
+      e = 0.0f;
+    }
+    const float2 c = lds2(mat + 8u * (wv & 7u));
+    // real event with probability mu(voxel)/mubar; the same uniform picks the type
+    const float scale = __uint_as_float(wv & ~7u) * imaj;   // 0 where no voxel was met
+    const float ic = c.x * s_c;
+    const float icp = fmaf(c.y, s_pe, ic);
+    const float t = u01(rr.y);
+    bool park = t < scale * ic;
+    if constexpr (GENERAL) {
+      if (!(t < scale * icp) && t < scale * fmaf(lds1(zr + 4u * (wv & 7u)), s_r, icp)) {
+        atomicAdd(&s_cnt[kCtrRayleigh], 1ull);
+        // Thomson angular shape (1 + cos^2)/2 by rejection; one block per trial.
+        for (int trial = 0;; ++trial) {
+          const uint4 r = draw(ctr, stream, hlo, hhi, p.key);
+          const float cth = fmaf(2.0f, u01(r.x), -1.0f);
+          const bool acc = 2.0f * u01(r.y) <= fmaf(cth, cth, 1.0f);
+          if (acc || trial + 1 >= kKahnTrialLimit) {
+            if (!acc) flags |= NM_DEV_RAYLEIGH_LIMIT;
+            rotate(ux, uy, uz, cth, fmaf(kTwoPi, u01(r.z), -3.14159265f));
+            rem = region_distance(p.g, maj < 0.0f, px, py, pz, ux, uy, uz);
+            break;
+          }
+        }
+      }
+    }
+    // the rare ends of a photon: absorbed, or stopped by the step limit
+    const bool limit = (GENERAL ? steps : ctr) >= (uint32_t)p.max_steps;
+    const bool photo = !park && t < scale * icp;
+    uint32_t dq = 0;
+    if (photo || limit) {
+      if (photo) {
+        atomicAdd(&s_cnt[kCtrPhoto], 1ull);
+        dq = (uint32_t)q_units(fabsf(e));
+        deposit += dq;
+        n_steps += GENERAL ? steps : ctr;
+        if (!WARP_AGG) atomicAdd(p.g.tally + v, (ull)dq);
+      } else if (e != 0.0f) {
+        atomicAdd(&s_cnt[kCtrKilledUnits], (ull)q_units(fabsf(e)));
+        atomicAdd(&s_cnt[kKilled], 1ull);
+        if (park) atomicAdd(&s_cnt[kCtrCompton], 1ull);
+        flags |= NM_DEV_STEP_LIMIT;
+        n_steps += GENERAL ? steps : ctr;
+      }
+      e = 0.0f;
+      park = false;
+    }
+    if (WARP_AGG) tally_flush<true>(p.g.tally + v, photo, dq, lane);
+    if constexpr (LAST) {
+      n_compton += __popc(__ballot_sync(kFull, park));
+      uint32_t dq2 = 0;
+      if (park) {
+        float4 cd = make_float4(ux, uy, uz, __uint_as_float(hlo));
+        e = scatter(e, cd, ctr, rr.z, rr.w, dq2);
+        ux = cd.x; uy = cd.y; uz = cd.z;
+        if (e == 0.0f) {
+          n_steps += GENERAL ? steps : ctr;
+        } else {
+          const RingEnergy f = ring_energy<GENERAL>(fabsf(e), tab, p.ln_e_lo, p.inv_dln_e);
+          s_c = f.s_c; s_pe = f.s_pe; s_r = f.s_r;
+          const bool o = maj < 0.0f;
+          maj = o ? f.maj_out : f.maj_in;
+          maj2 = o ? f.maj_in : f.maj_out;
+          rem = region_distance(p.g, o, px, py, pz, ux, uy, uz);
+        }
+      }
+      tally_flush<WARP_AGG>(p.g.tally + v, park, dq2, lane);
+      return 0u;
+    }
+    // exchanges: scattered photons, and near the end lanes without one
+    const bool swap = park || (ENDING && n_ring != 0 && e == 0.0f);
+    const unsigned sm = __ballot_sync(kFull, swap);
+    const uint32_t n_swap = __popc(sm), n_park = ENDING ? __popc(__ballot_sync(kFull, park)) : n_swap;
+    if (swap) {
+      const uint32_t i = (head + __popc(sm & lt_mask)) & (kRing - 1);
+      const float4 np = lds4(RING_AT(pos, i)), nd = lds4(RING_AT(dir, i)), nm = lds4(RING_AT(mid, i));
+      const float2 na = lds2(RING_AT8(aux, i));
+      sts4(RING_AT(pos, i), px, py, pz, e);
+      sts4(RING_AT(dir, i), ux, uy, uz, __uint_as_float(hlo));
+      sts4(RING_AT(mid, i), __uint_as_float(rr.z), __uint_as_float(rr.w), __int_as_float(v), maj);
+      sts1(RING_AT8(aux, i), __uint_as_float(ctr));
+      px = np.x; py = np.y; pz = np.z; e = np.w;
+      ux = nd.x; uy = nd.y; uz = nd.z; hlo = __float_as_uint(nd.w);
+      s_c = nm.x; s_pe = nm.y; maj = nm.z; rem = nm.w;
+      ctr = __float_as_uint(na.x); maj2 = na.y;
+      if constexpr (GENERAL) {
+        const float2 g = lds2(RING_AT8(gen, i));
+        sts1(RING_AT8(gen, i), __uint_as_float(steps));
+        steps = __float_as_uint(g.x);
+        s_r = g.y;
+      }
+    }
+    n_compton += n_park;
+    if (ENDING) n_ring += n_park - __popc(__ballot_sync(kFull, swap && e != 0.0f));
+    head += n_swap;
+    n_parked += n_swap;
+    __syncwarp();
+    return n_ring;
+  };
+
+  for (;;) {
+    if (n_parked >= 32) compton_pass();
+    if (s_left == 0) {
+      if (drained) break;
+      sample_sites();
+    }
+    // lanes without a photon take the site queue's next ones
+    const unsigned want = __ballot_sync(kFull, e == 0.0f);
+    const uint32_t rank = __popc(want & lt_mask);
+    if (e == 0.0f && rank < s_left) {
+      const uint32_t k = s_next + rank, j = pairs ? k >> 1 : k;
+      const uint32_t sign = pairs ? k << 31 : 0u;      // photon B (odd) flies opposite to A
+      const float4 sp = lds4(RING_AT(site_pos, j)), sd = lds4(RING_AT(site_dir, j));
+      const float2 sr = lds2(RING_AT8(site_rem, j));
+      px = sp.x; py = sp.y; pz = sp.z;
+      hlo = __float_as_uint(sp.w);
+      ux = __uint_as_float(__float_as_uint(sd.x) ^ sign);
+      uy = __uint_as_float(__float_as_uint(sd.y) ^ sign);
+      uz = __uint_as_float(__float_as_uint(sd.z) ^ sign);
+      rem = sign ? sr.x : sd.w;
+      e = __uint_as_float(__float_as_uint(p.e0) ^ sign);
+      s_c = s_f0.s_c;
+      s_pe = s_f0.s_pe;
+      maj = s_f0.maj_in;
+      maj2 = s_f0.maj_out;
+      if (sr.y < 0.0f) {
+        maj = s_f0.maj_out;
+        maj2 = s_f0.maj_in;
+      }
+      ctr = 0;
+      if (GENERAL) {
+        s_r = s_f0.s_r;
+        steps = 0;
+      }
+    }
+    const uint32_t n_pop = min((uint32_t)__popc(want), s_left);
+    s_next += n_pop;
+    s_left -= n_pop;
+    flight(std::integral_constant<int, 0>(), 0u);
+  }
+  // Every photon has been started: lanes without one take what the ring holds.
+  // Once the lanes can hold all that is left, they keep their photons and
+  // scatter them themselves: the last photons fly without waiting in the ring.
+  uint32_t n_ring = __popc(__ballot_sync(kFull, lds1(RING_AT(pos, lane) + 12) != 0.0f)) +
+                    __popc(__ballot_sync(kFull, lds1(RING_AT(pos, 32 + lane) + 12) != 0.0f));
+  while (n_ring + __popc(__ballot_sync(kFull, e != 0.0f)) > 32) {
+    if (n_parked >= 32) n_ring -= compton_pass();
+    n_ring = flight(std::integral_constant<int, 1>(), n_ring);
+  }
+  while (n_parked) compton_pass();
+  {
+    const unsigned lo = __ballot_sync(kFull, lds1(RING_AT(pos, lane) + 12) != 0.0f),
+                   hi = __ballot_sync(kFull, lds1(RING_AT(pos, 32 + lane) + 12) != 0.0f);
+    const uint32_t rank = __popc(__ballot_sync(kFull, e == 0.0f) & lt_mask), n_lo = __popc(lo);
+    if (e == 0.0f && rank < n_lo + __popc(hi))
+      take(rank < n_lo ? __fns(lo, 0, rank + 1) : 32 + __fns(hi, 0, rank - n_lo + 1));
+  }
+  while (__any_sync(kFull, e != 0.0f)) flight(std::integral_constant<int, 2>(), 0u);
+#undef RING_AT
+#undef RING_AT8
+
+  // ---- counters ---------------------------------------------------------------
+  const ull dep_sum = warp_sum(deposit), step_sum = warp_sum((ull)n_steps);
+  if (lane == 0) {
+    atomicAdd(&s_cnt[kCtrSteps], step_sum);
+    atomicAdd(&s_cnt[kCtrCompton], (ull)n_compton);
+    atomicAdd(&s_cnt[kBorn], (ull)n_born);
+    atomicAdd(&s_cnt[kDeposit], dep_sum);
+  }
+  const unsigned fl = __reduce_or_sync(kFull, flags);
+  if (lane == 0 && fl) atomicOr(p.status, fl);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    // every photon that started was absorbed, cut off, killed or escaped, and
+    // what it did not deposit went with it
+    s_cnt[kCtrEscapes] = s_cnt[kBorn] - s_cnt[kCtrPhoto] - s_cnt[kCtrCutoff] - s_cnt[kKilled];
+    s_cnt[kCtrEscapedUnits] = s_cnt[kBorn] * (ull)(uint32_t)p.q_e0 - s_cnt[kDeposit] - s_cnt[kCtrKilledUnits];
+  }
+  __syncthreads();
+  if (threadIdx.x < 8 && s_cnt[threadIdx.x]) atomicAdd(p.g.counters + threadIdx.x, s_cnt[threadIdx.x]);
+}
+
 // Scattering cosines at energy e as the transport's table sampler draws them
 // (counters 0..n-1 of stream 7, key k0 k1).
 __global__ void check_kn_table_kernel(const TransportParams p, float e, int64_t n, float* out) {
@@ -1000,9 +1427,8 @@ __global__ void check_source_kernel(const TransportParams p, uint64_t first, int
 
 // Dynamic shared memory: the site stash, the history lists when kept, and
 // (nuclide variant) the origin of the gamma lines.
-size_t transport_smem(int block, bool history, bool beta = false, bool siteq = false) {
-  return (((size_t)9 + (history ? 2 * kHistVoxels : 0) + (beta ? 3 : 0)) * block +
-          (siteq ? (size_t)(block / 32) * kQueueCap * kQueueWords : 0)) * sizeof(float);
+size_t transport_smem(int block, bool history, bool beta) {
+  return ((size_t)9 + (history ? 2 * kHistVoxels : 0) + (beta ? 3 : 0)) * block * sizeof(float);
 }
 
 template <bool A, bool R, bool G, bool M, bool H, bool B = false>
@@ -1010,14 +1436,10 @@ void* kernel_ptr() {
   return (void*)transport_kernel<A, R, G, M, H, B>;
 }
 
-template <bool M>
-void* pick_m(bool a, bool r, bool g) {
-  if (a) {
-    if (r) return g ? kernel_ptr<true, true, true, M, false>() : kernel_ptr<true, true, false, M, false>();
-    return g ? kernel_ptr<true, false, true, M, false>() : kernel_ptr<true, false, false, M, false>();
-  }
-  if (r) return g ? kernel_ptr<false, true, true, M, false>() : kernel_ptr<false, true, false, M, false>();
-  return g ? kernel_ptr<false, false, true, M, false>() : kernel_ptr<false, false, false, M, false>();
+template <bool G, bool M>
+void* pick_m(bool a, bool r) {
+  if (a) return r ? kernel_ptr<true, true, G, M, false>() : kernel_ptr<true, false, G, M, false>();
+  return r ? kernel_ptr<false, true, G, M, false>() : kernel_ptr<false, false, G, M, false>();
 }
 
 template <bool H>
@@ -1038,7 +1460,22 @@ void* pick(bool a, bool r, bool g, bool m, bool h, bool beta) {
     if (r) return g ? kernel_ptr<false, true, true, false, true>() : kernel_ptr<false, true, false, false, true>();
     return g ? kernel_ptr<false, false, true, false, true>() : kernel_ptr<false, false, false, false, true>();
   }
-  return m ? pick_m<true>(a, r, g) : pick_m<false>(a, r, g);
+  if (m) return g ? pick_m<true, true>(a, r) : pick_m<false, true>(a, r);
+  return g ? nullptr : pick_m<false, false>(a, r);   // one patient, regrouped: the ring kernel
+}
+
+// The ring kernel runs every single-patient regrouped launch of annihilation
+// photons (or a point source) without history statistics: 1e8 decays on the
+// benchmark phantom take 13.2 ms on it and 30.5 ms on the lane kernel.
+bool use_ring(bool regroup, bool multi, bool history, bool beta) { return regroup && !multi && !history && !beta; }
+
+void* pick_ring(bool a, bool general) {
+  if (a) return general ? (void*)transport_ring_kernel<true, true> : (void*)transport_ring_kernel<true, false>;
+  return general ? (void*)transport_ring_kernel<false, true> : (void*)transport_ring_kernel<false, false>;
+}
+
+size_t ring_smem(int block, bool general) {
+  return sizeof(RingTables) + (size_t)(block / 32) * (general ? sizeof(WarpStoreGeneral) : sizeof(WarpStore));
 }
 
 }  // namespace
@@ -1050,12 +1487,14 @@ bool nuclide_launch(const TransportParams& p) {
 cudaError_t launch_transport(const TransportParams& p, int grid, int block, bool warp_agg,
                              bool rayleigh, bool regroup, cudaStream_t s, bool multi, bool history) {
   const bool beta = !multi && nuclide_launch(p);
-  void* fn = pick(warp_agg, rayleigh, regroup, multi, history, beta);
+  const bool ring = use_ring(regroup, multi, history, beta);
+  const bool general = rayleigh || !p.kn_inv;
+  void* fn = ring ? pick_ring(warp_agg, general) : pick(warp_agg, rayleigh, regroup, multi, history, beta);
   if (!fn) return cudaErrorInvalidValue;
   void* args[] = {(void*)&p};
-  // the history lists and the site queues take the static + dynamic total
-  // past the 48 KB default
-  const size_t smem = transport_smem(block, history, beta, regroup && !multi && !history && !beta);
+  // the history lists and the rings take the static + dynamic total past the
+  // 48 KB default
+  const size_t smem = ring ? ring_smem(block, general) : transport_smem(block, history, beta);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) e = cudaLaunchKernel(fn, dim3(grid), dim3(block), args, smem, s);
   if (e != cudaSuccess) cudaGetLastError();  // a refused launch must not linger as the last error
@@ -1065,8 +1504,9 @@ cudaError_t launch_transport(const TransportParams& p, int grid, int block, bool
 int transport_max_blocks_per_sm(int block, bool warp_agg, bool rayleigh, bool regroup, bool multi, bool history,
                                 bool beta) {
   int n = 0;
-  void* fn = pick(warp_agg, rayleigh, regroup, multi, history, beta);
-  const size_t smem = transport_smem(block, history, beta, regroup && !multi && !history && !beta);
+  const bool ring = use_ring(regroup, multi, history, beta);
+  void* fn = ring ? pick_ring(warp_agg, rayleigh) : pick(warp_agg, rayleigh, regroup, multi, history, beta);
+  const size_t smem = ring ? ring_smem(block, rayleigh) : transport_smem(block, history, beta);
   if (!fn || cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, block, smem) != cudaSuccess) {
     cudaGetLastError();
