@@ -226,16 +226,15 @@ def run_gpu(args):
     value = decays / (ms * 1e-3)
     steps_dec = DECAYS_PER_STEP * args.steps
     transport_ms = c1["transport_ms"] - c0["transport_ms"]
-    n_batches = c1["batches"] - c0["batches"]
-    launch_ms = transport_ms / n_batches
+    # a step's batches share one transport launch
+    launch_ms = transport_ms / args.steps
     dsteps = c1["steps"] - c0["steps"]
     deps = (c1["compton"] - c0["compton"]) + (c1["photo"] - c0["photo"]) + (c1["cutoff"] - c0["cutoff"])
     per_decay = {"flight_steps": dsteps / steps_dec,
                  "interactions": (c1["compton"] - c0["compton"] + c1["photo"] - c0["photo"]) / steps_dec,
                  "positron_deposits": 1.0 if c1["emitted"] - c0["emitted"] > 2 * steps_dec * round(0.511 * 64e6) else 0.0,
                  "escapes": (c1["escapes"] - c0["escapes"]) / steps_dec}
-    roofline = transport_roofline(per_decay, DECAYS_PER_STEP / (n_batches / args.steps), launch_ms, clocks,
-                                  probes)
+    roofline = transport_roofline(per_decay, DECAYS_PER_STEP, launch_ms, clocks, probes)
     dose_map = torch.empty(SHAPE, dtype=torch.float32, device="cuda")
     nmdose.nm_dose_get(d.h, dose_map, None, None)
     d.close()
@@ -284,8 +283,8 @@ def run_gpu(args):
     if rank == 0 and ws == 1 and args.cpu_decays > 0:
         cpu = cpu_baseline(args.cpu_decays)
     if rank == 0:
-        # transport + fold + organ fold per batch
-        launches = 3 * (n_batches // args.steps) * args.steps
+        # transport + fold + organ fold per step
+        launches = 3 * args.steps
         line = {"metric": METRIC, "value": value, "unit": METRIC, "n_gpus": ws, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True,
                 "scaling": "weak", "vs_baseline": None, "dtype": "f32+int64", "data": "synthetic",
@@ -586,7 +585,7 @@ def run_reference(args):
 
 def run_profile(args):
     """One short run of the benchmark workload for ncu: create, then one
-    nm_dose_run of --decays decays in 2 batches (2 transport launches)."""
+    nm_dose_run of --decays decays in 2 batches (one transport launch)."""
     import torch
 
     from paper_2111_11687_gb300 import build, inputs, nmdose

@@ -150,11 +150,9 @@ typedef struct {
   int64_t killed;            /* energy units of photons stopped by max_steps */
   uint64_t steps;            /* flight steps (real + virtual) */
   uint64_t compton, photo, rayleigh, cutoff, escapes;
-  double transport_ms;       /* device time of the transport launches: per run call, from the first
-                                batch's start to the last transport's end (consecutive batches
-                                overlap on two streams, folds between them inside the span) */
-  double fold_ms;            /* device time of the batch folds (a fold waits for SMs while the other
-                                stream's transport holds them: an upper bound) */
+  double transport_ms;       /* device time of the transport launches (nm_dose_run_batch: of the
+                                whole call, shared by decays) */
+  double fold_ms;            /* device time of the batch folds (nm_dose_run) */
   uint32_t device_status;    /* OR of NM_DEV_* flags seen */
   int32_t block_threads, chunk, warp_aggregate, regroup, regroup_lanes, grid_blocks; /* tuning used */
   uint64_t history_splits;   /* history_sigma: histories whose deposits touched more voxels
@@ -193,7 +191,10 @@ nm_status nm_dose_create(nm_dose** out, const nm_grid* grid, const nm_materials*
                          const float* activity, const uint8_t* labels, const nm_options* opts);
 
 /* Simulates n_decays more histories (§2.1-2.2) in opts.batches batches of
- * near-equal size, folding each batch into the statistics.  History ids
+ * near-equal size, folding each batch into the statistics.  Up to 16 batches
+ * share a launch, each with a tally of its own: the first run of more than one
+ * batch adds 8 bytes per voxel and further batch to the handle, up to 16 GiB
+ * (fewer batches share a launch where memory is short).  History ids
  * continue across calls and every history's random numbers depend only on
  * (seed, history id) (Philox4x32-10), so the tally after run(a) + run(b) is
  * bit-identical to run(a + b); the batch uncertainty depends on the split.
@@ -204,10 +205,11 @@ nm_status nm_dose_run(nm_dose* h, uint64_t n_decays, uint64_t seed);
 /* Many patients in one launch (the paper runs one patient at a time; this is
  * the batched form of nm_dose_run).  Runs n_decays[i] more histories on each
  * handle hs[i] (i < n <= 64) with seed `seed`, in the handles' common number
- * of batches: per batch one persistent transport launch whose warps drain
- * per-patient work queues, moving to the next patient when one runs dry, then
- * every patient's fold; all batches are captured into one CUDA graph and
- * launched once on the first handle's stream.  Handles must be distinct and
+ * of batches: one persistent transport launch whose warps drain per-patient
+ * work queues, moving to the next patient when one runs dry, tallies every
+ * batch of every patient by itself (in several launches where the batch
+ * tallies would take more memory than the handles may), then every patient's
+ * fold, on the first handle's stream.  Handles must be distinct and
  * share materials, energies, batches, max_steps and device; grids may differ.
  * Each handle's tally is bit-identical to nm_dose_run(hs[i], n_decays[i],
  * seed).  The launch shape is the first handle's explicit options, else

@@ -315,13 +315,10 @@ struct nm_dose {
   ull* s2h_hi = nullptr;
   ull* counters = nullptr;     // kCtrCount
   unsigned* work = nullptr;
-  // Odd batches of a run go to a second stream with a tally and work counter
-  // of their own, so that a batch's transport starts on the SMs the previous
-  // one releases while its last photons finish (the folds stay in batch order).
-  ull* tb2 = nullptr;
-  unsigned* work2 = nullptr;
-  cudaStream_t side = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  // Batch tallies [slots][V], all zero between runs unless `dirty`: one from
+  // the start, as many as a run can use at once from the first run that does.
+  int slots = 1;
+  bool dirty = false;
   uint32_t* status = nullptr;
   uint32_t* rho_max_bits = nullptr;
   double* org_s1 = nullptr;
@@ -343,20 +340,15 @@ struct nm_dose {
   std::vector<float> minv_out_host;  // ... and of the one outside the tracking box
   float blo[3] = {0, 0, 0}, bhi[3] = {0, 0, 0};  // tracking box, voxel units
   bool tuned = false;             // launch shape chosen by the autotuner
-  double batch_graph_ms = 0;      // device time of graphs launched by nm_dose_run_batch
 
   ~nm_dose() {
     // nothing on the device may still use a buffer that is recycled
     cudaStreamSynchronize(stream);
-    if (side) cudaStreamSynchronize(side);
-    void* ptrs[] = {vox, density, labels, label_bad, alias, tb, tb2, work2, tsum, s2, kn, minv, minv_out, beta_tab, kn_inv, s2h_lo, s2h_hi, counters, work, status,
+    void* ptrs[] = {vox, density, labels, label_bad, alias, tb, tsum, s2, kn, minv, minv_out, beta_tab, kn_inv, s2h_lo, s2h_hi, counters, work, status,
                     rho_max_bits, org_s1, org_s2, organ_count, organ_partial, organ_out,
                     out_dose, out_sigma};
     for (void* p : ptrs) dfree(p);
     for (auto e : ev) cudaEventDestroy(e);
-    if (ev_fork) cudaEventDestroy(ev_fork);
-    if (ev_join) cudaEventDestroy(ev_join);
-    if (side) cudaStreamDestroy(side);
   }
 
   PatientGeom geom(uint64_t first, uint64_t n) const {
@@ -365,6 +357,8 @@ struct nm_dose {
     g.vox = vox;
     g.alias = alias;
     g.tally = tb;
+    g.slot_stride = (uint32_t)V;
+    g.split.slots = 1;
     g.counters = counters;
     g.work = work;
     g.n_active = (uint64_t)n_active;
@@ -796,14 +790,13 @@ nm_status nm_dose_create(nm_dose** out, const nm_grid* g, const nm_materials* mt
   }
 
   if ((e = dalloc(&h->vox, V)) || (e = dalloc(&h->density, V)) || (e = dalloc(&h->tb, V)) ||
-      (e = dalloc(&h->tb2, V)) || (e = dalloc(&h->work2, 1)) ||
       (e = dalloc(&h->tsum, V)) || (e = dalloc(&h->s2, V)) || (e = dalloc(&h->kn, kKnTable)) ||
       (e = dalloc(&h->minv, kKnTable)) || (e = dalloc(&h->minv_out, kKnTable)) ||
       (e = dalloc(&h->counters, kCtrCount)) || (e = dalloc(&h->work, 1)) ||
       (e = dalloc(&h->status, 1)) || (e = dalloc(&h->rho_max_bits, NM_MAX_MATERIALS)) ||
       (e = dalloc(&h->org_s1, kLabelSlots)) || (e = dalloc(&h->org_s2, kLabelSlots)) ||
       (e = dalloc(&h->organ_count, kLabelSlots)) ||
-      (e = dalloc(&h->organ_partial, (size_t)fold_blocks(V) * 2 * kLabelSlots)) ||
+      (e = dalloc(&h->organ_partial, std::max((size_t)finalize_blocks(V) * 2, (size_t)fold_blocks(V) * kMaxSlots) * kLabelSlots)) ||
       (e = dalloc(&h->organ_out, 4 * kLabelSlots)))
     return bail(cuda_fail(e, "device allocation"));
   if (labels && ((e = dalloc(&h->labels, V)) || (e = dalloc(&h->label_bad, 1))))
@@ -907,10 +900,6 @@ nm_status nm_dose_create(nm_dose** out, const nm_grid* g, const nm_materials* mt
   }
 
   e = cudaMemsetAsync(h->tb, 0, V * sizeof(ull), s);
-  if (!e) e = cudaMemsetAsync(h->tb2, 0, V * sizeof(ull), s);
-  if (!e) e = cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking);
-  if (!e) e = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);
-  if (!e) e = cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming);
   if (!e) e = cudaMemsetAsync(h->tsum, 0, V * sizeof(ull), s);
   if (!e) e = cudaMemsetAsync(h->s2, 0, V * sizeof(double), s);
   if (!e) e = cudaMemsetAsync(h->counters, 0, kCtrCount * sizeof(ull), s);
@@ -937,6 +926,63 @@ nm_status nm_dose_create(nm_dose** out, const nm_grid* g, const nm_materials* mt
   return NM_OK;
 }
 
+// Memory of one handle's batch tallies beyond the first, at most.
+static constexpr uint64_t kSlotBytes = 16ull << 30;
+
+// Batch tallies for `want` batches per launch, as far as kSlotBytes and the
+// device's memory go: at least the one the handle was made with.
+static nm_status ensure_slots(nm_dose* h, int want) {
+  const uint64_t each = (uint64_t)h->V * sizeof(ull);
+  // ... below 2^32 voxels in all
+  const int most = (int)std::min<uint64_t>({(uint64_t)kMaxSlots, std::max<uint64_t>(kSlotBytes / each, 1),
+                                            std::max<uint64_t>(((1ull << 32) - 1) / (uint64_t)h->V, 1)});
+  const int launches = (want + most - 1) / most;
+  want = (want + launches - 1) / launches;     // near-equal launches
+  if (want <= h->slots) return NM_OK;
+  ull* tb = nullptr;
+  const cudaError_t e = dalloc(&tb, (size_t)h->V * want);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();                 // one batch per launch then
+    return NM_OK;
+  }
+  if (e) return cuda_fail(e, "batch tallies");
+  if (cudaError_t m = cudaMemsetAsync(tb, 0, each * want, h->stream)) {
+    dfree(tb);
+    return cuda_fail(m, "batch tallies");
+  }
+  NM_CUDA(cudaStreamSynchronize(h->stream), "batch tallies");
+  dfree(h->tb);
+  h->tb = tb;
+  h->slots = want;
+  return NM_OK;
+}
+
+static FoldParams fold_params(const nm_dose* h) {
+  FoldParams fp;
+  memset(&fp, 0, sizeof fp);
+  fp.tb = h->tb; fp.tsum = h->tsum; fp.s2 = h->s2; fp.density = h->density;
+  fp.labels = h->labels; fp.V = h->V; fp.gy_per_unit_vol = h->gy_per_unit_vol();
+  fp.organ_partial = h->organ_partial; fp.org_s1 = h->org_s1; fp.org_s2 = h->org_s2;
+  fp.deposited = h->counters + kCtrDepositedUnits;
+  return fp;
+}
+
+// Batches of n histories in B near-equal batches that one launch takes from
+// batch b0 on: as many as there are tallies and 2^31 histories (the launch's
+// work counter) allow; 1 for a batch above that, which takes several launches,
+// and for batches of a few histories.
+static int launch_batches(uint64_t n, int B, int b0, int slots) {
+  if (n / B < kMinSplit) return 1;
+  uint64_t sum = 0;
+  int k = 0;
+  while (k < slots && b0 + k < B) {
+    sum += n / B + ((uint64_t)(b0 + k) < n % B ? 1 : 0);
+    if (sum > (1ull << 31)) break;
+    ++k;
+  }
+  return std::max(k, 1);
+}
+
 nm_status nm_dose_run(nm_dose* h, uint64_t n, uint64_t seed) {
   NvtxRange range("nm_dose_run");
   if (!h) return fail(NM_ERR_ARG, "handle is NULL");
@@ -950,75 +996,56 @@ nm_status nm_dose_run(nm_dose* h, uint64_t n, uint64_t seed) {
     return fail(NM_ERR_OVERFLOW, "history ids exhausted");
   const int B = (uint64_t)h->opt.batches < n ? h->opt.batches : (int)n;
   cudaStream_t s = h->stream;
-  while ((int)h->ev.size() < 4 * B) {
+  const nm_status es = ensure_slots(h, B);
+  if (es != NM_OK) return es;
+  int groups = 0;
+  for (int b = 0; b < B; b += launch_batches(n, B, b, h->slots)) ++groups;
+  while ((int)h->ev.size() < 3 * groups) {
     cudaEvent_t ev;
     NM_CUDA(cudaEventCreate(&ev), "cudaEventCreate");
     h->ev.push_back(ev);
   }
-  FoldParams fp;
-  fp.tb = h->tb; fp.tsum = h->tsum; fp.s2 = h->s2; fp.density = h->density;
-  fp.labels = h->labels; fp.V = h->V; fp.gy_per_unit_vol = h->gy_per_unit_vol();
-  fp.organ_partial = h->organ_partial; fp.org_s1 = h->org_s1; fp.org_s2 = h->org_s2;
-  fp.deposited = h->counters + kCtrDepositedUnits;
-  // Even batches run on the handle's stream, odd ones on the side stream,
-  // each with its own batch tally and work counter: a batch's transport takes
-  // the SMs the other stream's transport releases while its last photons
-  // finish.  Batch b's fold follows its transport (same stream) and the fold
-  // of batch b - 1 (an event across the streams), so the folds add the
-  // batches in order and every statistic is the one a single stream gives;
-  // batch b + 2 follows the fold of batch b, which zeroed its tally.
-  NM_CUDA(cudaEventRecord(h->ev_fork, s), "cudaEventRecord");
-  NM_CUDA(cudaStreamWaitEvent(h->side, h->ev_fork, 0), "cudaStreamWaitEvent");
-  for (int b = 0; b < B; ++b) {
-    NvtxRange batch_range("batch");
-    const uint64_t nb = n / B + ((uint64_t)b < n % B ? 1 : 0);
-    const bool odd = (b & 1) != 0;
-    cudaStream_t bs = odd ? h->side : s;
-    ull* const tally = odd ? h->tb2 : h->tb;
-    unsigned* const work = odd ? h->work2 : h->work;
-    NM_CUDA(cudaEventRecord(h->ev[4 * b + 0], bs), "cudaEventRecord");
-    // A launch hands out at most 2^31 histories (32-bit work counter).
-    for (uint64_t done = 0; done < nb;) {
-      const uint64_t part = std::min<uint64_t>(nb - done, 1ull << 31);
+  const bool was_dirty = h->dirty;      // a run before this one failed half-way
+  h->dirty = true;
+  // Groups of batches: one launch that tallies each batch in its own slot, then
+  // one fold of the slots in batch order.
+  const uint64_t q = n / B, r = n % B;
+  for (int b0 = 0, g = 0; b0 < B; ++g) {
+    NvtxRange batch_range("batches");
+    const int k = launch_batches(n, B, b0, h->slots);
+    const uint32_t big = (uint32_t)std::min<uint64_t>(r > (uint64_t)b0 ? r - b0 : 0, (uint64_t)k);
+    const uint64_t total = q * k + big;
+    FoldParams fp = fold_params(h);
+    fp.n_slots = k;
+    for (int b = 0; b < k; ++b) fp.set_batch(b, q + ((uint32_t)b < big ? 1 : 0));
+    NM_CUDA(cudaEventRecord(h->ev[3 * g + 0], s), "cudaEventRecord");
+    for (uint64_t done = 0; done < total;) {
+      const uint64_t part = std::min<uint64_t>(total - done, 1ull << 31);
       TransportParams p = h->params(h->id_next + done, part, seed);
-      p.g.tally = tally;
-      p.g.work = work;
+      if (k > 1) p.g.split = batch_split((uint32_t)k, big, (uint32_t)q);
       p.chunk = launch_chunk(h, part);
-      NM_CUDA(cudaMemsetAsync(work, 0, sizeof(unsigned), bs), "cudaMemsetAsync");
-      NM_CUDA(launch_transport(p, h->grid, h->block, h->warp_agg, h->rayleigh, h->regroup, bs, false,
+      NM_CUDA(cudaMemsetAsync(h->work, 0, sizeof(unsigned), s), "cudaMemsetAsync");
+      NM_CUDA(launch_transport(p, h->grid, h->block, h->warp_agg, h->rayleigh, h->regroup, s, false,
                                h->opt.history_sigma != 0),
               "transport launch");
       done += part;
     }
-    NM_CUDA(cudaEventRecord(h->ev[4 * b + 1], bs), "cudaEventRecord");
-    if (b > 0) NM_CUDA(cudaStreamWaitEvent(bs, h->ev[4 * (b - 1) + 3], 0), "cudaStreamWaitEvent");
-    fp.n_b = (double)nb;
-    fp.tb = tally;
-    NM_CUDA(cudaEventRecord(h->ev[4 * b + 2], bs), "cudaEventRecord");
-    NM_CUDA(launch_fold(fp, bs), "fold launch");
-    NM_CUDA(cudaEventRecord(h->ev[4 * b + 3], bs), "cudaEventRecord");
-    h->hist_next += nb;
-    h->id_next += nb;
-    h->n_batches += 1;
+    NM_CUDA(cudaEventRecord(h->ev[3 * g + 1], s), "cudaEventRecord");
+    NM_CUDA(launch_fold(fp, s), "fold launch");
+    NM_CUDA(cudaEventRecord(h->ev[3 * g + 2], s), "cudaEventRecord");
+    h->hist_next += total;
+    h->id_next += total;
+    h->n_batches += (uint64_t)k;
+    b0 += k;
   }
-  // the handle's stream continues after the side stream's last work
-  NM_CUDA(cudaEventRecord(h->ev_join, h->side), "cudaEventRecord");
-  NM_CUDA(cudaStreamWaitEvent(s, h->ev_join, 0), "cudaStreamWaitEvent");
   uint32_t st = 0;
   NM_CUDA(cudaMemcpyAsync(&st, h->status, 4, cudaMemcpyDeviceToHost, s), "status read");
   NM_CUDA(cudaStreamSynchronize(s), "nm_dose_run");
-  // transport time of the run: from the first batch's start to the last
-  // transport's end (the batches overlap on two streams; folds that run in
-  // between are inside the span)
-  float span = 0;
-  for (int b = 0; b < B; ++b) {
+  h->dirty = was_dirty;
+  for (int g = 0; g < groups; ++g) {
     float ms = 0;
-    if (cudaEventElapsedTime(&ms, h->ev[0], h->ev[4 * b + 1]) == cudaSuccess) span = std::max(span, ms);
-  }
-  h->transport_ms += span;
-  for (int b = 0; b < B; ++b) {
-    float ms = 0;
-    if (cudaEventElapsedTime(&ms, h->ev[4 * b + 2], h->ev[4 * b + 3]) == cudaSuccess) h->fold_ms += ms;
+    if (cudaEventElapsedTime(&ms, h->ev[3 * g], h->ev[3 * g + 1]) == cudaSuccess) h->transport_ms += ms;
+    if (cudaEventElapsedTime(&ms, h->ev[3 * g + 1], h->ev[3 * g + 2]) == cudaSuccess) h->fold_ms += ms;
   }
   h->status_seen |= st;
   if (st) {
@@ -1032,10 +1059,10 @@ nm_status nm_dose_run(nm_dose* h, uint64_t n, uint64_t seed) {
 }
 
 // ---------------------------------------------------------------------------
-// Many patients in one graph: per batch, one persistent multi-patient transport
-// launch in which every warp drains per-patient work queues (moving on to the
-// next patient when one runs dry), then each patient's fold.  The B batches
-// are captured into a CUDA graph once per call and launched as one graph.
+// Many patients in one launch: one persistent multi-patient transport launch in
+// which every warp drains per-patient work queues (moving on to the next
+// patient when one runs dry), every batch of every patient with a tally of its
+// own, then each patient's fold.
 // ---------------------------------------------------------------------------
 static bool same_physics(const nm_dose* a, const nm_dose* b) {
   if (a->n_mat != b->n_mat || a->rayleigh != b->rayleigh || a->e0 != b->e0 || a->cut != b->cut ||
@@ -1093,38 +1120,60 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
     minv[k] = m;
     minv[kKnTable + k] = mo;
   }
-  // Temporary device memory: per-batch patient tables, majorant, status.
-  PatientGeom* d_pat = nullptr;
-  float* d_minv = nullptr;
-  uint32_t* d_status = nullptr;
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
+  // Batches per launch: what every patient's batch tallies and 2^31 histories
+  // of each (its work counter) allow.
+  int slots = kMaxSlots;
+  for (int i = 0; i < n; ++i) {
+    const nm_status es = ensure_slots(hs[i], B);
+    if (es != NM_OK) return es;
+    slots = std::min(slots, hs[i]->slots);
+  }
+  auto batches_at = [&](int b0) {
+    int k = B;
+    for (int i = 0; i < n; ++i)
+      if (n_decays[i]) k = std::min(k, launch_batches(n_decays[i], B, b0, slots));
+    return k;
+  };
+  int groups = 0;
+  for (int b0 = 0; b0 < B; b0 += batches_at(b0)) ++groups;
+  // Temporary device memory: the launches' patient tables, then the majorants,
+  // the work counters and the status word.
+  const size_t pat_bytes = (size_t)std::max(groups, 1) * n * sizeof(PatientGeom);
+  const size_t tmp_bytes = pat_bytes + 2 * kKnTable * sizeof(float) + (kMaxBatchPatients + 1) * sizeof(uint32_t);
+  static_assert(sizeof(PatientGeom) % 8 == 0, "what follows the patient tables stays aligned");
+  uint8_t* tmp = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
-  nm_status st = NM_OK;
+  cudaError_t e;
   auto cleanup = [&]() {
-    if (exec) cudaGraphExecDestroy(exec);
-    if (graph) cudaGraphDestroy(graph);
+    cudaStreamSynchronize(s);           // nothing on the device may still use the buffer
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
-    if (d_pat) cudaFree(d_pat);
-    if (d_minv) cudaFree(d_minv);
-    if (d_status) cudaFree(d_status);
+    dfree(tmp);
   };
-  cudaError_t e;
-  std::vector<PatientGeom> pat((size_t)B * n);
+  std::vector<PatientGeom> pat((size_t)groups * n);
+  if ((e = dalloc(&tmp, tmp_bytes))) return cuda_fail(e, "nm_dose_run_batch: set-up");
+  PatientGeom* const d_pat = (PatientGeom*)tmp;
+  float* const d_minv = (float*)(tmp + pat_bytes);
+  unsigned* const d_work = (unsigned*)(d_minv + 2 * kKnTable);
+  uint32_t* const d_status = d_work + kMaxBatchPatients;
   std::vector<uint64_t> off(n, 0);
-  for (int b = 0; b < B; ++b)
+  for (int b0 = 0, g = 0; b0 < B; ++g) {
+    const int k = batches_at(b0);
     for (int i = 0; i < n; ++i) {
-      const uint64_t nb = n_decays[i] / B + ((uint64_t)b < n_decays[i] % B ? 1 : 0);
-      pat[(size_t)b * n + i] = hs[i]->geom(hs[i]->id_next + off[i], nb);
-      off[i] += nb;
-      if (nb >= (1ull << 31)) { cleanup(); return fail(NM_ERR_ARG, "handle %d: batches above 2^31 histories", i); }
+      const uint64_t q = n_decays[i] / B, r = n_decays[i] % B;
+      const uint64_t big = std::min<uint64_t>(r > (uint64_t)b0 ? r - b0 : 0, (uint64_t)k), total = q * k + big;
+      if (k == 1 && total >= (1ull << 31)) { cleanup(); return fail(NM_ERR_ARG, "handle %d: batches above 2^31 histories", i); }
+      PatientGeom& G = pat[(size_t)g * n + i];
+      G = hs[i]->geom(hs[i]->id_next + off[i], total);
+      if (k > 1) G.split = batch_split((uint32_t)k, (uint32_t)big, (uint32_t)q);
+      G.work = d_work + i;
+      off[i] += total;
     }
-  if ((e = cudaMalloc(&d_pat, pat.size() * sizeof(PatientGeom))) ||
-      (e = cudaMalloc(&d_minv, 2 * kKnTable * sizeof(float))) || (e = cudaMalloc(&d_status, 4)) ||
-      (e = cudaMemcpyAsync(d_pat, pat.data(), pat.size() * sizeof(PatientGeom), cudaMemcpyHostToDevice, s)) ||
-      (e = cudaMemcpyAsync(d_minv, minv.data(), 2 * kKnTable * sizeof(float), cudaMemcpyHostToDevice, s)) ||
-      (e = cudaMemsetAsync(d_status, 0, 4, s)) || (e = cudaStreamSynchronize(s))) {
+    b0 += k;
+  }
+  if ((e = cudaMemcpyAsync(d_minv, minv.data(), 2 * kKnTable * sizeof(float), cudaMemcpyHostToDevice, s)) ||
+      (e = cudaMemsetAsync(d_status, 0, 4, s)) || (e = cudaStreamSynchronize(s)) || (e = cudaEventCreate(&e0)) ||
+      (e = cudaEventCreate(&e1))) {
     cleanup();
     return cuda_fail(e, "nm_dose_run_batch: set-up");
   }
@@ -1147,9 +1196,11 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
   const bool free_shape = h0->opt.block_threads <= 0 || h0->opt.chunk <= 0 || h0->opt.regroup < 0;
   if (!have && free_shape) {
     // Trials on history ids above 2^62 of every patient, then cleared.
-    if ((e = cudaEventCreate(&e0)) || (e = cudaEventCreate(&e1))) { cleanup(); return cuda_fail(e, "events"); }
     std::vector<PatientGeom> tp(n);
-    for (int i = 0; i < n; ++i) tp[i] = hs[i]->geom(1ull << 62, (1ull << 22) / n + 1);
+    for (int i = 0; i < n; ++i) {
+      tp[i] = hs[i]->geom(1ull << 62, (1ull << 22) / n + 1);
+      tp[i].work = d_work + i;
+    }
     if ((e = cudaMemcpy(d_pat, tp.data(), n * sizeof(PatientGeom), cudaMemcpyHostToDevice))) {
       cleanup();
       return cuda_fail(e, "batch autotune");
@@ -1172,7 +1223,7 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
         p.patients = d_pat;
         p.chunk = c.chunk;
         p.regroup_compton = p.regroup_refill = c.lanes;
-        for (int i = 0; i < n; ++i) cudaMemsetAsync(hs[i]->work, 0, 4, s);
+        cudaMemsetAsync(d_work, 0, n * sizeof(unsigned), s);
         float ms = 0;
         if ((e = cudaEventRecord(e0, s)) ||
             (e = launch_transport(p, grid, c.block, c.warp_agg, h0->rayleigh, c.regroup, s, true)) ||
@@ -1190,12 +1241,8 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
                                   cudaMemcpyHostToDevice, s);
     }
     if (!e) e = cudaMemsetAsync(d_status, 0, 4, s);
+    if (!e) e = cudaStreamSynchronize(s);
     if (e) { cleanup(); return cuda_fail(e, "batch autotune"); }
-    if ((e = cudaMemcpyAsync(d_pat, pat.data(), pat.size() * sizeof(PatientGeom), cudaMemcpyHostToDevice, s)) ||
-        (e = cudaStreamSynchronize(s))) {
-      cleanup();
-      return cuda_fail(e, "batch autotune");
-    }
     std::lock_guard<std::mutex> lock(g_tune_mu);
     g_batch_tune[key] = sh;
   }
@@ -1203,64 +1250,50 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
   if (grid <= 0) { cleanup(); return fail(NM_ERR_ARG, "multi-patient kernel cannot launch"); }
   p.chunk = sh.chunk;
   p.regroup_compton = p.regroup_refill = sh.lanes;
-
-  // Capture: B x (reset queues, one transport launch over all patients, folds),
-  // on a private stream (the legacy default stream cannot be captured), after
-  // the handles' stream has drained.
-  cudaStream_t cs = nullptr;
-  if ((e = cudaStreamSynchronize(s)) || (e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking))) {
-    cleanup();
-    return cuda_fail(e, "capture stream");
+  std::vector<char> was_dirty(n);
+  for (int i = 0; i < n; ++i) {
+    was_dirty[i] = hs[i]->dirty;
+    hs[i]->dirty = true;
   }
-  auto cleanup_stream = [&]() { if (cs) cudaStreamDestroy(cs); cs = nullptr; };
-  if ((e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal))) {
-    cleanup_stream();
-    cleanup();
-    return cuda_fail(e, "stream capture");
-  }
-  for (int b = 0; b < B && !e; ++b) {
-    for (int i = 0; i < n && !e; ++i) e = cudaMemsetAsync(hs[i]->work, 0, sizeof(unsigned), cs);
-    p.patients = d_pat + (size_t)b * n;
-    if (!e) e = launch_transport(p, grid, sh.block, sh.warp_agg, h0->rayleigh, sh.regroup, cs, true);
+  if (!(e = cudaMemcpyAsync(d_pat, pat.data(), pat.size() * sizeof(PatientGeom), cudaMemcpyHostToDevice, s)))
+    e = cudaEventRecord(e0, s);
+  for (int b0 = 0, g = 0; b0 < B && !e; ++g) {
+    const int k = batches_at(b0);
+    p.patients = d_pat + (size_t)g * n;
+    e = cudaMemsetAsync(d_work, 0, n * sizeof(unsigned), s);
+    if (!e) e = launch_transport(p, grid, sh.block, sh.warp_agg, h0->rayleigh, sh.regroup, s, true);
     for (int i = 0; i < n && !e; ++i) {
-      const uint64_t nb = pat[(size_t)b * n + i].n_hist;
-      if (nb == 0) continue;
-      nm_dose* h = hs[i];
-      FoldParams fp;
-      fp.tb = h->tb; fp.tsum = h->tsum; fp.s2 = h->s2; fp.density = h->density;
-      fp.labels = h->labels; fp.V = h->V; fp.gy_per_unit_vol = h->gy_per_unit_vol();
-      fp.organ_partial = h->organ_partial; fp.org_s1 = h->org_s1; fp.org_s2 = h->org_s2;
-      fp.deposited = h->counters + kCtrDepositedUnits;
-      fp.n_b = (double)nb;
-      e = launch_fold(fp, cs);
+      const uint64_t q = n_decays[i] / B, r = n_decays[i] % B;
+      if (pat[(size_t)g * n + i].n_hist == 0) continue;
+      FoldParams fp = fold_params(hs[i]);
+      fp.n_slots = k;
+      for (int b = 0; b < k; ++b) fp.set_batch(b, q + ((uint64_t)(b0 + b) < r ? 1 : 0));
+      e = launch_fold(fp, s);
     }
+    b0 += k;
   }
-  cudaError_t ec = cudaStreamEndCapture(cs, &graph);
-  if (e || ec) { cleanup_stream(); cleanup(); return cuda_fail(e ? e : ec, "stream capture"); }
-  if ((e = cudaGraphInstantiate(&exec, graph, 0))) { cleanup_stream(); cleanup(); return cuda_fail(e, "graph instantiate"); }
-  if (!e0 && ((e = cudaEventCreate(&e0)) || (e = cudaEventCreate(&e1)))) { cleanup_stream(); cleanup(); return cuda_fail(e, "events"); }
   float ms = 0;
   uint32_t flags = 0;
-  if ((e = cudaEventRecord(e0, cs)) || (e = cudaGraphLaunch(exec, cs)) || (e = cudaEventRecord(e1, cs)) ||
-      (e = cudaMemcpyAsync(&flags, d_status, 4, cudaMemcpyDeviceToHost, cs)) ||
-      (e = cudaStreamSynchronize(cs)) || (e = cudaEventElapsedTime(&ms, e0, e1))) {
-    cleanup_stream();
+  if (!e) e = cudaEventRecord(e1, s);
+  if (!e) e = cudaMemcpyAsync(&flags, d_status, 4, cudaMemcpyDeviceToHost, s);
+  if (!e) e = cudaStreamSynchronize(s);
+  if (!e) e = cudaEventElapsedTime(&ms, e0, e1);
+  if (e) {
     cleanup();
-    return cuda_fail(e, "graph launch");
+    return cuda_fail(e, "nm_dose_run_batch");
   }
-  cleanup_stream();
+  for (int i = 0; i < n; ++i) hs[i]->dirty = was_dirty[i];
   for (int i = 0; i < n; ++i) {
     if (n_decays[i] == 0) continue;
     hs[i]->hist_next += n_decays[i];
     hs[i]->id_next += n_decays[i];
     hs[i]->n_batches += (uint64_t)std::min<uint64_t>(B, n_decays[i]);
-    hs[i]->transport_ms += ms * (double)n_decays[i] / (double)total;  // graph time, shared by decays
+    hs[i]->transport_ms += ms * (double)n_decays[i] / (double)total;  // the call's device time, shared by decays
     hs[i]->status_seen |= flags;
   }
-  h0->batch_graph_ms += ms;
   cleanup();
   if (flags) return fail(NM_ERR_DEVICE, "device check fired (flags 0x%x)", flags);
-  return st;
+  return NM_OK;
 }
 
 static nm_status finalize(nm_dose* h, float* dose, float* sigma) {
@@ -1590,9 +1623,9 @@ nm_status nm_dose_restore(nm_dose* h, const void* buf, uint64_t bytes) {
     NM_CUDA(cudaMemcpyAsync(h->s2h_lo, b + o.lo, V8, cudaMemcpyDefault, s), "restore");
     NM_CUDA(cudaMemcpyAsync(h->s2h_hi, b + o.hi, V8, cudaMemcpyDefault, s), "restore");
   }
-  NM_CUDA(cudaMemsetAsync(h->tb, 0, V8, s), "restore");
-  NM_CUDA(cudaMemsetAsync(h->tb2, 0, V8, s), "restore");
+  if (h->dirty) NM_CUDA(cudaMemsetAsync(h->tb, 0, V8 * h->slots, s), "restore");
   NM_CUDA(cudaStreamSynchronize(s), "nm_dose_restore");
+  h->dirty = false;
   h->hist_next = hd.hist_next;
   h->id_next = hd.id_next;
   h->n_batches = hd.n_batches;
@@ -1680,8 +1713,7 @@ nm_status nm_dose_counters(nm_dose* h, nm_counters* c) {
 nm_status nm_dose_reset(nm_dose* h) {
   if (!h) return fail(NM_ERR_ARG, "handle is NULL");
   cudaStream_t s = h->stream;
-  NM_CUDA(cudaMemsetAsync(h->tb, 0, h->V * sizeof(ull), s), "reset");
-  NM_CUDA(cudaMemsetAsync(h->tb2, 0, h->V * sizeof(ull), s), "reset");
+  if (h->dirty) NM_CUDA(cudaMemsetAsync(h->tb, 0, h->V * h->slots * sizeof(ull), s), "reset");
   NM_CUDA(cudaMemsetAsync(h->tsum, 0, h->V * sizeof(ull), s), "reset");
   NM_CUDA(cudaMemsetAsync(h->s2, 0, h->V * sizeof(double), s), "reset");
   NM_CUDA(cudaMemsetAsync(h->counters, 0, kCtrCount * sizeof(ull), s), "reset");
@@ -1692,6 +1724,7 @@ nm_status nm_dose_reset(nm_dose* h) {
     NM_CUDA(cudaMemsetAsync(h->s2h_hi, 0, h->V * sizeof(ull), s), "reset");
   }
   NM_CUDA(cudaStreamSynchronize(s), "reset");
+  h->dirty = false;
   h->hist_next = 0;
   h->id_next = 0;
   h->n_batches = 0;

@@ -20,7 +20,8 @@ constexpr double kJoulePerEv = 1.602176634e-19;
 constexpr float kTwoPi = 6.283185307179586f;
 constexpr int kKnTable = 1024;      // log-energy nodes of the Klein-Nishina table
 constexpr int kFoldThreads = 128;   // fold / finalize CTA size
-constexpr int kFoldTile = 8192;     // voxels per fold CTA
+constexpr int kFoldTile = 2048;     // voxels a fold CTA takes at a time
+constexpr int kFinalTile = 8192;    // voxels per finalize CTA
 constexpr int kLabelSlots = NM_MAX_LABELS + 1;
 
 // Fixed-point energy: round-to-nearest-even of the FP32 product E * 6.4e7.
@@ -93,11 +94,35 @@ struct MaterialCoef {
   float rho_max;  // largest density of this material in the grid (host side)
 };
 
+// Batches of one launch, each with a tally of its own (a slot): the first `big`
+// hold q + 1 histories of the launch, the others q.  est = 2^32 / (q + 1), so
+// that the high word of idx * est is the batch of history idx or, from q =
+// kMinSplit on and up to 2^31 histories, the one before (the estimate is short
+// by less than 1/2 + slots / q).
+struct BatchSplit {
+  uint32_t slots;             // batches of the launch; at most 1: no split
+  uint32_t big, q, est;
+  __host__ __device__ uint32_t start(uint32_t b) const { return b * q + (b < big ? b : big); }
+};
+constexpr uint32_t kMinSplit = 64;
+inline BatchSplit batch_split(uint32_t slots, uint32_t big, uint32_t q) {
+  return BatchSplit{slots, big, q, (uint32_t)(((uint64_t)1 << 32) / (q + 1))};
+}
+// Slot of history idx of the launch (split.slots > 1).
+__host__ __device__ __forceinline__ uint32_t batch_of(const BatchSplit& s, uint32_t idx) {
+  uint32_t b = (uint32_t)((ull)idx * s.est >> 32);
+  if (b + 1 < s.slots && idx >= s.start(b + 1)) ++b;
+  return b;
+}
+constexpr int kMaxSlots = 16;      // batches of one launch
+
 // Per-patient (per-grid) part of a transport launch.
 struct PatientGeom {
   const uint32_t* vox;        // packed voxel: density bits with the low 3 bits = material
   const uint4* alias;         // {prob bits, voxel, alias voxel, 0}
-  ull* tally;                 // batch tally, units
+  ull* tally;                 // batch tallies, units: slot b at tally + b slot_stride
+  uint32_t slot_stride;       // voxels
+  BatchSplit split;
   ull* counters;              // device counters (see CounterSlot)
   unsigned* work;             // histories handed out in this launch (< 2^32 per launch)
   uint64_t n_active;
@@ -237,22 +262,29 @@ struct AliasScratch {
 cudaError_t build_alias_table(const float* activity, int64_t V, AliasScratch scratch, uint4* table,
                               int64_t* n_active_host, uint32_t* status, cudaStream_t s);
 
-// Batch fold (per batch) and finalize.
+// Fold of a launch's batches, and finalize.
 struct FoldParams {
-  ull* tb;                  // batch tally, zeroed by the fold
+  ull* tb;                  // batch tallies, zeroed by the fold: slot b at tb + b V
+  int n_slots;              // 1 .. kMaxSlots
   ull* tsum;                // cumulative tally
   double* s2;               // sum over batches of T_b^2 / n_b
   const float* density;
   const uint8_t* labels;    // may be NULL
   int64_t V;
-  double n_b;               // histories in this batch
+  double n_b[kMaxSlots];    // histories in each batch; 0: none, the slot is empty
+  double inv_nb[kMaxSlots];
   double gy_per_unit_vol;   // J per unit / (1e-3 kg/g * voxel volume cm^3)
-  double* organ_partial;    // [blocks][kLabelSlots]
+  double* organ_partial;    // [n_slots][fold_blocks(V)][kLabelSlots]
   double* org_s1;           // [kLabelSlots] sum_b O_b
   double* org_s2;           // [kLabelSlots] sum_b O_b^2 / n_b
   ull* deposited;           // counter
+  void set_batch(int b, uint64_t n) {
+    n_b[b] = (double)n;
+    inv_nb[b] = n ? 1.0 / (double)n : 0.0;
+  }
 };
 int fold_blocks(int64_t V);
+int finalize_blocks(int64_t V);
 cudaError_t launch_fold(const FoldParams& p, cudaStream_t s);
 
 // Adds another shard's statistics (o_*) into a handle's (all device arrays;

@@ -1,6 +1,6 @@
 // Tally statistics (§2.1 dose and uncertainty maps, Eq. 1-3).
 //
-// Per batch b of n_b histories the fold moves the int64 batch tally T_b into
+// For each batch b of n_b histories the fold moves the int64 batch tally T_b into
 // the exact cumulative tally and accumulates, in FP64, S2 = sum_b T_b^2 / n_b
 // per voxel and the organ sums O_b = sum over the organ's voxels of the batch
 // dose.  With N = sum n_b histories and K batches the per-decay mean of a
@@ -9,6 +9,8 @@
 // the n_b-weighted form of the batch-means estimator.  Every reduction has a
 // fixed tree (per-thread columns in shared memory, then fixed warp trees, then
 // blocks in index order), so the statistics are the same on every run.
+#include <algorithm>
+
 #include "nm_internal.cuh"
 
 namespace nm {
@@ -33,80 +35,173 @@ __device__ void reduce_label_columns(const double (*acc)[kFoldThreads], double* 
   }
 }
 
-__global__ void __launch_bounds__(kFoldThreads) fold_kernel(const FoldParams p) {
-  __shared__ double acc[kLabelSlots][kFoldThreads];
+// Fold of a launch's NS (or fewer) batches in one pass over the voxels: per
+// voxel the slots' tallies are read together and added in batch order, so the
+// cumulative tally and S2 are read and written once for all of them, and they
+// are the bits of a fold per batch.
+//
+// Bound by DRAM (8 B per slot and voxel read; written, with the 37 B of
+// statistics, only where something was deposited) and, in densely hit volumes,
+// by FP64 (four operations per deposit-holding voxel and slot; this GPU does
+// about two per SM and clock).  A thread therefore loads NS x K tallies before
+// it uses any, and lone voxels of other batches cost nothing.
+//
+// Organ sums: a tile holds few labels, so each thread keeps a column of FP64
+// sums for kAccLabels of them per slot in shared memory; tiles with more labels
+// are read again for the next ones.  Columns are added in a fixed order.
+constexpr int kAccLabels = 4;
+
+template <int NS, bool LABELS>
+__global__ void __launch_bounds__(kFoldThreads) fold_kernel(const FoldParams p, int tiles_per_block) {
+  constexpr int K = NS <= 2 ? 8 : 4;       // voxels of a thread in flight
+  constexpr int kPer = kFoldTile / kFoldThreads;          // voxels of a thread per tile
+  extern __shared__ double acc[];                         // [NS][kAccLabels][kFoldThreads]
+  __shared__ double out[LABELS ? NS : 1][kLabelSlots];
+  __shared__ uint32_t s_mask[kFoldThreads / 32];
   __shared__ ull dep_w[kFoldThreads / 32];
-  for (int l = 0; l < kLabelSlots; ++l) acc[l][threadIdx.x] = 0.0;
-  const int64_t v0 = (int64_t)blockIdx.x * kFoldTile;
-  const int64_t v1 = v0 + kFoldTile < p.V ? v0 + kFoldTile : p.V;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (LABELS)
+    for (int i = tid; i < NS * kLabelSlots; i += kFoldThreads) out[i / kLabelSlots][i % kLabelSlots] = 0.0;
   ull dep = 0;
-  const double inv_nb = 1.0 / p.n_b;
-  // A thread's voxels v0 + tid + k kFoldThreads, kFold at a time: all their
-  // loads are issued before any update (a lone load per voxel left the kernel
-  // bound by DRAM latency), and the updates then follow in voxel order, so
-  // every sum is formed exactly as one voxel at a time would.
-  constexpr int kFold = 8;
-  for (int64_t vb = v0 + threadIdx.x; vb < v1; vb += (int64_t)kFold * kFoldThreads) {
-    ull t[kFold], ts[kFold];
-    double s2v[kFold];
-    float rho[kFold];
-    int lab[kFold];
+  const float gy = (float)p.gy_per_unit_vol;
+  const int64_t first = (int64_t)blockIdx.x * tiles_per_block * kFoldTile;
+  for (int ti = 0; ti < tiles_per_block; ++ti) {
+    const int64_t v0 = first + (int64_t)ti * kFoldTile;
+    if (v0 >= p.V) break;
+    const int64_t v1 = v0 + kFoldTile < p.V ? v0 + kFoldTile : p.V;
+    // labels of this thread's voxels v0 + tid + i kFoldThreads, and of the tile
+    uint32_t lab[kPer / 4] = {};
+    uint32_t mask = 0;
+    if (LABELS) {
 #pragma unroll
-    for (int j = 0; j < kFold; ++j) {
-      const int64_t v = vb + (int64_t)j * kFoldThreads;
-      t[j] = v < v1 ? p.tb[v] : 0ull;
+      for (int i = 0; i < kPer; ++i) {
+        const int64_t v = v0 + tid + (int64_t)i * kFoldThreads;
+        const uint32_t l = v < v1 ? p.labels[v] : 0u;
+        lab[i / 4] |= l << (8 * (i % 4));
+        mask |= 1u << l;
+      }
+      mask = __reduce_or_sync(0xffffffffu, mask);
+      if (lane == 0) s_mask[wid] = mask;
+      __syncthreads();
+      mask = s_mask[0] | s_mask[1] | s_mask[2] | s_mask[3];
     }
+    const int n_lab = LABELS ? __popc(mask) : 1;
+    for (int l0 = 0; l0 < n_lab; l0 += kAccLabels) {
+      const int n_acc = min(kAccLabels, n_lab - l0);
+      const bool last = l0 + kAccLabels >= n_lab;
+      if (LABELS)
+        for (int i = 0; i < p.n_slots; ++i)
+          for (int l = 0; l < n_acc; ++l) acc[(i * kAccLabels + l) * kFoldThreads + tid] = 0.0;
+#pragma unroll 1
+      for (int c = 0; c < kPer; c += K) {
+        ull t[NS][K];
+        ull any[K];
 #pragma unroll
-    for (int j = 0; j < kFold; ++j) {
-      const int64_t v = vb + (int64_t)j * kFoldThreads;
-      ts[j] = 0; s2v[j] = 0.0; rho[j] = 1.0f; lab[j] = 0;
-      if (t[j]) {
-        ts[j] = p.tsum[v];
-        s2v[j] = p.s2[v];
-        if (p.labels) {
-          lab[j] = p.labels[v];
-          rho[j] = p.density[v];
+        for (int b = 0; b < NS; ++b)
+#pragma unroll
+          for (int j = 0; j < K; ++j) {
+            const int64_t v = v0 + tid + (int64_t)(c + j) * kFoldThreads;
+            t[b][j] = b < p.n_slots && v < v1 ? p.tb[(int64_t)b * p.V + v] : 0ull;
+          }
+        ull ts[K];
+        double s2v[K];
+        float rho[K];
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+          any[j] = 0;
+#pragma unroll
+          for (int b = 0; b < NS; ++b) any[j] |= t[b][j];
+          ts[j] = 0; s2v[j] = 0.0; rho[j] = 1.0f;
+          if (any[j]) {
+            const int64_t v = v0 + tid + (int64_t)(c + j) * kFoldThreads;
+            if (l0 == 0) {
+              ts[j] = p.tsum[v];
+              s2v[j] = p.s2[v];
+            }
+            if (LABELS) rho[j] = p.density[v];
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+          if (!any[j]) continue;
+          const int64_t v = v0 + tid + (int64_t)(c + j) * kFoldThreads;
+          // Gy per unit in FP32 (GB300's FP64 divide is slow); the sum stays FP64
+          const double g = LABELS ? (double)__fdiv_rn(gy, rho[j]) : 0.0;
+          int la = -1;                                    // the voxel's column, if one of this pass
+          if (LABELS) {
+            const uint32_t l = (lab[(c + j) / 4] >> (8 * ((c + j) % 4))) & 255u;
+            la = __popc(mask & ((1u << l) - 1u)) - l0;
+            if (la >= kAccLabels) la = -1;
+          }
+#pragma unroll
+          for (int b = 0; b < NS; ++b) {
+            if (!t[b][j]) continue;
+            const double x = (double)t[b][j];
+            if (l0 == 0) {
+              ts[j] += t[b][j];
+              s2v[j] = s2v[j] + x * x * p.inv_nb[b];
+              dep += t[b][j];
+            }
+            if (LABELS && la >= 0) acc[(b * kAccLabels + la) * kFoldThreads + tid] += x * g;
+            if (last) p.tb[(int64_t)b * p.V + v] = 0;
+          }
+          if (l0 == 0) {
+            p.tsum[v] = ts[j];
+            p.s2[v] = s2v[j];
+          }
         }
       }
-    }
+      if (LABELS) {
+        __syncthreads();
+        // one warp per (slot, label): a fixed tree over the columns
+        for (int q = wid; q < p.n_slots * n_acc; q += kFoldThreads / 32) {
+          const int b = q / n_acc, l = q % n_acc;
+          const double* col = acc + (b * kAccLabels + l) * kFoldThreads;
+          double sum = 0.0;
 #pragma unroll
-    for (int j = 0; j < kFold; ++j) {
-      if (!t[j]) continue;
-      const int64_t v = vb + (int64_t)j * kFoldThreads;
-      p.tb[v] = 0;
-      p.tsum[v] = ts[j] + t[j];
-      const double x = (double)t[j];
-      p.s2[v] = s2v[j] + x * x * inv_nb;
-      dep += t[j];
-      // Gy per unit in FP32 (GB300's FP64 divide is slow); the sum stays FP64
-      if (p.labels) acc[lab[j]][threadIdx.x] += x * (double)__fdiv_rn((float)p.gy_per_unit_vol, rho[j]);
+          for (int j = 0; j < kFoldThreads / 32; ++j) sum += col[lane + 32 * j];
+          sum = warp_sum_d(sum);
+          if (lane == 0) out[b][__fns(mask, 0, l0 + l + 1)] += sum;
+        }
+        __syncthreads();
+      }
     }
   }
   // deposited-energy counter (integer, so the order of the adds does not matter)
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) dep += __shfl_xor_sync(0xffffffffu, dep, o);
-  if ((threadIdx.x & 31) == 0) dep_w[threadIdx.x >> 5] = dep;
+  if (lane == 0) dep_w[wid] = dep;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    ull s = 0;
-    for (int w = 0; w < kFoldThreads / 32; ++w) s += dep_w[w];
-    if (s) atomicAdd(p.deposited, s);
+  if (tid == 0) {
+    ull sum = 0;
+    for (int w = 0; w < kFoldThreads / 32; ++w) sum += dep_w[w];
+    if (sum) atomicAdd(p.deposited, sum);
   }
-  if (p.labels) reduce_label_columns(acc, p.organ_partial + (size_t)blockIdx.x * kLabelSlots);
+  if (LABELS)
+    for (int i = tid; i < p.n_slots * kLabelSlots; i += kFoldThreads)
+      p.organ_partial[((size_t)(i / kLabelSlots) * gridDim.x + blockIdx.x) * kLabelSlots + i % kLabelSlots] =
+          out[i / kLabelSlots][i % kLabelSlots];
 }
 
-// One warp per label: blocks in index order, lane-strided, then a fixed tree.
+// One CTA per label, one warp per slot: blocks lane-strided, then a fixed tree;
+// the slots are then added in batch order.
 __global__ void fold_organs_kernel(const FoldParams p, int n_blocks) {
-  const int lane = threadIdx.x & 31;
-  const int l = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (l >= kLabelSlots) return;
+  __shared__ double sum[kMaxSlots];
+  const int lane = threadIdx.x & 31, b = threadIdx.x >> 5, l = blockIdx.x;
   double s = 0.0;
-  for (int b = lane; b < n_blocks; b += 32) s += p.organ_partial[(size_t)b * kLabelSlots + l];
+  for (int i = lane; i < n_blocks; i += 32) s += p.organ_partial[((size_t)b * n_blocks + i) * kLabelSlots + l];
   s = warp_sum_d(s);
-  if (lane == 0) {
-    p.org_s1[l] += s;
-    p.org_s2[l] += s * s / p.n_b;
+  if (lane == 0) sum[b] = s;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  double s1 = p.org_s1[l], s2 = p.org_s2[l];
+  for (int i = 0; i < p.n_slots; ++i) {
+    if (!(p.n_b[i] > 0.0)) continue;
+    s1 += sum[i];
+    s2 += sum[i] * sum[i] / p.n_b[i];
   }
+  p.org_s1[l] = s1;
+  p.org_s2[l] = s2;
 }
 
 __global__ void __launch_bounds__(kFoldThreads) finalize_kernel(const FinalizeParams p) {
@@ -114,8 +209,8 @@ __global__ void __launch_bounds__(kFoldThreads) finalize_kernel(const FinalizePa
   double(*acc_d)[kFoldThreads] = (double(*)[kFoldThreads])sm;
   double(*acc_e)[kFoldThreads] = (double(*)[kFoldThreads])(sm + kLabelSlots * kFoldThreads);
   for (int l = 0; l < kLabelSlots; ++l) acc_d[l][threadIdx.x] = acc_e[l][threadIdx.x] = 0.0;
-  const int64_t v0 = (int64_t)blockIdx.x * kFoldTile;
-  const int64_t v1 = v0 + kFoldTile < p.V ? v0 + kFoldTile : p.V;
+  const int64_t v0 = (int64_t)blockIdx.x * kFinalTile;
+  const int64_t v1 = v0 + kFinalTile < p.V ? v0 + kFinalTile : p.V;
   // FP64 where cancellation needs it (the variance: S2 - Tsum^2/N) and in the
   // organ sums; the rest in FP32, whose precision the FP32 outputs have anyway
   // (GB300's FP64 rate is a small fraction of its FP32 rate).
@@ -185,8 +280,8 @@ __global__ void __launch_bounds__(kFoldThreads) map_organ_kernel(const float* __
                                                                  double* __restrict__ part) {
   __shared__ double acc[kLabelSlots][kFoldThreads];
   for (int l = 0; l < kLabelSlots; ++l) acc[l][threadIdx.x] = 0.0;
-  const int64_t v0 = (int64_t)blockIdx.x * kFoldTile;
-  const int64_t v1 = v0 + kFoldTile < V ? v0 + kFoldTile : V;
+  const int64_t v0 = (int64_t)blockIdx.x * kFinalTile;
+  const int64_t v1 = v0 + kFinalTile < V ? v0 + kFinalTile : V;
   for (int64_t v = v0 + threadIdx.x; v < v1; v += kFoldThreads) {
     const int l = labels[v];
     if (l < kLabelSlots) acc[l][threadIdx.x] += (double)dose[v];
@@ -234,7 +329,7 @@ cudaError_t launch_history_sigma(const ull* tsum, const ull* s2h_lo, const ull* 
 
 cudaError_t launch_map_organ_means(const float* dose, const uint8_t* labels, int64_t V, double* part,
                                    const long long* count, double* out, cudaStream_t s) {
-  const int nb = fold_blocks(V);
+  const int nb = finalize_blocks(V);
   map_organ_kernel<<<nb, kFoldThreads, 0, s>>>(dose, labels, V, part);
   map_organ_final_kernel<<<(kLabelSlots + 3) / 4, 128, 0, s>>>(part, nb, count, out);
   return cudaGetLastError();
@@ -304,17 +399,48 @@ cudaError_t launch_dose_only(const FinalizeParams& p, int sms, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-int fold_blocks(int64_t V) { return (int)((V + kFoldTile - 1) / kFoldTile); }
+int finalize_blocks(int64_t V) { return (int)((V + kFinalTile - 1) / kFinalTile); }
 
-cudaError_t launch_fold(const FoldParams& p, cudaStream_t s) {
-  const int nb = fold_blocks(p.V);
-  fold_kernel<<<nb, kFoldThreads, 0, s>>>(p);
-  if (p.labels) fold_organs_kernel<<<(kLabelSlots + 3) / 4, 128, 0, s>>>(p, nb);
+// Tiles of a fold CTA: few enough CTAs for a small pass over their organ
+// sums, one tile each while that leaves every SM with work.
+static int fold_tiles(int64_t V) {
+  const int64_t tiles = (V + kFoldTile - 1) / kFoldTile;
+  return (int)std::max<int64_t>(1, (tiles + 16 * 152 - 1) / (16 * 152));
+}
+int fold_blocks(int64_t V) {
+  const int64_t per = (int64_t)fold_tiles(V) * kFoldTile;
+  return (int)((V + per - 1) / per);
+}
+
+template <int NS>
+static cudaError_t launch_fold_t(const FoldParams& p, cudaStream_t s) {
+  const int nb = fold_blocks(p.V), tiles = fold_tiles(p.V);
+  if (!p.labels) {
+    fold_kernel<NS, false><<<nb, kFoldThreads, 0, s>>>(p, tiles);
+    return cudaGetLastError();
+  }
+  const size_t smem = (size_t)NS * kAccLabels * kFoldThreads * sizeof(double);
+  // per call: cheap, and correct for every device and calling thread
+  const cudaError_t e =
+      cudaFuncSetAttribute(fold_kernel<NS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  fold_kernel<NS, true><<<nb, kFoldThreads, smem, s>>>(p, tiles);
+  fold_organs_kernel<<<kLabelSlots, 32 * p.n_slots, 0, s>>>(p, nb);
   return cudaGetLastError();
 }
 
+cudaError_t launch_fold(const FoldParams& p, cudaStream_t s) {
+  // the smallest variant that holds the slots (registers grow with it)
+  if (p.n_slots < 1 || p.n_slots > kMaxSlots) return cudaErrorInvalidValue;
+  if (p.n_slots == 1) return launch_fold_t<1>(p, s);
+  if (p.n_slots == 2) return launch_fold_t<2>(p, s);
+  if (p.n_slots <= 5) return launch_fold_t<5>(p, s);
+  if (p.n_slots <= 10) return launch_fold_t<10>(p, s);
+  return launch_fold_t<kMaxSlots>(p, s);
+}
+
 cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t s) {
-  const int nb = fold_blocks(p.V);
+  const int nb = finalize_blocks(p.V);
   const size_t smem = 2 * kLabelSlots * kFoldThreads * sizeof(double);
   // per call: cheap, and correct for every device and calling thread
   cudaError_t e = cudaFuncSetAttribute(finalize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -3,7 +3,9 @@
 // grid, Klein-Nishina Compton (Kahn's sampler), photoelectric absorption,
 // optional Rayleigh, 10 keV photon cutoff, int64 fixed-point tally.
 //
-// One persistent launch per batch, in two kernels.  In transport_ring_kernel
+// One persistent launch for all batches of a run, each with a tally of its own
+// (a launch's last photons then leave SMs idle once, not once per batch), in
+// two kernels.  In transport_ring_kernel
 // (annihilation photons or a point source, one patient: the default) a warp's
 // lanes hand photons on to each other through a ring in shared memory.  In
 // transport_kernel (several patients, history statistics, other decays, or
@@ -372,6 +374,11 @@ __device__ __forceinline__ void tally_flush(ull* cell, bool has, uint32_t dq, ui
   }
 }
 
+// The tally of the batch that history idx of the launch belongs to.
+__device__ __forceinline__ ull* batch_tally(const PatientGeom& G, uint32_t idx) {
+  return G.split.slots > 1 ? G.tally + batch_of(G.split, idx) * G.slot_stride : G.tally;
+}
+
 __device__ __forceinline__ ull warp_sum(ull x) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
@@ -510,6 +517,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
   Energy f = s_f0;
   int32_t qe = 0;
   int cv = 0;                            // voxel of a pending Compton event
+  ull* tal = p.g.tally;                  // tally of this lane's history's batch
   uint32_t hlo = 0, hhi = 0, stream = 0, ctr = 0;
   bool out = false;                      // outside the tracking box
   float rem = 0.f;                       // cm to the region boundary along (ux, uy, uz)
@@ -610,8 +618,9 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
             cpi = npi;
           }
           pi = npi;
-          if (HIST && hn) hist_flush(hl, hn, p.g.tally, p.s2h_lo, p.s2h_hi);   // the previous history ends
+          if (HIST && hn) hist_flush(hl, hn, tal, p.s2h_lo, p.s2h_hi);   // the previous history ends
           const PatientGeom& G = MULTI ? s_geom[pi] : p.g;
+          tal = batch_tally(G, idx);
           const uint64_t h = G.hist_begin + idx;
           hlo = (uint32_t)h;
           hhi = (uint32_t)(h >> 32);
@@ -635,10 +644,10 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
             pair = positron_track(G, p.key, hlo, hhi, st.v, st.x, st.y, st.z, q0, q_left,
                                   [&](int v, uint32_t dq) {
                                     if (HIST)
-                                      hist_add(hl, hn, (uint32_t)v, dq, p.g.tally, p.s2h_lo, p.s2h_hi,
+                                      hist_add(hl, hn, (uint32_t)v, dq, tal, p.s2h_lo, p.s2h_hi,
                                                p.g.counters + kCtrHistSplits);
                                     else
-                                      atomicAdd(G.tally + v, (ull)dq);
+                                      atomicAdd(tal + v, (ull)dq);
                                   });
             atomicAdd(&s_cnt[MULTI ? pi : 0][8], (ull)q0);
             if (!pair) escaped += (ull)q_left + (p.annihilate ? 2ull * (ull)(uint32_t)p.q_e0 : 0ull);
@@ -646,10 +655,10 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
           if (BETA && G.source_mode == NM_SOURCE_DECAY && G.q_positron > 0 && !p.annihilate) {
             // no annihilation photon to carry the local deposit: tally it here
             if (HIST)
-              hist_add(hl, hn, (uint32_t)st.v, (uint32_t)G.q_positron, p.g.tally, p.s2h_lo, p.s2h_hi,
+              hist_add(hl, hn, (uint32_t)st.v, (uint32_t)G.q_positron, tal, p.s2h_lo, p.s2h_hi,
                        p.g.counters + kCtrHistSplits);
             else
-              atomicAdd(G.tally + st.v, (ull)(uint32_t)G.q_positron);
+              atomicAdd(tal + st.v, (ull)(uint32_t)G.q_positron);
           }
           if (BETA && !p.annihilate && G.source_mode == NM_SOURCE_DECAY) pair = false;
           if (pair) {
@@ -669,11 +678,11 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
             pending_b = true;
             if (HIST) {
               if (G.q_positron > 0)
-                hist_add(hl, hn, (uint32_t)st.v, (uint32_t)G.q_positron, p.g.tally, p.s2h_lo, p.s2h_hi,
+                hist_add(hl, hn, (uint32_t)st.v, (uint32_t)G.q_positron, tal, p.s2h_lo, p.s2h_hi,
                          p.g.counters + kCtrHistSplits);
             } else {
               has = G.q_positron > 0;
-              cell = G.tally + st.v;
+              cell = tal + st.v;
             }
           }
           }
@@ -711,9 +720,9 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
         // The scattered photons tally their deposit now and take their next
         // flight step in this same iteration instead of idling through it.
         if (HIST) {
-          if (has) hist_add(hl, hn, (uint32_t)dv, dq, p.g.tally, p.s2h_lo, p.s2h_hi, p.g.counters + kCtrHistSplits);
+          if (has) hist_add(hl, hn, (uint32_t)dv, dq, tal, p.s2h_lo, p.s2h_hi, p.g.counters + kCtrHistSplits);
         } else {
-          tally_flush<WARP_AGG>(G.tally + dv, has, dq, lane);
+          tally_flush<WARP_AGG>(tal + dv, has, dq, lane);
         }
         has = false;
         dq = 0;
@@ -804,12 +813,12 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
       }
     }
     if (HIST) {
-      if (has) hist_add(hl, hn, (uint32_t)dv, dq, p.g.tally, p.s2h_lo, p.s2h_hi, p.g.counters + kCtrHistSplits);
+      if (has) hist_add(hl, hn, (uint32_t)dv, dq, tal, p.s2h_lo, p.s2h_hi, p.g.counters + kCtrHistSplits);
     } else {
-      tally_flush<WARP_AGG>(G.tally + dv, has, dq, lane);
+      tally_flush<WARP_AGG>(tal + dv, has, dq, lane);
     }
   }
-  if (HIST && hn) hist_flush(hl, hn, p.g.tally, p.s2h_lo, p.s2h_hi);
+  if (HIST && hn) hist_flush(hl, hn, tal, p.s2h_lo, p.s2h_hi);
 
   // ---- counters ---------------------------------------------------------------
   if (MULTI) {
@@ -959,6 +968,7 @@ struct RingTables {
   float4 tab[kKnTable];
   float2 mat[NM_MAX_MATERIALS];   // za, zp
   float zr[NM_MAX_MATERIALS];
+  uint32_t next[kMaxSlots];       // first history of the launch past batch b
 };
 static_assert(sizeof(RingTables) % 16 == 0, "the warps' stores follow");
 
@@ -980,6 +990,8 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
     tb.mat[threadIdx.x] = make_float2(m.za, m.zp);
     tb.zr[threadIdx.x] = m.zr;
   }
+  if (threadIdx.x < kMaxSlots)
+    tb.next[threadIdx.x] = threadIdx.x + 1 < p.g.split.slots ? p.g.split.start(threadIdx.x + 1) : 0xffffffffu;
   if (threadIdx.x < 12) s_cnt[threadIdx.x] = 0;
   __syncthreads();
   uint32_t tables, store;                // volatile: kept, not formed again at every use
@@ -988,7 +1000,7 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
                : "=r"(store)
                : "r"(tables + (uint32_t)sizeof(RingTables) + (threadIdx.x >> 5) * (uint32_t)sizeof(Store)));
   const uint32_t tab = tables + offsetof(RingTables, tab), mat = tables + offsetof(RingTables, mat),
-                 zr = tables + offsetof(RingTables, zr);
+                 zr = tables + offsetof(RingTables, zr), next = tables + offsetof(RingTables, next);
   if (threadIdx.x == 0) s_f0 = ring_energy<GENERAL>(p.e0, tab, p.ln_e_lo, p.inv_dln_e);
   __syncthreads();
   constexpr int kBorn = 8, kKilled = 9, kDeposit = 10;
@@ -1019,6 +1031,13 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
   uint32_t n_steps = 0;                  // flight steps of the photons this lane saw end
   ull deposit = 0;                       // energy of the deposits this lane made
 
+  // Tally cell of voxel v in the batch of history idx of the launch (batch_of,
+  // from the table of batch ends; all batches' voxels count below 2^32).
+  auto tally_cell = [&](uint32_t idx, uint32_t v) -> ull* {
+    uint32_t b = __umulhi(idx, p.g.split.est);
+    if (idx >= __float_as_uint(lds1(next + 4u * b))) ++b;
+    return p.g.tally + (b * p.g.slot_stride + v);
+  };
   // The Compton event of a photon of signed energy ce with direction and
   // history cd, drawn with the flight step's words rk and rp: its deposit dq,
   // its new direction; returns its new energy, 0 below the cutoff.
@@ -1057,7 +1076,7 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
     if (cp.w != 0.0f && lane < n_parked) {
       float4 cd = lds4(RING_AT(dir, i));
       const float4 cm = lds4(RING_AT(mid, i));
-      cell = p.g.tally + __float_as_int(cm.z);
+      cell = tally_cell(__float_as_uint(cd.w) - h0, __float_as_uint(cm.z));
       uint32_t cctr = 0;
       if constexpr (GENERAL) cctr = __float_as_uint(lds1(RING_AT8(aux, i)));
       const float ce = scatter(cp.w, cd, cctr, __float_as_uint(cm.x), __float_as_uint(cm.y), dq);
@@ -1145,7 +1164,7 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
       sts2(RING_AT8(site_rem, lane), rb, o ? -1.0f : 1.0f);
       if (pairs) {
         has = p.g.q_positron > 0;
-        cell = p.g.tally + st.v;
+        cell = tally_cell(idx, (uint32_t)st.v);
       }
     }
     tally_flush<WARP_AGG>(cell, has, (uint32_t)p.g.q_positron, lane);
@@ -1228,7 +1247,7 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
         dq = (uint32_t)q_units(fabsf(e));
         deposit += dq;
         n_steps += GENERAL ? steps : ctr;
-        if (!WARP_AGG) atomicAdd(p.g.tally + v, (ull)dq);
+        if (!WARP_AGG) atomicAdd(tally_cell(hlo - h0, (uint32_t)v), (ull)dq);
       } else if (e != 0.0f) {
         atomicAdd(&s_cnt[kCtrKilledUnits], (ull)q_units(fabsf(e)));
         atomicAdd(&s_cnt[kKilled], 1ull);
@@ -1239,7 +1258,7 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
       e = 0.0f;
       park = false;
     }
-    if (WARP_AGG) tally_flush<true>(p.g.tally + v, photo, dq, lane);
+    if (WARP_AGG) tally_flush<true>(photo ? tally_cell(hlo - h0, (uint32_t)v) : nullptr, photo, dq, lane);
     if constexpr (LAST) {
       n_compton += __popc(__ballot_sync(kFull, park));
       uint32_t dq2 = 0;
@@ -1258,7 +1277,7 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
           rem = region_distance(p.g, o, px, py, pz, ux, uy, uz);
         }
       }
-      tally_flush<WARP_AGG>(p.g.tally + v, park, dq2, lane);
+      tally_flush<WARP_AGG>(park ? tally_cell(hlo - h0, (uint32_t)v) : nullptr, park, dq2, lane);
       return 0u;
     }
     // exchanges: scattered photons, and near the end lanes without one
