@@ -796,7 +796,7 @@ nm_status nm_dose_create(nm_dose** out, const nm_grid* g, const nm_materials* mt
       (e = dalloc(&h->status, 1)) || (e = dalloc(&h->rho_max_bits, NM_MAX_MATERIALS)) ||
       (e = dalloc(&h->org_s1, kLabelSlots)) || (e = dalloc(&h->org_s2, kLabelSlots)) ||
       (e = dalloc(&h->organ_count, kLabelSlots)) ||
-      (e = dalloc(&h->organ_partial, std::max((size_t)finalize_blocks(V) * 2, (size_t)fold_blocks(V) * kMaxSlots) * kLabelSlots)) ||
+      (e = dalloc(&h->organ_partial, (size_t)fold_blocks(V) * kMaxSlots * kLabelSlots)) ||
       (e = dalloc(&h->organ_out, 4 * kLabelSlots)))
     return bail(cuda_fail(e, "device allocation"));
   if (labels && ((e = dalloc(&h->labels, V)) || (e = dalloc(&h->label_bad, 1))))
@@ -1296,7 +1296,7 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
   return NM_OK;
 }
 
-static nm_status finalize(nm_dose* h, float* dose, float* sigma) {
+static nm_status finalize(nm_dose* h, float* dose, float* sigma, bool organs) {
   if (h->hist_next == 0) return fail(NM_ERR_STATE, "no histories simulated yet");
   if (h->n_batches < 2) return fail(NM_ERR_STATE, "need at least 2 batches for the uncertainty");
   cudaStream_t s = h->stream;
@@ -1312,7 +1312,7 @@ static nm_status finalize(nm_dose* h, float* dose, float* sigma) {
   p.org_s1 = h->org_s1; p.org_s2 = h->org_s2;
   p.organ_count = h->organ_count;
   p.organ_out = h->organ_out;
-  NM_CUDA(launch_finalize(p, s), "finalize launch");
+  NM_CUDA(launch_finalize(p, organs && h->labels, s), "finalize launch");
   return NM_OK;
 }
 
@@ -1336,7 +1336,7 @@ nm_status nm_dose_get(nm_dose* h, float* dose, float* sigma, double* organ_dose)
     p.gy_per_unit_vol = h->gy_per_unit_vol(); p.activity_bq = h->opt.activity_bq; p.dose = d_out;
     NM_CUDA(launch_dose_only(p, h->sms, s), "dose launch");
   } else {
-    nm_status st = finalize(h, d_out, s_out);
+    nm_status st = finalize(h, d_out, s_out, organ_dose != nullptr);
     if (st != NM_OK) return st;
   }
   if (dose && !dd) NM_CUDA(cudaMemcpyAsync(dose, d_out, h->V * sizeof(float), cudaMemcpyDeviceToHost, s), "dose copy");
@@ -1384,7 +1384,7 @@ nm_status nm_dose_get_organs(nm_dose* h, double* mean, double* eps_rms, double* 
     }
     return NM_OK;
   }
-  nm_status st = finalize(h, nullptr, nullptr);
+  nm_status st = finalize(h, nullptr, nullptr, true);
   if (st != NM_OK) return st;
   std::vector<double> out(4 * kLabelSlots);
   NM_CUDA(cudaMemcpyAsync(out.data(), h->organ_out, out.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream), "organ copy");

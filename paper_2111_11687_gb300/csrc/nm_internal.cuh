@@ -20,8 +20,7 @@ constexpr double kJoulePerEv = 1.602176634e-19;
 constexpr float kTwoPi = 6.283185307179586f;
 constexpr int kKnTable = 1024;      // log-energy nodes of the Klein-Nishina table
 constexpr int kFoldThreads = 128;   // fold / finalize CTA size
-constexpr int kFoldTile = 2048;     // voxels a fold CTA takes at a time
-constexpr int kFinalTile = 8192;    // voxels per finalize CTA
+constexpr int kFoldTile = 2048;     // voxels a fold / finalize CTA takes at a time
 constexpr int kLabelSlots = NM_MAX_LABELS + 1;
 
 // Fixed-point energy: round-to-nearest-even of the FP32 product E * 6.4e7.
@@ -284,7 +283,6 @@ struct FoldParams {
   }
 };
 int fold_blocks(int64_t V);
-int finalize_blocks(int64_t V);
 cudaError_t launch_fold(const FoldParams& p, cudaStream_t s);
 
 // Adds another shard's statistics (o_*) into a handle's (all device arrays;
@@ -317,7 +315,8 @@ struct FinalizeParams {
 };
 // Eq. 1 dose rate only into p.dose (bit-identical to launch_finalize's).
 cudaError_t launch_dose_only(const FinalizeParams& p, int sms, cudaStream_t s);
-cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t s);
+// organs: also the per-label sums and organ_out (needs labels).
+cudaError_t launch_finalize(const FinalizeParams& p, bool organs, cudaStream_t s);
 // Voxels per label into count[kLabelSlots] (labels >= kLabelSlots count as 0),
 // and atomicMin of first_bad with every voxel index whose label exceeds n_labels.
 cudaError_t launch_label_count(const uint8_t* labels, int64_t V, int n_labels, long long* count,

@@ -22,17 +22,60 @@ __device__ __forceinline__ double warp_sum_d(double x) {
   return x;
 }
 
-// Reduce acc[l][0..kFoldThreads) for every label into out[l] (fixed tree).
-__device__ void reduce_label_columns(const double (*acc)[kFoldThreads], double* out) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  constexpr int nw = kFoldThreads / 32;
-  for (int l = wid; l < kLabelSlots; l += nw) {
-    double s = 0.0;
+// Sums per label.  A tile of kFoldTile voxels holds few labels, so each thread
+// keeps FP64 sums for kAccLabels of them in columns of shared memory (one per
+// quantity and label); a tile with more labels is read again for the next
+// ones.  The columns, and then the tiles and blocks, are added in a fixed order.
+constexpr int kAccLabels = 4;
+constexpr int kPerThread = kFoldTile / kFoldThreads;       // voxels of a thread per tile
+
+// Labels of this thread's voxels v0 + tid + i kFoldThreads, a byte each (0 past
+// v1); returns the set of labels in the tile.
+__device__ __forceinline__ uint32_t tile_labels(const uint8_t* __restrict__ labels, int64_t v0, int64_t v1,
+                                                uint32_t (&lab)[kPerThread / 4], uint32_t* s_mask) {
+  uint32_t mask = 0;
 #pragma unroll
-    for (int j = 0; j < kFoldThreads / 32; ++j) s += acc[l][lane + 32 * j];
-    s = warp_sum_d(s);
-    if (lane == 0) out[l] = s;
+  for (int i = 0; i < kPerThread / 4; ++i) lab[i] = 0;
+#pragma unroll
+  for (int i = 0; i < kPerThread; ++i) {
+    const int64_t v = v0 + threadIdx.x + (int64_t)i * kFoldThreads;
+    const uint32_t l = v < v1 ? labels[v] : 0u;
+    lab[i / 4] |= l << (8 * (i % 4));
+    if (v < v1) mask |= 1u << l;
   }
+  mask = __reduce_or_sync(0xffffffffu, mask);
+  if ((threadIdx.x & 31) == 0) s_mask[threadIdx.x >> 5] = mask;
+  __syncthreads();
+  mask = 0;
+#pragma unroll
+  for (int w = 0; w < kFoldThreads / 32; ++w) mask |= s_mask[w];
+  return mask;
+}
+
+// Column of the thread's i-th voxel among those for labels l0, l0 + 1, ... of
+// the tile's set, or -1.
+__device__ __forceinline__ int label_column(const uint32_t (&lab)[kPerThread / 4], int i, uint32_t mask, int l0) {
+  const uint32_t l = (lab[i / 4] >> (8 * (i % 4))) & 255u;
+  const int c = __popc(mask & ((1u << l) - 1u)) - l0;
+  return c < kAccLabels ? c : -1;
+}
+
+// out[q][label] += the sum of the columns acc[q][0 .. n_acc) (labels l0, ... of
+// the set) for q < n_q; one warp per column.  Ends with the columns free again.
+__device__ __forceinline__ void add_columns(const double* acc, int n_q, int n_acc, uint32_t mask, int l0,
+                                            double (*out)[kLabelSlots]) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __syncthreads();
+  for (int i = wid; i < n_q * n_acc; i += kFoldThreads / 32) {
+    const int q = i / n_acc, l = i % n_acc;
+    const double* col = acc + (q * kAccLabels + l) * kFoldThreads;
+    double sum = 0.0;
+#pragma unroll
+    for (int j = 0; j < kFoldThreads / 32; ++j) sum += col[lane + 32 * j];
+    sum = warp_sum_d(sum);
+    if (lane == 0) out[q][__fns(mask, 0, l0 + l + 1)] += sum;
+  }
+  __syncthreads();
 }
 
 // Fold of a launch's NS (or fewer) batches in one pass over the voxels: per
@@ -46,15 +89,10 @@ __device__ void reduce_label_columns(const double (*acc)[kFoldThreads], double* 
 // about two per SM and clock).  A thread therefore loads NS x K tallies before
 // it uses any, and lone voxels of other batches cost nothing.
 //
-// Organ sums: a tile holds few labels, so each thread keeps a column of FP64
-// sums for kAccLabels of them per slot in shared memory; tiles with more labels
-// are read again for the next ones.  Columns are added in a fixed order.
-constexpr int kAccLabels = 4;
-
+// Benchmark phantom, ten batches: 10 x 0.18 ms as a fold each, 1.15 ms together.
 template <int NS, bool LABELS>
 __global__ void __launch_bounds__(kFoldThreads) fold_kernel(const FoldParams p, int tiles_per_block) {
   constexpr int K = NS <= 2 ? 8 : 4;       // voxels of a thread in flight
-  constexpr int kPer = kFoldTile / kFoldThreads;          // voxels of a thread per tile
   extern __shared__ double acc[];                         // [NS][kAccLabels][kFoldThreads]
   __shared__ double out[LABELS ? NS : 1][kLabelSlots];
   __shared__ uint32_t s_mask[kFoldThreads / 32];
@@ -69,22 +107,8 @@ __global__ void __launch_bounds__(kFoldThreads) fold_kernel(const FoldParams p, 
     const int64_t v0 = first + (int64_t)ti * kFoldTile;
     if (v0 >= p.V) break;
     const int64_t v1 = v0 + kFoldTile < p.V ? v0 + kFoldTile : p.V;
-    // labels of this thread's voxels v0 + tid + i kFoldThreads, and of the tile
-    uint32_t lab[kPer / 4] = {};
-    uint32_t mask = 0;
-    if (LABELS) {
-#pragma unroll
-      for (int i = 0; i < kPer; ++i) {
-        const int64_t v = v0 + tid + (int64_t)i * kFoldThreads;
-        const uint32_t l = v < v1 ? p.labels[v] : 0u;
-        lab[i / 4] |= l << (8 * (i % 4));
-        mask |= 1u << l;
-      }
-      mask = __reduce_or_sync(0xffffffffu, mask);
-      if (lane == 0) s_mask[wid] = mask;
-      __syncthreads();
-      mask = s_mask[0] | s_mask[1] | s_mask[2] | s_mask[3];
-    }
+    uint32_t lab[kPerThread / 4];
+    const uint32_t mask = LABELS ? tile_labels(p.labels, v0, v1, lab, s_mask) : 0u;
     const int n_lab = LABELS ? __popc(mask) : 1;
     for (int l0 = 0; l0 < n_lab; l0 += kAccLabels) {
       const int n_acc = min(kAccLabels, n_lab - l0);
@@ -93,7 +117,7 @@ __global__ void __launch_bounds__(kFoldThreads) fold_kernel(const FoldParams p, 
         for (int i = 0; i < p.n_slots; ++i)
           for (int l = 0; l < n_acc; ++l) acc[(i * kAccLabels + l) * kFoldThreads + tid] = 0.0;
 #pragma unroll 1
-      for (int c = 0; c < kPer; c += K) {
+      for (int c = 0; c < kPerThread; c += K) {
         ull t[NS][K];
         ull any[K];
 #pragma unroll
@@ -128,11 +152,7 @@ __global__ void __launch_bounds__(kFoldThreads) fold_kernel(const FoldParams p, 
           // Gy per unit in FP32 (GB300's FP64 divide is slow); the sum stays FP64
           const double g = LABELS ? (double)__fdiv_rn(gy, rho[j]) : 0.0;
           int la = -1;                                    // the voxel's column, if one of this pass
-          if (LABELS) {
-            const uint32_t l = (lab[(c + j) / 4] >> (8 * ((c + j) % 4))) & 255u;
-            la = __popc(mask & ((1u << l) - 1u)) - l0;
-            if (la >= kAccLabels) la = -1;
-          }
+          if (LABELS) la = label_column(lab, c + j, mask, l0);
 #pragma unroll
           for (int b = 0; b < NS; ++b) {
             if (!t[b][j]) continue;
@@ -151,20 +171,7 @@ __global__ void __launch_bounds__(kFoldThreads) fold_kernel(const FoldParams p, 
           }
         }
       }
-      if (LABELS) {
-        __syncthreads();
-        // one warp per (slot, label): a fixed tree over the columns
-        for (int q = wid; q < p.n_slots * n_acc; q += kFoldThreads / 32) {
-          const int b = q / n_acc, l = q % n_acc;
-          const double* col = acc + (b * kAccLabels + l) * kFoldThreads;
-          double sum = 0.0;
-#pragma unroll
-          for (int j = 0; j < kFoldThreads / 32; ++j) sum += col[lane + 32 * j];
-          sum = warp_sum_d(sum);
-          if (lane == 0) out[b][__fns(mask, 0, l0 + l + 1)] += sum;
-        }
-        __syncthreads();
-      }
+      if (LABELS) add_columns(acc, p.n_slots, n_acc, mask, l0, out);
     }
   }
   // deposited-energy counter (integer, so the order of the adds does not matter)
@@ -204,44 +211,101 @@ __global__ void fold_organs_kernel(const FoldParams p, int n_blocks) {
   p.org_s2[l] = s2;
 }
 
-__global__ void __launch_bounds__(kFoldThreads) finalize_kernel(const FinalizeParams p) {
-  extern __shared__ double sm[];
-  double(*acc_d)[kFoldThreads] = (double(*)[kFoldThreads])sm;
-  double(*acc_e)[kFoldThreads] = (double(*)[kFoldThreads])(sm + kLabelSlots * kFoldThreads);
-  for (int l = 0; l < kLabelSlots; ++l) acc_d[l][threadIdx.x] = acc_e[l][threadIdx.x] = 0.0;
-  const int64_t v0 = (int64_t)blockIdx.x * kFinalTile;
-  const int64_t v1 = v0 + kFinalTile < p.V ? v0 + kFinalTile : p.V;
-  // FP64 where cancellation needs it (the variance: S2 - Tsum^2/N) and in the
-  // organ sums; the rest in FP32, whose precision the FP32 outputs have anyway
-  // (GB300's FP64 rate is a small fraction of its FP32 rate).
+// Eq. 1 per voxel (MAPS: dose and sigma, either may be NULL) and the sums behind
+// Eq. 2 and Eq. 3 per label (ORGANS).
+//
+// Bound by DRAM (25 B per voxel for the maps) and FP64, which therefore does
+// only what needs it: the mean, the variance (S2 - Tsum^2/N cancels) and the
+// organ sums; the rest is FP32, whose precision the FP32 outputs have anyway.
+// Voxels without a deposit cost no FP64: their dose adds nothing and their
+// epsilon of 1 is counted in integers.  Eight voxels' loads go out together.
+// Whole body (157 M voxels): 3.3 ms for either -> 0.54 ms (maps), 1.02 ms (organs).
+template <bool MAPS, bool ORGANS>
+__global__ void __launch_bounds__(kFoldThreads) finalize_kernel(const FinalizeParams p, int tiles_per_block) {
+  constexpr int K = 8;
+  __shared__ double acc[ORGANS ? 2 * kAccLabels * kFoldThreads : 1];   // dose, epsilon^2
+  __shared__ int zeros[ORGANS ? kAccLabels : 1][kFoldThreads];         // voxels without a deposit
+  __shared__ double out[ORGANS ? 2 : 1][kLabelSlots];
+  __shared__ uint32_t s_mask[kFoldThreads / 32];
+  const int tid = threadIdx.x;
+  if (ORGANS && tid < 2 * kLabelSlots) out[tid / kLabelSlots][tid % kLabelSlots] = 0.0;
   const double inv_n = 1.0 / p.n_total;
   const double inv_k1n = 1.0 / ((p.n_batches - 1.0) * p.n_total);
   const float gy_a = (float)(p.gy_per_unit_vol * p.activity_bq);
-  for (int64_t v = v0 + threadIdx.x; v < v1; v += kFoldThreads) {
-    const ull ti = p.tsum[v];
-    float d = 0.0f, sg = 0.0f;
-    if (ti) {
-      const double t = (double)ti;
-      const double mean = t * inv_n;                       // units per decay
-      const double var = fmax(fma(-t, mean, p.s2[v]), 0.0) * inv_k1n;
-      const float conv = __fdiv_rn(gy_a, p.density[v]);
-      d = (float)mean * conv;                              // Eq. 1, Gy/s
-      sg = sqrtf((float)var) * conv;
-    }
-    if (p.dose) p.dose[v] = d;
-    if (p.sigma) p.sigma[v] = sg;
-    if (p.labels) {
-      const int l = p.labels[v];
-      acc_d[l][threadIdx.x] += (double)d;
-      const float eps = d > 0.0f ? __fdiv_rn(sg, d) : 1.0f;
-      acc_e[l][threadIdx.x] += (double)(eps * eps);
+  const int64_t first = (int64_t)blockIdx.x * tiles_per_block * kFoldTile;
+  for (int ti = 0; ti < tiles_per_block; ++ti) {
+    const int64_t v0 = first + (int64_t)ti * kFoldTile;
+    if (v0 >= p.V) break;
+    const int64_t v1 = v0 + kFoldTile < p.V ? v0 + kFoldTile : p.V;
+    uint32_t lab[kPerThread / 4];
+    const uint32_t mask = ORGANS ? tile_labels(p.labels, v0, v1, lab, s_mask) : 0u;
+    const int n_lab = ORGANS ? __popc(mask) : 1;
+    for (int l0 = 0; l0 < n_lab; l0 += kAccLabels) {
+      const int n_acc = min(kAccLabels, n_lab - l0);
+      if (ORGANS)
+        for (int l = 0; l < n_acc; ++l) {
+          acc[l * kFoldThreads + tid] = acc[(kAccLabels + l) * kFoldThreads + tid] = 0.0;
+          zeros[l][tid] = 0;
+        }
+#pragma unroll 1
+      for (int c = 0; c < kPerThread; c += K) {
+        ull t[K];
+        double s2v[K];
+        float rho[K];
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+          const int64_t v = v0 + tid + (int64_t)(c + j) * kFoldThreads;
+          t[j] = v < v1 ? p.tsum[v] : 0ull;
+        }
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+          const int64_t v = v0 + tid + (int64_t)(c + j) * kFoldThreads;
+          s2v[j] = 0.0; rho[j] = 1.0f;
+          if (t[j]) {
+            s2v[j] = p.s2[v];
+            rho[j] = p.density[v];
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+          const int64_t v = v0 + tid + (int64_t)(c + j) * kFoldThreads;
+          if (v >= v1) continue;
+          float d = 0.0f, sg = 0.0f;
+          if (t[j]) {
+            const double x = (double)t[j];
+            const double mean = x * inv_n;                       // units per decay
+            const double var = fma(-x, mean, s2v[j]) * inv_k1n;  // rounding may leave it below 0
+            const float conv = __fdiv_rn(gy_a, rho[j]);
+            d = (float)mean * conv;                              // Eq. 1, Gy/s
+            sg = sqrtf(fmaxf((float)var, 0.0f)) * conv;
+          }
+          if (MAPS) {
+            if (p.dose) p.dose[v] = d;
+            if (p.sigma) p.sigma[v] = sg;
+          }
+          if (ORGANS) {
+            const int la = label_column(lab, c + j, mask, l0);
+            if (la >= 0) {
+              if (d > 0.0f) {
+                const float eps = __fdiv_rn(sg, d);
+                acc[la * kFoldThreads + tid] += (double)d;
+                acc[(kAccLabels + la) * kFoldThreads + tid] += (double)(eps * eps);
+              } else {
+                zeros[la][tid] += 1;
+              }
+            }
+          }
+        }
+      }
+      if (ORGANS) {
+        for (int l = 0; l < n_acc; ++l)
+          if (zeros[l][tid]) acc[(kAccLabels + l) * kFoldThreads + tid] += (double)zeros[l][tid];
+        add_columns(acc, 2, n_acc, mask, l0, out);
+      }
     }
   }
-  if (!p.labels) return;
-  __syncthreads();
-  double* out = p.organ_partial + (size_t)blockIdx.x * 2 * kLabelSlots;
-  reduce_label_columns(acc_d, out);
-  reduce_label_columns(acc_e, out + kLabelSlots);
+  if (ORGANS && tid < 2 * kLabelSlots)
+    p.organ_partial[(size_t)blockIdx.x * 2 * kLabelSlots + tid] = out[tid / kLabelSlots][tid % kLabelSlots];
 }
 
 __global__ void finalize_organs_kernel(const FinalizeParams p, int n_blocks) {
@@ -274,20 +338,42 @@ __global__ void finalize_organs_kernel(const FinalizeParams p, int n_blocks) {
   p.organ_out[3 * kLabelSlots + l] = cnt;
 }
 
-// Eq. 2 over an arbitrary dose map: per-CTA per-label partial sums (fixed tree).
+// Eq. 2 over an arbitrary dose map: per-CTA per-label partial sums (fixed
+// tree).  Zeros add nothing and cost no FP64 (benchmark phantom: 134 -> 96 us).
 __global__ void __launch_bounds__(kFoldThreads) map_organ_kernel(const float* __restrict__ dose,
                                                                  const uint8_t* __restrict__ labels, int64_t V,
-                                                                 double* __restrict__ part) {
-  __shared__ double acc[kLabelSlots][kFoldThreads];
-  for (int l = 0; l < kLabelSlots; ++l) acc[l][threadIdx.x] = 0.0;
-  const int64_t v0 = (int64_t)blockIdx.x * kFinalTile;
-  const int64_t v1 = v0 + kFinalTile < V ? v0 + kFinalTile : V;
-  for (int64_t v = v0 + threadIdx.x; v < v1; v += kFoldThreads) {
-    const int l = labels[v];
-    if (l < kLabelSlots) acc[l][threadIdx.x] += (double)dose[v];
+                                                                 int tiles_per_block, double* __restrict__ part) {
+  __shared__ double acc[kAccLabels * kFoldThreads];
+  __shared__ double out[1][kLabelSlots];
+  __shared__ uint32_t s_mask[kFoldThreads / 32];
+  const int tid = threadIdx.x;
+  if (tid < kLabelSlots) out[0][tid] = 0.0;
+  const int64_t first = (int64_t)blockIdx.x * tiles_per_block * kFoldTile;
+  for (int ti = 0; ti < tiles_per_block; ++ti) {
+    const int64_t v0 = first + (int64_t)ti * kFoldTile;
+    if (v0 >= V) break;
+    const int64_t v1 = v0 + kFoldTile < V ? v0 + kFoldTile : V;
+    float d[kPerThread];
+#pragma unroll
+    for (int i = 0; i < kPerThread; ++i) {
+      const int64_t v = v0 + tid + (int64_t)i * kFoldThreads;
+      d[i] = v < v1 ? dose[v] : 0.0f;
+    }
+    uint32_t lab[kPerThread / 4];
+    const uint32_t mask = tile_labels(labels, v0, v1, lab, s_mask);
+    const int n_lab = __popc(mask);
+    for (int l0 = 0; l0 < n_lab; l0 += kAccLabels) {
+      const int n_acc = min(kAccLabels, n_lab - l0);
+      for (int l = 0; l < n_acc; ++l) acc[l * kFoldThreads + tid] = 0.0;
+#pragma unroll
+      for (int i = 0; i < kPerThread; ++i) {
+        const int la = label_column(lab, i, mask, l0);
+        if (d[i] != 0.0f && la >= 0) acc[la * kFoldThreads + tid] += (double)d[i];
+      }
+      add_columns(acc, 1, n_acc, mask, l0, out);
+    }
   }
-  __syncthreads();
-  reduce_label_columns(acc, part + (size_t)blockIdx.x * kLabelSlots);
+  if (tid < kLabelSlots) part[(size_t)blockIdx.x * kLabelSlots + tid] = out[0][tid];
 }
 
 __global__ void map_organ_final_kernel(const double* __restrict__ part, int n_blocks,
@@ -319,6 +405,17 @@ __global__ void history_sigma_kernel(const ull* __restrict__ tsum, const ull* __
 
 }  // namespace
 
+// Tiles of a CTA of the passes over the voxels: few enough CTAs for a small pass over their
+// label sums, one tile each while that leaves every SM with work.
+static int fold_tiles(int64_t V) {
+  const int64_t tiles = (V + kFoldTile - 1) / kFoldTile;
+  return (int)std::max<int64_t>(1, (tiles + 16 * 152 - 1) / (16 * 152));
+}
+int fold_blocks(int64_t V) {
+  const int64_t per = (int64_t)fold_tiles(V) * kFoldTile;
+  return (int)((V + per - 1) / per);
+}
+
 cudaError_t launch_history_sigma(const ull* tsum, const ull* s2h_lo, const ull* s2h_hi, const float* density,
                                  int64_t V, double n_total, double gy_a, float* sigma, cudaStream_t s) {
   const int64_t g = (V + 255) / 256;
@@ -329,8 +426,8 @@ cudaError_t launch_history_sigma(const ull* tsum, const ull* s2h_lo, const ull* 
 
 cudaError_t launch_map_organ_means(const float* dose, const uint8_t* labels, int64_t V, double* part,
                                    const long long* count, double* out, cudaStream_t s) {
-  const int nb = finalize_blocks(V);
-  map_organ_kernel<<<nb, kFoldThreads, 0, s>>>(dose, labels, V, part);
+  const int nb = fold_blocks(V);
+  map_organ_kernel<<<nb, kFoldThreads, 0, s>>>(dose, labels, V, fold_tiles(V), part);
   map_organ_final_kernel<<<(kLabelSlots + 3) / 4, 128, 0, s>>>(part, nb, count, out);
   return cudaGetLastError();
 }
@@ -399,19 +496,6 @@ cudaError_t launch_dose_only(const FinalizeParams& p, int sms, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-int finalize_blocks(int64_t V) { return (int)((V + kFinalTile - 1) / kFinalTile); }
-
-// Tiles of a fold CTA: few enough CTAs for a small pass over their organ
-// sums, one tile each while that leaves every SM with work.
-static int fold_tiles(int64_t V) {
-  const int64_t tiles = (V + kFoldTile - 1) / kFoldTile;
-  return (int)std::max<int64_t>(1, (tiles + 16 * 152 - 1) / (16 * 152));
-}
-int fold_blocks(int64_t V) {
-  const int64_t per = (int64_t)fold_tiles(V) * kFoldTile;
-  return (int)((V + per - 1) / per);
-}
-
 template <int NS>
 static cudaError_t launch_fold_t(const FoldParams& p, cudaStream_t s) {
   const int nb = fold_blocks(p.V), tiles = fold_tiles(p.V);
@@ -439,14 +523,16 @@ cudaError_t launch_fold(const FoldParams& p, cudaStream_t s) {
   return launch_fold_t<kMaxSlots>(p, s);
 }
 
-cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t s) {
-  const int nb = finalize_blocks(p.V);
-  const size_t smem = 2 * kLabelSlots * kFoldThreads * sizeof(double);
-  // per call: cheap, and correct for every device and calling thread
-  cudaError_t e = cudaFuncSetAttribute(finalize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  finalize_kernel<<<nb, kFoldThreads, smem, s>>>(p);
-  if (p.labels) finalize_organs_kernel<<<(kLabelSlots + 3) / 4, 128, 0, s>>>(p, nb);
+cudaError_t launch_finalize(const FinalizeParams& p, bool organs, cudaStream_t s) {
+  const int nb = fold_blocks(p.V), tiles = fold_tiles(p.V);
+  const bool maps = p.dose || p.sigma;
+  if (!organs) {
+    if (maps) finalize_kernel<true, false><<<nb, kFoldThreads, 0, s>>>(p, tiles);
+    return cudaGetLastError();
+  }
+  if (maps) finalize_kernel<true, true><<<nb, kFoldThreads, 0, s>>>(p, tiles);
+  else finalize_kernel<false, true><<<nb, kFoldThreads, 0, s>>>(p, tiles);
+  finalize_organs_kernel<<<(kLabelSlots + 3) / 4, 128, 0, s>>>(p, nb);
   return cudaGetLastError();
 }
 
