@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstring>
 #include <deque>
+#include <functional>
 #include <map>
 #include <mutex>
 #include <string>
@@ -100,8 +101,8 @@ std::vector<float> build_beta_inverse_cdf(const double* t_maxs, const double* in
   const double h = t_max / kPanels;
   std::vector<double> mix(kPanels + 1, 0.0), den(kPanels + 1);   // mixture and branch at the panel edges
   for (int b = 0; b < n; ++b) {
-    double norm = 0.0;
     for (int i = 0; i <= kPanels; ++i) den[i] = density(i * h, t_maxs[b]);
+    double norm = 0.0;
     for (int i = 0; i < kPanels; ++i) norm += 0.5 * h * (den[i] + den[i + 1]);
     const double weight = norm > 0.0 ? inten[b] / itot / norm : 0.0;
     for (int i = 0; i <= kPanels; ++i) mix[i] += weight * den[i];
@@ -597,11 +598,9 @@ typedef std::tuple<int, int, int, int, int, int, int, int, int, int, int, int> T
 static std::mutex g_tune_mu;
 static std::map<TuneKey, Shape> g_tune_cache;
 
-static int grid_for_shape(const nm_dose* h, const Shape& sh, bool multi) {
-  const int per_sm = transport_max_blocks_per_sm(sh.block, sh.warp_agg, h->rayleigh, sh.regroup, multi,
-                                                 !multi && h->opt.history_sigma != 0,
-                                                 !multi && h->nuclide);
-  return per_sm * h->sms;
+static int grid_for_shape(const nm_dose* h, const Shape& sh) {
+  return h->sms * transport_max_blocks_per_sm(sh.block, sh.warp_agg, h->rayleigh, sh.regroup,
+                                              h->opt.history_sigma != 0, h->nuclide);
 }
 
 // Histories per work grab of a launch of n: the handle's chunk, but where it is
@@ -609,11 +608,9 @@ static int grid_for_shape(const nm_dose* h, const Shape& sh, bool multi) {
 // launch of 1e5 in chunks of 256 keeps 391 of 4864 warps busy (point source in
 // water, 1e6 histories in ten batches: 0.85 ms in chunks of 256, 0.50 in chunks
 // of 32, 0.59 in chunks of 16).
-static int launch_chunk(const nm_dose* h, uint64_t n) {
-  if (h->opt.chunk > 0) return h->chunk;
-  const uint64_t warps = (uint64_t)h->grid * (h->block / 32);
+static int launch_chunk(int chunk, uint64_t warps, uint64_t n) {
   const uint64_t share = n / (2 * warps) / 32 * 32;
-  return (int)std::min<uint64_t>(h->chunk, std::max<uint64_t>(share, 32));
+  return (int)std::min<uint64_t>(chunk, std::max<uint64_t>(share, 32));
 }
 
 static void apply_shape(nm_dose* h, const Shape& sh) {
@@ -622,7 +619,7 @@ static void apply_shape(nm_dose* h, const Shape& sh) {
   h->warp_agg = sh.warp_agg;
   h->regroup = sh.regroup;
   h->regroup_lanes = sh.lanes;
-  h->grid = grid_for_shape(h, sh, false);
+  h->grid = grid_for_shape(h, sh);
 }
 
 static nm_status autotune(nm_dose* h, Shape sh, bool free_block, bool free_chunk, bool free_agg,
@@ -659,8 +656,7 @@ static nm_status autotune(nm_dose* h, Shape sh, bool free_block, bool free_chunk
     TransportParams p = h->params(first, n_trial, 0x7475u);
     NM_CUDA(cudaMemsetAsync(h->work, 0, sizeof(unsigned), s), "autotune");
     NM_CUDA(cudaEventRecord(e0, s), "autotune");
-    NM_CUDA(launch_transport(p, h->grid, h->block, h->warp_agg, h->rayleigh, h->regroup, s, false,
-                             h->opt.history_sigma != 0),
+    NM_CUDA(launch_transport(p, h->grid, h->block, h->warp_agg, h->rayleigh, h->regroup, s, h->opt.history_sigma != 0),
             "autotune");
     NM_CUDA(cudaEventRecord(e1, s), "autotune");
     NM_CUDA(cudaEventSynchronize(e1), "autotune");
@@ -1002,6 +998,53 @@ static int launch_batches(uint64_t n, int B, int b0, int slots) {
   return std::max(k, 1);
 }
 
+// Enqueues n histories of h in B batches on stream s with the launch shape of
+// `like`: per group of batches one launch that tallies each batch in its own
+// slot, then one fold of the slots in batch order.  minv: the majorants
+// [2][kKnTable] to fly with, NULL = the handle's.  mark() is called before a
+// launch, after it and after its fold.
+static cudaError_t enqueue_run(nm_dose* h, uint64_t n, int B, uint64_t seed, const nm_dose* like, const float* minv,
+                               cudaStream_t s, const std::function<cudaError_t()>& mark) {
+  const uint64_t q = n / B, r = n % B;
+  uint64_t id = h->id_next;
+  cudaError_t e = cudaSuccess;
+  for (int b0 = 0; b0 < B && !e;) {
+    NvtxRange batch_range("batches");
+    const int k = launch_batches(n, B, b0, h->slots);
+    const uint32_t big = (uint32_t)std::min<uint64_t>(r > (uint64_t)b0 ? r - b0 : 0, (uint64_t)k);
+    const uint64_t total = q * k + big;
+    FoldParams fp = fold_params(h);
+    fp.n_slots = k;
+    for (int b = 0; b < k; ++b) fp.set_batch(b, q + ((uint32_t)b < big ? 1 : 0));
+    e = mark();
+    for (uint64_t done = 0; done < total && !e;) {
+      const uint64_t part = std::min<uint64_t>(total - done, 1ull << 31);
+      TransportParams p = h->params(id + done, part, seed);
+      if (k > 1) p.g.split = batch_split((uint32_t)k, big, (uint32_t)q);
+      if (minv) {
+        p.minv = minv;
+        p.minv_out = minv + kKnTable;
+      }
+      const int warps = like->block / 32;
+      p.chunk = like->opt.chunk > 0 ? like->chunk : launch_chunk(like->chunk, (uint64_t)like->grid * warps, part);
+      p.regroup_compton = p.regroup_refill = like->regroup_lanes;
+      // no more CTAs than have a chunk to take
+      const uint64_t want = (part + (uint64_t)p.chunk * warps - 1) / ((uint64_t)p.chunk * warps);
+      e = cudaMemsetAsync(h->work, 0, sizeof(unsigned), s);
+      if (!e)
+        e = launch_transport(p, (int)std::min<uint64_t>((uint64_t)like->grid, want), like->block, like->warp_agg,
+                             h->rayleigh, like->regroup, s, h->opt.history_sigma != 0);
+      done += part;
+    }
+    if (!e) e = mark();
+    if (!e) e = launch_fold(fp, s);
+    if (!e) e = mark();
+    id += total;
+    b0 += k;
+  }
+  return e;
+}
+
 nm_status nm_dose_run(nm_dose* h, uint64_t n, uint64_t seed) {
   NvtxRange range("nm_dose_run");
   if (!h) return fail(NM_ERR_ARG, "handle is NULL");
@@ -1017,54 +1060,30 @@ nm_status nm_dose_run(nm_dose* h, uint64_t n, uint64_t seed) {
   cudaStream_t s = h->stream;
   const nm_status es = ensure_slots(h, B);
   if (es != NM_OK) return es;
-  int groups = 0;
-  for (int b = 0; b < B; b += launch_batches(n, B, b, h->slots)) ++groups;
-  while ((int)h->ev.size() < 3 * groups) {
-    cudaEvent_t ev;
-    NM_CUDA(cudaEventCreate(&ev), "cudaEventCreate");
-    h->ev.push_back(ev);
-  }
   const bool was_dirty = h->dirty;      // a run before this one failed half-way
   h->dirty = true;
-  // Groups of batches: one launch that tallies each batch in its own slot, then
-  // one fold of the slots in batch order.
-  const uint64_t q = n / B, r = n % B;
-  for (int b0 = 0, g = 0; b0 < B; ++g) {
-    NvtxRange batch_range("batches");
-    const int k = launch_batches(n, B, b0, h->slots);
-    const uint32_t big = (uint32_t)std::min<uint64_t>(r > (uint64_t)b0 ? r - b0 : 0, (uint64_t)k);
-    const uint64_t total = q * k + big;
-    FoldParams fp = fold_params(h);
-    fp.n_slots = k;
-    for (int b = 0; b < k; ++b) fp.set_batch(b, q + ((uint32_t)b < big ? 1 : 0));
-    NM_CUDA(cudaEventRecord(h->ev[3 * g + 0], s), "cudaEventRecord");
-    for (uint64_t done = 0; done < total;) {
-      const uint64_t part = std::min<uint64_t>(total - done, 1ull << 31);
-      TransportParams p = h->params(h->id_next + done, part, seed);
-      if (k > 1) p.g.split = batch_split((uint32_t)k, big, (uint32_t)q);
-      p.chunk = launch_chunk(h, part);
-      NM_CUDA(cudaMemsetAsync(h->work, 0, sizeof(unsigned), s), "cudaMemsetAsync");
-      NM_CUDA(launch_transport(p, h->grid, h->block, h->warp_agg, h->rayleigh, h->regroup, s, false,
-                               h->opt.history_sigma != 0),
-              "transport launch");
-      done += part;
+  // per launch: transport start and end, fold end
+  size_t used = 0;
+  const cudaError_t e = enqueue_run(h, n, B, seed, h, nullptr, s, [&]() -> cudaError_t {
+    if (used == h->ev.size()) {
+      cudaEvent_t ev;
+      if (cudaError_t c = cudaEventCreate(&ev)) return c;
+      h->ev.push_back(ev);
     }
-    NM_CUDA(cudaEventRecord(h->ev[3 * g + 1], s), "cudaEventRecord");
-    NM_CUDA(launch_fold(fp, s), "fold launch");
-    NM_CUDA(cudaEventRecord(h->ev[3 * g + 2], s), "cudaEventRecord");
-    h->hist_next += total;
-    h->id_next += total;
-    h->n_batches += (uint64_t)k;
-    b0 += k;
-  }
+    return cudaEventRecord(h->ev[used++], s);
+  });
+  NM_CUDA(e, "nm_dose_run");
+  h->hist_next += n;
+  h->id_next += n;
+  h->n_batches += (uint64_t)B;
   uint32_t st = 0;
   NM_CUDA(cudaMemcpyAsync(&st, h->status, 4, cudaMemcpyDeviceToHost, s), "status read");
   NM_CUDA(cudaStreamSynchronize(s), "nm_dose_run");
   h->dirty = was_dirty;
-  for (int g = 0; g < groups; ++g) {
+  for (size_t g = 0; g < used; g += 3) {
     float ms = 0;
-    if (cudaEventElapsedTime(&ms, h->ev[3 * g], h->ev[3 * g + 1]) == cudaSuccess) h->transport_ms += ms;
-    if (cudaEventElapsedTime(&ms, h->ev[3 * g + 1], h->ev[3 * g + 2]) == cudaSuccess) h->fold_ms += ms;
+    if (cudaEventElapsedTime(&ms, h->ev[g], h->ev[g + 1]) == cudaSuccess) h->transport_ms += ms;
+    if (cudaEventElapsedTime(&ms, h->ev[g + 1], h->ev[g + 2]) == cudaSuccess) h->fold_ms += ms;
   }
   h->status_seen |= st;
   if (st) {
@@ -1078,10 +1097,11 @@ nm_status nm_dose_run(nm_dose* h, uint64_t n, uint64_t seed) {
 }
 
 // ---------------------------------------------------------------------------
-// Many patients in one launch: one persistent multi-patient transport launch in
-// which every warp drains per-patient work queues (moving on to the next
-// patient when one runs dry), every batch of every patient with a tally of its
-// own, then each patient's fold.
+// Many patients in one call: each patient's launches and folds go to one of a
+// few streams, so that a patient's transport fills the SMs that others' last
+// photons and folds leave, and small patients run side by side.  (One launch
+// over all patients' queues, whose lanes carried their patient, took 23.3 ms
+// for eight patients of 1e7; the patients' own launches take 14.2 ms, folds included.)
 // ---------------------------------------------------------------------------
 static bool same_physics(const nm_dose* a, const nm_dose* b) {
   if (a->n_mat != b->n_mat || a->rayleigh != b->rayleigh || a->e0 != b->e0 || a->cut != b->cut ||
@@ -1095,15 +1115,13 @@ static bool same_physics(const nm_dose* a, const nm_dose* b) {
   return true;
 }
 
-typedef std::tuple<int, int, long long, long long> BatchKey;
-static std::map<BatchKey, Shape> g_batch_tune;
+constexpr int kBatchStreams = 4;
 
 extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint64_t* n_decays,
                                        uint64_t seed) {
   NvtxRange range("nm_dose_run_batch");
   if (!hs || !n_decays || n < 1 || n > kMaxBatchPatients)
     return fail(NM_ERR_ARG, "need 1..%d handles and their decay counts", kMaxBatchPatients);
-  long long vox_sum = 0, vox_hash = 0;
   for (int i = 0; i < n; ++i) {
     if (!hs[i]) return fail(NM_ERR_ARG, "handle %d is NULL", i);
     for (int j = 0; j < i; ++j)
@@ -1118,8 +1136,6 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
     if (hs[i]->hist_next > lim || n_decays[i] > lim - hs[i]->hist_next ||
         hs[i]->id_next + n_decays[i] > (1ull << 62))
       return fail(NM_ERR_OVERFLOW, "handle %d: too many histories", i);
-    vox_sum += hs[i]->V;
-    vox_hash = vox_hash * 1000003 + hs[i]->V;
   }
   nm_dose* h0 = hs[0];
   cudaStream_t s = h0->stream;
@@ -1139,164 +1155,64 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
     minv[k] = m;
     minv[kKnTable + k] = mo;
   }
-  // Batches per launch: what every patient's batch tallies and 2^31 histories
-  // of each (its work counter) allow.
-  int slots = kMaxSlots;
+  for (int i = 0; i < n; ++i)
+    if (n_decays[i] / B + (n_decays[i] % B ? 1 : 0) >= (1ull << 31))
+      return fail(NM_ERR_ARG, "handle %d: batches above 2^31 histories", i);
   for (int i = 0; i < n; ++i) {
-    const nm_status es = ensure_slots(hs[i], B);
+    const nm_status es = ensure_slots(hs[i], (int)std::min<uint64_t>(B, n_decays[i]));
     if (es != NM_OK) return es;
-    slots = std::min(slots, hs[i]->slots);
   }
-  auto batches_at = [&](int b0) {
-    int k = B;
-    for (int i = 0; i < n; ++i)
-      if (n_decays[i]) k = std::min(k, launch_batches(n_decays[i], B, b0, slots));
-    return k;
-  };
-  int groups = 0;
-  for (int b0 = 0; b0 < B; b0 += batches_at(b0)) ++groups;
-  // Temporary device memory: the launches' patient tables, then the majorants,
-  // the work counters and the status word.
-  const size_t pat_bytes = (size_t)std::max(groups, 1) * n * sizeof(PatientGeom);
-  const size_t tmp_bytes = pat_bytes + 2 * kKnTable * sizeof(float) + (kMaxBatchPatients + 1) * sizeof(uint32_t);
-  static_assert(sizeof(PatientGeom) % 8 == 0, "what follows the patient tables stays aligned");
-  uint8_t* tmp = nullptr;
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  cudaError_t e;
+  float* d_minv = nullptr;
+  cudaStream_t st[kBatchStreams] = {};
+  cudaEvent_t e0 = nullptr, e1 = nullptr, join = nullptr;
   auto cleanup = [&]() {
-    cudaStreamSynchronize(s);           // nothing on the device may still use the buffer
-    if (e0) cudaEventDestroy(e0);
-    if (e1) cudaEventDestroy(e1);
-    dfree(tmp);
-  };
-  std::vector<PatientGeom> pat((size_t)groups * n);
-  if ((e = dalloc(&tmp, tmp_bytes))) return cuda_fail(e, "nm_dose_run_batch: set-up");
-  PatientGeom* const d_pat = (PatientGeom*)tmp;
-  float* const d_minv = (float*)(tmp + pat_bytes);
-  unsigned* const d_work = (unsigned*)(d_minv + 2 * kKnTable);
-  uint32_t* const d_status = d_work + kMaxBatchPatients;
-  std::vector<uint64_t> off(n, 0);
-  for (int b0 = 0, g = 0; b0 < B; ++g) {
-    const int k = batches_at(b0);
-    for (int i = 0; i < n; ++i) {
-      const uint64_t q = n_decays[i] / B, r = n_decays[i] % B;
-      const uint64_t big = std::min<uint64_t>(r > (uint64_t)b0 ? r - b0 : 0, (uint64_t)k), total = q * k + big;
-      if (k == 1 && total >= (1ull << 31)) { cleanup(); return fail(NM_ERR_ARG, "handle %d: batches above 2^31 histories", i); }
-      PatientGeom& G = pat[(size_t)g * n + i];
-      G = hs[i]->geom(hs[i]->id_next + off[i], total);
-      if (k > 1) G.split = batch_split((uint32_t)k, (uint32_t)big, (uint32_t)q);
-      G.work = d_work + i;
-      off[i] += total;
-    }
-    b0 += k;
-  }
-  if ((e = cudaMemcpyAsync(d_minv, minv.data(), 2 * kKnTable * sizeof(float), cudaMemcpyHostToDevice, s)) ||
-      (e = cudaMemsetAsync(d_status, 0, 4, s)) || (e = cudaStreamSynchronize(s)) || (e = cudaEventCreate(&e0)) ||
-      (e = cudaEventCreate(&e1))) {
-    cleanup();
-    return cuda_fail(e, "nm_dose_run_batch: set-up");
-  }
-  TransportParams p = h0->params(0, 0, seed);
-  p.minv = d_minv;
-  p.minv_out = d_minv + kKnTable;
-  p.status = d_status;
-  p.n_patients = n;
-
-  // Launch shape of the multi-patient kernel: the first handle's explicit
-  // options, else timed trials on this batch (cached per batch geometry).
-  Shape sh{h0->block, h0->chunk, h0->warp_agg, h0->regroup, h0->regroup_lanes};
-  const BatchKey key{h0->device, n, vox_sum, vox_hash};
-  bool have = false;
-  {
-    std::lock_guard<std::mutex> lock(g_tune_mu);
-    auto it = g_batch_tune.find(key);
-    if (it != g_batch_tune.end()) { sh = it->second; have = true; }
-  }
-  const bool free_shape = h0->opt.block_threads <= 0 || h0->opt.chunk <= 0 || h0->opt.regroup < 0;
-  if (!have && free_shape) {
-    // Trials on history ids above 2^62 of every patient, then cleared.
-    std::vector<PatientGeom> tp(n);
-    for (int i = 0; i < n; ++i) {
-      tp[i] = hs[i]->geom(1ull << 62, (1ull << 22) / n + 1);
-      tp[i].work = d_work + i;
-    }
-    if ((e = cudaMemcpy(d_pat, tp.data(), n * sizeof(PatientGeom), cudaMemcpyHostToDevice))) {
-      cleanup();
-      return cuda_fail(e, "batch autotune");
-    }
-    // Trials add to the handles' counters: keep them to restore afterwards.
-    std::vector<ull> saved((size_t)n * kCtrCount);
-    for (int i = 0; i < n && !e; ++i)
-      e = cudaMemcpy(&saved[(size_t)i * kCtrCount], hs[i]->counters, kCtrCount * sizeof(ull), cudaMemcpyDeviceToHost);
-    if (e) { cleanup(); return cuda_fail(e, "batch autotune"); }
-    float best = 1e30f;
-    Shape cand[] = {{128, 256, sh.warp_agg, 1, 12}, {256, 256, sh.warp_agg, 1, 12},
-                    {512, 256, sh.warp_agg, 1, 12}, {256, 64, sh.warp_agg, 1, 12},
-                    {256, 1024, sh.warp_agg, 1, 12}, {256, 256, sh.warp_agg, 1, 8},
-                    {256, 256, sh.warp_agg, 1, 16}, {256, 256, sh.warp_agg, 0, 12}};
-    Shape pick = sh;
-    for (int rep = 0; rep < 2; ++rep)
-      for (const Shape& c : cand) {
-        const int grid = grid_for_shape(h0, c, true);
-        if (grid <= 0) continue;
-        p.patients = d_pat;
-        p.chunk = c.chunk;
-        p.regroup_compton = p.regroup_refill = c.lanes;
-        cudaMemsetAsync(d_work, 0, n * sizeof(unsigned), s);
-        float ms = 0;
-        if ((e = cudaEventRecord(e0, s)) ||
-            (e = launch_transport(p, grid, c.block, c.warp_agg, h0->rayleigh, c.regroup, s, true)) ||
-            (e = cudaEventRecord(e1, s)) || (e = cudaEventSynchronize(e1)) ||
-            (e = cudaEventElapsedTime(&ms, e0, e1))) {
-          cleanup();
-          return cuda_fail(e, "batch autotune");
-        }
-        if (rep == 1 && ms < best) { best = ms; pick = c; }
+    for (cudaStream_t& c : st)
+      if (c) {
+        cudaStreamSynchronize(c);
+        cudaStreamDestroy(c);
       }
-    sh = pick;
-    for (int i = 0; i < n && !e; ++i) {
-      e = cudaMemsetAsync(hs[i]->tb, 0, hs[i]->V * sizeof(ull), s);
-      if (!e) e = cudaMemcpyAsync(hs[i]->counters, &saved[(size_t)i * kCtrCount], kCtrCount * sizeof(ull),
-                                  cudaMemcpyHostToDevice, s);
-    }
-    if (!e) e = cudaMemsetAsync(d_status, 0, 4, s);
-    if (!e) e = cudaStreamSynchronize(s);
-    if (e) { cleanup(); return cuda_fail(e, "batch autotune"); }
-    std::lock_guard<std::mutex> lock(g_tune_mu);
-    g_batch_tune[key] = sh;
+    cudaStreamSynchronize(s);           // nothing on the device may still use the buffer
+    for (cudaEvent_t c : {e0, e1, join})
+      if (c) cudaEventDestroy(c);
+    dfree(d_minv);
+  };
+  cudaError_t e = dalloc(&d_minv, 2 * kKnTable);
+  if (!e) e = cudaMemcpyAsync(d_minv, minv.data(), 2 * kKnTable * sizeof(float), cudaMemcpyHostToDevice, s);
+  if (!e) e = cudaEventCreate(&e0);
+  if (!e) e = cudaEventCreate(&e1);
+  if (!e) e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
+  const int n_streams = std::min(n, kBatchStreams);
+  if (!e) e = cudaEventRecord(e0, s);
+  for (int j = 0; j < n_streams && !e; ++j) {
+    e = cudaStreamCreateWithFlags(&st[j], cudaStreamNonBlocking);
+    if (!e) e = cudaStreamWaitEvent(st[j], e0, 0);
   }
-  const int grid = grid_for_shape(h0, sh, true);
-  if (grid <= 0) { cleanup(); return fail(NM_ERR_ARG, "multi-patient kernel cannot launch"); }
-  p.chunk = sh.chunk;
-  p.regroup_compton = p.regroup_refill = sh.lanes;
   std::vector<char> was_dirty(n);
   for (int i = 0; i < n; ++i) {
     was_dirty[i] = hs[i]->dirty;
     hs[i]->dirty = true;
   }
-  if (!(e = cudaMemcpyAsync(d_pat, pat.data(), pat.size() * sizeof(PatientGeom), cudaMemcpyHostToDevice, s)))
-    e = cudaEventRecord(e0, s);
-  for (int b0 = 0, g = 0; b0 < B && !e; ++g) {
-    const int k = batches_at(b0);
-    p.patients = d_pat + (size_t)g * n;
-    e = cudaMemsetAsync(d_work, 0, n * sizeof(unsigned), s);
-    if (!e) e = launch_transport(p, grid, sh.block, sh.warp_agg, h0->rayleigh, sh.regroup, s, true);
-    for (int i = 0; i < n && !e; ++i) {
-      const uint64_t q = n_decays[i] / B, r = n_decays[i] % B;
-      if (pat[(size_t)g * n + i].n_hist == 0) continue;
-      FoldParams fp = fold_params(hs[i]);
-      fp.n_slots = k;
-      for (int b = 0; b < k; ++b) fp.set_batch(b, q + ((uint64_t)(b0 + b) < r ? 1 : 0));
-      e = launch_fold(fp, s);
-    }
-    b0 += k;
+  // the launch shape is the first handle's
+  for (int i = 0; i < n && !e; ++i)
+    if (n_decays[i])
+      e = enqueue_run(hs[i], n_decays[i], (int)std::min<uint64_t>(B, n_decays[i]), seed, h0, d_minv,
+                      st[i % n_streams], [] { return cudaSuccess; });
+  for (int j = 0; j < n_streams && !e; ++j) {
+    e = cudaEventRecord(join, st[j]);
+    if (!e) e = cudaStreamWaitEvent(s, join, 0);
   }
   float ms = 0;
-  uint32_t flags = 0;
+  std::vector<uint32_t> flag(n, 0);
   if (!e) e = cudaEventRecord(e1, s);
-  if (!e) e = cudaMemcpyAsync(&flags, d_status, 4, cudaMemcpyDeviceToHost, s);
+  for (int i = 0; i < n && !e; ++i) e = cudaMemcpyAsync(&flag[i], hs[i]->status, 4, cudaMemcpyDeviceToHost, s);
   if (!e) e = cudaStreamSynchronize(s);
   if (!e) e = cudaEventElapsedTime(&ms, e0, e1);
+  uint32_t flags = 0;
+  for (int i = 0; i < n && !e; ++i)
+    if (flag[i]) {
+      flags |= flag[i];
+      e = cudaMemsetAsync(hs[i]->status, 0, 4, s);
+    }
   if (e) {
     cleanup();
     return cuda_fail(e, "nm_dose_run_batch");

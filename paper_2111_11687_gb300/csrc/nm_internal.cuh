@@ -115,7 +115,7 @@ __host__ __device__ __forceinline__ uint32_t batch_of(const BatchSplit& s, uint3
 }
 constexpr int kMaxSlots = 16;      // batches of one launch
 
-// Per-patient (per-grid) part of a transport launch.
+// The grid's part of a transport launch.
 struct PatientGeom {
   const uint32_t* vox;        // packed voxel: density bits with the low 3 bits = material
   const uint4* alias;         // {prob bits, voxel, alias voxel, 0}
@@ -144,9 +144,7 @@ struct PatientGeom {
 };
 
 struct TransportParams {
-  PatientGeom g;              // the patient of a single-patient launch
-  const PatientGeom* patients;  // multi-patient launch: n_patients entries (device memory)
-  int n_patients;
+  PatientGeom g;
   uint32_t* status;           // NM_DEV_* flags
   const float* kn;            // kKnTable nodes of N_A * sigma_KN(E)
   const float* minv;          // kKnTable bins: 1 / majorant (cm) on [E_i, E_i+1)
@@ -164,12 +162,11 @@ struct TransportParams {
   int max_steps;
   int regroup_compton;        // regrouped variant: lanes that must wait before a Compton pass
   int regroup_refill;         // regrouped variant: lanes that must wait before a refill pass
-  // History-by-history statistics (single-patient launches): per voxel the
+  // History-by-history statistics: per voxel the
   // 128-bit sum over histories of each history's squared total deposit.
   ull* s2h_lo;
   ull* s2h_hi;
-  // Decay of another radionuclide (single-patient launches, the nuclide
-  // variant): whether the annihilation pair is emitted, and the gamma lines
+  // Decay of another radionuclide (the nuclide variant): whether the annihilation pair is emitted, and the gamma lines
   // (energy, fixed-point energy, emission probability per decay).
   int annihilate;
   int n_gamma;
@@ -197,21 +194,19 @@ void set_error_message(const char* msg);
 nm_status check_problem(const nm_grid* g, const nm_materials* mt, const nm_options& o, const float* activity);
 
 // ---- launchers (host side), one translation unit each ---------------------
-// history: history-by-history statistics (needs !warp_agg and !multi); a
-// single-patient launch whose p.g.beta_tab is set runs the beta+ variant
-// (needs !warp_agg).
+// history: history-by-history statistics (needs !warp_agg); a launch whose
+// p.g.beta_tab is set runs the beta+ variant (needs !warp_agg).
 cudaError_t launch_transport(const TransportParams& p, int grid, int block, bool warp_agg,
-                             bool rayleigh, bool regroup, cudaStream_t s, bool multi = false,
-                             bool history = false);
-// True for a single-patient launch that needs the nuclide variant (a beta
-// spectrum, gamma lines or no annihilation pair).
+                             bool rayleigh, bool regroup, cudaStream_t s, bool history = false);
+// True for a launch that needs the nuclide variant (a beta spectrum, gamma
+// lines or no annihilation pair).
 bool nuclide_launch(const TransportParams& p);
 // Per-voxel time-integrated activity (trapezoid between time points, linear
 // uptake before the first, physical decay after the last), FP64 per voxel.
 cudaError_t launch_time_integral(const float* const* act, const double* t_s, int n, int64_t V, double tail_s,
                                  float* out, double* block_sums, int blocks, cudaStream_t s);
 int transport_max_blocks_per_sm(int block, bool warp_agg, bool rayleigh, bool regroup,
-                                bool multi = false, bool history = false, bool beta = false);
+                                bool history = false, bool beta = false);
 cudaError_t launch_check_philox(const uint4* ctr, const uint2* key, int64_t n, uint4* out,
                                 cudaStream_t s);
 // Klein-Nishina inverse-CDF table [kKnInvE][kKnInvU + 1] of x = 1 - cos(theta)

@@ -6,10 +6,9 @@
 // One persistent launch for all batches of a run, each with a tally of its own
 // (a launch's last photons then leave SMs idle once, not once per batch), in
 // two kernels.  In transport_ring_kernel
-// (annihilation photons or a point source, one patient: the default) a warp's
+// (annihilation photons or a point source: the default) a warp's
 // lanes hand photons on to each other through a ring in shared memory.  In
-// transport_kernel (several patients, history statistics, other decays, or
-// `regroup` off) each lane owns one photon; a lane whose photon ends takes the
+// transport_kernel (history statistics, other decays, or `regroup` off) each lane owns one photon; a lane whose photon ends takes the
 // decay's second photon or, with the rest of its warp, refills from a
 // warp-private pool of history ids that one lane grabs from a global counter
 // in chunks.  Every iteration of the loop is one flight step for every live
@@ -459,34 +458,28 @@ __device__ __forceinline__ void hist_add(const HistList& L, int& n, uint32_t v, 
   ++n;
 }
 
-template <bool WARP_AGG, bool RAYLEIGH, bool REGROUP, bool MULTI, bool HIST, bool BETA>
+template <bool WARP_AGG, bool RAYLEIGH, bool REGROUP, bool HIST, bool BETA>
 __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams p) {
-  static_assert(!HIST || (!WARP_AGG && !MULTI), "history statistics: one patient, lane-wise deposits");
-  static_assert(!BETA || (!WARP_AGG && !MULTI), "beta+ spectrum: one patient, lane-wise deposits");
+  static_assert(!HIST || !WARP_AGG, "history statistics: lane-wise deposits");
+  static_assert(!BETA || !WARP_AGG, "beta+ spectrum: lane-wise deposits");
   __shared__ float s_kn[kKnTable];
   __shared__ float s_minv[kKnTable];
   __shared__ float s_minv_out[kKnTable];
   __shared__ MaterialCoef s_mat[NM_MAX_MATERIALS];
   __shared__ Energy s_f0;
   __shared__ float s_inv0_out;              // 1 / majorant outside the box at e0
-  // Per patient, indexed by CounterSlot: the rare events (photo, cutoff,
-  // rayleigh, killed units) counted here directly, and (multi) the lanes'
-  // register counters handed over when a lane changes patient.
-  __shared__ unsigned long long s_cnt[MULTI ? kMaxBatchPatients : 1][10];  // [8]: positron, [9]: gamma units
-  __shared__ PatientGeom s_geom[MULTI ? kMaxBatchPatients : 1];
+  // Indexed by CounterSlot: the rare events (photo, cutoff, rayleigh, killed units).
+  __shared__ unsigned long long s_cnt[10];  // [8]: positron, [9]: gamma units
   extern __shared__ float s_site[];         // [9][blockDim]: decay site, photon A direction, photon B's
                                             // distance to its region boundary, a pending Compton's two words;
                                             // then the history lists (HIST) and the gamma origin (BETA)
-  const int n_pat = MULTI ? p.n_patients : 1;
   for (int i = threadIdx.x; i < kKnTable; i += blockDim.x) {
     s_kn[i] = p.kn[i];
     s_minv[i] = p.minv[i];
     s_minv_out[i] = p.minv_out[i];
   }
   if (threadIdx.x < NM_MAX_MATERIALS) s_mat[threadIdx.x] = p.mat[threadIdx.x];
-  for (int i = threadIdx.x; i < n_pat * 10; i += blockDim.x) s_cnt[i / 10][i % 10] = 0;
-  if (MULTI)
-    for (int i = threadIdx.x; i < n_pat; i += blockDim.x) s_geom[i] = p.patients[i];
+  if (threadIdx.x < 10) s_cnt[threadIdx.x] = 0;
   __syncthreads();
   if (threadIdx.x == 0) {
     s_f0 = energy_factors<RAYLEIGH>(p.e0, s_kn, s_minv, p.ln_e_lo, p.inv_dln_e);
@@ -505,12 +498,9 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
 
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t lt_mask = (1u << lane) - 1u;
-  // Warp-uniform work pool [pool_next, pool_end) of patient wp; the warps start
-  // spread over the patients.
+  // Warp-uniform work pool [pool_next, pool_end).
   uint32_t pool_next = 0, pool_end = 0;
-  int wp = MULTI ? (int)((blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) % n_pat) : 0;
-  int pi = 0;                            // this lane's patient
-  int cpi = 0;                           // patient the lane's counters belong to
+  const PatientGeom& G = p.g;
   bool done = false, alive = false, pending_b = false, pending_c = false;
   float px = 0.f, py = 0.f, pz = 0.f, ux = 0.f, uy = 0.f, uz = 0.f;
   float e = 0.f;
@@ -534,8 +524,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
       ux = -site[3 * nb]; uy = -site[4 * nb]; uz = -site[5 * nb];
       e = p.e0; qe = p.q_e0; f = s_f0;
       stream = kStreamPhotonB; ctr = 0; steps = 0;
-      const PatientGeom& GB = MULTI ? s_geom[pi] : p.g;
-      out = outside_box(GB, px, py, pz);
+      out = outside_box(G, px, py, pz);
       rem = site[6 * nb];
       if (out) f.inv_mubar = s_inv0_out;
     } else if (BETA && !alive && gmask) {
@@ -552,7 +541,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
       __sincosf(fmaf(kTwoPi, u01(rd.y), -3.14159265f), &sp, &cp);
       ux = sn * cp; uy = sn * sp; uz = c;
       e = p.gamma_e[j]; qe = p.gamma_q[j];
-      atomicAdd(&s_cnt[0][9], (ull)(uint32_t)qe);
+      atomicAdd(&s_cnt[9], (ull)(uint32_t)qe);
       out = outside_box(p.g, px, py, pz);
       f = energy_factors<RAYLEIGH>(e, s_kn, out ? s_minv_out : s_minv, p.ln_e_lo, p.inv_dln_e);
       rem = region_distance(p.g, out, px, py, pz, ux, uy, uz);
@@ -570,25 +559,16 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
       const uint32_t cnt = __popc(need);
       const uint32_t avail = pool_end - pool_next;
       uint32_t fresh = 0, fresh_end = 0;
-      int nwp = wp;
       if (avail < cnt) {
-        // Grab a chunk from the current patient's queue; a drained queue moves
-        // the warp on to the next patient.
         if (lane == 0) {
-          for (int t = 0; t < n_pat; ++t) {
-            const PatientGeom& Q = MULTI ? s_geom[nwp] : p.g;
-            const unsigned f0 = atomicAdd(Q.work, (unsigned)p.chunk);
-            if ((uint64_t)f0 < Q.n_hist) {
-              fresh = f0;
-              fresh_end = (uint32_t)min((uint64_t)f0 + (uint64_t)p.chunk, Q.n_hist);
-              break;
-            }
-            if (MULTI) nwp = nwp + 1 < n_pat ? nwp + 1 : 0;
+          const unsigned f0 = atomicAdd(G.work, (unsigned)p.chunk);
+          if ((uint64_t)f0 < G.n_hist) {
+            fresh = f0;
+            fresh_end = (uint32_t)min((uint64_t)f0 + (uint64_t)p.chunk, G.n_hist);
           }
         }
         fresh = __shfl_sync(kFull, fresh, 0);
         fresh_end = __shfl_sync(kFull, fresh_end, 0);
-        nwp = __shfl_sync(kFull, nwp, 0);
       }
       bool has = false;
       ull* cell = nullptr;
@@ -596,30 +576,16 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
         const uint32_t rank = __popc(need & lt_mask);
         uint32_t idx = 0;
         bool got = true;
-        int npi = wp;
         if (rank < avail) {
           idx = pool_next + rank;
         } else if (fresh + (rank - avail) < fresh_end) {
           idx = fresh + (rank - avail);
-          npi = nwp;
         } else {
           got = false;
           if (fresh_end == 0) done = true;   // every queue is drained
         }
         if (got) {
-          if (MULTI && npi != cpi) {
-            // counters belong to one patient: hand them over before switching
-            atomicAdd(&s_cnt[cpi][kCtrSteps], (ull)n_steps);
-            atomicAdd(&s_cnt[cpi][kCtrCompton], (ull)n_compton);
-            atomicAdd(&s_cnt[cpi][kCtrEscapes], (ull)n_esc);
-            atomicAdd(&s_cnt[cpi][kCtrEscapedUnits], escaped);
-            n_steps = n_compton = n_esc = 0;
-            escaped = 0;
-            cpi = npi;
-          }
-          pi = npi;
           if (HIST && hn) hist_flush(hl, hn, tal, p.s2h_lo, p.s2h_hi);   // the previous history ends
-          const PatientGeom& G = MULTI ? s_geom[pi] : p.g;
           tal = batch_tally(G, idx);
           const uint64_t h = G.hist_begin + idx;
           hlo = (uint32_t)h;
@@ -649,7 +615,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
                                     else
                                       atomicAdd(tal + v, (ull)dq);
                                   });
-            atomicAdd(&s_cnt[MULTI ? pi : 0][8], (ull)q0);
+            atomicAdd(&s_cnt[8], (ull)q0);
             if (!pair) escaped += (ull)q_left + (p.annihilate ? 2ull * (ull)(uint32_t)p.q_e0 : 0ull);
           }
           if (BETA && G.source_mode == NM_SOURCE_DECAY && G.q_positron > 0 && !p.annihilate) {
@@ -691,15 +657,13 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
       if (avail < cnt) {
         pool_next = min(fresh + (cnt - avail), fresh_end);
         pool_end = fresh_end;
-        wp = nwp;
       } else {
         pool_next += cnt;
       }
-      tally_flush<WARP_AGG>(cell, has, (uint32_t)(MULTI ? s_geom[pi].q_positron : p.g.q_positron), lane);
+      tally_flush<WARP_AGG>(cell, has, (uint32_t)G.q_positron, lane);
     }
     if (!__any_sync(kFull, alive || !done)) break;
 
-    const PatientGeom& G = MULTI ? s_geom[pi] : p.g;
     bool has = false;
     int dv = 0;
     uint32_t dq = 0;
@@ -712,7 +676,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
           pending_c = false;
           const uint32_t* words = reinterpret_cast<const uint32_t*>(site);
           compton<RAYLEIGH>(p, s_kn, out ? s_minv_out : s_minv, e, qe, f, ux, uy, uz, ctr, stream, hlo, hhi,
-                            alive, dq, flags, s_cnt[MULTI ? pi : 0], words[7 * nb], words[8 * nb]);
+                            alive, dq, flags, s_cnt, words[7 * nb], words[8 * nb]);
           rem = region_distance(G, out, px, py, pz, ux, uy, uz);
           has = true;
           dv = cv;
@@ -778,19 +742,19 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
             words[8 * nb] = rr.w;
           } else {
             compton<RAYLEIGH>(p, s_kn, out ? s_minv_out : s_minv, e, qe, f, ux, uy, uz, ctr, stream, hlo,
-                              hhi, alive, dq, flags, s_cnt[MULTI ? pi : 0], rr.z, rr.w);
+                              hhi, alive, dq, flags, s_cnt, rr.z, rr.w);
             rem = region_distance(G, out, px, py, pz, ux, uy, uz);
             has = true;
             dv = v;
           }
         } else if (t < scale * icp) {
-          atomicAdd(&s_cnt[MULTI ? pi : 0][kCtrPhoto], 1ull);
+          atomicAdd(&s_cnt[kCtrPhoto], 1ull);
           has = true;
           dv = v;
           dq = (uint32_t)qe;
           alive = false;
         } else if (RAYLEIGH && t < scale * fmaf(c.zr, f.s_r, icp)) {
-          atomicAdd(&s_cnt[MULTI ? pi : 0][kCtrRayleigh], 1ull);
+          atomicAdd(&s_cnt[kCtrRayleigh], 1ull);
           // Thomson angular shape (1 + cos^2)/2 by rejection; one block per trial.
           for (int trial = 0;; ++trial) {
             const uint4 r = draw(ctr, stream, hlo, hhi, p.key);
@@ -806,7 +770,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
         }
       }
       if (alive && steps >= p.max_steps) {
-        atomicAdd(&s_cnt[MULTI ? pi : 0][kCtrKilledUnits], (ull)qe);
+        atomicAdd(&s_cnt[kCtrKilledUnits], (ull)qe);
         flags |= NM_DEV_STEP_LIMIT;
         alive = false;
         pending_c = false;
@@ -821,12 +785,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
   if (HIST && hn) hist_flush(hl, hn, tal, p.s2h_lo, p.s2h_hi);
 
   // ---- counters ---------------------------------------------------------------
-  if (MULTI) {
-    atomicAdd(&s_cnt[cpi][kCtrSteps], (ull)n_steps);
-    atomicAdd(&s_cnt[cpi][kCtrCompton], (ull)n_compton);
-    atomicAdd(&s_cnt[cpi][kCtrEscapes], (ull)n_esc);
-    atomicAdd(&s_cnt[cpi][kCtrEscapedUnits], escaped);
-  } else {
+  {
     // warp sums, one atomic per warp per counter
     ull sm = warp_sum((ull)n_steps);
     if (lane == 0 && sm) atomicAdd(p.g.counters + kCtrSteps, sm);
@@ -840,12 +799,9 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
   const unsigned fl = __reduce_or_sync(kFull, flags);
   if (lane == 0 && fl) atomicOr(p.status, fl);
   __syncthreads();
-  for (int i = threadIdx.x; i < n_pat * 10; i += blockDim.x) {
-    const int q = i / 10, k = i % 10;   // k is the CounterSlot, 8 the positron and 9 the gamma units
-    if (s_cnt[q][k])
-      atomicAdd((MULTI ? s_geom[q].counters : p.g.counters) +
-                    (k < 8 ? k : k == 8 ? (int)kCtrPositronUnits : (int)kCtrGammaUnits),
-                s_cnt[q][k]);
+  if (threadIdx.x < 10 && s_cnt[threadIdx.x]) {
+    const int k = threadIdx.x;           // the CounterSlot; 8 the positron and 9 the gamma units
+    atomicAdd(p.g.counters + (k < 8 ? k : k == 8 ? (int)kCtrPositronUnits : (int)kCtrGammaUnits), s_cnt[k]);
   }
 }
 
@@ -1450,43 +1406,35 @@ size_t transport_smem(int block, bool history, bool beta) {
   return ((size_t)9 + (history ? 2 * kHistVoxels : 0) + (beta ? 3 : 0)) * block * sizeof(float);
 }
 
-template <bool A, bool R, bool G, bool M, bool H, bool B = false>
+template <bool A, bool R, bool G, bool H, bool B = false>
 void* kernel_ptr() {
-  return (void*)transport_kernel<A, R, G, M, H, B>;
+  return (void*)transport_kernel<A, R, G, H, B>;
 }
 
-template <bool G, bool M>
-void* pick_m(bool a, bool r) {
-  if (a) return r ? kernel_ptr<true, true, G, M, false>() : kernel_ptr<true, false, G, M, false>();
-  return r ? kernel_ptr<false, true, G, M, false>() : kernel_ptr<false, false, G, M, false>();
+template <bool H, bool B>
+void* pick_lanes(bool r, bool g) {
+  if (r) return g ? kernel_ptr<false, true, true, H, B>() : kernel_ptr<false, true, false, H, B>();
+  return g ? kernel_ptr<false, false, true, H, B>() : kernel_ptr<false, false, false, H, B>();
 }
 
-template <bool H>
-void* pick_beta(bool r, bool g) {
-  if (r) return g ? kernel_ptr<false, true, true, false, H, true>() : kernel_ptr<false, true, false, false, H, true>();
-  return g ? kernel_ptr<false, false, true, false, H, true>() : kernel_ptr<false, false, false, false, H, true>();
-}
-
-// History statistics and the beta+ spectrum exist only without warp
-// aggregation and for one patient.
-void* pick(bool a, bool r, bool g, bool m, bool h, bool beta) {
-  if (beta) {
-    if (a || m) return nullptr;
-    return h ? pick_beta<true>(r, g) : pick_beta<false>(r, g);
+// The lane kernel.  History statistics and the beta+ spectrum exist only
+// without warp aggregation; without either, regrouped launches are the ring
+// kernel's.
+void* pick(bool a, bool r, bool g, bool h, bool beta) {
+  if (beta || h) {
+    if (a) return nullptr;
+    if (!beta) return pick_lanes<true, false>(r, g);
+    return h ? pick_lanes<true, true>(r, g) : pick_lanes<false, true>(r, g);
   }
-  if (h) {
-    if (a || m) return nullptr;
-    if (r) return g ? kernel_ptr<false, true, true, false, true>() : kernel_ptr<false, true, false, false, true>();
-    return g ? kernel_ptr<false, false, true, false, true>() : kernel_ptr<false, false, false, false, true>();
-  }
-  if (m) return g ? pick_m<true, true>(a, r) : pick_m<false, true>(a, r);
-  return g ? nullptr : pick_m<false, false>(a, r);   // one patient, regrouped: the ring kernel
+  if (g) return nullptr;
+  if (a) return r ? kernel_ptr<true, true, false, false>() : kernel_ptr<true, false, false, false>();
+  return r ? kernel_ptr<false, true, false, false>() : kernel_ptr<false, false, false, false>();
 }
 
-// The ring kernel runs every single-patient regrouped launch of annihilation
+// The ring kernel runs every regrouped launch of annihilation
 // photons (or a point source) without history statistics: 1e8 decays on the
 // benchmark phantom take 13.2 ms on it and 30.5 ms on the lane kernel.
-bool use_ring(bool regroup, bool multi, bool history, bool beta) { return regroup && !multi && !history && !beta; }
+bool use_ring(bool regroup, bool history, bool beta) { return regroup && !history && !beta; }
 
 void* pick_ring(bool a, bool general) {
   if (a) return general ? (void*)transport_ring_kernel<true, true> : (void*)transport_ring_kernel<true, false>;
@@ -1504,11 +1452,11 @@ bool nuclide_launch(const TransportParams& p) {
 }
 
 cudaError_t launch_transport(const TransportParams& p, int grid, int block, bool warp_agg,
-                             bool rayleigh, bool regroup, cudaStream_t s, bool multi, bool history) {
-  const bool beta = !multi && nuclide_launch(p);
-  const bool ring = use_ring(regroup, multi, history, beta);
+                             bool rayleigh, bool regroup, cudaStream_t s, bool history) {
+  const bool beta = nuclide_launch(p);
+  const bool ring = use_ring(regroup, history, beta);
   const bool general = rayleigh || !p.kn_inv;
-  void* fn = ring ? pick_ring(warp_agg, general) : pick(warp_agg, rayleigh, regroup, multi, history, beta);
+  void* fn = ring ? pick_ring(warp_agg, general) : pick(warp_agg, rayleigh, regroup, history, beta);
   if (!fn) return cudaErrorInvalidValue;
   void* args[] = {(void*)&p};
   // the history lists and the rings take the static + dynamic total past the
@@ -1520,11 +1468,10 @@ cudaError_t launch_transport(const TransportParams& p, int grid, int block, bool
   return e;
 }
 
-int transport_max_blocks_per_sm(int block, bool warp_agg, bool rayleigh, bool regroup, bool multi, bool history,
-                                bool beta) {
+int transport_max_blocks_per_sm(int block, bool warp_agg, bool rayleigh, bool regroup, bool history, bool beta) {
   int n = 0;
-  const bool ring = use_ring(regroup, multi, history, beta);
-  void* fn = ring ? pick_ring(warp_agg, rayleigh) : pick(warp_agg, rayleigh, regroup, multi, history, beta);
+  const bool ring = use_ring(regroup, history, beta);
+  void* fn = ring ? pick_ring(warp_agg, rayleigh) : pick(warp_agg, rayleigh, regroup, history, beta);
   const size_t smem = ring ? ring_smem(block, rayleigh) : transport_smem(block, history, beta);
   if (!fn || cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, block, smem) != cudaSuccess) {
