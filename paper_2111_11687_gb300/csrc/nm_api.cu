@@ -371,6 +371,10 @@ struct nm_dose {
     for (auto e : ev) cudaEventDestroy(e);
   }
 
+  int kind() const {
+    return nuclide_kind(opt.source_mode == NM_SOURCE_DECAY, beta_tab != nullptr, annihilate != 0, n_gamma);
+  }
+
   PatientGeom geom(uint64_t first, uint64_t n) const {
     PatientGeom g;
     memset(&g, 0, sizeof g);
@@ -600,7 +604,7 @@ static std::map<TuneKey, Shape> g_tune_cache;
 
 static int grid_for_shape(const nm_dose* h, const Shape& sh) {
   return h->sms * transport_max_blocks_per_sm(sh.block, sh.warp_agg, h->rayleigh, sh.regroup,
-                                              h->opt.history_sigma != 0, h->nuclide);
+                                              h->opt.history_sigma != 0, h->kind());
 }
 
 // Histories per work grab of a launch of n: the handle's chunk, but where it is
@@ -627,7 +631,7 @@ static nm_status autotune(nm_dose* h, Shape sh, bool free_block, bool free_chunk
   const TuneKey key{h->device, h->nx, h->ny, h->nz, h->opt.source_mode, h->rayleigh,
                     (free_block ? 1 : 0) | (free_chunk ? 2 : 0) | (free_agg ? 4 : 0) |
                         (free_regroup ? 8 : 0) | (free_lanes ? 16 : 0) | (h->opt.history_sigma ? 32 : 0) |
-                        (h->nuclide ? 64 : 0),
+                        ((h->kind() + 1) << 6),
                     free_block ? 0 : sh.block, free_chunk ? 0 : sh.chunk, free_agg ? 0 : sh.warp_agg,
                     free_regroup ? 0 : sh.regroup, free_lanes ? 0 : sh.lanes};
   {
@@ -677,7 +681,7 @@ static nm_status autotune(nm_dose* h, Shape sh, bool free_block, bool free_chunk
   };
   // The ring kernel regroups by itself, 32 photons at a time, so it has no lane
   // count to choose, and regrouping off (the lane kernel) is never faster.
-  const bool ring = !h->opt.history_sigma && !h->nuclide && sh.regroup;
+  const bool ring = !h->opt.history_sigma && h->kind() >= 0 && sh.regroup;
   for (int pass = 0; pass < 2 && st == NM_OK; ++pass) {
     if ((free_regroup || free_lanes) && !ring) {
       const int lanes[] = {8, 12, 16};

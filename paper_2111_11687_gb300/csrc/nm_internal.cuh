@@ -198,15 +198,16 @@ nm_status check_problem(const nm_grid* g, const nm_materials* mt, const nm_optio
 // p.g.beta_tab is set runs the beta+ variant (needs !warp_agg).
 cudaError_t launch_transport(const TransportParams& p, int grid, int block, bool warp_agg,
                              bool rayleigh, bool regroup, cudaStream_t s, bool history = false);
-// True for a launch that needs the nuclide variant (a beta spectrum, gamma
-// lines or no annihilation pair).
-bool nuclide_launch(const TransportParams& p);
+// Kind of decay that a launch transports, for the choice of its kernel: 0 an
+// annihilation pair from the decay site (or a point source's photon), 1 from
+// the end of a positron's track, 2 gamma lines, -1 a pair and gamma lines.
+int nuclide_kind(bool decay, bool beta_track, bool annihilate, int n_gamma);
 // Per-voxel time-integrated activity (trapezoid between time points, linear
 // uptake before the first, physical decay after the last), FP64 per voxel.
 cudaError_t launch_time_integral(const float* const* act, const double* t_s, int n, int64_t V, double tail_s,
                                  float* out, double* block_sums, int blocks, cudaStream_t s);
 int transport_max_blocks_per_sm(int block, bool warp_agg, bool rayleigh, bool regroup,
-                                bool history = false, bool beta = false);
+                                bool history = false, int nuclide = 0);
 cudaError_t launch_check_philox(const uint4* ctr, const uint2* key, int64_t n, uint4* out,
                                 cudaStream_t s);
 // Klein-Nishina inverse-CDF table [kKnInvE][kKnInvU + 1] of x = 1 - cos(theta)

@@ -859,15 +859,34 @@ struct WarpStore {
   uint2 aux[kRing];
   float2 site_rem[kSiteQueue];
 };
-struct WarpStoreGeneral : WarpStore {
+struct GenStore {
   uint2 gen[kRing];             // flight steps (the counter also counts other draws), Rayleigh factor
 };
-static_assert(sizeof(WarpStore) % 16 == 0 && sizeof(WarpStoreGeneral) % 16 == 0, "warps' stores stay 16-byte aligned");
+// Gamma lines (kGammas): the queue holds single photons, which differ in
+// energy: s_c, s_pe and the majorants of each, and in the place of site_rem
+// its energy and its counter word.  More photons than the queue holds wait as
+// (history, lines still to be emitted).
+struct GammaStore {
+  float4 site_mid[kSiteQueue];
+  uint2 defer[kSiteQueue];
+};
 
-template <bool GENERAL>
-struct StoreOf { typedef WarpStore type; };
-template <>
-struct StoreOf<true> { typedef WarpStoreGeneral type; };
+// What a decay gives (nuclide_kind): the annihilation pair of a positron that
+// stays where it is (or a point source's photon), of one that is tracked, or
+// gamma lines (and a tracked or local beta particle).
+enum Nuclide { kPair = 0, kTracked = 1, kGammas = 2 };
+
+// Layout of a warp's store: the parts its variant needs, one after the other.
+template <bool GENERAL, int NUC>
+struct StoreOf {
+  static constexpr uint32_t kGen = sizeof(WarpStore);
+  static constexpr uint32_t kGamma = kGen + (GENERAL ? sizeof(GenStore) : 0);
+  static constexpr uint32_t kBytes = kGamma + (NUC == kGammas ? sizeof(GammaStore) : 0);
+  static_assert(kBytes % 16 == 0 && kGamma % 16 == 0, "warps' stores stay 16-byte aligned");
+};
+// The Philox counter word of a gamma line's photon: its stream above the counter.
+constexpr int kStreamShift = 27;
+constexpr uint32_t kCtrMask = (1u << kStreamShift) - 1u;
 
 // Shared-memory accesses by 32-bit address (the compiler forms the address of
 // a shared array anew at every use).
@@ -930,11 +949,16 @@ static_assert(sizeof(RingTables) % 16 == 0, "the warps' stores follow");
 
 // GENERAL: Rayleigh scattering and Kahn's sampler, whose trials draw from the
 // photon's counter; otherwise the counter is the number of flight steps.
-template <bool WARP_AGG, bool GENERAL>
+template <bool WARP_AGG, bool GENERAL, int NUC>
 __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportParams p) {
-  typedef typename StoreOf<GENERAL>::type Store;
+  typedef StoreOf<GENERAL, NUC> Store;
+  static_assert(NUC == kPair || !WARP_AGG, "tracks deposit lane by lane");
+  constexpr bool GAMMAS = NUC == kGammas;
   __shared__ RingEnergy s_f0;                  // at the source energy
-  __shared__ unsigned long long s_cnt[12];     // [0..7]: CounterSlot; photons started, killed; energy deposited
+  // [0..7]: CounterSlot; photons started, killed; energy they deposited; of
+  // decays: energy of the beta particles, of the gamma lines, taken out of the
+  // grid by tracks (with the photons that then do not start)
+  __shared__ unsigned long long s_cnt[14];
   extern __shared__ __align__(16) unsigned char s_dyn[];   // tables, then a Store per warp
   RingTables& tb = *reinterpret_cast<RingTables*>(s_dyn);
   for (int i = threadIdx.x; i < kKnTable; i += blockDim.x) {
@@ -948,24 +972,27 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
   }
   if (threadIdx.x < kMaxSlots)
     tb.next[threadIdx.x] = threadIdx.x + 1 < p.g.split.slots ? p.g.split.start(threadIdx.x + 1) : 0xffffffffu;
-  if (threadIdx.x < 12) s_cnt[threadIdx.x] = 0;
+  if (threadIdx.x < 14) s_cnt[threadIdx.x] = 0;
   __syncthreads();
   uint32_t tables, store;                // volatile: kept, not formed again at every use
   asm volatile("mov.u32 %0, %1;" : "=r"(tables) : "r"((uint32_t)__cvta_generic_to_shared(s_dyn)));
   asm volatile("mov.u32 %0, %1;"
                : "=r"(store)
-               : "r"(tables + (uint32_t)sizeof(RingTables) + (threadIdx.x >> 5) * (uint32_t)sizeof(Store)));
+               : "r"(tables + (uint32_t)sizeof(RingTables) + (threadIdx.x >> 5) * Store::kBytes));
   const uint32_t tab = tables + offsetof(RingTables, tab), mat = tables + offsetof(RingTables, mat),
                  zr = tables + offsetof(RingTables, zr), next = tables + offsetof(RingTables, next);
   if (threadIdx.x == 0) s_f0 = ring_energy<GENERAL>(p.e0, tab, p.ln_e_lo, p.inv_dln_e);
   __syncthreads();
-  constexpr int kBorn = 8, kKilled = 9, kDeposit = 10;
+  constexpr int kBorn = 8, kKilled = 9, kDeposit = 10, kBeta = 11, kGamma = 12, kLost = 13;
 
   const uint32_t lane = threadIdx.x & 31u;
   uint32_t lt_mask;                      // volatile: kept, not fetched again at every use
   asm volatile("mov.u32 %0, %%lanemask_lt;" : "=r"(lt_mask));
 #define RING_AT(word, slot) (store + (uint32_t)offsetof(WarpStore, word) + 16u * (slot))
-#define RING_AT8(word, slot) (store + (uint32_t)offsetof(Store, word) + 8u * (slot))
+#define RING_AT8(word, slot) (store + (uint32_t)offsetof(WarpStore, word) + 8u * (slot))
+#define RING_GEN(slot) (store + Store::kGen + 8u * (slot))
+#define GAMMA_MID(slot) (store + Store::kGamma + (uint32_t)offsetof(GammaStore, site_mid) + 16u * (slot))
+#define GAMMA_DEFER(slot) (store + Store::kGamma + (uint32_t)offsetof(GammaStore, defer) + 8u * (slot))
   sts1(RING_AT(pos, lane) + 12, 0.0f);   // every slot starts empty
   sts1(RING_AT(pos, 32 + lane) + 12, 0.0f);
   __syncwarp();
@@ -978,7 +1005,8 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
   uint32_t pool_next = 0, pool_end = 0;  // histories of the launch grabbed and not yet sampled
   bool drained = false;                  // every history has been handed out
   uint32_t n_born = 0, n_compton = 0;
-  const bool pairs = p.g.source_mode == NM_SOURCE_DECAY;   // two photons per history
+  const bool pairs = NUC == kTracked || (NUC == kPair && p.g.source_mode == NM_SOURCE_DECAY);   // two photons per entry
+  bool deferred = false;                 // lines of sampled decays are still to be emitted
   // this lane's photon (none while e = 0; photon B while e < 0)
   float px = 0.f, py = 0.f, pz = 0.f, ux = 0.f, uy = 0.f, uz = 0.f, e = 0.f, rem = 0.f;
   float s_c = 0.f, s_pe = 0.f, s_r = 0.f, maj = 1.f, maj2 = 1.f;
@@ -987,6 +1015,8 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
   uint32_t n_steps = 0;                  // flight steps of the photons this lane saw end
   ull deposit = 0;                       // energy of the deposits this lane made
 
+  // Flight steps from the counter word: a gamma line's photon drew its direction first.
+  auto steps_of = [](uint32_t c) -> uint32_t { return GAMMAS ? (c & kCtrMask) - 1u : c; };
   // Tally cell of voxel v in the batch of history idx of the launch (batch_of,
   // from the table of batch ends; all batches' voxels count below 2^32).
   auto tally_cell = [&](uint32_t idx, uint32_t v) -> ull* {
@@ -1004,8 +1034,10 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
       x = kn_table_x(p, e1, rk);
     } else {
       const uint32_t clo = __float_as_uint(cd.w);
-      x = kahn_x(e1 * kInvElectronMassMeV, cctr, ce < 0.0f ? kStreamPhotonB : kStreamPhotonA, clo,
-                 h0_hi + (clo < h0 ? 1u : 0u), p.key, rp, flags);
+      uint32_t cnt = GAMMAS ? cctr & kCtrMask : cctr;
+      const uint32_t stream = GAMMAS ? cctr >> kStreamShift : ce < 0.0f ? kStreamPhotonB : kStreamPhotonA;
+      x = kahn_x(e1 * kInvElectronMassMeV, cnt, stream, clo, h0_hi + (clo < h0 ? 1u : 0u), p.key, rp, flags);
+      cctr = GAMMAS ? (cctr & ~kCtrMask) | cnt : cnt;
     }
     const float e2 = __fdividef(e1, fmaf(e1 * kInvElectronMassMeV, x, 1.0f));
     rotate(cd.x, cd.y, cd.z, 1.0f - x, fmaf(kTwoPi, u01(rp), -3.14159265f));
@@ -1039,8 +1071,8 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
       sts1(RING_AT(pos, i) + 12, ce);
       if (ce == 0.0f) {
         gone = true;
-        if constexpr (GENERAL) n_steps += __float_as_uint(lds1(RING_AT8(gen, i)));
-        else n_steps += __float_as_uint(lds1(RING_AT8(aux, i)));
+        if constexpr (GENERAL) n_steps += __float_as_uint(lds1(RING_GEN(i)));
+        else n_steps += steps_of(__float_as_uint(lds1(RING_AT8(aux, i))));
       } else {
         const RingEnergy f = ring_energy<GENERAL>(fabsf(ce), tab, p.ln_e_lo, p.inv_dln_e);
         const bool cout = cm.w < 0.0f;
@@ -1050,7 +1082,7 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
         sts1(RING_AT8(aux, i) + 4, cout ? f.maj_in : f.maj_out);
         if constexpr (GENERAL) {
           sts1(RING_AT8(aux, i), __uint_as_float(cctr));
-          sts1(RING_AT8(gen, i) + 4, f.s_r);
+          sts1(RING_GEN(i) + 4, f.s_r);
         }
       }
     }
@@ -1070,62 +1102,143 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
     s_c = nm.x; s_pe = nm.y; maj = nm.z; rem = nm.w;
     ctr = __float_as_uint(na.x); maj2 = na.y;
     if constexpr (GENERAL) {
-      const float2 g = lds2(RING_AT8(gen, i));
+      const float2 g = lds2(RING_GEN(i));
       steps = __float_as_uint(g.x);
       s_r = g.y;
     }
   };
 
   // ---- site queue: 32 new decays, one per lane --------------------------------
+  // Adds the warp's q (below 2^31 each) to a shared counter.
+  auto add_units = [&](int slot, uint32_t q) {
+    const ull sum = (ull)__reduce_add_sync(kFull, q & 0xffffu) + ((ull)__reduce_add_sync(kFull, q >> 16) << 16);
+    if (lane == 0 && sum) atomicAdd(&s_cnt[slot], sum);
+  };
   auto sample_sites = [&]() {
-    const uint32_t avail = pool_end - pool_next;
-    uint32_t fresh = 0, fresh_end = 0;
-    if (avail < 32) {
-      if (lane == 0) {
-        const unsigned f0 = atomicAdd(p.g.work, (unsigned)p.chunk);
-        if ((uint64_t)f0 < p.g.n_hist) {
-          fresh = f0;
-          fresh_end = (uint32_t)min((uint64_t)f0 + (uint64_t)p.chunk, p.g.n_hist);
-        }
-      }
-      fresh = __shfl_sync(kFull, fresh, 0);
-      fresh_end = __shfl_sync(kFull, fresh_end, 0);
-    }
-    uint32_t idx = 0;
+    uint32_t idx = 0, lines = 0;
     bool got = true;
-    if (lane < avail) {
-      idx = pool_next + lane;
-    } else if (fresh + (lane - avail) < fresh_end) {
-      idx = fresh + (lane - avail);
+    if (!(GAMMAS && deferred)) {
+      const uint32_t avail = pool_end - pool_next;
+      uint32_t fresh = 0, fresh_end = 0;
+      if (avail < 32) {
+        if (lane == 0) {
+          const unsigned f = atomicAdd(p.g.work, (unsigned)p.chunk);
+          if ((uint64_t)f < p.g.n_hist) {
+            fresh = f;
+            fresh_end = (uint32_t)min((uint64_t)f + (uint64_t)p.chunk, p.g.n_hist);
+          }
+        }
+        fresh = __shfl_sync(kFull, fresh, 0);
+        fresh_end = __shfl_sync(kFull, fresh_end, 0);
+      }
+      if (lane < avail) {
+        idx = pool_next + lane;
+      } else if (fresh + (lane - avail) < fresh_end) {
+        idx = fresh + (lane - avail);
+      } else {
+        got = false;
+      }
+      if (avail < 32) {
+        pool_next = min(fresh + (32u - avail), fresh_end);
+        pool_end = fresh_end;
+        drained = fresh_end == 0;
+      } else {
+        pool_next += 32;
+      }
     } else {
-      got = false;
+      const float2 d = lds2(GAMMA_DEFER(lane));
+      idx = __float_as_uint(d.x);
+      lines = __float_as_uint(d.y);
+      got = lines != 0u;
     }
-    if (avail < 32) {
-      pool_next = min(fresh + (32u - avail), fresh_end);
-      pool_end = fresh_end;
-      drained = fresh_end == 0;
-    } else {
-      pool_next += 32;
-    }
+    const uint64_t h = p.g.hist_begin + idx;
+    const uint32_t slo = (uint32_t)h, shi = (uint32_t)(h >> 32);
     bool has = false;
     ull* cell = nullptr;
+    Site st{};
     if (got) {
-      const uint64_t h = p.g.hist_begin + idx;
-      const Site st = sample_site(p.g, p.key, (uint32_t)h, (uint32_t)(h >> 32));
-      const bool o = outside_box(p.g, st.x, st.y, st.z);
-      float ra, rb;
-      region_distance_pair(p.g, o, st.x, st.y, st.z, st.u, st.v_, st.w, ra, rb);
-      sts4(RING_AT(site_pos, lane), st.x, st.y, st.z, __uint_as_float((uint32_t)h));
-      sts4(RING_AT(site_dir, lane), st.u, st.v_, st.w, ra);
-      sts2(RING_AT8(site_rem, lane), rb, o ? -1.0f : 1.0f);
+      st = sample_site(p.g, p.key, slo, shi);
       if (pairs) {
         has = p.g.q_positron > 0;
         cell = tally_cell(idx, (uint32_t)st.v);
       }
     }
+    float sx = st.x, sy = st.y, sz = st.z;   // where the photons start: the decay, or the end of the positron's track
+    if constexpr (NUC != kPair) {
+      uint32_t q0 = 0, q_left = 0;
+      bool stays = true;
+      if (got && !(GAMMAS && deferred)) {
+        if constexpr (GAMMAS) {
+          uint32_t gc = 0;
+          for (int j0 = 0; j0 < p.n_gamma; j0 += 4) {
+            const uint4 rg = draw(gc, kStreamGammaSelect, slo, shi, p.key);
+            const uint32_t w4[4] = {rg.x, rg.y, rg.z, rg.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              if (j0 + k < p.n_gamma && u01(w4[k]) < p.gamma_y[j0 + k]) lines |= 1u << (j0 + k);
+          }
+          has = p.g.q_positron > 0;
+          cell = tally_cell(idx, (uint32_t)st.v);
+        }
+        if (NUC == kTracked || p.g.beta_tab) {
+          ull* const tal = tally_cell(idx, 0u);
+          float tx = st.x, ty = st.y, tz = st.z;
+          stays = positron_track(p.g, p.key, slo, shi, st.v, tx, ty, tz, q0, q_left,
+                                 [&](int v, uint32_t dq) { atomicAdd(tal + v, (ull)dq); });
+          if (NUC == kTracked) {
+            sx = tx; sy = ty; sz = tz;
+          }
+        }
+      }
+      add_units(kBeta, q0);
+      if (!stays) atomicAdd(&s_cnt[kLost], (ull)q_left + (NUC == kTracked ? 2ull * (ull)(uint32_t)p.q_e0 : 0ull));
+      if (NUC == kTracked) got = got && stays;
+    }
     tally_flush<WARP_AGG>(cell, has, (uint32_t)p.g.q_positron, lane);
+    const bool o = outside_box(p.g, sx, sy, sz);
     s_next = 0;
-    s_left = (uint32_t)__popc(__ballot_sync(kFull, got)) << (pairs ? 1 : 0);   // lanes 0 .. got - 1
+    if constexpr (GAMMAS) {
+      // one photon per lane and round, as far as the queue goes
+      s_left = 0;
+      for (;;) {
+        const unsigned m = __ballot_sync(kFull, lines != 0u);
+        if (m == 0u || s_left == kSiteQueue) break;
+        const uint32_t slot = s_left + __popc(m & lt_mask);
+        uint32_t q = 0;
+        if (lines && slot < kSiteQueue) {
+          const int j = __ffs(lines) - 1;
+          lines &= lines - 1;
+          uint32_t c = 0;
+          const uint4 rd = draw(c, kStreamGamma0 + (uint32_t)j, slo, shi, p.key);
+          const float cz = fmaf(2.0f, u01(rd.x), -1.0f);
+          const float sn = sqrtf(fmaxf(0.0f, fmaf(-cz, cz, 1.0f)));
+          float sp, cp;
+          __sincosf(fmaf(kTwoPi, u01(rd.y), -3.14159265f), &sp, &cp);
+          const float gx = sn * cp, gy = sn * sp, ge = p.gamma_e[j];
+          q = (uint32_t)p.gamma_q[j];
+          const RingEnergy f = ring_energy<GENERAL>(ge, tab, p.ln_e_lo, p.inv_dln_e);
+          sts4(RING_AT(site_pos, slot), sx, sy, sz, __uint_as_float(slo));
+          sts4(RING_AT(site_dir, slot), gx, gy, cz, region_distance(p.g, o, sx, sy, sz, gx, gy, cz));
+          sts2(RING_AT8(site_rem, slot), ge, __uint_as_float(((kStreamGamma0 + (uint32_t)j) << kStreamShift) | c));
+          sts4(GAMMA_MID(slot), f.s_c, f.s_pe, o ? f.maj_out : f.maj_in, o ? f.maj_in : f.maj_out);
+        }
+        add_units(kGamma, q);
+        s_left = min(s_left + (uint32_t)__popc(m), (uint32_t)kSiteQueue);
+      }
+      deferred = __any_sync(kFull, lines != 0u);
+      if (deferred) sts2(GAMMA_DEFER(lane), __uint_as_float(idx), __uint_as_float(lines));
+    } else {
+      const unsigned m = __ballot_sync(kFull, got);
+      if (got) {
+        const uint32_t slot = __popc(m & lt_mask);
+        float ra, rb;
+        region_distance_pair(p.g, o, sx, sy, sz, st.u, st.v_, st.w, ra, rb);
+        sts4(RING_AT(site_pos, slot), sx, sy, sz, __uint_as_float(slo));
+        sts4(RING_AT(site_dir, slot), st.u, st.v_, st.w, ra);
+        sts2(RING_AT8(site_rem, slot), rb, o ? -1.0f : 1.0f);
+      }
+      s_left = (uint32_t)__popc(m) << (pairs ? 1 : 0);
+    }
     n_born += s_left;
     __syncwarp();
   };
@@ -1139,8 +1252,10 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
     const bool fly = e != 0.0f;
     // words x and y of the step's block; z and w serve the Compton angle if
     // the step finds a scatter
-    const uint32_t hhi = h0_hi + (hlo < h0 ? 1u : 0u), stream = kStreamPhotonA + (__float_as_uint(e) >> 31);
-    const uint4 rr = draw(ctr, stream, hlo, hhi, p.key);
+    const uint32_t hhi = h0_hi + (hlo < h0 ? 1u : 0u);
+    const uint32_t stream = GAMMAS ? ctr >> kStreamShift : kStreamPhotonA + (__float_as_uint(e) >> 31);
+    const uint4 rr = philox4x32_10(make_uint4(GAMMAS ? ctr & kCtrMask : ctr, stream, hlo, hhi), p.key);
+    ++ctr;
     const float imaj = fabsf(maj);
     float s = -__logf(u01(rr.x)) * imaj;   // cm
     const bool cross = s >= rem;           // flight cut at the region boundary
@@ -1166,7 +1281,7 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
       if (maj > 0.0f) rem = region_distance(p.g, false, px, py, pz, ux, uy, uz);
     }
     if (fly && !in_grid) {                 // escapes
-      n_steps += GENERAL ? steps : ctr;
+      n_steps += GENERAL ? steps : steps_of(ctr);
       e = 0.0f;
     }
     const float2 c = lds2(mat + 8u * (wv & 7u));
@@ -1181,7 +1296,8 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
         atomicAdd(&s_cnt[kCtrRayleigh], 1ull);
         // Thomson angular shape (1 + cos^2)/2 by rejection; one block per trial.
         for (int trial = 0;; ++trial) {
-          const uint4 r = draw(ctr, stream, hlo, hhi, p.key);
+          const uint4 r = philox4x32_10(make_uint4(GAMMAS ? ctr & kCtrMask : ctr, stream, hlo, hhi), p.key);
+          ++ctr;
           const float cth = fmaf(2.0f, u01(r.x), -1.0f);
           const bool acc = 2.0f * u01(r.y) <= fmaf(cth, cth, 1.0f);
           if (acc || trial + 1 >= kKahnTrialLimit) {
@@ -1194,7 +1310,7 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
       }
     }
     // the rare ends of a photon: absorbed, or stopped by the step limit
-    const bool limit = (GENERAL ? steps : ctr) >= (uint32_t)p.max_steps;
+    const bool limit = (GENERAL ? steps : steps_of(ctr)) >= (uint32_t)p.max_steps;
     const bool photo = !park && t < scale * icp;
     uint32_t dq = 0;
     if (photo || limit) {
@@ -1202,14 +1318,14 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
         atomicAdd(&s_cnt[kCtrPhoto], 1ull);
         dq = (uint32_t)q_units(fabsf(e));
         deposit += dq;
-        n_steps += GENERAL ? steps : ctr;
+        n_steps += GENERAL ? steps : steps_of(ctr);
         if (!WARP_AGG) atomicAdd(tally_cell(hlo - h0, (uint32_t)v), (ull)dq);
       } else if (e != 0.0f) {
         atomicAdd(&s_cnt[kCtrKilledUnits], (ull)q_units(fabsf(e)));
         atomicAdd(&s_cnt[kKilled], 1ull);
         if (park) atomicAdd(&s_cnt[kCtrCompton], 1ull);
         flags |= NM_DEV_STEP_LIMIT;
-        n_steps += GENERAL ? steps : ctr;
+        n_steps += GENERAL ? steps : steps_of(ctr);
       }
       e = 0.0f;
       park = false;
@@ -1223,7 +1339,7 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
         e = scatter(e, cd, ctr, rr.z, rr.w, dq2);
         ux = cd.x; uy = cd.y; uz = cd.z;
         if (e == 0.0f) {
-          n_steps += GENERAL ? steps : ctr;
+          n_steps += GENERAL ? steps : steps_of(ctr);
         } else {
           const RingEnergy f = ring_energy<GENERAL>(fabsf(e), tab, p.ln_e_lo, p.inv_dln_e);
           s_c = f.s_c; s_pe = f.s_pe; s_r = f.s_r;
@@ -1253,8 +1369,8 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
       s_c = nm.x; s_pe = nm.y; maj = nm.z; rem = nm.w;
       ctr = __float_as_uint(na.x); maj2 = na.y;
       if constexpr (GENERAL) {
-        const float2 g = lds2(RING_AT8(gen, i));
-        sts1(RING_AT8(gen, i), __uint_as_float(steps));
+        const float2 g = lds2(RING_GEN(i));
+        sts1(RING_GEN(i), __uint_as_float(steps));
         steps = __float_as_uint(g.x);
         s_r = g.y;
       }
@@ -1270,7 +1386,7 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
   for (;;) {
     if (n_parked >= 32) compton_pass();
     if (s_left == 0) {
-      if (drained) break;
+      if (drained && !(GAMMAS && deferred)) break;
       sample_sites();
     }
     // lanes without a photon take the site queue's next ones
@@ -1286,21 +1402,31 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
       ux = __uint_as_float(__float_as_uint(sd.x) ^ sign);
       uy = __uint_as_float(__float_as_uint(sd.y) ^ sign);
       uz = __uint_as_float(__float_as_uint(sd.z) ^ sign);
-      rem = sign ? sr.x : sd.w;
-      e = __uint_as_float(__float_as_uint(p.e0) ^ sign);
-      s_c = s_f0.s_c;
-      s_pe = s_f0.s_pe;
-      maj = s_f0.maj_in;
-      maj2 = s_f0.maj_out;
-      if (sr.y < 0.0f) {
-        maj = s_f0.maj_out;
-        maj2 = s_f0.maj_in;
+      if constexpr (GAMMAS) {
+        const float4 m = lds4(GAMMA_MID(j));
+        rem = sd.w;
+        e = sr.x;
+        s_c = m.x; s_pe = m.y; maj = m.z; maj2 = m.w;
+        ctr = __float_as_uint(sr.y);
+        if (GENERAL) {
+          const float ie = __fdividef(1.0f, e);
+          s_r = ie * ie;
+        }
+      } else {
+        rem = sign ? sr.x : sd.w;
+        e = __uint_as_float(__float_as_uint(p.e0) ^ sign);
+        s_c = s_f0.s_c;
+        s_pe = s_f0.s_pe;
+        maj = s_f0.maj_in;
+        maj2 = s_f0.maj_out;
+        if (sr.y < 0.0f) {
+          maj = s_f0.maj_out;
+          maj2 = s_f0.maj_in;
+        }
+        ctr = 0;
+        if (GENERAL) s_r = s_f0.s_r;
       }
-      ctr = 0;
-      if (GENERAL) {
-        s_r = s_f0.s_r;
-        steps = 0;
-      }
+      if (GENERAL) steps = 0;
     }
     const uint32_t n_pop = min((uint32_t)__popc(want), s_left);
     s_next += n_pop;
@@ -1327,6 +1453,9 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
   while (__any_sync(kFull, e != 0.0f)) flight(std::integral_constant<int, 2>(), 0u);
 #undef RING_AT
 #undef RING_AT8
+#undef RING_GEN
+#undef GAMMA_MID
+#undef GAMMA_DEFER
 
   // ---- counters ---------------------------------------------------------------
   const ull dep_sum = warp_sum(deposit), step_sum = warp_sum((ull)n_steps);
@@ -1343,7 +1472,10 @@ __global__ void __launch_bounds__(512, 2) transport_ring_kernel(const TransportP
     // every photon that started was absorbed, cut off, killed or escaped, and
     // what it did not deposit went with it
     s_cnt[kCtrEscapes] = s_cnt[kBorn] - s_cnt[kCtrPhoto] - s_cnt[kCtrCutoff] - s_cnt[kKilled];
-    s_cnt[kCtrEscapedUnits] = s_cnt[kBorn] * (ull)(uint32_t)p.q_e0 - s_cnt[kDeposit] - s_cnt[kCtrKilledUnits];
+    s_cnt[kCtrEscapedUnits] = (GAMMAS ? s_cnt[kGamma] : s_cnt[kBorn] * (ull)(uint32_t)p.q_e0) - s_cnt[kDeposit] -
+                              s_cnt[kCtrKilledUnits] + s_cnt[kLost];
+    if (NUC != kPair && s_cnt[kBeta]) atomicAdd(p.g.counters + kCtrPositronUnits, s_cnt[kBeta]);
+    if (GAMMAS && s_cnt[kGamma]) atomicAdd(p.g.counters + kCtrGammaUnits, s_cnt[kGamma]);
   }
   __syncthreads();
   if (threadIdx.x < 8 && s_cnt[threadIdx.x]) atomicAdd(p.g.counters + threadIdx.x, s_cnt[threadIdx.x]);
@@ -1431,48 +1563,60 @@ void* pick(bool a, bool r, bool g, bool h, bool beta) {
   return r ? kernel_ptr<false, true, false, false>() : kernel_ptr<false, false, false, false>();
 }
 
-// The ring kernel runs every regrouped launch of annihilation
-// photons (or a point source) without history statistics: 1e8 decays on the
-// benchmark phantom take 13.2 ms on it and 30.5 ms on the lane kernel.
-bool use_ring(bool regroup, bool history, bool beta) { return regroup && !history && !beta; }
+// The ring kernel runs every regrouped launch without history statistics but
+// that of a nuclide which gives both an annihilation pair and gamma lines: 1e8
+// decays on the benchmark phantom take 13.2 ms on it and 30.5 ms on the lane
+// kernel; 2e7 on the 4 mm phantom with tracked positrons 3.7 and (regrouped)
+// 7.4 ms, of 131I 2.9 and 6.0, of 177Lu 1.4 and 3.0.
+bool use_ring(bool regroup, bool history, int nuc) { return regroup && !history && nuc >= 0; }
 
-void* pick_ring(bool a, bool general) {
-  if (a) return general ? (void*)transport_ring_kernel<true, true> : (void*)transport_ring_kernel<true, false>;
-  return general ? (void*)transport_ring_kernel<false, true> : (void*)transport_ring_kernel<false, false>;
+void* pick_ring(bool a, bool general, int nuc) {
+  if (nuc == kTracked)
+    return general ? (void*)transport_ring_kernel<false, true, kTracked> : (void*)transport_ring_kernel<false, false, kTracked>;
+  if (nuc == kGammas)
+    return general ? (void*)transport_ring_kernel<false, true, kGammas> : (void*)transport_ring_kernel<false, false, kGammas>;
+  if (a) return general ? (void*)transport_ring_kernel<true, true, kPair> : (void*)transport_ring_kernel<true, false, kPair>;
+  return general ? (void*)transport_ring_kernel<false, true, kPair> : (void*)transport_ring_kernel<false, false, kPair>;
 }
 
-size_t ring_smem(int block, bool general) {
-  return sizeof(RingTables) + (size_t)(block / 32) * (general ? sizeof(WarpStoreGeneral) : sizeof(WarpStore));
+size_t ring_smem(int block, bool general, int nuc) {
+  const uint32_t warp = nuc == kGammas ? (general ? StoreOf<true, kGammas>::kBytes : StoreOf<false, kGammas>::kBytes)
+                                       : (general ? StoreOf<true, kPair>::kBytes : StoreOf<false, kPair>::kBytes);
+  return sizeof(RingTables) + (size_t)(block / 32) * warp;
 }
 
 }  // namespace
 
-bool nuclide_launch(const TransportParams& p) {
-  return p.g.beta_tab != nullptr || p.n_gamma > 0 || (p.g.source_mode == NM_SOURCE_DECAY && !p.annihilate);
+int nuclide_kind(bool decay, bool beta_track, bool annihilate, int n_gamma) {
+  if (!decay) return kPair;
+  if (annihilate) return n_gamma > 0 ? -1 : beta_track ? kTracked : kPair;
+  return kGammas;
 }
 
 cudaError_t launch_transport(const TransportParams& p, int grid, int block, bool warp_agg,
                              bool rayleigh, bool regroup, cudaStream_t s, bool history) {
-  const bool beta = nuclide_launch(p);
-  const bool ring = use_ring(regroup, history, beta);
+  const int nuc = nuclide_kind(p.g.source_mode == NM_SOURCE_DECAY, p.g.beta_tab != nullptr, p.annihilate != 0, p.n_gamma);
+  if (nuc != kPair && warp_agg) return cudaErrorInvalidValue;
+  const bool ring = use_ring(regroup, history, nuc);
   const bool general = rayleigh || !p.kn_inv;
-  void* fn = ring ? pick_ring(warp_agg, general) : pick(warp_agg, rayleigh, regroup, history, beta);
+  void* fn = ring ? pick_ring(warp_agg, general, nuc) : pick(warp_agg, rayleigh, regroup, history, nuc != kPair);
   if (!fn) return cudaErrorInvalidValue;
   void* args[] = {(void*)&p};
   // the history lists and the rings take the static + dynamic total past the
   // 48 KB default
-  const size_t smem = ring ? ring_smem(block, general) : transport_smem(block, history, beta);
+  const size_t smem = ring ? ring_smem(block, general, nuc) : transport_smem(block, history, nuc != kPair);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) e = cudaLaunchKernel(fn, dim3(grid), dim3(block), args, smem, s);
   if (e != cudaSuccess) cudaGetLastError();  // a refused launch must not linger as the last error
   return e;
 }
 
-int transport_max_blocks_per_sm(int block, bool warp_agg, bool rayleigh, bool regroup, bool history, bool beta) {
+int transport_max_blocks_per_sm(int block, bool warp_agg, bool rayleigh, bool regroup, bool history, int nuc) {
   int n = 0;
-  const bool ring = use_ring(regroup, history, beta);
-  void* fn = ring ? pick_ring(warp_agg, rayleigh) : pick(warp_agg, rayleigh, regroup, history, beta);
-  const size_t smem = ring ? ring_smem(block, rayleigh) : transport_smem(block, history, beta);
+  if (nuc != kPair && warp_agg) return 0;
+  const bool ring = use_ring(regroup, history, nuc);
+  void* fn = ring ? pick_ring(warp_agg, rayleigh, nuc) : pick(warp_agg, rayleigh, regroup, history, nuc != kPair);
+  const size_t smem = ring ? ring_smem(block, rayleigh, nuc) : transport_smem(block, history, nuc != kPair);
   if (!fn || cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, block, smem) != cudaSuccess) {
     cudaGetLastError();

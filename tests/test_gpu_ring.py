@@ -2,8 +2,9 @@
 lane kernel (regroup = 0): the same histories give the same tally and counters
 bit for bit, from a single decay to more than a warp's ring holds, with every
 sampler and physics option, from sources inside and outside the tracking box,
-across the 2^32 boundary of the history ids, and when photons hit the step
-limit."""
+across the 2^32 boundary of the history ids, when photons hit the step limit,
+and for decays with tracked positrons or gamma lines (more lines per decay than
+the site queue holds included)."""
 import numpy as np
 import pytest
 
@@ -30,8 +31,10 @@ def phantom(nm):
     return ph, den, mat
 
 
-def _run(nm, phantom, n, regroup, first=0, rayleigh=0, everywhere=False, **kw):
-    from paper_2111_11687_gb300 import inputs
+def _run(nm, phantom, n, regroup, first=0, rayleigh=0, everywhere=False, decay=None, **kw):
+    from paper_2111_11687_gb300 import inputs, nuclides
+    if decay:
+        kw.update(DECAYS[decay] if isinstance(DECAYS[decay], dict) else getattr(nuclides, DECAYS[decay]))
     ph, den, mat = phantom
     gm = nm.Materials(inputs.MATERIAL_Z_OVER_A, inputs.MATERIAL_ZEFF, inputs.PE_COEFF, inputs.PE_EXP,
                       rayleigh=rayleigh, rayleigh_coeff=1e-4)
@@ -56,6 +59,16 @@ CASES = ([dict(n=n) for n in (1, 2, 31, 32, 33, 64, 65, 127, 1000, 70_001)] +
              dict(first=2**32 - 7_001), dict(max_steps=3), dict(max_steps=4, kn_sampler=1), dict(batches=1),
              dict(source_mode=1, point=(20.0, 25.0, 40.0)), dict(source_mode=1, point=(0.5, 0.5, 0.5)),
              dict(positron_mev=0.0))])
+
+
+EIGHT = dict(no_annihilation=1, positron_mev=0.1, gamma_lines=[(0.05 + 0.1 * j, 1.0) for j in range(8)])
+DECAYS = {"18F tracked": "F18_TRACKED", "177Lu": "LU177", "131I": "I131", "eight lines": EIGHT,
+          "no photon": dict(no_annihilation=1, positron_mev=0.2),
+          "pair and line": dict(gamma_lines=[(0.9, 0.7)])}
+CASES += [dict(n=n, decay=d) for d in DECAYS for n in (1, 33, 9_001)]
+CASES += [dict(n=9_001, decay=d, **kw) for d in ("18F tracked", "131I", "eight lines")
+          for kw in (dict(rayleigh=1), dict(kn_sampler=1), dict(everywhere=True), dict(first=2**32 - 3_001),
+                     dict(block_threads=256, chunk=64), dict(max_steps=4))]
 
 
 @pytest.mark.parametrize("case", CASES, ids=lambda c: "-".join(f"{k}{v}" for k, v in c.items()))
