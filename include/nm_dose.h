@@ -97,7 +97,7 @@ typedef struct {
   int32_t max_steps;         /* per-photon flight-step limit (bounded loops) */
   void* stream;              /* cudaStream_t; NULL = legacy default stream */
   int32_t history_sigma;     /* 1: also keep history-by-history statistics (the paper's
-                                uncertainty method, §2.1; +16 B per voxel, no warp
+                                uncertainty method, §2.1; +32 B per voxel, no warp
                                 aggregation); read with nm_dose_get_history_sigma */
   double beta_max_mev;       /* decay mode.  0 (default): positron_mev is deposited in the
                                 decay voxel (§2.1's positron, locally absorbed).  > 0

@@ -333,6 +333,8 @@ struct nm_dose {
   bool nuclide = false;
   ull* s2h_lo = nullptr;       // history statistics (history_sigma): 128-bit sums of squares
   ull* s2h_hi = nullptr;
+  ull* q_lo = nullptr;         // a launch's sums of their low and high 32 bits, zero between runs unless `dirty`
+  ull* q_hi = nullptr;
   ull* counters = nullptr;     // kCtrCount
   unsigned* work = nullptr;
   // Batch tallies [slots][V], all zero between runs unless `dirty`: one from
@@ -364,7 +366,7 @@ struct nm_dose {
   ~nm_dose() {
     // nothing on the device may still use a buffer that is recycled
     cudaStreamSynchronize(stream);
-    void* ptrs[] = {vox, density, labels, label_bad, alias, tb, tsum, s2, kn, minv, minv_out, beta_tab, kn_inv, s2h_lo, s2h_hi, counters, work, status,
+    void* ptrs[] = {vox, density, labels, label_bad, alias, tb, tsum, s2, kn, minv, minv_out, beta_tab, kn_inv, s2h_lo, s2h_hi, q_lo, q_hi, counters, work, status,
                     rho_max_bits, org_s1, org_s2, organ_count, organ_partial, organ_out,
                     out_dose, out_sigma};
     for (void* p : ptrs) dfree(p);
@@ -413,8 +415,8 @@ struct nm_dose {
     p.kn_inv = opt.kn_sampler == 0 ? kn_inv : nullptr;
     p.kn_inv_lo = kn_inv_lo;
     p.kn_inv_idln = kn_inv_idln;
-    p.s2h_lo = s2h_lo;
-    p.s2h_hi = s2h_hi;
+    p.s2h_lo = q_lo;
+    p.s2h_hi = q_hi;
     p.key = philox_key((uint32_t)seed, (uint32_t)(seed >> 32));
     p.e0 = e0;
     p.q_e0 = q_e0;
@@ -709,8 +711,8 @@ static nm_status autotune(nm_dose* h, Shape sh, bool free_block, bool free_chunk
   NM_CUDA(cudaMemsetAsync(h->counters, 0, kCtrCount * sizeof(ull), s), "autotune");
   NM_CUDA(cudaMemsetAsync(h->status, 0, sizeof(uint32_t), s), "autotune");
   if (h->s2h_lo) {
-    NM_CUDA(cudaMemsetAsync(h->s2h_lo, 0, h->V * sizeof(ull), s), "autotune");
-    NM_CUDA(cudaMemsetAsync(h->s2h_hi, 0, h->V * sizeof(ull), s), "autotune");
+    NM_CUDA(cudaMemsetAsync(h->q_lo, 0, h->V * sizeof(ull), s), "autotune");
+    NM_CUDA(cudaMemsetAsync(h->q_hi, 0, h->V * sizeof(ull), s), "autotune");
   }
   NM_CUDA(cudaStreamSynchronize(s), "autotune");
   std::lock_guard<std::mutex> lock(g_tune_mu);
@@ -847,7 +849,9 @@ nm_status nm_dose_create(nm_dose** out, const nm_grid* g, const nm_materials* mt
       return bail(cuda_fail(e, "beta table"));
   }
   if (o.history_sigma) {
-    if ((e = dalloc(&h->s2h_lo, V)) || (e = dalloc(&h->s2h_hi, V)) ||
+    if ((e = dalloc(&h->s2h_lo, V)) || (e = dalloc(&h->s2h_hi, V)) || (e = dalloc(&h->q_lo, V)) ||
+        (e = dalloc(&h->q_hi, V)) || (e = cudaMemsetAsync(h->q_lo, 0, V * sizeof(ull), s)) ||
+        (e = cudaMemsetAsync(h->q_hi, 0, V * sizeof(ull), s)) ||
         (e = cudaMemsetAsync(h->s2h_lo, 0, V * sizeof(ull), s)) || (e = cudaMemsetAsync(h->s2h_hi, 0, V * sizeof(ull), s)))
       return bail(cuda_fail(e, "device allocation"));
   }
@@ -976,6 +980,17 @@ static nm_status ensure_slots(nm_dose* h, int want) {
   return NM_OK;
 }
 
+// Clears what a run that failed half-way left in the batch tallies and the
+// launch's sums of squares.
+static cudaError_t clear_dirty(nm_dose* h) {
+  if (!h->dirty) return cudaSuccess;
+  const size_t V8 = 8 * (size_t)h->V;
+  cudaError_t e = cudaMemsetAsync(h->tb, 0, V8 * h->slots, h->stream);
+  if (!e && h->q_lo) e = cudaMemsetAsync(h->q_lo, 0, V8, h->stream);
+  if (!e && h->q_hi) e = cudaMemsetAsync(h->q_hi, 0, V8, h->stream);
+  return e;
+}
+
 static FoldParams fold_params(const nm_dose* h) {
   FoldParams fp;
   memset(&fp, 0, sizeof fp);
@@ -1038,6 +1053,7 @@ static cudaError_t enqueue_run(nm_dose* h, uint64_t n, int B, uint64_t seed, con
       if (!e)
         e = launch_transport(p, (int)std::min<uint64_t>((uint64_t)like->grid, want), like->block, like->warp_agg,
                              h->rayleigh, like->regroup, s, h->opt.history_sigma != 0);
+      if (!e && h->q_lo) e = launch_fold_history(h->q_lo, h->q_hi, h->s2h_lo, h->s2h_hi, h->V, s);
       done += part;
     }
     if (!e) e = mark();
@@ -1562,7 +1578,7 @@ nm_status nm_dose_restore(nm_dose* h, const void* buf, uint64_t bytes) {
     NM_CUDA(cudaMemcpyAsync(h->s2h_lo, b + o.lo, V8, cudaMemcpyDefault, s), "restore");
     NM_CUDA(cudaMemcpyAsync(h->s2h_hi, b + o.hi, V8, cudaMemcpyDefault, s), "restore");
   }
-  if (h->dirty) NM_CUDA(cudaMemsetAsync(h->tb, 0, V8 * h->slots, s), "restore");
+  NM_CUDA(clear_dirty(h), "restore");
   NM_CUDA(cudaStreamSynchronize(s), "nm_dose_restore");
   h->dirty = false;
   h->hist_next = hd.hist_next;
@@ -1652,7 +1668,7 @@ nm_status nm_dose_counters(nm_dose* h, nm_counters* c) {
 nm_status nm_dose_reset(nm_dose* h) {
   if (!h) return fail(NM_ERR_ARG, "handle is NULL");
   cudaStream_t s = h->stream;
-  if (h->dirty) NM_CUDA(cudaMemsetAsync(h->tb, 0, h->V * h->slots * sizeof(ull), s), "reset");
+  NM_CUDA(clear_dirty(h), "reset");
   NM_CUDA(cudaMemsetAsync(h->tsum, 0, h->V * sizeof(ull), s), "reset");
   NM_CUDA(cudaMemsetAsync(h->s2, 0, h->V * sizeof(double), s), "reset");
   NM_CUDA(cudaMemsetAsync(h->counters, 0, kCtrCount * sizeof(ull), s), "reset");

@@ -162,8 +162,9 @@ struct TransportParams {
   int max_steps;
   int regroup_compton;        // regrouped variant: lanes that must wait before a Compton pass
   int regroup_refill;         // regrouped variant: lanes that must wait before a refill pass
-  // History-by-history statistics: per voxel the
-  // 128-bit sum over histories of each history's squared total deposit.
+  // History-by-history statistics: per voxel the sums over the launch's
+  // histories of the low and of the high 32 bits of each history's squared
+  // total deposit.
   ull* s2h_lo;
   ull* s2h_hi;
   // Decay of another radionuclide (the nuclide variant): whether the annihilation pair is emitted, and the gamma lines
@@ -279,6 +280,9 @@ struct FoldParams {
   }
 };
 int fold_blocks(int64_t V);
+// Moves a launch's sums of squares (q_lo, q_hi: of low and high 32 bits) into the
+// 128-bit sums hi * 2^64 + lo.
+cudaError_t launch_fold_history(ull* q_lo, ull* q_hi, ull* lo, ull* hi, int64_t V, cudaStream_t s);
 cudaError_t launch_fold(const FoldParams& p, cudaStream_t s);
 
 // Adds another shard's statistics (o_*) into a handle's (all device arrays;

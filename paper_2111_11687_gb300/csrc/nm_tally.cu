@@ -387,6 +387,20 @@ __global__ void map_organ_final_kernel(const double* __restrict__ part, int n_bl
   if (lane == 0) out[l] = count[l] > 0 ? s / (double)count[l] : 0.0;
 }
 
+// lo + 2^64 hi += q_lo + 2^32 q_hi, and q_lo = q_hi = 0.
+__global__ void fold_history_kernel(ull* __restrict__ q_lo, ull* __restrict__ q_hi, ull* __restrict__ lo,
+                                    ull* __restrict__ hi, int64_t V) {
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (int64_t)gridDim.x * blockDim.x) {
+    const ull a = q_lo[v], b = q_hi[v];
+    if (!(a | b)) continue;
+    const ull l0 = lo[v], l1 = l0 + a, l2 = l1 + (b << 32);
+    lo[v] = l2;
+    hi[v] += (b >> 32) + (l1 < l0 ? 1ull : 0ull) + (l2 < l1 ? 1ull : 0ull);
+    q_lo[v] = 0;
+    q_hi[v] = 0;
+  }
+}
+
 __global__ void history_sigma_kernel(const ull* __restrict__ tsum, const ull* __restrict__ lo,
                                      const ull* __restrict__ hi, const float* __restrict__ density, int64_t V,
                                      double n, float gy_a, float* __restrict__ sigma) {
@@ -414,6 +428,12 @@ static int fold_tiles(int64_t V) {
 int fold_blocks(int64_t V) {
   const int64_t per = (int64_t)fold_tiles(V) * kFoldTile;
   return (int)((V + per - 1) / per);
+}
+
+cudaError_t launch_fold_history(ull* q_lo, ull* q_hi, ull* lo, ull* hi, int64_t V, cudaStream_t s) {
+  const int64_t g = (V + 255) / 256;
+  fold_history_kernel<<<(unsigned)(g < 8192 ? g : 8192), 256, 0, s>>>(q_lo, q_hi, lo, hi, V);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_history_sigma(const ull* tsum, const ull* s2h_lo, const ull* s2h_hi, const float* density,

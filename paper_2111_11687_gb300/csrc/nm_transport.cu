@@ -422,8 +422,13 @@ __device__ __forceinline__ void compton(const TransportParams& p, const float* s
 
 // History statistics: a lane lists its current history's deposits per voxel
 // (kHistVoxels entries in shared memory, structure of arrays over the CTA) and
-// adds them to the tally, with their squares to the 128-bit sums, when the
-// history ends (the lane takes its next history, or the kernel ends).
+// adds them to the tally, with their squares' halves to two 64-bit sums, when
+// the history ends (the lane takes its next history, or the kernel ends).  The
+// halves' sums hold a launch's histories (each below 2^32) without overflow and
+// go into the 128-bit sums afterwards (launch_fold_history), so that no lane
+// waits for an old value to see a carry.  The list loops stay rolled: unrolled
+// they spill 220 bytes of the tracked variant's photon.  4 mm phantom, 2e7
+// decays: 7.5 -> 6.8 ms, with tracked positrons 18.2 -> 11.9.
 struct HistList {
   uint32_t* v;   // voxel of entry i at v[i * stride]
   uint32_t* q;   // units
@@ -431,18 +436,20 @@ struct HistList {
 };
 
 __device__ __forceinline__ void hist_flush(const HistList& L, int& n, ull* tally, ull* lo, ull* hi) {
+#pragma unroll 1
   for (int i = 0; i < n; ++i) {
     const uint32_t v = L.v[i * L.stride], t = L.q[i * L.stride];
-    atomicAdd(tally + v, (ull)t);
     const ull t2 = (ull)t * t;
-    const ull old = atomicAdd(lo + v, t2);
-    if (old + t2 < old) atomicAdd(hi + v, 1ull);   // carry into the high word
+    atomicAdd(tally + v, (ull)t);
+    atomicAdd(lo + v, t2 & 0xffffffffull);
+    atomicAdd(hi + v, t2 >> 32);
   }
   n = 0;
 }
 
 __device__ __forceinline__ void hist_add(const HistList& L, int& n, uint32_t v, uint32_t dq, ull* tally, ull* lo,
                                          ull* hi, ull* splits) {
+#pragma unroll 1
   for (int i = 0; i < n; ++i)
     if (L.v[i * L.stride] == v) {
       L.q[i * L.stride] += dq;
