@@ -331,8 +331,10 @@ nm_status nm_check_kn_table(double e_mev, double cut_mev, double e0_mev, int64_t
 /* Device memory released by destroyed handles and by the library's per-call
  * temporaries is kept (up to 8 GiB, per device and buffer size) and handed to
  * the next allocation of the same size on the same device, so that a handle
- * created after one of the same grid maps no new memory.  This call returns
- * every kept buffer to the device (cudaFree); buffers of live handles are not
+ * created after one of the same grid maps no new memory; scratch of the
+ * denoiser and its convolutions comes from a memory pool that keeps up to
+ * 512 MiB per device.  This call returns
+ * all of it to the device; buffers of live handles are not
  * affected.  A failed allocation releases them by itself before it retries.
  * Safe to call at any time from any thread.  Kept buffers belong to the
  * device's context: destroy the handles and call this before cudaDeviceReset

@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "nm_internal.cuh"
+#include "nm_scratch.cuh"
 #include "nm_trace.h"
 
 using namespace nm;
@@ -205,6 +206,16 @@ cudaError_t dalloc(T** p, size_t n) {
   }
   c.live[(void*)*p] = std::make_pair(dev, bytes);
   return cudaSuccess;
+}
+
+// Memory pools of stream_alloc, one per device, made at its first use there.
+struct StreamPools {
+  std::mutex mu;
+  std::map<int, cudaMemPool_t> pool;
+};
+StreamPools& stream_pools() {
+  static StreamPools* p = new StreamPools();   // never destroyed, as the buffer cache
+  return *p;
 }
 
 // Returns a dalloc'd buffer; the caller guarantees that no device work still
@@ -489,6 +500,33 @@ const char* nm_last_error(void) { return g_err.c_str(); }
 }  // extern "C"
 
 void nm::set_error_message(const char* msg) { g_err = msg; }
+
+cudaError_t nm::stream_alloc(void** p, size_t bytes, cudaStream_t s) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e) return e;
+  StreamPools& sp = stream_pools();
+  std::lock_guard<std::mutex> lock(sp.mu);
+  auto it = sp.pool.find(dev);
+  if (it == sp.pool.end()) {
+    cudaMemPoolProps props;
+    memset(&props, 0, sizeof props);
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    uint64_t keep = kPoolKeep;
+    if ((e = cudaMemPoolCreate(&pool, &props))) return e;
+    if ((e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep))) {
+      cudaMemPoolDestroy(pool);
+      return e;
+    }
+    it = sp.pool.emplace(dev, pool).first;
+  }
+  return cudaMallocFromPoolAsync(p, bytes, it->second, s);
+}
+
+cudaError_t nm::stream_free(void* p, cudaStream_t s) { return cudaFreeAsync(p, s); }
 
 // Checks shared by every entry point that takes a phantom: grid sizes and
 // spacing, material constants, energies and options.  The positron energy is
@@ -1731,9 +1769,15 @@ nm_status nm_check_kahn(double e_mev, int64_t n, uint64_t seed, float* cos_out) 
 void nm_debug_fail_alloc(int32_t n) { g_fail_alloc.store(n > 0 ? n : 0); }
 
 void nm_release_cached_memory(void) {
-  BufferCache& c = buffer_cache();
-  std::lock_guard<std::mutex> lock(c.mu);
-  release_cache_locked(c);
+  {
+    BufferCache& c = buffer_cache();
+    std::lock_guard<std::mutex> lock(c.mu);
+    release_cache_locked(c);
+  }
+  StreamPools& sp = stream_pools();
+  std::lock_guard<std::mutex> lock(sp.mu);
+  for (auto& kv : sp.pool) cudaMemPoolDestroy(kv.second);   // lives on until its last buffer is freed
+  sp.pool.clear();
 }
 
 nm_status nm_check_wait_timeout(int64_t max_cycles) {

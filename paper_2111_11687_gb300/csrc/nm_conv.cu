@@ -20,6 +20,7 @@
 #include <algorithm>
 
 #include "nm_internal.cuh"
+#include "nm_scratch.cuh"
 #include "nm_tc.cuh"
 
 namespace nm {
@@ -437,14 +438,14 @@ cudaError_t launch_fwd_t(const ConvGeom& g, const __nv_bfloat16* x0, const __nv_
     return cudaGetLastError();
   }
   float* part = nullptr;
-  if ((e = cudaMallocAsync((void**)&part, (size_t)splits * g.m * COUT * sizeof(float), s))) return e;
+  if ((e = stream_alloc((void**)&part, (size_t)splits * g.m * COUT * sizeof(float), s))) return e;
   conv_fwd_kernel<COUT><<<dim3((unsigned)grid, splits), kThreads, smem, s>>>(g, x0, x1, w, bias, y, relu, part, per,
                                                                            status);
   const long long n = g.m * COUT;
   split_finish_kernel<<<(unsigned)((n + 255) / 256 < 8192 ? (n + 255) / 256 : 8192), 256, 0, s>>>(
       part, splits, g.m, COUT, bias, relu, y);
   e = cudaGetLastError();
-  cudaFreeAsync(part, s);
+  stream_free(part, s);
   return e;
 }
 

@@ -49,6 +49,7 @@
 #include <mutex>
 
 #include "nm_internal.cuh"
+#include "nm_scratch.cuh"
 #include "nm_tc.cuh"
 
 namespace nm {
@@ -539,7 +540,7 @@ cudaError_t launch_tile(const nm_conv3d_desc& d, const void* x, const void* w, c
     return cudaErrorInvalidValue;
   bf16* wt = nullptr;
   const size_t welems = (size_t)nchunks * COUT * 432;
-  cudaError_t e = cudaMallocAsync((void**)&wt, welems * sizeof(bf16), s);
+  cudaError_t e = stream_alloc((void**)&wt, welems * sizeof(bf16), s);
   if (e != cudaSuccess) return e;
   tile_weights_kernel<<<(unsigned)std::min<size_t>((welems + 255) / 256, 4096), 256, 0, s>>>(
       (const bf16*)w, cin, conv_kpad(cin), COUT, nchunks, SWZ ? 1 : 0, wt);
@@ -559,7 +560,7 @@ cudaError_t launch_tile(const nm_conv3d_desc& d, const void* x, const void* w, c
                                                                                       status);
     e = cudaGetLastError();
   }
-  cudaFreeAsync(wt, s);
+  stream_free(wt, s);
   return e;
 }
 

@@ -3,6 +3,7 @@
 #include <cstring>
 
 #include "nm_internal.cuh"
+#include "nm_scratch.cuh"
 
 using namespace nm;
 
@@ -37,7 +38,7 @@ nm_status finish(uint32_t* status, cudaStream_t s, const char* what) {
   uint32_t flags = 0;
   cudaError_t e = cudaMemcpyAsync(&flags, status, 4, cudaMemcpyDeviceToHost, s);
   if (!e) e = cudaStreamSynchronize(s);
-  cudaFreeAsync(status, s);
+  stream_free(status, s);
   if (e) return cuda_err(e, what);
   if (flags) return err(NM_ERR_DEVICE, "tensor-core wait timed out");
   return NM_OK;
@@ -58,11 +59,11 @@ nm_status nm_conv3d_fwd(const nm_conv3d_desc* d, const uint16_t* x0, const uint1
     return err(NM_ERR_ARG, "nm_conv3d_fwd: operands must be 16-byte aligned");
   cudaStream_t s = (cudaStream_t)stream;
   uint32_t* status = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&status, 4, s);
+  cudaError_t e = stream_alloc((void**)&status, 4, s);
   if (!e) e = cudaMemsetAsync(status, 0, 4, s);
   if (!e) e = conv3d_fwd(*d, x0, d->c1 ? x1 : nullptr, w, bias, y, relu, status, s);
   if (e) {
-    if (status) cudaFreeAsync(status, s);
+    if (status) stream_free(status, s);
     return cuda_err(e, "nm_conv3d_fwd");
   }
   return finish(status, s, "nm_conv3d_fwd");
@@ -81,14 +82,14 @@ nm_status nm_conv3d_dgrad(const nm_conv3d_desc* d, const uint16_t* dy, const uin
   uint32_t* status = nullptr;
   void* wb = nullptr;
   const size_t wb_bytes = (size_t)b.cout * conv_kpad(b.c0) * 2;
-  cudaError_t e = cudaMallocAsync((void**)&status, 4, s);
-  if (!e) e = cudaMallocAsync(&wb, wb_bytes, s);
+  cudaError_t e = stream_alloc((void**)&status, 4, s);
+  if (!e) e = stream_alloc(&wb, wb_bytes, s);
   if (!e) e = cudaMemsetAsync(status, 0, 4, s);
   if (!e) e = conv3d_flip_weights(*d, w, wb, s);
   if (!e) e = conv3d_fwd(b, dy, nullptr, wb, nullptr, dx, 0, status, s);
-  if (wb) cudaFreeAsync(wb, s);
+  if (wb) stream_free(wb, s);
   if (e) {
-    if (status) cudaFreeAsync(status, s);
+    if (status) stream_free(status, s);
     return cuda_err(e, "nm_conv3d_dgrad");
   }
   return finish(status, s, "nm_conv3d_dgrad");
@@ -103,13 +104,13 @@ nm_status nm_conv3d_wgrad(const nm_conv3d_desc* d, const uint16_t* x0, const uin
   cudaStream_t s = (cudaStream_t)stream;
   uint32_t* status = nullptr;
   void* ws = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&status, 4, s);
-  if (!e) e = cudaMallocAsync(&ws, conv_wgrad_workspace(*d), s);
+  cudaError_t e = stream_alloc((void**)&status, 4, s);
+  if (!e) e = stream_alloc(&ws, conv_wgrad_workspace(*d), s);
   if (!e) e = cudaMemsetAsync(status, 0, 4, s);
   if (!e) e = conv3d_wgrad(*d, x0, d->c1 ? x1 : nullptr, dy, dw, db, ws, status, s);
-  if (ws) cudaFreeAsync(ws, s);
+  if (ws) stream_free(ws, s);
   if (e) {
-    if (status) cudaFreeAsync(status, s);
+    if (status) stream_free(status, s);
     return cuda_err(e, "nm_conv3d_wgrad");
   }
   return finish(status, s, "nm_conv3d_wgrad");

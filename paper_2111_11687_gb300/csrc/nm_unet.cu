@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "nm_internal.cuh"
+#include "nm_scratch.cuh"
 #include "nm_trace.h"
 
 using namespace nm;
@@ -572,7 +573,7 @@ nm_status body_stats(const float* dose, const float* activity, const float* dens
   double* part = nullptr;
   int* dbox = nullptr;
   const size_t pbytes = kStatBlocks * 3 * sizeof(double);
-  CK(cudaMallocAsync((void**)&part, pbytes + 8 * sizeof(int), s), "body statistics");
+  CK(stream_alloc((void**)&part, pbytes + 8 * sizeof(int), s), "body statistics");
   if (box_out) {
     dbox = (int*)((char*)part + pbytes);
     const int init[6] = {INT_MAX, INT_MAX, INT_MAX, -1, -1, -1};
@@ -582,7 +583,7 @@ nm_status body_stats(const float* dose, const float* activity, const float* dens
   body_stats_kernel<<<kStatBlocks, 256, 0, s>>>(dose, activity, density, roi, nx, ny, n, part, dbox);
   cudaError_t e = cudaMemcpyAsync(r.data(), part, pbytes, cudaMemcpyDeviceToHost, s);
   if (!e && box_out) e = cudaMemcpyAsync(box_out, dbox, 6 * sizeof(int), cudaMemcpyDeviceToHost, s);
-  cudaFreeAsync(part, s);
+  stream_free(part, s);
   if (!e) e = cudaStreamSynchronize(s);
   if (e) return cfail(e, "body statistics");
   double v[2] = {0, 0}, c = 0;
@@ -854,6 +855,10 @@ nm_status run_steps(nm_denoiser* h, cudaGraphExec_t& exec, int& key_slot, int ke
     if (exec) cudaGraphExecDestroy(exec);
     exec = nullptr;
     if (!h->cap_stream) CK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking), "graph stream");
+    // the scratch pool must exist before the capture (it is made at first use)
+    void* probe = nullptr;
+    CK(stream_alloc(&probe, 256, s), "graph capture");
+    CK(stream_free(probe, s), "graph capture");
     CK(cudaStreamSynchronize(s), "graph capture");
     CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal), "graph capture");
     h->s = h->cap_stream;
@@ -1209,7 +1214,7 @@ nm_status nm_denoise_apply_roi(nm_denoiser* h, const float* dose, const float* d
   nm_denoiser* c = nullptr;
   if ((st = inference_instance(h, D, H, W, &c)) != NM_OK) return st;
   int* dcorn = nullptr;
-  CK(cudaMallocAsync((void**)&dcorn, 3 * sizeof(int), s), "apply");
+  CK(stream_alloc((void**)&dcorn, 3 * sizeof(int), s), "apply");
   for (int z0 = box[2]; z0 <= box[5] && st == NM_OK; z0 += tc) {
     const int core = std::min(tc, box[5] + 1 - z0);
     const int corner[3] = {box[0] - mg, box[1] - mg, z0 - mg};
@@ -1225,7 +1230,7 @@ nm_status nm_denoise_apply_roi(nm_denoiser* h, const float* dose, const float* d
     // the corner buffer is reused by the next slab
     CK(cudaStreamSynchronize(s), "apply");
   }
-  cudaFreeAsync(dcorn, s);
+  stream_free(dcorn, s);
   if (st != NM_OK) return st;
   CK(cudaGetLastError(), "apply");
   return check_status(h);
