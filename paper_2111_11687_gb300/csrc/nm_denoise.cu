@@ -4,6 +4,7 @@
 
 #include "nm_internal.cuh"
 #include "nm_scratch.cuh"
+#include "nm_wgrad.cuh"
 
 using namespace nm;
 
@@ -33,11 +34,15 @@ nm_status cuda_err(cudaError_t e, const char* what) {
   return e == cudaErrorMemoryAllocation ? NM_ERR_OOM : NM_ERR_CUDA;
 }
 
+cudaError_t read_flags(uint32_t* flags, const uint32_t* status, cudaStream_t s) {
+  const cudaError_t e = cudaMemcpyAsync(flags, status, 4, cudaMemcpyDeviceToHost, s);
+  return e ? e : cudaStreamSynchronize(s);
+}
+
 // Reads back a device status word, frees it, and maps flags to a status.
 nm_status finish(uint32_t* status, cudaStream_t s, const char* what) {
   uint32_t flags = 0;
-  cudaError_t e = cudaMemcpyAsync(&flags, status, 4, cudaMemcpyDeviceToHost, s);
-  if (!e) e = cudaStreamSynchronize(s);
+  cudaError_t e = read_flags(&flags, status, s);
   stream_free(status, s);
   if (e) return cuda_err(e, what);
   if (flags) return err(NM_ERR_DEVICE, "tensor-core wait timed out");
@@ -103,12 +108,32 @@ nm_status nm_conv3d_wgrad(const nm_conv3d_desc* d, const uint16_t* x0, const uin
     return err(NM_ERR_ARG, "nm_conv3d_wgrad: operands must be device pointers");
   cudaStream_t s = (cudaStream_t)stream;
   uint32_t* status = nullptr;
-  void* ws = nullptr;
   cudaError_t e = stream_alloc((void**)&status, 4, s);
-  if (!e) e = stream_alloc(&ws, conv_wgrad_workspace(*d), s);
   if (!e) e = cudaMemsetAsync(status, 0, 4, s);
-  if (!e) e = conv3d_wgrad(*d, x0, d->c1 ? x1 : nullptr, dy, dw, db, ws, status, s);
-  if (ws) stream_free(ws, s);
+  // a single layer takes the row kernel where it can; a network's training
+  // keeps the order of sums its runs began with (nm_wgrad_rows.cu)
+  bool rows = conv_wgrad_rows_ok(*d) && aligned16(dw);
+  if (!e && rows) {
+    uint32_t flags = 0;
+    void* ws = nullptr;
+    e = stream_alloc(&ws, conv_wgrad_rows_workspace(*d), s);
+    if (!e) e = conv3d_wgrad_rows(*d, x0, dy, dw, db, ws, status, s);
+    if (ws) stream_free(ws, s);
+    if (!e) e = read_flags(&flags, status, s);
+    if (!e && flags == kWgradNonFinite) {
+      rows = false;
+      e = cudaMemsetAsync(status, 0, 4, s);
+    } else if (!e) {
+      stream_free(status, s);
+      return flags ? err(NM_ERR_DEVICE, "tensor-core wait timed out") : NM_OK;
+    }
+  }
+  if (!e && !rows) {
+    void* ws = nullptr;
+    e = stream_alloc(&ws, conv_wgrad_workspace(*d), s);
+    if (!e) e = conv3d_wgrad(*d, x0, d->c1 ? x1 : nullptr, dy, dw, db, ws, status, s);
+    if (ws) stream_free(ws, s);
+  }
   if (e) {
     if (status) stream_free(status, s);
     return cuda_err(e, "nm_conv3d_wgrad");

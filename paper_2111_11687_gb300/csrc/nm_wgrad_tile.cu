@@ -40,6 +40,7 @@
 
 #include "nm_internal.cuh"
 #include "nm_tc.cuh"
+#include "nm_wgrad.cuh"
 
 namespace nm {
 namespace {
@@ -67,7 +68,6 @@ constexpr uint32_t kXBytes = kXRows * 32;
 constexpr uint32_t kYBytes = kYRows * 32;
 constexpr int kThreads = 192;
 constexpr long long kWaitCycles = 4ll << 30;
-constexpr int kBiasBlocks = 256;
 
 static_assert(kXRows >= kRows && kYRows >= kYBox, "tile rows");
 
@@ -436,15 +436,21 @@ cudaError_t launch_wgrad_tile(const nm_conv3d_desc& d, const void* x, const void
   wgrad_tile_kernel<COUT, G, DY><<<grid, kThreads, L::kSmem, s>>>(mx, my, g, part, status);
   const long long n = (long long)g.kpad * COUT;
   wgrad_tile_reduce<<<(unsigned)((n + 31) / 32), 256, 0, s>>>(part, grid, g.kpad, 27 * d.c0, COUT, dw);
-  if (db) {
-    const long long m = (long long)d.n * d.d * d.h * d.w;
-    bias_grad_partial<COUT><<<kBiasBlocks, 256, 0, s>>>((const bf16*)dy, m, bpart);
-    bias_grad_final<<<COUT, 32, 0, s>>>(bpart, kBiasBlocks, COUT, db);
-  }
+  if (db) bias_grad(d, dy, bpart, db, s);
   return cudaGetLastError();
 }
 
 }  // namespace
+
+void bias_grad(const nm_conv3d_desc& d, const void* dy, float* bpart, float* db, cudaStream_t s) {
+  const long long m = (long long)d.n * d.d * d.h * d.w;
+  const bf16* g = (const bf16*)dy;
+  if (d.cout == 16) bias_grad_partial<16><<<kBiasBlocks, 256, 0, s>>>(g, m, bpart);
+  else if (d.cout == 32) bias_grad_partial<32><<<kBiasBlocks, 256, 0, s>>>(g, m, bpart);
+  else if (d.cout == 64) bias_grad_partial<64><<<kBiasBlocks, 256, 0, s>>>(g, m, bpart);
+  else bias_grad_partial<128><<<kBiasBlocks, 256, 0, s>>>(g, m, bpart);
+  bias_grad_final<<<d.cout, 32, 0, s>>>(bpart, kBiasBlocks, d.cout, db);
+}
 
 bool conv_wgrad_tile_ok(const nm_conv3d_desc& d) {
   return d.c1 == 0 && !d.src0_coarse && d.c0 % 8 == 0 && (d.cout == 16 || d.cout == 32);
