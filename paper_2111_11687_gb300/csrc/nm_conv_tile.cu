@@ -9,7 +9,7 @@
 // of tap (dz, dy, dx) is the same tile shifted by (dz*PY + dy)*PX + dx rows: a
 // different start address in the descriptor.  GEMM rows run over the padded
 // tile's centre indices; rows whose centre is a halo voxel are computed and
-// dropped (20 % for a 16 x 16 x 2 tile, 27 % for 16 x 16 x 4).
+// dropped (20 % for a 16 x 16 x 2 tile).
 //
 // The kernel is persistent and warp-specialised (one CTA per SM):
 //   warp 0    one thread issues TMA loads: per 16-channel chunk two 5-D tiled
@@ -57,7 +57,7 @@ namespace {
 
 typedef __nv_bfloat16 bf16;
 
-constexpr int TX = 16, TY = 16;
+constexpr int TX = 16;
 constexpr uint32_t kSboB = 27 * 16 / 8 * 128;               // 8 weight rows of 27 x 16 channels
 constexpr int kEpiParts = 3;                               // epilogue warps per TMEM lane quarter
 constexpr int kEpiThreads = 128 * kEpiParts;               // warps 2 .. 1 + 4 kEpiParts
@@ -68,7 +68,7 @@ constexpr long long kWaitCycles = 4ll << 30;
 // Every 128-row M-tile accumulates its 27 taps in order, so the M-tiles are
 // the independent MMA chains in flight: 16-output layers, whose small MMAs
 // are bound by that chain latency, take deeper tiles (more M-tiles).
-template <int COUT, int TZ, bool SWZ, bool PACK = false>
+template <int COUT, int TZ, int TY, bool SWZ, bool PACK = false>
 struct TileLayout {
   static constexpr int PX = TX + 2, PY = TY + 2, PZ = TZ + 2;
   static constexpr int kRows = PX * PY * PZ;                // padded tile voxels
@@ -130,24 +130,24 @@ struct TileHead {
 };
 
 struct TileGrid {
-  int n, d, h, w, tz, tiles_x, tiles_y, tiles_z;
+  int n, d, h, w, ty, tz, tiles_x, tiles_y, tiles_z;
   long long tiles;
   __device__ void coords(long long t, int& b, int& x0, int& y0, int& z0) const {
     x0 = (int)(t % tiles_x) * TX; t /= tiles_x;
-    y0 = (int)(t % tiles_y) * TY; t /= tiles_y;
+    y0 = (int)(t % tiles_y) * ty; t /= tiles_y;
     z0 = (int)(t % tiles_z) * tz;
     b = (int)(t / tiles_z);
   }
 };
 
-template <int COUT, int TZ, bool SWZ, bool PACK>
+template <int COUT, int TZ, int TY, bool SWZ, bool PACK>
 __global__ void __launch_bounds__(kThreads, 1) conv_tile_kernel(const __grid_constant__ CUtensorMap tmx,
                                                                 const TileGrid g, int nchunks,
                                                                 const bf16* __restrict__ wt,
                                                                 const float* __restrict__ bias,
                                                                 bf16* __restrict__ y, int ldy, int relu,
                                                                 const TileHead hd, uint32_t* status) {
-  typedef TileLayout<COUT, TZ, SWZ, PACK> L;
+  typedef TileLayout<COUT, TZ, TY, SWZ, PACK> L;
   constexpr int NC = L::kNcol;
   constexpr int S = L::kStages, NA = L::kNacc;
   constexpr int PX = L::PX, PY = L::PY, kMt = L::kMt, kCmin = L::kCmin, kCmax = L::kCmax;
@@ -518,10 +518,10 @@ int sm_count() {
 
 // y: output voxel v's channels at y + v ldy (ldy = COUT, or the full width
 // when a wider convolution is computed COUT outputs at a time).
-template <int COUT, int TZ, bool SWZ, bool PACK = false>
+template <int COUT, int TZ, int TY, bool SWZ, bool PACK = false>
 cudaError_t launch_tile(const nm_conv3d_desc& d, const void* x, const void* w, const float* bias, void* y,
-                        int relu, const TileHead& hd, uint32_t* status, cudaStream_t s, int ldy = COUT) {
-  typedef TileLayout<COUT, TZ, SWZ, PACK> L;
+                        int relu, const TileHead& hd, uint32_t* status, cudaStream_t s, int ldy) {
+  typedef TileLayout<COUT, TZ, TY, SWZ, PACK> L;
   const int cin = d.c0;
   const int nchunks = (cin + 15) / 16;
   // the input as a 5-D tensor (c, x, y, z, n); boxes of 8 channels x the padded tile
@@ -548,20 +548,44 @@ cudaError_t launch_tile(const nm_conv3d_desc& d, const void* x, const void* w, c
   g.n = d.n; g.d = d.d; g.h = d.h; g.w = d.w;
   g.tiles_x = (d.w + TX - 1) / TX;
   g.tiles_y = (d.h + TY - 1) / TY;
+  g.ty = TY;
   g.tz = TZ;
   g.tiles_z = (d.d + TZ - 1) / TZ;
   g.tiles = (long long)g.tiles_x * g.tiles_y * g.tiles_z * g.n;
-  e = cudaFuncSetAttribute(conv_tile_kernel<COUT, TZ, SWZ, PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  e = cudaFuncSetAttribute(conv_tile_kernel<COUT, TZ, TY, SWZ, PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)L::kSmem);
   if (e == cudaSuccess) {
     const long long grid = std::min<long long>(g.tiles, sm_count());
-    conv_tile_kernel<COUT, TZ, SWZ, PACK><<<(unsigned)grid, kThreads, L::kSmem, s>>>(map, g, nchunks, wt, bias,
+    conv_tile_kernel<COUT, TZ, TY, SWZ, PACK><<<(unsigned)grid, kThreads, L::kSmem, s>>>(map, g, nchunks, wt, bias,
                                                                                       (bf16*)y, ldy, relu, hd,
                                                                                       status);
     e = cudaGetLastError();
   }
   stream_free(wt, s);
   return e;
+}
+
+// The tile of a layer by how full it leaves the chip: 16 x 16 x 2 voxels are
+// five M-tiles of MMAs (the fewest rows computed and dropped), 16 x 16 x 1
+// three, 16 x 8 x 1 two; a launch lasts as many of them as its fullest CTA has,
+// and a tile's set-up and epilogue about as long as one more.  An output's
+// additions come in the same order in all three.  Microseconds a call in the
+// three forms: 4 x 16^3 voxels, 64 -> 64 channels 52, 46, 39 (the kernel 27 in
+// the first, 14 in the last); 32^3, 32 -> 32 39, 35, 37; 40^3, 64 -> 64 75, 66,
+// 61; 2 x 32^3, 32 -> 32 39, 40, 49; 4 x 32^3 49, 53, 61; 2 x 50 x 37 x 61,
+// 96 -> 32 138, 162, 197.
+template <int COUT, bool PACK = false>
+cudaError_t launch_fitting(const nm_conv3d_desc& d, const void* x, const void* w, const float* bias, void* y,
+                           int relu, const TileHead& hd, uint32_t* status, cudaStream_t s, int ldy = COUT) {
+  const long long sms = sm_count();
+  auto turns = [&](int tz, int ty, int mt) {
+    const long long tiles = (long long)((d.w + TX - 1) / TX) * ((d.h + ty - 1) / ty) * ((d.d + tz - 1) / tz) * d.n;
+    return (tiles + sms - 1) / sms * (mt + 1);
+  };
+  const long long a = turns(2, 16, 5), b = turns(1, 16, 3), c = turns(1, 8, 2);
+  if (a < b && a < c) return launch_tile<COUT, 2, 16, true, PACK>(d, x, w, bias, y, relu, hd, status, s, ldy);
+  if (b < c) return launch_tile<COUT, 1, 16, true, PACK>(d, x, w, bias, y, relu, hd, status, s, ldy);
+  return launch_tile<COUT, 1, 8, true, PACK>(d, x, w, bias, y, relu, hd, status, s, ldy);
 }
 
 }  // namespace
@@ -605,13 +629,12 @@ static bool packed_tiles() {
 
 cudaError_t conv3d_fwd_tile(const nm_conv3d_desc& d, const void* x, const void* w, const float* bias, void* y,
                             int relu, uint32_t* status, cudaStream_t s) {
-  constexpr bool kSwz = true;
   const TileHead none{nullptr, nullptr, 0, nullptr};
-  if (d.cout == 16 && packed_tiles()) return launch_tile<16, 2, kSwz, true>(d, x, w, bias, y, relu, none, status, s);
-  if (d.cout == 16) return launch_tile<16, 4, kSwz>(d, x, w, bias, y, relu, none, status, s);
-  if (d.cout == 32) return launch_tile<32, 2, kSwz>(d, x, w, bias, y, relu, none, status, s);
-  if (d.cout == 48) return launch_tile<48, 2, kSwz>(d, x, w, bias, y, relu, none, status, s);
-  if (d.cout == 64) return launch_tile<64, 2, kSwz>(d, x, w, bias, y, relu, none, status, s);
+  if (d.cout == 16 && packed_tiles()) return launch_fitting<16, true>(d, x, w, bias, y, relu, none, status, s);
+  if (d.cout == 16) return launch_tile<16, 4, 16, true>(d, x, w, bias, y, relu, none, status, s, 16);
+  if (d.cout == 32) return launch_fitting<32>(d, x, w, bias, y, relu, none, status, s);
+  if (d.cout == 48) return launch_fitting<48>(d, x, w, bias, y, relu, none, status, s);
+  if (d.cout == 64) return launch_fitting<64>(d, x, w, bias, y, relu, none, status, s);
   // 96 and 192 outputs (input gradients of the decoders' two-source layers):
   // 48 or 64 output channels per launch, written at the full channel stride
   const int P = d.cout == 96 ? 48 : 64;
@@ -621,8 +644,8 @@ cudaError_t conv3d_fwd_tile(const nm_conv3d_desc& d, const void* x, const void* 
     const void* wp = (const bf16*)w + (size_t)p * P * conv_kpad(d.c0);
     const float* bp = bias ? bias + p * P : nullptr;
     void* yp = (bf16*)y + p * P;
-    const cudaError_t e = P == 48 ? launch_tile<48, 2, kSwz>(dp, x, wp, bp, yp, relu, none, status, s, d.cout)
-                                  : launch_tile<64, 2, kSwz>(dp, x, wp, bp, yp, relu, none, status, s, d.cout);
+    const cudaError_t e = P == 48 ? launch_fitting<48>(dp, x, wp, bp, yp, relu, none, status, s, d.cout)
+                                  : launch_fitting<64>(dp, x, wp, bp, yp, relu, none, status, s, d.cout);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -633,8 +656,8 @@ cudaError_t conv3d_fwd_tile_head(const nm_conv3d_desc& d, const void* x, const v
                                  cudaStream_t s) {
   if (d.cout != 16 || !conv_tile_ok(d)) return cudaErrorInvalidValue;
   const TileHead hd{head_w, (const bf16*)xin, cx, yh};
-  if (packed_tiles()) return launch_tile<16, 2, true, true>(d, x, w, bias, nullptr, 1, hd, status, s);
-  return launch_tile<16, 4, true>(d, x, w, bias, nullptr, 1, hd, status, s);
+  if (packed_tiles()) return launch_fitting<16, true>(d, x, w, bias, nullptr, 1, hd, status, s);
+  return launch_tile<16, 4, 16, true>(d, x, w, bias, nullptr, 1, hd, status, s, 16);
 }
 
 }  // namespace nm
