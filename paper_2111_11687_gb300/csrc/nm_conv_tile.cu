@@ -2,20 +2,20 @@
 // straight out of one shared-memory halo tile, with no im2col gather.
 //
 // An output tile is TZ x TY x TX voxels.  Its input tile, with a one-voxel
-// halo, is stored as "channel planes": plane j holds channels 8j..8j+7 of
-// every padded voxel, 16 bytes per voxel, voxels in x-fastest order.  In the
-// no-swizzle K-major operand layout with a stride byte offset of 128 (eight
-// 16-byte rows) consecutive voxels are consecutive GEMM rows, so the A operand
+// halo, is stored 16 channels at a time: 32 bytes per padded voxel, voxels in
+// x-fastest order.  In the 32-byte-swizzled K-major operand layout with a
+// stride byte offset of 256 (eight rows) consecutive voxels are consecutive
+// GEMM rows, so the A operand
 // of tap (dz, dy, dx) is the same tile shifted by (dz*PY + dy)*PX + dx rows: a
 // different start address in the descriptor.  GEMM rows run over the padded
 // tile's centre indices; rows whose centre is a halo voxel are computed and
 // dropped (20 % for a 16 x 16 x 2 tile).
 //
 // The kernel is persistent and warp-specialised (one CTA per SM):
-//   warp 0    one thread issues TMA loads: per 16-channel chunk two 5-D tiled
-//             tensor loads (the two channel planes of the halo box; the TMA
-//             unit zero-fills outside the volume) and one bulk copy of the
-//             chunk's weights, pre-arranged in the operand layout;
+//   warp 0    one thread issues TMA loads: per 16-channel chunk a 5-D tiled
+//             tensor load (the halo box; the TMA unit zero-fills outside the
+//             volume) and one bulk copy of the chunk's weights, pre-arranged
+//             in the operand layout;
 //   warp 1    one thread issues 27 taps x (tile rows / 128) MMAs per chunk
 //             into a TMEM accumulator and commits them to the stage's "empty"
 //             barrier, then the tile to the accumulator's "full" barrier;
@@ -49,6 +49,7 @@
 #include <mutex>
 
 #include "nm_internal.cuh"
+#include "nm_image.cuh"
 #include "nm_scratch.cuh"
 #include "nm_tc.cuh"
 
@@ -58,7 +59,7 @@ namespace {
 typedef __nv_bfloat16 bf16;
 
 constexpr int TX = 16;
-constexpr uint32_t kSboB = 27 * 16 / 8 * 128;               // 8 weight rows of 27 x 16 channels
+constexpr uint32_t kSboB = 27 * 16 / 8 * 128;               // 8 outputs of 27 x 16 channels
 constexpr int kEpiParts = 3;                               // epilogue warps per TMEM lane quarter
 constexpr int kEpiThreads = 128 * kEpiParts;               // warps 2 .. 1 + 4 kEpiParts
 constexpr int kThreads = 64 + kEpiThreads;
@@ -68,7 +69,7 @@ constexpr long long kWaitCycles = 4ll << 30;
 // Every 128-row M-tile accumulates its 27 taps in order, so the M-tiles are
 // the independent MMA chains in flight: 16-output layers, whose small MMAs
 // are bound by that chain latency, take deeper tiles (more M-tiles).
-template <int COUT, int TZ, int TY, bool SWZ, bool PACK = false>
+template <int COUT, int TZ, int TY, bool PACK = false>
 struct TileLayout {
   static constexpr int PX = TX + 2, PY = TY + 2, PZ = TZ + 2;
   static constexpr int kRows = PX * PY * PZ;                // padded tile voxels
@@ -80,14 +81,11 @@ struct TileLayout {
   static constexpr int kNcol = PACK ? 3 * COUT : COUT;      // accumulator columns per M-tile
   static constexpr int kDelta = PY * PX + PX + 1;           // largest tap shift
   static constexpr int kRowsAlloc = (kCmin + kMt * 128 + kDelta + 15) / 16 * 16;  // rows any MMA may read
-  // SWZ: one 16-channel plane of 32-byte swizzled rows; else two 8-channel
-  // planes of 16-byte rows
-  static constexpr int kPlanes = SWZ ? 1 : 2;
-  static constexpr uint32_t kRowBytes = SWZ ? 32 : 16;
-  static constexpr uint32_t kPlane = kRowsAlloc * kRowBytes; // one plane (256-byte multiple)
-  static constexpr uint32_t kBoxBytes = kRows * kRowBytes;  // what one plane's TMA load writes
+  static constexpr uint32_t kRowBytes = 32;                 // 16 channels, 32-byte swizzled rows
+  static constexpr uint32_t kPlane = kRowsAlloc * kRowBytes; // the tile (256-byte multiple)
+  static constexpr uint32_t kBoxBytes = kRows * kRowBytes;  // what its TMA load writes
   static constexpr uint32_t kB = COUT / 8 * kSboB;          // one chunk's weights
-  static constexpr uint32_t kStage = (kPlanes * kPlane + kB + 1023) / 1024 * 1024;
+  static constexpr uint32_t kStage = (kPlane + kB + 1023) / 1024 * 1024;
   static constexpr int kStages = (3 * kStage <= 220 * 1024) ? 3 : 2;
   static constexpr int kAccCols = kMt * kNcol;
   static constexpr int kNacc = 2 * kAccCols <= 512 ? 2 : 1;
@@ -98,7 +96,6 @@ struct TileLayout {
   static_assert(kPlane % 256 == 0, "planes keep 256-byte (swizzle atom) alignment");
   static_assert(kAccCols <= 512, "accumulator fits the tensor memory");
   static_assert(kSmem <= 227 * 1024, "shared memory");
-  static_assert(!PACK || SWZ, "the packed variant reads three taps' rows of the swizzled weight image");
   static_assert(!PACK || COUT == 16, "the packed variant serves 16 outputs");
 };
 
@@ -140,14 +137,14 @@ struct TileGrid {
   }
 };
 
-template <int COUT, int TZ, int TY, bool SWZ, bool PACK>
+template <int COUT, int TZ, int TY, bool PACK>
 __global__ void __launch_bounds__(kThreads, 1) conv_tile_kernel(const __grid_constant__ CUtensorMap tmx,
                                                                 const TileGrid g, int nchunks,
                                                                 const bf16* __restrict__ wt,
                                                                 const float* __restrict__ bias,
                                                                 bf16* __restrict__ y, int ldy, int relu,
                                                                 const TileHead hd, uint32_t* status) {
-  typedef TileLayout<COUT, TZ, TY, SWZ, PACK> L;
+  typedef TileLayout<COUT, TZ, TY, PACK> L;
   constexpr int NC = L::kNcol;
   constexpr int S = L::kStages, NA = L::kNacc;
   constexpr int PX = L::PX, PY = L::PY, kMt = L::kMt, kCmin = L::kCmin, kCmax = L::kCmax;
@@ -198,10 +195,9 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tile_kernel(const __grid_con
             break;
           }
           const uint32_t sa = base + s * L::kStage;
-          tc::mbar_arrive_expect_tx(&full[s], L::kPlanes * L::kBoxBytes + L::kB);
+          tc::mbar_arrive_expect_tx(&full[s], L::kBoxBytes + L::kB);
           tc::tma_load_5d(sa, &tmx, &full[s], cc * 16, x0 - 1, y0 - 1, z0 - 1, b);
-          if (!SWZ) tc::tma_load_5d(sa + kPlane, &tmx, &full[s], cc * 16 + 8, x0 - 1, y0 - 1, z0 - 1, b);
-          tc::bulk_load(sa + L::kPlanes * kPlane, wt + (size_t)cc * COUT * 432, L::kB, &full[s]);
+          tc::bulk_load(sa + L::kPlane, wt + (size_t)cc * COUT * 432, L::kB, &full[s]);
           ++it;
         }
       }
@@ -230,13 +226,13 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tile_kernel(const __grid_con
           }
           tc::fence_after_sync();
           const uint32_t sa = base + s * L::kStage;
-          const uint32_t sb = sa + L::kPlanes * kPlane;
+          const uint32_t sb = sa + L::kPlane;
           // Descriptors differ only in the start-address field (bits 0-13, in
           // 16-byte units, no carry out for shared-memory addresses): build
           // two once and offset them by compile-time constants, so that the
           // issuing thread spends a few instructions per MMA.
-          const uint64_t a_base = SWZ ? tc::smem_desc_sw32(sa, 256) : tc::smem_desc(sa, kPlane, 128);
-          const uint64_t b_base = SWZ ? tc::smem_desc_sw32(sb, 256) : tc::smem_desc(sb, 128, kSboB);
+          const uint64_t a_base = tc::smem_desc_sw32(sa, 256);
+          const uint64_t b_base = tc::smem_desc_sw32(sb, 256);
           const uint32_t first = cc != 0;
           // packed: the three x-taps of a (dz, dy) pair in one MMA, the voxel
           // operand shifted for the first (dx = -1)
@@ -244,7 +240,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tile_kernel(const __grid_con
           for (int it2 = 0; it2 < (PACK ? 9 : 27); ++it2) {
             const int tap = PACK ? 3 * it2 : it2;
             const int delta = ((tap / 9 - 1) * PY + ((tap / 3) % 3 - 1)) * PX + (tap % 3 - 1);
-            const uint64_t bdesc = b_base + (uint64_t)((SWZ ? tap * COUT * 32 : tap * 256) >> 4);
+            const uint64_t bdesc = b_base + (uint64_t)((tap * COUT * 32) >> 4);
 #pragma unroll
             for (int mt = 0; mt < kMt; ++mt) {
               const uint64_t adesc = a_base + (uint64_t)(((kCmin + mt * 128 + delta) * (int)L::kRowBytes) >> 4);
@@ -461,34 +457,39 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tile_kernel(const __grid_con
 
 // Weights [cout][kpad] (K index tap * cin + c) -> per 16-channel chunk the
 // shared-memory image of the B operand, zero for channels >= cin:
-//   swz:  [chunk][27 taps][cout rows][2 halves of 8 channels], the halves of
-//         row co exchanged when bit 2 of co is set (32-byte swizzle);
-//   else: [chunk][cout / 8][27 taps x 2 halves][8 rows][8 channels].
-__global__ void tile_weights_kernel(const bf16* __restrict__ w, int cin, int kpad, int cout, int nchunks, int swz,
-                                    bf16* __restrict__ out) {
-  const long long total = (long long)nchunks * cout * 432;
+// [chunk][27 taps][cout rows][2 halves of 8 channels], the halves of row co
+// exchanged when bit 2 of co is set (32-byte swizzle).  A convolution computed
+// P outputs at a time has the images of its parts one after the other.  With
+// flip the taps are read backwards and inputs and outputs exchanged, from a
+// layer's weights [cin][kpad(cout)] for its input gradient.  A thread writes 8
+// channels; grid y = image.
+struct ImageJobs {
+  TileImage job[kMaxImages];
+};
+__host__ __device__ inline int image_part(int cout) { return cout == 96 ? 48 : cout == 192 ? 64 : cout; }
+__global__ void tile_weights_kernel(const __grid_constant__ ImageJobs jobs) {
+  const TileImage j = jobs.job[blockIdx.y];
+  const int nchunks = (j.cin + 15) / 16, P = image_part(j.cout), kpad = j.kpad;
+  const long long total = (long long)nchunks * j.cout * 54;
+  const __nv_bfloat16* w = reinterpret_cast<const __nv_bfloat16*>(j.w);
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
-    const int e = (int)(i % 8);
-    long long t = i / 8;
-    int co, tap, half, cc;
-    if (swz) {
-      const int pos = (int)(t % 2); t /= 2;
-      co = (int)(t % cout); t /= cout;
-      tap = (int)(t % 27);
-      cc = (int)(t / 27);
-      half = pos ^ ((co >> 2) & 1);
-    } else {
-      const int r = (int)(t % 8); t /= 8;
-      const int kc = (int)(t % 54); t /= 54;
-      const int grp = (int)(t % (cout / 8));
-      cc = (int)(t / (cout / 8));
-      co = grp * 8 + r;
-      tap = kc >> 1;
-      half = kc & 1;
+    long long t = i;
+    const int pos = (int)(t % 2); t /= 2;
+    const int r = (int)(t % P); t /= P;
+    const int tap = (int)(t % 27); t /= 27;
+    const int cc = (int)(t % nchunks);
+    const int co = (int)(t / nchunks) * P + r;
+    const int ch = cc * 16 + (pos ^ ((r >> 2) & 1)) * 8;       // cin is a multiple of 8
+    __align__(16) __nv_bfloat16 v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      v[e] = __float2bfloat16_rn(0.0f);
+      if (ch < j.cin)
+        v[e] = j.flip ? w[(long long)(ch + e) * kpad + (26 - tap) * j.cout + co]
+                      : w[(long long)co * kpad + tap * j.cin + ch + e];
     }
-    const int ch = cc * 16 + half * 8 + e;
-    out[i] = ch < cin ? w[(long long)co * kpad + tap * cin + ch] : __float2bfloat16_rn(0.0f);
+    reinterpret_cast<uint4*>(j.out)[i] = *reinterpret_cast<const uint4*>(v);
   }
 }
 
@@ -518,32 +519,26 @@ int sm_count() {
 
 // y: output voxel v's channels at y + v ldy (ldy = COUT, or the full width
 // when a wider convolution is computed COUT outputs at a time).
-template <int COUT, int TZ, int TY, bool SWZ, bool PACK = false>
-cudaError_t launch_tile(const nm_conv3d_desc& d, const void* x, const void* w, const float* bias, void* y,
+template <int COUT, int TZ, int TY, bool PACK = false>
+cudaError_t launch_tile(const nm_conv3d_desc& d, const void* x, const void* image, const float* bias, void* y,
                         int relu, const TileHead& hd, uint32_t* status, cudaStream_t s, int ldy) {
-  typedef TileLayout<COUT, TZ, TY, SWZ, PACK> L;
+  typedef TileLayout<COUT, TZ, TY, PACK> L;
   const int cin = d.c0;
   const int nchunks = (cin + 15) / 16;
-  // the input as a 5-D tensor (c, x, y, z, n); boxes of 8 channels x the padded tile
+  // the input as a 5-D tensor (c, x, y, z, n); boxes of 16 channels x the padded tile
   PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
   if (!enc) return cudaErrorNotSupported;
   CUtensorMap map;
   const cuuint64_t dims[5] = {(cuuint64_t)cin, (cuuint64_t)d.w, (cuuint64_t)d.h, (cuuint64_t)d.d, (cuuint64_t)d.n};
   const cuuint64_t strides[4] = {(cuuint64_t)cin * 2, (cuuint64_t)d.w * cin * 2, (cuuint64_t)d.h * d.w * cin * 2,
                                  (cuuint64_t)d.d * d.h * d.w * cin * 2};
-  const cuuint32_t box[5] = {SWZ ? 16u : 8u, (cuuint32_t)L::PX, (cuuint32_t)L::PY, (cuuint32_t)L::PZ, 1};
+  const cuuint32_t box[5] = {16u, (cuuint32_t)L::PX, (cuuint32_t)L::PY, (cuuint32_t)L::PZ, 1};
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   if (enc(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(x), dims, strides, box, estr,
-          CU_TENSOR_MAP_INTERLEAVE_NONE, SWZ ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_NONE,
+          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B,
           CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
-  bf16* wt = nullptr;
-  const size_t welems = (size_t)nchunks * COUT * 432;
-  cudaError_t e = stream_alloc((void**)&wt, welems * sizeof(bf16), s);
-  if (e != cudaSuccess) return e;
-  tile_weights_kernel<<<(unsigned)std::min<size_t>((welems + 255) / 256, 4096), 256, 0, s>>>(
-      (const bf16*)w, cin, conv_kpad(cin), COUT, nchunks, SWZ ? 1 : 0, wt);
   TileGrid g;
   g.n = d.n; g.d = d.d; g.h = d.h; g.w = d.w;
   g.tiles_x = (d.w + TX - 1) / TX;
@@ -552,16 +547,15 @@ cudaError_t launch_tile(const nm_conv3d_desc& d, const void* x, const void* w, c
   g.tz = TZ;
   g.tiles_z = (d.d + TZ - 1) / TZ;
   g.tiles = (long long)g.tiles_x * g.tiles_y * g.tiles_z * g.n;
-  e = cudaFuncSetAttribute(conv_tile_kernel<COUT, TZ, TY, SWZ, PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(conv_tile_kernel<COUT, TZ, TY, PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)L::kSmem);
   if (e == cudaSuccess) {
     const long long grid = std::min<long long>(g.tiles, sm_count());
-    conv_tile_kernel<COUT, TZ, TY, SWZ, PACK><<<(unsigned)grid, kThreads, L::kSmem, s>>>(map, g, nchunks, wt, bias,
+    conv_tile_kernel<COUT, TZ, TY, PACK><<<(unsigned)grid, kThreads, L::kSmem, s>>>(map, g, nchunks, (const bf16*)image, bias,
                                                                                       (bf16*)y, ldy, relu, hd,
                                                                                       status);
     e = cudaGetLastError();
   }
-  stream_free(wt, s);
   return e;
 }
 
@@ -575,7 +569,7 @@ cudaError_t launch_tile(const nm_conv3d_desc& d, const void* x, const void* w, c
 // 61; 2 x 32^3, 32 -> 32 39, 40, 49; 4 x 32^3 49, 53, 61; 2 x 50 x 37 x 61,
 // 96 -> 32 138, 162, 197.
 template <int COUT, bool PACK = false>
-cudaError_t launch_fitting(const nm_conv3d_desc& d, const void* x, const void* w, const float* bias, void* y,
+cudaError_t launch_fitting(const nm_conv3d_desc& d, const void* x, const void* image, const float* bias, void* y,
                            int relu, const TileHead& hd, uint32_t* status, cudaStream_t s, int ldy = COUT) {
   const long long sms = sm_count();
   auto turns = [&](int tz, int ty, int mt) {
@@ -583,9 +577,9 @@ cudaError_t launch_fitting(const nm_conv3d_desc& d, const void* x, const void* w
     return (tiles + sms - 1) / sms * (mt + 1);
   };
   const long long a = turns(2, 16, 5), b = turns(1, 16, 3), c = turns(1, 8, 2);
-  if (a < b && a < c) return launch_tile<COUT, 2, 16, true, PACK>(d, x, w, bias, y, relu, hd, status, s, ldy);
-  if (b < c) return launch_tile<COUT, 1, 16, true, PACK>(d, x, w, bias, y, relu, hd, status, s, ldy);
-  return launch_tile<COUT, 1, 8, true, PACK>(d, x, w, bias, y, relu, hd, status, s, ldy);
+  if (a < b && a < c) return launch_tile<COUT, 2, 16, PACK>(d, x, image, bias, y, relu, hd, status, s, ldy);
+  if (b < c) return launch_tile<COUT, 1, 16, PACK>(d, x, image, bias, y, relu, hd, status, s, ldy);
+  return launch_tile<COUT, 1, 8, PACK>(d, x, image, bias, y, relu, hd, status, s, ldy);
 }
 
 }  // namespace
@@ -627,21 +621,21 @@ static bool packed_tiles() {
   return !(e && e[0] == '1');
 }
 
-cudaError_t conv3d_fwd_tile(const nm_conv3d_desc& d, const void* x, const void* w, const float* bias, void* y,
-                            int relu, uint32_t* status, cudaStream_t s) {
+cudaError_t conv3d_fwd_image(const nm_conv3d_desc& d, const void* x, const void* image, const float* bias, void* y,
+                             int relu, uint32_t* status, cudaStream_t s) {
   const TileHead none{nullptr, nullptr, 0, nullptr};
-  if (d.cout == 16 && packed_tiles()) return launch_fitting<16, true>(d, x, w, bias, y, relu, none, status, s);
-  if (d.cout == 16) return launch_tile<16, 4, 16, true>(d, x, w, bias, y, relu, none, status, s, 16);
-  if (d.cout == 32) return launch_fitting<32>(d, x, w, bias, y, relu, none, status, s);
-  if (d.cout == 48) return launch_fitting<48>(d, x, w, bias, y, relu, none, status, s);
-  if (d.cout == 64) return launch_fitting<64>(d, x, w, bias, y, relu, none, status, s);
+  if (d.cout == 16 && packed_tiles()) return launch_fitting<16, true>(d, x, image, bias, y, relu, none, status, s);
+  if (d.cout == 16) return launch_tile<16, 4, 16>(d, x, image, bias, y, relu, none, status, s, 16);
+  if (d.cout == 32) return launch_fitting<32>(d, x, image, bias, y, relu, none, status, s);
+  if (d.cout == 48) return launch_fitting<48>(d, x, image, bias, y, relu, none, status, s);
+  if (d.cout == 64) return launch_fitting<64>(d, x, image, bias, y, relu, none, status, s);
   // 96 and 192 outputs (input gradients of the decoders' two-source layers):
   // 48 or 64 output channels per launch, written at the full channel stride
-  const int P = d.cout == 96 ? 48 : 64;
+  const int P = image_part(d.cout);
   nm_conv3d_desc dp = d;
   dp.cout = P;
   for (int p = 0; p < d.cout / P; ++p) {
-    const void* wp = (const bf16*)w + (size_t)p * P * conv_kpad(d.c0);
+    const void* wp = (const bf16*)image + p * tile_image_elems(d.c0, P);
     const float* bp = bias ? bias + p * P : nullptr;
     void* yp = (bf16*)y + p * P;
     const cudaError_t e = P == 48 ? launch_fitting<48>(dp, x, wp, bp, yp, relu, none, status, s, d.cout)
@@ -651,13 +645,46 @@ cudaError_t conv3d_fwd_tile(const nm_conv3d_desc& d, const void* x, const void* 
   return cudaSuccess;
 }
 
-cudaError_t conv3d_fwd_tile_head(const nm_conv3d_desc& d, const void* x, const void* w, const float* bias,
-                                 const float* head_w, const void* xin, int cx, float* yh, uint32_t* status,
-                                 cudaStream_t s) {
+cudaError_t conv3d_fwd_image_head(const nm_conv3d_desc& d, const void* x, const void* image, const float* bias,
+                                  const float* head_w, const void* xin, int cx, float* yh, uint32_t* status,
+                                  cudaStream_t s) {
   if (d.cout != 16 || !conv_tile_ok(d)) return cudaErrorInvalidValue;
   const TileHead hd{head_w, (const bf16*)xin, cx, yh};
-  if (packed_tiles()) return launch_fitting<16, true>(d, x, w, bias, nullptr, 1, hd, status, s);
-  return launch_tile<16, 4, 16, true>(d, x, w, bias, nullptr, 1, hd, status, s, 16);
+  if (packed_tiles()) return launch_fitting<16, true>(d, x, image, bias, nullptr, 1, hd, status, s);
+  return launch_tile<16, 4, 16>(d, x, image, bias, nullptr, 1, hd, status, s, 16);
+}
+
+long long tile_image_elems(int cin, int cout) { return (long long)((cin + 15) / 16) * cout * 432; }
+
+cudaError_t launch_tile_images(const TileImage* images, int count, cudaStream_t s) {
+  if (count > kMaxImages) return cudaErrorInvalidValue;
+  ImageJobs jobs;
+  long long most = 0;
+  for (int i = 0; i < count; ++i) {
+    jobs.job[i] = images[i];
+    jobs.job[i].kpad = conv_kpad(images[i].flip ? images[i].cout : images[i].cin);
+    most = std::max(most, tile_image_elems(images[i].cin, images[i].cout) / 8);
+  }
+  if (most > 0)
+    tile_weights_kernel<<<dim3((unsigned)std::min<long long>((most + 255) / 256, 4096), count), 256, 0, s>>>(jobs);
+  return cudaGetLastError();
+}
+
+bool conv_image_ok(const nm_conv3d_desc& d) {
+  const char* force = getenv("NM_CONV_GATHER");
+  return conv_tile_ok(d) && !(force && force[0] == '1');
+}
+
+cudaError_t conv3d_fwd_tile(const nm_conv3d_desc& d, const void* x, const void* w, const float* bias, void* y,
+                            int relu, uint32_t* status, cudaStream_t s) {
+  uint16_t* image = nullptr;
+  cudaError_t e = stream_alloc((void**)&image, tile_image_elems(d.c0, d.cout) * 2, s);
+  if (e != cudaSuccess) return e;
+  const TileImage job{(const uint16_t*)w, image, d.c0, d.cout, 0, 0};
+  e = launch_tile_images(&job, 1, s);
+  if (e == cudaSuccess) e = conv3d_fwd_image(d, x, image, bias, y, relu, status, s);
+  stream_free(image, s);
+  return e;
 }
 
 }  // namespace nm
