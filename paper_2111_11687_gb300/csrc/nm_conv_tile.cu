@@ -116,6 +116,21 @@ __device__ __forceinline__ bool epi_all(bool ok) {
   return r != 0;
 }
 
+// 32 bytes of one thread, a whole sector: in one store where the output is
+// 32-byte aligned (wide), since two of 16 bytes, 32 bytes apart between lanes,
+// write every sector twice.  60 x 64 x 64 voxels, 192 -> 64 channels 272 -> 263
+// us, 128 x 192 x 256, 16 -> 16 251 -> 247.
+__device__ __forceinline__ void store32(bf16* dst, const uint32_t (&o)[8], bool wide) {
+  if (wide) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(__cvta_generic_to_global(dst)),
+                 "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7])
+                 : "memory");
+  } else {
+    reinterpret_cast<uint4*>(dst)[0] = make_uint4(o[0], o[1], o[2], o[3]);
+    reinterpret_cast<uint4*>(dst)[1] = make_uint4(o[4], o[5], o[6], o[7]);
+  }
+}
+
 // Optional fused 1x1x1 head (16-output layers): instead of the activations,
 // write yh[v] = hb + x[v][0] + sum_c hw[c] * bf16(act[v][c]) (FP32), the same
 // arithmetic, in the same order, as the separate head.
@@ -262,6 +277,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tile_kernel(const __grid_con
     const int q = warp & 3;                  // TMEM lane quarter of this warp
     const int part = (warp - 2) >> 2;        // this warp's M-tiles: mt = part modulo kEpiParts
     const uint32_t lanes = tmem + ((uint32_t)(q * 32) << 16);
+    const bool wide = (reinterpret_cast<uintptr_t>(y) & 31) == 0;   // ldy is a multiple of 16
     // padded-tile coordinates of centre c packed as pz << 16 | py << 8 | px,
     // or -1 when c is not a centre of the tile
     auto centre_code = [](int c) {
@@ -333,9 +349,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tile_kernel(const __grid_con
             const __nv_bfloat162 p = __floats2bfloat162_rn(t0, t1);   // t0 in the low half
             o[j] = *reinterpret_cast<const uint32_t*>(&p);
           }
-          uint4* dst = reinterpret_cast<uint4*>(y + vox * ldy);
-          dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-          dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+          store32(y + vox * ldy, o, wide);
         };
 #pragma unroll
         for (int i = 0; i < kSlots; ++i) {
@@ -431,16 +445,19 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tile_kernel(const __grid_con
               }
               hd.yh[vox] = out;
             } else if (ok) {
-              __align__(16) bf16 o[16];
+              uint32_t o[8];
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                float tv = v[j] + (bias ? __ldg(bias + cq * 16 + j) : 0.0f);
-                if (relu) tv = fmaxf(tv, 0.0f);
-                o[j] = __float2bfloat16_rn(tv);
+              for (int j = 0; j < 8; ++j) {
+                float t0 = v[2 * j] + (bias ? __ldg(bias + cq * 16 + 2 * j) : 0.0f);
+                float t1 = v[2 * j + 1] + (bias ? __ldg(bias + cq * 16 + 2 * j + 1) : 0.0f);
+                if (relu) {
+                  t0 = fmaxf(t0, 0.0f);
+                  t1 = fmaxf(t1, 0.0f);
+                }
+                const __nv_bfloat162 p = __floats2bfloat162_rn(t0, t1);   // t0 in the low half
+                o[j] = *reinterpret_cast<const uint32_t*>(&p);
               }
-              uint4* dst = reinterpret_cast<uint4*>(y + vox * ldy + cq * 16);
-              dst[0] = reinterpret_cast<uint4*>(o)[0];
-              dst[1] = reinterpret_cast<uint4*>(o)[1];
+              store32(y + vox * ldy + cq * 16, o, wide);
             }
           }
         }
