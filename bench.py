@@ -132,7 +132,7 @@ def batch_phantoms(n):
 
 def batched_perf(torch, nm, phs, decays, steps, warmup):
     """nm_dose_run_batch over the uneven patients: every patient gets `decays`
-    decays per step in one CUDA graph of persistent multi-patient launches."""
+    decays per step, the patients' launches side by side on four streams."""
     from paper_2111_11687_gb300 import inputs
     gm = _materials_gpu(nm)
     hs = []
@@ -290,7 +290,7 @@ def run_gpu(args):
                 "scaling": "weak", "vs_baseline": None, "dtype": "f32+int64", "data": "synthetic",
                 "config": {"workload": WORKLOAD, "decays_per_step": DECAYS_PER_STEP, "grid": list(SHAPE[::-1]),
                            "voxel_mm": [x * 10 for x in SPACING], "batches": 10,
-                           "l2": "working set (tallies 2x157 MB + grid 79 MB + alias 41 MB) exceeds the 129 MB L2",
+                           "l2": "working set (tallies 11x157 MB + grid 79 MB + alias 41 MB) exceeds the 129 MB L2",
                            "parallelism": f"histories sharded over {ws} GPU(s)"},
                 "gpu_launches": launches, "roofline": roofline, "clocks": clocks, "e2e": e2e,
                 "cpu_baseline": cpu, "denoiser": den, "batched": batched, "time_to_2pct": ttt,
@@ -451,7 +451,7 @@ def transport_roofline(per_decay, decays_per_launch, launch_ms, clocks, probes, 
             "traffic": traffic,
             "traffic_source": "from_profile: profiles/transport_kernel_adult_phantom.md (same kernel source)"
             if traffic is not None else None,
-            "peak_source": "measured" if peaks else "fallback", "kernel": "transport_kernel",
+            "peak_source": "measured" if peaks else "fallback", "kernel": "transport_ring_kernel",
             "launch_ms": launch_ms, "decays_per_launch": decays_per_launch, "bytes_per_decay": bytes_per_decay,
             "per_decay": per_decay, "ceilings": ceilings, "probes": probes}
 

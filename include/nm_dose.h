@@ -93,7 +93,10 @@ typedef struct {
   int32_t warp_aggregate;    /* warp-aggregated tally atomics: -1 auto, 0 off, 1 on */
   int32_t regroup;           /* event regrouping in the transport: -1 auto, 0 off, 1 on */
   int32_t regroup_lanes;     /* lanes of a warp that must wait for a Compton or a
-                                new-history pass before it runs (1..32); 0 = auto */
+                                new-history pass before it runs (1..32); 0 = auto.
+                                For history statistics and decays with both annihilation
+                                photons and lines; other runs hand photons between lanes
+                                and do not use it */
   int32_t max_steps;         /* per-photon flight-step limit (bounded loops) */
   void* stream;              /* cudaStream_t; NULL = legacy default stream */
   int32_t history_sigma;     /* 1: also keep history-by-history statistics (the paper's
