@@ -28,6 +28,7 @@ namespace {
 
 constexpr int kBM = 128;        // GEMM rows per CTA
 constexpr int kKS = 64;         // K elements per stage (4 MMAs of K = 16)
+constexpr int kWS = 32;         // voxels per stage of the weight gradient (2 MMAs)
 constexpr int kThreads = 128;
 constexpr long long kWaitCycles = 4ll << 30;  // about 2 s at 2 GHz
 
@@ -49,12 +50,20 @@ struct Row {
 
 __device__ __forceinline__ Row make_row(const ConvGeom& g, long long m) {
   Row r;
-  const int x = (int)(m % g.w);
-  long long t = m / g.w;
-  const int y = (int)(t % g.h);
-  t /= g.h;
-  const int z = (int)(t % g.d);
-  const int b = (int)(t / g.d);
+  int x, y, z, b;
+  if (g.m >> 31 == 0) {                    // 32-bit divisions where they do
+    unsigned t = (unsigned)m;
+    x = (int)(t % (unsigned)g.w); t /= (unsigned)g.w;
+    y = (int)(t % (unsigned)g.h); t /= (unsigned)g.h;
+    z = (int)(t % (unsigned)g.d);
+    b = (int)(t / (unsigned)g.d);
+  } else {
+    long long t = m;
+    x = (int)(t % g.w); t /= g.w;
+    y = (int)(t % g.h); t /= g.h;
+    z = (int)(t % g.d);
+    b = (int)(t / g.d);
+  }
   if (g.coarse) {
     const int dd = g.d >> 1, hh = g.h >> 1, ww = g.w >> 1;
     r.off0 = ((((long long)b * dd + (z >> 1)) * hh + (y >> 1)) * ww + (x >> 1)) * g.c0;
@@ -68,9 +77,8 @@ __device__ __forceinline__ Row make_row(const ConvGeom& g, long long m) {
   const uint32_t my = (y > 0 ? 1u : 0u) | 2u | (y < g.h - 1 ? 4u : 0u);
   const uint32_t mx = (x > 0 ? 1u : 0u) | 2u | (x < g.w - 1 ? 4u : 0u);
   uint32_t vm = 1u << 30;  // the row is a voxel of the volume
-#pragma unroll
-  for (int t2 = 0; t2 < 27; ++t2)
-    if (((mz >> (t2 / 9)) & 1u) && ((my >> ((t2 / 3) % 3)) & 1u) && ((mx >> (t2 % 3)) & 1u)) vm |= 1u << t2;
+  const uint32_t plane = (my & 1u ? mx : 0u) | (my & 2u ? mx << 3 : 0u) | (my & 4u ? mx << 6 : 0u);
+  vm |= (mz & 1u ? plane : 0u) | (mz & 2u ? plane << 9 : 0u) | (mz & 4u ? plane << 18 : 0u);
   r.vmask = vm;
   return r;
 }
@@ -265,8 +273,8 @@ __global__ void __launch_bounds__(kThreads) conv_wgrad_kernel(ConvGeom g, const 
                                                               float* __restrict__ part, long long vox_per_split,
                                                               uint32_t* status) {
   constexpr int kNcols = COUT < 32 ? 32 : COUT;
-  constexpr uint32_t kABytes = kBM * kKS * 2;
-  constexpr uint32_t kBBytes = COUT * kKS * 2;
+  constexpr uint32_t kABytes = kBM * kWS * 2;
+  constexpr uint32_t kBBytes = COUT * kWS * 2;
   constexpr uint32_t kSboA = (kBM / 8) * 128;       // distance of K-adjacent core matrices of A
   constexpr uint32_t kSboB = (COUT / 8) * 128;      // ... and of B
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -294,7 +302,7 @@ __global__ void __launch_bounds__(kThreads) conv_wgrad_kernel(ConvGeom g, const 
   const long long p_begin = (long long)blockIdx.y * vox_per_split;
   long long p_end = p_begin + vox_per_split;
   if (p_end > g.m) p_end = g.m;
-  const int nstages = p_begin < p_end ? (int)((p_end - p_begin + kKS - 1) / kKS) : 0;
+  const int nstages = p_begin < p_end ? (int)((p_end - p_begin + kWS - 1) / kWS) : 0;
   constexpr uint32_t idesc = tc::idesc_bf16_f32(kBM, COUT, true, true);
   bool timeout = false;
   int issued = 0;
@@ -305,25 +313,25 @@ __global__ void __launch_bounds__(kThreads) conv_wgrad_kernel(ConvGeom g, const 
     if (__syncthreads_or(timeout)) { timeout = true; break; }
     uint8_t* a = sa + buf * kABytes;
     uint8_t* bm = sb + buf * kBBytes;
-    // A: 64 voxels x 16 chunks (8 GEMM rows each); a thread owns one voxel
-    // (tid % 64) and every other chunk.
+    // A: 32 voxels x 16 chunks (8 GEMM rows each); a thread owns one voxel
+    // (tid % 32) and every fourth chunk.
     {
-      const int pl = tid & 63;
-      const long long p = p_begin + s * kKS + pl;
+      const int pl = tid & 31;
+      const long long p = p_begin + s * kWS + pl;
       Row row;
       if (p < p_end) row = make_row(g, p);
       else row.vmask = 0u;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int rc = 2 * i + (tid >> 6);
+      for (int i = 0; i < 4; ++i) {
+        const int rc = 4 * i + (tid >> 5);
         const uint4 v = gather8(g, x0, x1, row, ktab[(k0 >> 3) + rc], s_d0, s_d1);
         *reinterpret_cast<uint4*>(a + rc * 128 + (pl >> 3) * kSboA + (pl & 7) * 16) = v;
       }
     }
-    // B: 64 voxels x COUT/8 chunks of dY.
-    for (int q = tid; q < kKS * (COUT / 8); q += kThreads) {
+    // B: 32 voxels x COUT/8 chunks of dY.
+    for (int q = tid; q < kWS * (COUT / 8); q += kThreads) {
       const int pl = q / (COUT / 8), rc = q % (COUT / 8);
-      const long long p = p_begin + s * kKS + pl;
+      const long long p = p_begin + s * kWS + pl;
       uint4 v = make_uint4(0, 0, 0, 0);
       if (p < p_end) v = __ldg(reinterpret_cast<const uint4*>(dy + p * COUT + rc * 8));
       *reinterpret_cast<uint4*>(bm + rc * 128 + (pl >> 3) * kSboB + (pl & 7) * 16) = v;
@@ -334,7 +342,7 @@ __global__ void __launch_bounds__(kThreads) conv_wgrad_kernel(ConvGeom g, const 
       tc::fence_after_sync();
       const uint32_t a0 = tc::smem_u32(a), b0 = tc::smem_u32(bm);
 #pragma unroll
-      for (int kk = 0; kk < kKS / 16; ++kk)
+      for (int kk = 0; kk < kWS / 16; ++kk)
         // MN-major, no swizzle: the leading byte offset steps along K (8 voxels),
         // the stride byte offset along MN (8 rows).
         tc::mma_bf16(tmem, tc::smem_desc(a0 + kk * 2 * kSboA, kSboA, 128),
@@ -379,6 +387,7 @@ __global__ void wgrad_reduce_kernel(const float* __restrict__ part, int splits, 
   if (i >= (long long)kpad * cout) return;
   const int k = (int)(i / cout), co = (int)(i % cout);
   float s = 0.0f;
+#pragma unroll 8
   for (int t = 0; t < splits; ++t) s += part[((long long)t * kpad + k) * cout + co];
   if (k == kreal && db) db[co] = s;
   dw[(long long)co * kpad + k] = k < kreal ? s : 0.0f;
@@ -449,12 +458,15 @@ cudaError_t launch_fwd_t(const ConvGeom& g, const __nv_bfloat16* x0, const __nv_
   return e;
 }
 
-// The weight-gradient buffers are over-allocated to 96 KB: every read the
-// MMAs can make from the stage buffers stays inside the CTA's allocation.
+// Two stages, and as much again at the least (40 KB, 48 with 128 outputs): five
+// CTAs of up to 64 outputs share an SM, four of 128 outputs (their tensor
+// memory), so that the splits of conv_wgrad_splits, about four per SM and a few
+// over, run at once.  Stages of 64 voxels and 96 KB left room for two, and the
+// launch took three turns: 4 x 16^3 voxels, 64 -> 64 channels 72 -> 46 us.
 template <int COUT>
 size_t wgrad_smem(int kpad) {
-  const size_t need = fwd_smem_base<COUT>() > 96 * 1024 ? fwd_smem_base<COUT>() : 96 * 1024;
-  return need + (size_t)(kpad / 8) * 4;
+  static_assert(4 * (kBM + COUT) * kWS <= (COUT == 128 ? 48 : 40) * 1024, "two stages");
+  return (COUT == 128 ? 48 : 40) * 1024 + (size_t)(kpad / 8) * 4;
 }
 
 template <int COUT>
