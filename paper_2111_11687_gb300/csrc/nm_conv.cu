@@ -458,7 +458,7 @@ cudaError_t launch_fwd_t(const ConvGeom& g, const __nv_bfloat16* x0, const __nv_
   return e;
 }
 
-// Two stages, and as much again at the least (40 KB, 48 with 128 outputs): five
+// Two stages and some slack (40 KB, 48 with 128 outputs): five
 // CTAs of up to 64 outputs share an SM, four of 128 outputs (their tensor
 // memory), so that the splits of conv_wgrad_splits, about four per SM and a few
 // over, run at once.  Stages of 64 voxels and 96 KB left room for two, and the

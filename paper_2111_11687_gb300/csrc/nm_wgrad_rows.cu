@@ -31,7 +31,7 @@
 //   What bounds it is the MMA rate: MMAs of 48 to 144 columns run at about 90
 // cycles each, the operands' shared-memory reads and the issue.  2 x 50 x 37 x
 // 61 voxels, 96 -> 32 channels: 105 us (351 in the shifted-window kernel), the
-// call 157 (522); 2 x 40 x 60 x 60, 128 -> 64: 390 us, the call 440 (2321 with
+// call 157 (522); 2 x 40 x 60 x 60, 128 -> 64: 390 us, the call 440 (1318 with
 // the gather kernel).
 //   warp 0    TMA producer: dY atoms and X planes of each tile into a stage ring;
 //   warp 1    MMA issuer;
@@ -431,10 +431,15 @@ bool conv_wgrad_rows_ok(const nm_conv3d_desc& d) {
   // Two chunks: 636 there, 240 here (32 -> 32); three: 283 and 150 (48 -> 16).
   if (d.cout == 16 || d.cout == 32) return d.c0 > 16;
   // 64 and 128 outputs: a small layer is launches, and the gather kernel has
-  // fewer.  Both sides of the line: 800 voxels, 64 -> 64 channels 42 us a call
-  // with the gather, 46 here; 2048 voxels, 64 -> 128 channels 62 and 54; 4096,
-  // 64 -> 64 66 and 53; 288,000, 128 -> 64 2321 and 440.
-  return (d.cout == 64 || d.cout == 128) && (long long)d.n * d.d * d.h * d.w * d.c0 >= 1 << 17;
+  // fewer; its cost grows with voxels x inputs, this one's has a read-out of 27 x
+  // inputs x outputs in it.  Microseconds a call with the gather and here, below
+  // and above each line.  64 outputs: 800 voxels of 64 inputs 42, 46; 4096 of 64
+  // 60, 53; 32,000 of 32 73, 78; 65,340 of 32 104, 83; 288,000 of 128 1318, 440.
+  // 128 outputs: 16,384 of 128 128, 178; 54,000 of 64 182, 214; 55,296 of 128 332,
+  // 312; 81,120 of 128 565, 462.
+  const long long work = (long long)d.n * d.d * d.h * d.w * d.c0;
+  if (d.cout == 64) return work >= (d.c0 >= 64 ? 1 << 17 : 1 << 20);
+  return d.cout == 128 && work >= 1 << 22;
 }
 
 size_t conv_wgrad_rows_workspace(const nm_conv3d_desc& d) {

@@ -19,10 +19,10 @@ pytestmark = pytest.mark.gpu
     (1, 2, 7, 13, 80, 16),       # five chunks in groups of two: the last group half empty
     (1, 5, 17, 29, 32, 32),      # a z-tap a pass
     (2, 1, 9, 1, 144, 32),       # columns; nine chunks by three
-    (2, 9, 23, 29, 16, 64),      # one chunk
+    (2, 28, 33, 36, 16, 64),     # one chunk
     (1, 10, 13, 15, 80, 64),     # 64 outputs, the last group half empty
-    (1, 13, 36, 43, 8, 128),     # half a chunk
-    (1, 6, 24, 43, 48, 128),
+    (2, 52, 70, 73, 8, 128),     # half a chunk
+    (1, 20, 64, 70, 48, 128),
     (3, 16, 48, 70, 32, 32),     # more tiles than SMs: several tiles a CTA
     (4, 24, 73, 99, 32, 16),     # 3840 tiles, 26 a CTA: two sums each, added to the partial in turn
     (2, 22, 40, 43, 128, 64),    # the SMs shared among the passes
