@@ -855,7 +855,7 @@ nm_status nm_dose_create(nm_dose** out, const nm_grid* g, const nm_materials* mt
       (e = dalloc(&h->status, 1)) || (e = dalloc(&h->rho_max_bits, NM_MAX_MATERIALS)) ||
       (e = dalloc(&h->org_s1, kLabelSlots)) || (e = dalloc(&h->org_s2, kLabelSlots)) ||
       (e = dalloc(&h->organ_count, kLabelSlots)) ||
-      (e = dalloc(&h->organ_partial, (size_t)fold_blocks(V) * kMaxSlots * kLabelSlots)) ||
+      (e = dalloc(&h->organ_partial, (size_t)organ_tiles(V) * 2 * kLabelSlots)) ||
       (e = dalloc(&h->organ_out, 4 * kLabelSlots)))
     return bail(cuda_fail(e, "device allocation"));
   if (labels && ((e = dalloc(&h->labels, V)) || (e = dalloc(&h->label_bad, 1))))
@@ -1001,19 +1001,24 @@ static nm_status ensure_slots(nm_dose* h, int want) {
   want = (want + launches - 1) / launches;     // near-equal launches
   if (want <= h->slots) return NM_OK;
   ull* tb = nullptr;
-  const cudaError_t e = dalloc(&tb, (size_t)h->V * want);
-  if (e == cudaErrorMemoryAllocation) {
+  double* part = nullptr;
+  cudaError_t e = dalloc(&tb, (size_t)h->V * want);
+  if (!e && want > 2) e = dalloc(&part, (size_t)organ_tiles(h->V) * want * kLabelSlots);
+  if (!e) e = cudaMemsetAsync(tb, 0, each * want, h->stream);
+  if (!e) e = cudaStreamSynchronize(h->stream);
+  if (e) {
+    dfree(tb);
+    dfree(part);
+    if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "batch tallies");
     cudaGetLastError();                 // one batch per launch then
     return NM_OK;
   }
-  if (e) return cuda_fail(e, "batch tallies");
-  if (cudaError_t m = cudaMemsetAsync(tb, 0, each * want, h->stream)) {
-    dfree(tb);
-    return cuda_fail(m, "batch tallies");
-  }
-  NM_CUDA(cudaStreamSynchronize(h->stream), "batch tallies");
   dfree(h->tb);
   h->tb = tb;
+  if (part) {
+    dfree(h->organ_partial);
+    h->organ_partial = part;
+  }
   h->slots = want;
   return NM_OK;
 }
@@ -1033,7 +1038,7 @@ static FoldParams fold_params(const nm_dose* h) {
   FoldParams fp;
   memset(&fp, 0, sizeof fp);
   fp.tb = h->tb; fp.tsum = h->tsum; fp.s2 = h->s2; fp.density = h->density;
-  fp.labels = h->labels; fp.V = h->V; fp.gy_per_unit_vol = h->gy_per_unit_vol();
+  fp.labels = h->labels; fp.V = h->V; fp.sms = h->sms; fp.gy_per_unit_vol = h->gy_per_unit_vol();
   fp.organ_partial = h->organ_partial; fp.org_s1 = h->org_s1; fp.org_s2 = h->org_s2;
   fp.deposited = h->counters + kCtrDepositedUnits;
   return fp;
@@ -1305,7 +1310,7 @@ static nm_status finalize(nm_dose* h, float* dose, float* sigma, bool organs) {
   p.org_s1 = h->org_s1; p.org_s2 = h->org_s2;
   p.organ_count = h->organ_count;
   p.organ_out = h->organ_out;
-  NM_CUDA(launch_finalize(p, organs && h->labels, s), "finalize launch");
+  NM_CUDA(launch_finalize(p, organs && h->labels, h->sms, s), "finalize launch");
   return NM_OK;
 }
 

@@ -19,8 +19,8 @@ constexpr double kAvogadro = 6.02214076e23;
 constexpr double kJoulePerEv = 1.602176634e-19;
 constexpr float kTwoPi = 6.283185307179586f;
 constexpr int kKnTable = 1024;      // log-energy nodes of the Klein-Nishina table
-constexpr int kFoldThreads = 128;   // fold / finalize CTA size
-constexpr int kFoldTile = 2048;     // voxels a fold / finalize CTA takes at a time
+constexpr int kFoldThreads = 128;   // columns of a tile's organ sums, and CTA size of the fold
+constexpr int kFoldTile = 8192;     // voxels of a tile of the organ sums
 constexpr int kLabelSlots = NM_MAX_LABELS + 1;
 
 // Fixed-point energy: round-to-nearest-even of the FP32 product E * 6.4e7.
@@ -267,10 +267,11 @@ struct FoldParams {
   const float* density;
   const uint8_t* labels;    // may be NULL
   int64_t V;
+  int sms;
   double n_b[kMaxSlots];    // histories in each batch; 0: none, the slot is empty
   double inv_nb[kMaxSlots];
   double gy_per_unit_vol;   // J per unit / (1e-3 kg/g * voxel volume cm^3)
-  double* organ_partial;    // [n_slots][fold_blocks(V)][kLabelSlots]
+  double* organ_partial;    // [n_slots][kLabelSlots][organ_tiles(V)]
   double* org_s1;           // [kLabelSlots] sum_b O_b
   double* org_s2;           // [kLabelSlots] sum_b O_b^2 / n_b
   ull* deposited;           // counter
@@ -279,7 +280,7 @@ struct FoldParams {
     inv_nb[b] = n ? 1.0 / (double)n : 0.0;
   }
 };
-int fold_blocks(int64_t V);
+int organ_tiles(int64_t V);
 // Moves a launch's sums of squares (q_lo, q_hi: of low and high 32 bits) into the
 // 128-bit sums hi * 2^64 + lo.
 cudaError_t launch_fold_history(ull* q_lo, ull* q_hi, ull* lo, ull* hi, int64_t V, cudaStream_t s);
@@ -307,7 +308,7 @@ struct FinalizeParams {
   double activity_bq;
   float* dose;              // may be NULL
   float* sigma;             // may be NULL
-  double* organ_partial;    // [blocks][2][kLabelSlots]
+  double* organ_partial;    // [2][kLabelSlots][organ_tiles(V)]
   const double* org_s1;
   const double* org_s2;
   const long long* organ_count;  // [kLabelSlots]
@@ -316,7 +317,7 @@ struct FinalizeParams {
 // Eq. 1 dose rate only into p.dose (bit-identical to launch_finalize's).
 cudaError_t launch_dose_only(const FinalizeParams& p, int sms, cudaStream_t s);
 // organs: also the per-label sums and organ_out (needs labels).
-cudaError_t launch_finalize(const FinalizeParams& p, bool organs, cudaStream_t s);
+cudaError_t launch_finalize(const FinalizeParams& p, bool organs, int sms, cudaStream_t s);
 // Voxels per label into count[kLabelSlots] (labels >= kLabelSlots count as 0),
 // and atomicMin of first_bad with every voxel index whose label exceeds n_labels.
 cudaError_t launch_label_count(const uint8_t* labels, int64_t V, int n_labels, long long* count,

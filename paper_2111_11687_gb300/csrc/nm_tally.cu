@@ -7,8 +7,8 @@
 // voxel is x = Tsum / N and the batch estimate of its variance is
 //   var(x) = (S2 - Tsum^2 / N) / ((K - 1) N),
 // the n_b-weighted form of the batch-means estimator.  Every reduction has a
-// fixed tree (per-thread columns in shared memory, then fixed warp trees, then
-// blocks in index order), so the statistics are the same on every run.
+// fixed tree (columns of a tile, then fixed warp trees, then tiles in index
+// order), so the statistics are the same on every run.
 #include <algorithm>
 
 #include "nm_internal.cuh"
@@ -22,60 +22,57 @@ __device__ __forceinline__ double warp_sum_d(double x) {
   return x;
 }
 
-// Sums per label.  A tile of kFoldTile voxels holds few labels, so each thread
-// keeps FP64 sums for kAccLabels of them in columns of shared memory (one per
-// quantity and label); a tile with more labels is read again for the next
-// ones.  The columns, and then the tiles and blocks, are added in a fixed order.
-constexpr int kAccLabels = 4;
-constexpr int kPerThread = kFoldTile / kFoldThreads;       // voxels of a thread per tile
+// Sums per label keep one order, whatever kernel forms them, since the variance
+// of an organ's mean cancels and turns their last bits into leading ones of a
+// small sigma: a tile is kFoldTile voxels; column t of a label sums, in voxel
+// order, those of its voxels t, t + 128, ... of the tile; the tile's partial is
+// columns 0 .. 127 (column_sum), and the label's sum is the partials of all
+// tiles (tile_sum).  Partials: [quantity or slot][label][tile].
+constexpr int kColumn = kFoldTile / kFoldThreads;          // voxels of a column
+constexpr int kSub = 2048;                                 // voxels a CTA of 128 threads has in flight
+constexpr int kSubs = kFoldTile / kSub;
+constexpr int kPerThread = kSub / kFoldThreads;
 
-// Labels of this thread's voxels v0 + tid + i kFoldThreads, a byte each (0 past
-// v1); returns the set of labels in the tile.
-__device__ __forceinline__ uint32_t tile_labels(const uint8_t* __restrict__ labels, int64_t v0, int64_t v1,
-                                                uint32_t (&lab)[kPerThread / 4], uint32_t* s_mask) {
+__device__ __forceinline__ double column_sum(const double* col, int lane) {
+  double sum = 0.0;
+#pragma unroll
+  for (int j = 0; j < kFoldThreads / 32; ++j) sum += col[lane + 32 * j];
+  return warp_sum_d(sum);
+}
+
+__device__ __forceinline__ double tile_sum(const double* __restrict__ part, int n_tiles, int lane) {
+  double s = 0.0;
+#pragma unroll 8
+  for (int i = lane; i < n_tiles; i += 32) s += part[i];
+  return warp_sum_d(s);
+}
+
+// The tile's labels into shared memory, and the set of them that each warp met
+// in each sub-tile.  Ends with a barrier.
+template <int THREADS>
+__device__ __forceinline__ void tile_labels(const uint8_t* __restrict__ labels, int64_t v0, int64_t V, uint8_t* s_lab,
+                                            uint32_t (*s_mask)[THREADS / 32]) {
+#pragma unroll 1
+  for (int s = 0; s < kSubs; ++s) {
+    uint32_t mask = 0;
+#pragma unroll
+    for (int i = 0; i < kSub / THREADS; ++i) {
+      const int k = s * kSub + i * THREADS + threadIdx.x;
+      const uint32_t l = v0 + k < V ? labels[v0 + k] : 0u;
+      s_lab[k] = (uint8_t)l;
+      if (v0 + k < V) mask |= 1u << l;
+    }
+    mask = __reduce_or_sync(0xffffffffu, mask);
+    if ((threadIdx.x & 31) == 0) s_mask[s][threadIdx.x >> 5] = mask;
+  }
+  __syncthreads();
+}
+template <int THREADS>
+__device__ __forceinline__ uint32_t label_set(const uint32_t (*s_mask)[THREADS / 32], int s) {
   uint32_t mask = 0;
 #pragma unroll
-  for (int i = 0; i < kPerThread / 4; ++i) lab[i] = 0;
-#pragma unroll
-  for (int i = 0; i < kPerThread; ++i) {
-    const int64_t v = v0 + threadIdx.x + (int64_t)i * kFoldThreads;
-    const uint32_t l = v < v1 ? labels[v] : 0u;
-    lab[i / 4] |= l << (8 * (i % 4));
-    if (v < v1) mask |= 1u << l;
-  }
-  mask = __reduce_or_sync(0xffffffffu, mask);
-  if ((threadIdx.x & 31) == 0) s_mask[threadIdx.x >> 5] = mask;
-  __syncthreads();
-  mask = 0;
-#pragma unroll
-  for (int w = 0; w < kFoldThreads / 32; ++w) mask |= s_mask[w];
+  for (int w = 0; w < THREADS / 32; ++w) mask |= s_mask[s][w];
   return mask;
-}
-
-// Column of the thread's i-th voxel among those for labels l0, l0 + 1, ... of
-// the tile's set, or -1.
-__device__ __forceinline__ int label_column(const uint32_t (&lab)[kPerThread / 4], int i, uint32_t mask, int l0) {
-  const uint32_t l = (lab[i / 4] >> (8 * (i % 4))) & 255u;
-  const int c = __popc(mask & ((1u << l) - 1u)) - l0;
-  return c < kAccLabels ? c : -1;
-}
-
-// out[q][label] += the sum of the columns acc[q][0 .. n_acc) (labels l0, ... of
-// the set) for q < n_q; one warp per column.  Ends with the columns free again.
-__device__ __forceinline__ void add_columns(const double* acc, int n_q, int n_acc, uint32_t mask, int l0,
-                                            double (*out)[kLabelSlots]) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  __syncthreads();
-  for (int i = wid; i < n_q * n_acc; i += kFoldThreads / 32) {
-    const int q = i / n_acc, l = i % n_acc;
-    const double* col = acc + (q * kAccLabels + l) * kFoldThreads;
-    double sum = 0.0;
-#pragma unroll
-    for (int j = 0; j < kFoldThreads / 32; ++j) sum += col[lane + 32 * j];
-    sum = warp_sum_d(sum);
-    if (lane == 0) out[q][__fns(mask, 0, l0 + l + 1)] += sum;
-  }
-  __syncthreads();
 }
 
 // Fold of a launch's NS (or fewer) batches in one pass over the voxels: per
@@ -87,35 +84,56 @@ __device__ __forceinline__ void add_columns(const double* acc, int n_q, int n_ac
 // statistics, only where something was deposited) and, in densely hit volumes,
 // by FP64 (four operations per deposit-holding voxel and slot; this GPU does
 // about two per SM and clock).  A thread therefore loads NS x K tallies before
-// it uses any, and lone voxels of other batches cost nothing.
+// it uses any, and lone voxels of other batches cost nothing.  256 x 253 x 300
+// voxels, 6e6 decays in ten batches: 0.50 ms (ten folds 1.3).
 //
-// Benchmark phantom, ten batches: 10 x 0.18 ms as a fold each, 1.15 ms together.
+// With labels a CTA takes a whole tile, for the order of its organ sums, in
+// columns for fold_columns(NS) labels at a time; a tile with more labels is
+// gone through again, sub-tiles without any of the next ones left out.
+__host__ __device__ constexpr int fold_columns(int ns) { return ns == 1 ? 32 : ns == 2 ? 16 : ns <= 5 ? 8 : 4; }
+
 template <int NS, bool LABELS>
-__global__ void __launch_bounds__(kFoldThreads) fold_kernel(const FoldParams p, int tiles_per_block) {
+__global__ void __launch_bounds__(kFoldThreads) fold_kernel(const FoldParams p, int subs) {
   constexpr int K = NS <= 2 ? 8 : 4;       // voxels of a thread in flight
-  extern __shared__ double acc[];                         // [NS][kAccLabels][kFoldThreads]
-  __shared__ double out[LABELS ? NS : 1][kLabelSlots];
-  __shared__ uint32_t s_mask[kFoldThreads / 32];
+  constexpr int C = fold_columns(NS);
+  extern __shared__ double acc[];                         // [NS][C][kFoldThreads]
+  __shared__ uint8_t s_lab[LABELS ? kFoldTile : 1];
+  __shared__ uint32_t s_mask[kSubs][kFoldThreads / 32];
   __shared__ ull dep_w[kFoldThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  if (LABELS)
-    for (int i = tid; i < NS * kLabelSlots; i += kFoldThreads) out[i / kLabelSlots][i % kLabelSlots] = 0.0;
+  const int64_t first = (int64_t)blockIdx.x * subs * kSub;
   ull dep = 0;
   const float gy = (float)p.gy_per_unit_vol;
-  const int64_t first = (int64_t)blockIdx.x * tiles_per_block * kFoldTile;
-  for (int ti = 0; ti < tiles_per_block; ++ti) {
-    const int64_t v0 = first + (int64_t)ti * kFoldTile;
-    if (v0 >= p.V) break;
-    const int64_t v1 = v0 + kFoldTile < p.V ? v0 + kFoldTile : p.V;
-    uint32_t lab[kPerThread / 4];
-    const uint32_t mask = LABELS ? tile_labels(p.labels, v0, v1, lab, s_mask) : 0u;
-    const int n_lab = LABELS ? __popc(mask) : 1;
-    for (int l0 = 0; l0 < n_lab; l0 += kAccLabels) {
-      const int n_acc = min(kAccLabels, n_lab - l0);
-      const bool last = l0 + kAccLabels >= n_lab;
-      if (LABELS)
-        for (int i = 0; i < p.n_slots; ++i)
-          for (int l = 0; l < n_acc; ++l) acc[(i * kAccLabels + l) * kFoldThreads + tid] = 0.0;
+  uint32_t labels_left = 1u;                              // of the tile; one pass without labels
+  if (LABELS) {
+    tile_labels<kFoldThreads>(p.labels, first, p.V, s_lab, s_mask);
+    labels_left = 0;
+    for (int s = 0; s < kSubs; ++s) labels_left |= label_set<kFoldThreads>(s_mask, s);
+    for (int i = tid; i < p.n_slots * kLabelSlots; i += kFoldThreads)
+      if (!(labels_left >> (i % kLabelSlots) & 1u)) p.organ_partial[(size_t)i * gridDim.x + blockIdx.x] = 0.0;
+  }
+  while (labels_left) {
+    // the next labels, lowest first
+    uint32_t group = labels_left;
+    if (LABELS) {
+      for (int i = 0; i < C; ++i) labels_left &= labels_left - 1;
+      group &= ~labels_left;
+      for (int i = 0; i < p.n_slots; ++i)
+        for (int l = 0; l < __popc(group); ++l) acc[(i * C + l) * kFoldThreads + tid] = 0.0;
+    } else {
+      labels_left = 0;
+    }
+    for (int s = 0; s < subs; ++s) {
+      const int64_t v0 = first + (int64_t)s * kSub;
+      if (v0 >= p.V) break;
+      const int64_t v1 = v0 + kSub < p.V ? v0 + kSub : p.V;
+      bool fresh = true, last = true;                     // first and last time at these voxels
+      if (LABELS) {
+        const uint32_t here = label_set<kFoldThreads>(s_mask, s);
+        if (!(here & group)) continue;
+        fresh = (here & ((group & -group) - 1u)) == 0;
+        last = (here & labels_left) == 0;
+      }
 #pragma unroll 1
       for (int c = 0; c < kPerThread; c += K) {
         ull t[NS][K];
@@ -138,7 +156,7 @@ __global__ void __launch_bounds__(kFoldThreads) fold_kernel(const FoldParams p, 
           ts[j] = 0; s2v[j] = 0.0; rho[j] = 1.0f;
           if (any[j]) {
             const int64_t v = v0 + tid + (int64_t)(c + j) * kFoldThreads;
-            if (l0 == 0) {
+            if (fresh) {
               ts[j] = p.tsum[v];
               s2v[j] = p.s2[v];
             }
@@ -152,26 +170,42 @@ __global__ void __launch_bounds__(kFoldThreads) fold_kernel(const FoldParams p, 
           // Gy per unit in FP32 (GB300's FP64 divide is slow); the sum stays FP64
           const double g = LABELS ? (double)__fdiv_rn(gy, rho[j]) : 0.0;
           int la = -1;                                    // the voxel's column, if one of this pass
-          if (LABELS) la = label_column(lab, c + j, mask, l0);
+          if (LABELS) {
+            const uint32_t l = s_lab[s * kSub + tid + (c + j) * kFoldThreads];
+            if (group >> l & 1u) la = __popc(group & ((1u << l) - 1u));
+          }
 #pragma unroll
           for (int b = 0; b < NS; ++b) {
             if (!t[b][j]) continue;
             const double x = (double)t[b][j];
-            if (l0 == 0) {
+            if (fresh) {
               ts[j] += t[b][j];
               s2v[j] = s2v[j] + x * x * p.inv_nb[b];
               dep += t[b][j];
             }
-            if (LABELS && la >= 0) acc[(b * kAccLabels + la) * kFoldThreads + tid] += x * g;
+            if (LABELS && la >= 0) {
+              double* const a = acc + (b * C + la) * kFoldThreads + tid;
+              *a = fma(x, g, *a);
+            }
             if (last) p.tb[(int64_t)b * p.V + v] = 0;
           }
-          if (l0 == 0) {
+          if (fresh) {
             p.tsum[v] = ts[j];
             p.s2[v] = s2v[j];
           }
         }
       }
-      if (LABELS) add_columns(acc, p.n_slots, n_acc, mask, l0, out);
+    }
+    if (LABELS) {
+      const int n = __popc(group);
+      __syncthreads();
+      for (int i = wid; i < p.n_slots * n; i += kFoldThreads / 32) {
+        const int b = i / n, l = i % n;
+        const double sum = column_sum(acc + (b * C + l) * kFoldThreads, lane);
+        if (lane == 0)
+          p.organ_partial[((size_t)b * kLabelSlots + __fns(group, 0, l + 1)) * gridDim.x + blockIdx.x] = sum;
+      }
+      __syncthreads();
     }
   }
   // deposited-energy counter (integer, so the order of the adds does not matter)
@@ -184,20 +218,57 @@ __global__ void __launch_bounds__(kFoldThreads) fold_kernel(const FoldParams p, 
     for (int w = 0; w < kFoldThreads / 32; ++w) sum += dep_w[w];
     if (sum) atomicAdd(p.deposited, sum);
   }
-  if (LABELS)
-    for (int i = tid; i < p.n_slots * kLabelSlots; i += kFoldThreads)
-      p.organ_partial[((size_t)(i / kLabelSlots) * gridDim.x + blockIdx.x) * kLabelSlots + i % kLabelSlots] =
-          out[i / kLabelSlots][i % kLabelSlots];
 }
 
-// One CTA per label, one warp per slot: blocks lane-strided, then a fixed tree;
-// the slots are then added in batch order.
-__global__ void fold_organs_kernel(const FoldParams p, int n_blocks) {
+// The organ sums of a launch's batches alone, a CTA per tile and slot, ahead of
+// a fold without labels: where the tiles are too few for the chip.
+__global__ void __launch_bounds__(kFoldThreads) fold_slot_organs_kernel(const FoldParams p) {
+  constexpr int K = 16;
+  __shared__ double acc[kLabelSlots * kFoldThreads];
+  __shared__ uint8_t s_lab[kFoldTile];
+  __shared__ uint32_t s_mask[kSubs][kFoldThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, b = blockIdx.y;
+  const int64_t v0 = (int64_t)blockIdx.x * kFoldTile;
+  const ull* const tb = p.tb + (int64_t)b * p.V;
+  const float gy = (float)p.gy_per_unit_vol;
+  tile_labels<kFoldThreads>(p.labels, v0, p.V, s_lab, s_mask);
+  uint32_t set = 0;
+  for (int s = 0; s < kSubs; ++s) set |= label_set<kFoldThreads>(s_mask, s);
+  const int n = __popc(set);
+  for (int l = 0; l < n; ++l) acc[l * kFoldThreads + tid] = 0.0;
+#pragma unroll 1
+  for (int c = 0; c < kColumn; c += K) {
+    ull t[K];
+    float rho[K];
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+      const int64_t v = v0 + tid + (int64_t)(c + j) * kFoldThreads;
+      t[j] = v < p.V ? tb[v] : 0ull;
+    }
+#pragma unroll
+    for (int j = 0; j < K; ++j)
+      rho[j] = t[j] ? p.density[v0 + tid + (int64_t)(c + j) * kFoldThreads] : 1.0f;
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+      if (!t[j]) continue;
+      const uint32_t l = s_lab[tid + (c + j) * kFoldThreads];
+      double* const a = acc + __popc(set & ((1u << l) - 1u)) * kFoldThreads + tid;
+      *a = fma((double)t[j], (double)__fdiv_rn(gy, rho[j]), *a);
+    }
+  }
+  __syncthreads();
+  for (int l = wid; l < kLabelSlots; l += kFoldThreads / 32) {
+    double sum = 0.0;
+    if (set >> l & 1u) sum = column_sum(acc + __popc(set & ((1u << l) - 1u)) * kFoldThreads, lane);
+    if (lane == 0) p.organ_partial[((size_t)b * kLabelSlots + l) * gridDim.x + blockIdx.x] = sum;
+  }
+}
+
+// One CTA per label, one warp per slot; the slots are then added in batch order.
+__global__ void fold_organs_kernel(const FoldParams p, int n_tiles) {
   __shared__ double sum[kMaxSlots];
   const int lane = threadIdx.x & 31, b = threadIdx.x >> 5, l = blockIdx.x;
-  double s = 0.0;
-  for (int i = lane; i < n_blocks; i += 32) s += p.organ_partial[((size_t)b * n_blocks + i) * kLabelSlots + l];
-  s = warp_sum_d(s);
+  const double s = tile_sum(p.organ_partial + ((size_t)b * kLabelSlots + l) * n_tiles, n_tiles, lane);
   if (lane == 0) sum[b] = s;
   __syncthreads();
   if (threadIdx.x != 0) return;
@@ -211,114 +282,203 @@ __global__ void fold_organs_kernel(const FoldParams p, int n_blocks) {
   p.org_s2[l] = s2;
 }
 
-// Eq. 1 per voxel (MAPS: dose and sigma, either may be NULL) and the sums behind
-// Eq. 2 and Eq. 3 per label (ORGANS).
+// Eq. 1 of a voxel with tally t > 0: FP64 where cancellation needs it (the
+// mean and the variance, S2 - Tsum^2/N), the rest in FP32, whose precision the
+// FP32 outputs have anyway.
+__device__ __forceinline__ void voxel_dose(ull t, double s2, float rho, double inv_n, double inv_k1n, float gy_a,
+                                           float& d, float& sg) {
+  const double x = (double)t;
+  const double mean = x * inv_n;                       // units per decay
+  const double var = fma(-x, mean, s2) * inv_k1n;      // rounding may leave it below 0
+  const float conv = __fdiv_rn(gy_a, rho);
+  d = (float)mean * conv;                              // Eq. 1, Gy/s
+  sg = sqrtf(fmaxf((float)var, 0.0f)) * conv;
+}
+
+// Eq. 1 per voxel: dose and sigma, either may be NULL.
 //
-// Bound by DRAM (25 B per voxel for the maps) and FP64, which therefore does
-// only what needs it: the mean, the variance (S2 - Tsum^2/N cancels) and the
-// organ sums; the rest is FP32, whose precision the FP32 outputs have anyway.
-// Voxels without a deposit cost no FP64: their dose adds nothing and their
-// epsilon of 1 is counted in integers.  Eight voxels' loads go out together.
-// Whole body (157 M voxels): 3.3 ms for either -> 0.54 ms (maps), 1.02 ms (organs).
-template <bool MAPS, bool ORGANS>
-__global__ void __launch_bounds__(kFoldThreads) finalize_kernel(const FinalizeParams p, int tiles_per_block) {
+// Bound by DRAM (25 B per voxel) and FP64.  Voxels without a deposit cost no
+// FP64; eight voxels' loads go out together.  Whole body (157 M voxels): 3.3 ms
+// -> 0.54 ms.
+__global__ void __launch_bounds__(kFoldThreads) finalize_maps_kernel(const FinalizeParams p, int subs) {
   constexpr int K = 8;
-  __shared__ double acc[ORGANS ? 2 * kAccLabels * kFoldThreads : 1];   // dose, epsilon^2
-  __shared__ int zeros[ORGANS ? kAccLabels : 1][kFoldThreads];         // voxels without a deposit
-  __shared__ double out[ORGANS ? 2 : 1][kLabelSlots];
-  __shared__ uint32_t s_mask[kFoldThreads / 32];
-  const int tid = threadIdx.x;
-  if (ORGANS && tid < 2 * kLabelSlots) out[tid / kLabelSlots][tid % kLabelSlots] = 0.0;
   const double inv_n = 1.0 / p.n_total;
   const double inv_k1n = 1.0 / ((p.n_batches - 1.0) * p.n_total);
   const float gy_a = (float)(p.gy_per_unit_vol * p.activity_bq);
-  const int64_t first = (int64_t)blockIdx.x * tiles_per_block * kFoldTile;
-  for (int ti = 0; ti < tiles_per_block; ++ti) {
-    const int64_t v0 = first + (int64_t)ti * kFoldTile;
-    if (v0 >= p.V) break;
-    const int64_t v1 = v0 + kFoldTile < p.V ? v0 + kFoldTile : p.V;
-    uint32_t lab[kPerThread / 4];
-    const uint32_t mask = ORGANS ? tile_labels(p.labels, v0, v1, lab, s_mask) : 0u;
-    const int n_lab = ORGANS ? __popc(mask) : 1;
-    for (int l0 = 0; l0 < n_lab; l0 += kAccLabels) {
-      const int n_acc = min(kAccLabels, n_lab - l0);
-      if (ORGANS)
-        for (int l = 0; l < n_acc; ++l) {
-          acc[l * kFoldThreads + tid] = acc[(kAccLabels + l) * kFoldThreads + tid] = 0.0;
-          zeros[l][tid] = 0;
-        }
+  for (int s = 0; s < subs; ++s) {
+    const int64_t v0 = ((int64_t)blockIdx.x * subs + s) * kSub + threadIdx.x;
 #pragma unroll 1
-      for (int c = 0; c < kPerThread; c += K) {
-        ull t[K];
-        double s2v[K];
-        float rho[K];
+    for (int c = 0; c < kPerThread; c += K) {
+      ull t[K];
+      double s2v[K];
+      float rho[K];
 #pragma unroll
-        for (int j = 0; j < K; ++j) {
-          const int64_t v = v0 + tid + (int64_t)(c + j) * kFoldThreads;
-          t[j] = v < v1 ? p.tsum[v] : 0ull;
-        }
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-          const int64_t v = v0 + tid + (int64_t)(c + j) * kFoldThreads;
-          s2v[j] = 0.0; rho[j] = 1.0f;
-          if (t[j]) {
-            s2v[j] = p.s2[v];
-            rho[j] = p.density[v];
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-          const int64_t v = v0 + tid + (int64_t)(c + j) * kFoldThreads;
-          if (v >= v1) continue;
-          float d = 0.0f, sg = 0.0f;
-          if (t[j]) {
-            const double x = (double)t[j];
-            const double mean = x * inv_n;                       // units per decay
-            const double var = fma(-x, mean, s2v[j]) * inv_k1n;  // rounding may leave it below 0
-            const float conv = __fdiv_rn(gy_a, rho[j]);
-            d = (float)mean * conv;                              // Eq. 1, Gy/s
-            sg = sqrtf(fmaxf((float)var, 0.0f)) * conv;
-          }
-          if (MAPS) {
-            if (p.dose) p.dose[v] = d;
-            if (p.sigma) p.sigma[v] = sg;
-          }
-          if (ORGANS) {
-            const int la = label_column(lab, c + j, mask, l0);
-            if (la >= 0) {
-              if (d > 0.0f) {
-                const float eps = __fdiv_rn(sg, d);
-                acc[la * kFoldThreads + tid] += (double)d;
-                acc[(kAccLabels + la) * kFoldThreads + tid] += (double)(eps * eps);
-              } else {
-                zeros[la][tid] += 1;
-              }
-            }
-          }
-        }
+      for (int j = 0; j < K; ++j) {
+        const int64_t v = v0 + (int64_t)(c + j) * kFoldThreads;
+        t[j] = v < p.V ? p.tsum[v] : 0ull;
       }
-      if (ORGANS) {
-        for (int l = 0; l < n_acc; ++l)
-          if (zeros[l][tid]) acc[(kAccLabels + l) * kFoldThreads + tid] += (double)zeros[l][tid];
-        add_columns(acc, 2, n_acc, mask, l0, out);
+#pragma unroll
+      for (int j = 0; j < K; ++j) {
+        const int64_t v = v0 + (int64_t)(c + j) * kFoldThreads;
+        s2v[j] = t[j] ? p.s2[v] : 0.0;
+        rho[j] = t[j] ? p.density[v] : 1.0f;
+      }
+#pragma unroll
+      for (int j = 0; j < K; ++j) {
+        const int64_t v = v0 + (int64_t)(c + j) * kFoldThreads;
+        if (v >= p.V) continue;
+        float d = 0.0f, sg = 0.0f;
+        if (t[j]) voxel_dose(t[j], s2v[j], rho[j], inv_n, inv_k1n, gy_a, d, sg);
+        if (p.dose) p.dose[v] = d;
+        if (p.sigma) p.sigma[v] = sg;
       }
     }
   }
-  if (ORGANS && tid < 2 * kLabelSlots)
-    p.organ_partial[(size_t)blockIdx.x * 2 * kLabelSlots + tid] = out[tid / kLabelSlots][tid % kLabelSlots];
 }
 
-__global__ void finalize_organs_kernel(const FinalizeParams p, int n_blocks) {
+// x as FP64, without the FP64 pipe where x is normal.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x);
+  if (((u >> 23) & 255u) - 1u >= 254u) return (double)x;
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+
+// a + 1 rounded to nearest even, without the FP64 pipe from 1 to 2^40 and at 0:
+// the mantissa plus one unit and, past the binade, half of that with the bit
+// that drops out.
+__device__ __forceinline__ double add_one(double a) {
+  const ull b = (ull)__double_as_longlong(a), one = 1023ull << 52;
+  if (b == 0) return 1.0;
+  if (b - one >= 40ull << 52) return a + 1.0;
+  const uint32_t ex = (uint32_t)(b >> 52);
+  const ull m = ((b & ((1ull << 52) - 1)) | 1ull << 52) + (1ull << (52 + 1023 - ex));
+  const ull h = m >> 1;
+  const ull r = m >> 53 ? h + (m & h & 1ull) + ((ull)ex << 52) : m + ((ull)(ex - 1) << 52);
+  return __longlong_as_double((long long)r);
+}
+
+// Partials of the NQ quantities staged in s_val (dose; then epsilon^2) for every
+// label of the tile, by 512 threads: thread t of a group of 128 goes through
+// column t's voxels once for one quantity and every WIDE-th label, the label
+// at hand in a register, the others in `col`.  Zero doses add nothing.
+constexpr int kOrganThreads = 512;
+constexpr int kOrganColumns = 32;
+struct OrganColumns {
+  double col[kOrganColumns][kFoldThreads];
+};
+template <int NQ, int WIDE>
+__device__ __forceinline__ void tile_partials(const float (*s_val)[kFoldTile], const uint8_t* s_lab, uint32_t set,
+                                              OrganColumns& s, double* __restrict__ part) {
+  constexpr int kMine = kOrganColumns / (NQ * WIDE), kRound = WIDE * kMine;   // columns of a group; labels of a round
+  static_assert(NQ * WIDE <= kOrganThreads / kFoldThreads, "a group each");
+  const int t = threadIdx.x & (kFoldThreads - 1), r = threadIdx.x >> 7, q = r % NQ, mine = r / NQ;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, n = __popc(set);
+  if (threadIdx.x < NQ * kLabelSlots && !(set >> (threadIdx.x % kLabelSlots) & 1u))
+    part[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = 0.0;
+  for (int k0 = 0; k0 < n; k0 += kRound) {
+    double(*const col)[kFoldThreads] = s.col + r * kMine;
+    if (r < NQ * WIDE) {
+      for (int c = 0; c < kMine && k0 + c * WIDE + mine < n; ++c) col[c][t] = 0.0;
+      double a = 0.0;                                    // of column `at`
+      int at = 0;
+#pragma unroll 1
+      for (int i0 = 0; i0 < kColumn; i0 += 16) {
+        float x[16];
+        int rank[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          x[i] = s_val[q][t + (i0 + i) * kFoldThreads];
+          rank[i] = __popc(set & ((1u << s_lab[t + (i0 + i) * kFoldThreads]) - 1u)) - k0;
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          if (x[i] == 0.0f || (unsigned)rank[i] % WIDE != mine || (unsigned)rank[i] >= (unsigned)kRound) continue;
+          if (rank[i] / WIDE != at) {
+            col[at][t] = a;
+            at = rank[i] / WIDE;
+            a = col[at][t];
+          }
+          if (q == 1 && x[i] == 1.0f) a = add_one(a);
+          else a += widen(x[i]);
+        }
+      }
+      col[at][t] = a;
+    }
+    __syncthreads();
+    for (int i = wid; i < NQ * min(kRound, n - k0); i += kOrganThreads / 32) {
+      const int qi = i % NQ, k = i / NQ;
+      const double sum = column_sum(s.col[(k % WIDE * NQ + qi) * kMine + k / WIDE], lane);
+      if (lane == 0) part[((size_t)qi * kLabelSlots + __fns(set, 0, k0 + k + 1)) * gridDim.x + blockIdx.x] = sum;
+    }
+    __syncthreads();
+  }
+}
+
+// Eq. 1 maps (MAPS) and the sums behind Eq. 2 and Eq. 3 per label.  A CTA takes
+// a tile: 512 threads form dose and epsilon^2 of its voxels in any order, eight
+// voxels' loads of each in flight, and then the columns from shared memory.
+// Bound by FP64 (six operations per voxel with a deposit, and two of the sums).
+// Microseconds a call of Eq. 2 and 3, host and copies with it: 256 x 253 x 300
+// voxels 505 -> 229, 64 x 61 x 75 84 -> 55.
+template <int NQ>
+struct OrganStage {
+  OrganColumns c;
+  float val[NQ][kFoldTile];
+  uint8_t lab[kFoldTile];
+};
+template <bool MAPS>
+__global__ void __launch_bounds__(kOrganThreads, 2) finalize_organ_tiles_kernel(const FinalizeParams p) {
+  constexpr int K = 8;
+  extern __shared__ __align__(16) unsigned char s_dyn[];
+  OrganStage<2>& st = *reinterpret_cast<OrganStage<2>*>(s_dyn);
+  __shared__ uint32_t s_mask[kSubs][kOrganThreads / 32];
+  const double inv_n = 1.0 / p.n_total;
+  const double inv_k1n = 1.0 / ((p.n_batches - 1.0) * p.n_total);
+  const float gy_a = (float)(p.gy_per_unit_vol * p.activity_bq);
+  const int64_t v0 = (int64_t)blockIdx.x * kFoldTile;
+#pragma unroll 1
+  for (int c = 0; c < kFoldTile / kOrganThreads; c += K) {
+    ull t[K];
+    double s2v[K];
+    float rho[K];
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+      const int64_t v = v0 + threadIdx.x + (c + j) * kOrganThreads;
+      t[j] = v < p.V ? p.tsum[v] : 0ull;
+    }
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+      const int64_t v = v0 + threadIdx.x + (c + j) * kOrganThreads;
+      s2v[j] = t[j] ? p.s2[v] : 0.0;
+      rho[j] = t[j] ? p.density[v] : 1.0f;
+    }
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+      const int k = threadIdx.x + (c + j) * kOrganThreads;
+      const int64_t v = v0 + k;
+      float d = 0.0f, sg = 0.0f;
+      if (t[j]) voxel_dose(t[j], s2v[j], rho[j], inv_n, inv_k1n, gy_a, d, sg);
+      const float eps = d > 0.0f ? __fdiv_rn(sg, d) : 1.0f;
+      st.val[0][k] = d;
+      st.val[1][k] = v < p.V ? eps * eps : 0.0f;
+      if (MAPS && v < p.V) {
+        if (p.dose) p.dose[v] = d;
+        if (p.sigma) p.sigma[v] = sg;
+      }
+    }
+  }
+  tile_labels<kOrganThreads>(p.labels, v0, p.V, st.lab, s_mask);
+  uint32_t set = 0;
+  for (int s = 0; s < kSubs; ++s) set |= label_set<kOrganThreads>(s_mask, s);
+  tile_partials<2, 1>(st.val, st.lab, set, st.c, p.organ_partial);
+}
+
+__global__ void finalize_organs_kernel(const FinalizeParams p, int n_tiles) {
   const int lane = threadIdx.x & 31;
   const int l = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (l >= kLabelSlots) return;
-  double sd = 0.0, se = 0.0;
-  for (int b = lane; b < n_blocks; b += 32) {
-    sd += p.organ_partial[(size_t)b * 2 * kLabelSlots + l];
-    se += p.organ_partial[(size_t)b * 2 * kLabelSlots + kLabelSlots + l];
-  }
-  sd = warp_sum_d(sd);
-  se = warp_sum_d(se);
+  const double sd = tile_sum(p.organ_partial + (size_t)l * n_tiles, n_tiles, lane);
+  const double se = tile_sum(p.organ_partial + (size_t)(kLabelSlots + l) * n_tiles, n_tiles, lane);
   if (lane != 0) return;
   const double cnt = (double)p.organ_count[l];
   double mean = 0.0, eps = 0.0, sig = 0.0;
@@ -338,52 +498,32 @@ __global__ void finalize_organs_kernel(const FinalizeParams p, int n_blocks) {
   p.organ_out[3 * kLabelSlots + l] = cnt;
 }
 
-// Eq. 2 over an arbitrary dose map: per-CTA per-label partial sums (fixed
-// tree).  Zeros add nothing and cost no FP64 (benchmark phantom: 134 -> 96 us).
-__global__ void __launch_bounds__(kFoldThreads) map_organ_kernel(const float* __restrict__ dose,
-                                                                 const uint8_t* __restrict__ labels, int64_t V,
-                                                                 int tiles_per_block, double* __restrict__ part) {
-  __shared__ double acc[kAccLabels * kFoldThreads];
-  __shared__ double out[1][kLabelSlots];
-  __shared__ uint32_t s_mask[kFoldThreads / 32];
-  const int tid = threadIdx.x;
-  if (tid < kLabelSlots) out[0][tid] = 0.0;
-  const int64_t first = (int64_t)blockIdx.x * tiles_per_block * kFoldTile;
-  for (int ti = 0; ti < tiles_per_block; ++ti) {
-    const int64_t v0 = first + (int64_t)ti * kFoldTile;
-    if (v0 >= V) break;
-    const int64_t v1 = v0 + kFoldTile < V ? v0 + kFoldTile : V;
-    float d[kPerThread];
+// Eq. 2 over an arbitrary dose map: partials per label and tile.  256 x 253 x
+// 300 voxels 165 -> 118 us a call.
+__global__ void __launch_bounds__(kOrganThreads) map_organ_kernel(const float* __restrict__ dose,
+                                                                  const uint8_t* __restrict__ labels, int64_t V,
+                                                                  double* __restrict__ part) {
+  extern __shared__ __align__(16) unsigned char s_dyn[];
+  OrganStage<1>& st = *reinterpret_cast<OrganStage<1>*>(s_dyn);
+  __shared__ uint32_t s_mask[kSubs][kOrganThreads / 32];
+  const int64_t v0 = (int64_t)blockIdx.x * kFoldTile;
 #pragma unroll
-    for (int i = 0; i < kPerThread; ++i) {
-      const int64_t v = v0 + tid + (int64_t)i * kFoldThreads;
-      d[i] = v < v1 ? dose[v] : 0.0f;
-    }
-    uint32_t lab[kPerThread / 4];
-    const uint32_t mask = tile_labels(labels, v0, v1, lab, s_mask);
-    const int n_lab = __popc(mask);
-    for (int l0 = 0; l0 < n_lab; l0 += kAccLabels) {
-      const int n_acc = min(kAccLabels, n_lab - l0);
-      for (int l = 0; l < n_acc; ++l) acc[l * kFoldThreads + tid] = 0.0;
-#pragma unroll
-      for (int i = 0; i < kPerThread; ++i) {
-        const int la = label_column(lab, i, mask, l0);
-        if (d[i] != 0.0f && la >= 0) acc[la * kFoldThreads + tid] += (double)d[i];
-      }
-      add_columns(acc, 1, n_acc, mask, l0, out);
-    }
+  for (int i = 0; i < kFoldTile / kOrganThreads; ++i) {
+    const int k = threadIdx.x + i * kOrganThreads;
+    st.val[0][k] = v0 + k < V ? dose[v0 + k] : 0.0f;
   }
-  if (tid < kLabelSlots) part[(size_t)blockIdx.x * kLabelSlots + tid] = out[0][tid];
+  tile_labels<kOrganThreads>(labels, v0, V, st.lab, s_mask);
+  uint32_t set = 0;
+  for (int s = 0; s < kSubs; ++s) set |= label_set<kOrganThreads>(s_mask, s);
+  tile_partials<1, 4>(st.val, st.lab, set, st.c, part);
 }
 
-__global__ void map_organ_final_kernel(const double* __restrict__ part, int n_blocks,
+__global__ void map_organ_final_kernel(const double* __restrict__ part, int n_tiles,
                                        const long long* __restrict__ count, double* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const int l = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (l >= kLabelSlots) return;
-  double s = 0.0;
-  for (int b = lane; b < n_blocks; b += 32) s += part[(size_t)b * kLabelSlots + l];
-  s = warp_sum_d(s);
+  const double s = tile_sum(part + (size_t)l * n_tiles, n_tiles, lane);
   if (lane == 0) out[l] = count[l] > 0 ? s / (double)count[l] : 0.0;
 }
 
@@ -419,16 +559,15 @@ __global__ void history_sigma_kernel(const ull* __restrict__ tsum, const ull* __
 
 }  // namespace
 
-// Tiles of a CTA of the passes over the voxels: few enough CTAs for a small pass over their
-// label sums, one tile each while that leaves every SM with work.
-static int fold_tiles(int64_t V) {
-  const int64_t tiles = (V + kFoldTile - 1) / kFoldTile;
-  return (int)std::max<int64_t>(1, (tiles + 16 * 152 - 1) / (16 * 152));
+int organ_tiles(int64_t V) { return (int)((V + kFoldTile - 1) / kFoldTile); }
+
+// Sub-tiles of a CTA of the passes without labels: one each while that leaves
+// about 16 CTAs an SM.
+static int pass_subs(int64_t V, int sms) {
+  const int64_t subs = (V + kSub - 1) / kSub;
+  return (int)std::max<int64_t>(1, (subs + 16 * sms - 1) / (16 * sms));
 }
-int fold_blocks(int64_t V) {
-  const int64_t per = (int64_t)fold_tiles(V) * kFoldTile;
-  return (int)((V + per - 1) / per);
-}
+static int pass_blocks(int64_t V, int subs) { return (int)((V + (int64_t)subs * kSub - 1) / ((int64_t)subs * kSub)); }
 
 cudaError_t launch_fold_history(ull* q_lo, ull* q_hi, ull* lo, ull* hi, int64_t V, cudaStream_t s) {
   const int64_t g = (V + 255) / 256;
@@ -446,9 +585,12 @@ cudaError_t launch_history_sigma(const ull* tsum, const ull* s2h_lo, const ull* 
 
 cudaError_t launch_map_organ_means(const float* dose, const uint8_t* labels, int64_t V, double* part,
                                    const long long* count, double* out, cudaStream_t s) {
-  const int nb = fold_blocks(V);
-  map_organ_kernel<<<nb, kFoldThreads, 0, s>>>(dose, labels, V, fold_tiles(V), part);
-  map_organ_final_kernel<<<(kLabelSlots + 3) / 4, 128, 0, s>>>(part, nb, count, out);
+  const int n = organ_tiles(V);
+  const cudaError_t e =
+      cudaFuncSetAttribute(map_organ_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(OrganStage<1>));
+  if (e != cudaSuccess) return e;
+  map_organ_kernel<<<n, kOrganThreads, sizeof(OrganStage<1>), s>>>(dose, labels, V, part);
+  map_organ_final_kernel<<<(kLabelSlots + 3) / 4, 128, 0, s>>>(part, n, count, out);
   return cudaGetLastError();
 }
 
@@ -516,20 +658,27 @@ cudaError_t launch_dose_only(const FinalizeParams& p, int sms, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Tiles per SM from which the fold takes whole tiles (fold_kernel); below, the
+// organ sums go by tile and slot, and the rest by sub-tile.  Microseconds by
+// slot and whole: one slot, 38 tiles 27 and 29, 300 tiles 39 and 35; ten slots,
+// 300 tiles 150 and 220, 1200 tiles 441 and 349.
+constexpr int split_tiles(int ns) { return ns <= 2 ? 1 : 4; }
+
 template <int NS>
 static cudaError_t launch_fold_t(const FoldParams& p, cudaStream_t s) {
-  const int nb = fold_blocks(p.V), tiles = fold_tiles(p.V);
-  if (!p.labels) {
-    fold_kernel<NS, false><<<nb, kFoldThreads, 0, s>>>(p, tiles);
-    return cudaGetLastError();
+  const int tiles = organ_tiles(p.V), subs = pass_subs(p.V, p.sms);
+  if (!p.labels || tiles < split_tiles(NS) * p.sms) {
+    if (p.labels) fold_slot_organs_kernel<<<dim3(tiles, p.n_slots), kFoldThreads, 0, s>>>(p);
+    fold_kernel<NS, false><<<pass_blocks(p.V, subs), kFoldThreads, 0, s>>>(p, subs);
+  } else {
+    const size_t smem = (size_t)NS * fold_columns(NS) * kFoldThreads * sizeof(double);
+    // per call: cheap, and correct for every device and calling thread
+    const cudaError_t e =
+        cudaFuncSetAttribute(fold_kernel<NS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    fold_kernel<NS, true><<<tiles, kFoldThreads, smem, s>>>(p, kSubs);
   }
-  const size_t smem = (size_t)NS * kAccLabels * kFoldThreads * sizeof(double);
-  // per call: cheap, and correct for every device and calling thread
-  const cudaError_t e =
-      cudaFuncSetAttribute(fold_kernel<NS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  fold_kernel<NS, true><<<nb, kFoldThreads, smem, s>>>(p, tiles);
-  fold_organs_kernel<<<kLabelSlots, 32 * p.n_slots, 0, s>>>(p, nb);
+  if (p.labels) fold_organs_kernel<<<kLabelSlots, 32 * p.n_slots, 0, s>>>(p, tiles);
   return cudaGetLastError();
 }
 
@@ -543,16 +692,22 @@ cudaError_t launch_fold(const FoldParams& p, cudaStream_t s) {
   return launch_fold_t<kMaxSlots>(p, s);
 }
 
-cudaError_t launch_finalize(const FinalizeParams& p, bool organs, cudaStream_t s) {
-  const int nb = fold_blocks(p.V), tiles = fold_tiles(p.V);
+template <bool MAPS>
+static cudaError_t launch_organ_tiles(const FinalizeParams& p, cudaStream_t s) {
+  const int tiles = organ_tiles(p.V);
+  const cudaError_t e = cudaFuncSetAttribute(finalize_organ_tiles_kernel<MAPS>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(OrganStage<2>));
+  if (e != cudaSuccess) return e;
+  finalize_organ_tiles_kernel<MAPS><<<tiles, kOrganThreads, sizeof(OrganStage<2>), s>>>(p);
+  finalize_organs_kernel<<<(kLabelSlots + 3) / 4, 128, 0, s>>>(p, tiles);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_finalize(const FinalizeParams& p, bool organs, int sms, cudaStream_t s) {
   const bool maps = p.dose || p.sigma;
-  if (!organs) {
-    if (maps) finalize_kernel<true, false><<<nb, kFoldThreads, 0, s>>>(p, tiles);
-    return cudaGetLastError();
-  }
-  if (maps) finalize_kernel<true, true><<<nb, kFoldThreads, 0, s>>>(p, tiles);
-  else finalize_kernel<false, true><<<nb, kFoldThreads, 0, s>>>(p, tiles);
-  finalize_organs_kernel<<<(kLabelSlots + 3) / 4, 128, 0, s>>>(p, nb);
+  if (organs) return maps ? launch_organ_tiles<true>(p, s) : launch_organ_tiles<false>(p, s);
+  const int subs = pass_subs(p.V, sms);
+  if (maps) finalize_maps_kernel<<<pass_blocks(p.V, subs), kFoldThreads, 0, s>>>(p, subs);
   return cudaGetLastError();
 }
 
