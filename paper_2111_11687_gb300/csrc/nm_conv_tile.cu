@@ -665,7 +665,7 @@ cudaError_t conv3d_fwd_image(const nm_conv3d_desc& d, const void* x, const void*
 cudaError_t conv3d_fwd_image_head(const nm_conv3d_desc& d, const void* x, const void* image, const float* bias,
                                   const float* head_w, const void* xin, int cx, float* yh, uint32_t* status,
                                   cudaStream_t s) {
-  if (d.cout != 16 || !conv_tile_ok(d)) return cudaErrorInvalidValue;
+  if (d.cout != 16 || !conv_image_ok(d)) return cudaErrorInvalidValue;
   const TileHead hd{head_w, (const bf16*)xin, cx, yh};
   if (packed_tiles()) return launch_fitting<16, true>(d, x, image, bias, nullptr, 1, hd, status, s);
   return launch_tile<16, 4, 16>(d, x, image, bias, nullptr, 1, hd, status, s, 16);

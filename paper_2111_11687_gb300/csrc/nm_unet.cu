@@ -704,7 +704,8 @@ nm_status forward(nm_denoiser* h, bool train, bool fuse_head = false, bool* fuse
                                                        la.c0, la.c1, h->cap_x[li - 2]);
       CK(keep(li - 2, nullptr, h->da[i]), "capture");
     }
-    if (i == 0 && fuse_head && lb.cout == 16 && conv_tile_ok(h->desc(lb))) {
+    // fused where the layer has an image (lay_out_weights)
+    if (i == 0 && fuse_head && lb.cout == 16 && conv_image_ok(h->desc(lb))) {
       CK(conv3d_fwd_image_head(h->desc(lb), h->da[0], h->images + lb.fwd_image, h->w + lb.b_off, h->w + h->head_off, h->x_in,
                               h->cx, h->y, h->status, s),
          "conv");
