@@ -202,7 +202,10 @@ nm_status nm_dose_create(nm_dose** out, const nm_grid* grid, const nm_materials*
  * (seed, history id) (Philox4x32-10), so the tally after run(a) + run(b) is
  * bit-identical to run(a + b); the batch uncertainty depends on the split.
  * NM_ERR_OVERFLOW if the cumulative tally could exceed 2^63 units;
- * NM_ERR_DEVICE if a device check fired (the batch is still folded). */
+ * NM_ERR_DEVICE if a device check fired (the batch is still folded).  After
+ * another error the handle holds the batches of the launches before the failed
+ * one, counted in its histories; if that one's fold had begun, runs and
+ * read-outs return NM_ERR_STATE until nm_dose_reset or nm_dose_restore. */
 nm_status nm_dose_run(nm_dose* h, uint64_t n_decays, uint64_t seed);
 
 /* Many patients in one call (the paper runs one patient at a time; this is
@@ -350,6 +353,11 @@ void nm_release_cached_memory(void);
  * of memory; 0 switches it off.  The failing call returns NM_ERR_OOM and frees
  * what it had allocated. */
 void nm_debug_fail_alloc(int32_t n);
+
+/* Fault injection: the n-th step that nm_dose_run or nm_dose_run_batch hands to
+ * the device from now on fails on the host instead (NM_ERR_CUDA); 0 switches it
+ * off. */
+void nm_debug_fail_enqueue(int32_t n);
 
 /* Runs one bounded device wait on an mbarrier that nothing completes (the
  * wait of the tensor-core kernels) with a limit of max_cycles SM clocks:

@@ -148,8 +148,16 @@ std::vector<float> beta_inverse_cdf(double t_max, int z) {
 }
 
 // Fault injection for the tests: the n-th device allocation from now (through
-// dalloc) fails as if the device were out of memory (0 = off).
-std::atomic<int> g_fail_alloc{0};
+// dalloc) fails as if the device were out of memory, the n-th step of a run
+// (enqueue_run) fails instead of going to the device (0 = off).
+std::atomic<int> g_fail_alloc{0}, g_fail_enqueue{0};
+
+bool fail_now(std::atomic<int>& left) {
+  int k = left.load();
+  while (k > 0 && !left.compare_exchange_weak(k, k - 1)) {
+  }
+  return k == 1;
+}
 
 // Device buffers of handles and of per-call temporaries are recycled: dfree
 // keeps a buffer (once nothing on the device can still use it) for the next
@@ -177,10 +185,7 @@ void release_cache_locked(BufferCache& c) {
 
 template <class T>
 cudaError_t dalloc(T** p, size_t n) {
-  int k = g_fail_alloc.load();
-  while (k > 0 && !g_fail_alloc.compare_exchange_weak(k, k - 1)) {
-  }
-  if (k == 1) {
+  if (fail_now(g_fail_alloc)) {
     *p = nullptr;
     return cudaErrorMemoryAllocation;
   }
@@ -344,14 +349,20 @@ struct nm_dose {
   bool nuclide = false;
   ull* s2h_lo = nullptr;       // history statistics (history_sigma): 128-bit sums of squares
   ull* s2h_hi = nullptr;
-  ull* q_lo = nullptr;         // a launch's sums of their low and high 32 bits, zero between runs unless `dirty`
+  ull* q_lo = nullptr;         // a launch's sums of their low and high 32 bits, zero between runs unless `broken`
   ull* q_hi = nullptr;
-  ull* counters = nullptr;     // kCtrCount
-  unsigned* work = nullptr;
-  // Batch tallies [slots][V], all zero between runs unless `dirty`: one from
+  // Counters, kCtrCount and a zero; the same before the launch under way, and
+  // in the place of the zero the launch's work counter: one copy before a launch
+  // sets both.
+  ull* counters = nullptr;
+  ull* kept = nullptr;
+  unsigned* work = nullptr;    // in kept
+  // Batch tallies [slots][V], all zero between runs unless `broken`: one from
   // the start, as many as a run can use at once from the first run that does.
   int slots = 1;
-  bool dirty = false;
+  // A run ended in the middle of a fold: the statistics are not those of the
+  // histories counted, and runs and read-outs are refused until reset or restore.
+  bool broken = false;
   uint32_t* status = nullptr;
   uint32_t* rho_max_bits = nullptr;
   double* org_s1 = nullptr;
@@ -377,7 +388,7 @@ struct nm_dose {
   ~nm_dose() {
     // nothing on the device may still use a buffer that is recycled
     cudaStreamSynchronize(stream);
-    void* ptrs[] = {vox, density, labels, label_bad, alias, tb, tsum, s2, kn, minv, minv_out, beta_tab, kn_inv, s2h_lo, s2h_hi, q_lo, q_hi, counters, work, status,
+    void* ptrs[] = {vox, density, labels, label_bad, alias, tb, tsum, s2, kn, minv, minv_out, beta_tab, kn_inv, s2h_lo, s2h_hi, q_lo, q_hi, counters, kept, status,
                     rho_max_bits, org_s1, org_s2, organ_count, organ_partial, organ_out,
                     out_dose, out_sigma};
     for (void* p : ptrs) dfree(p);
@@ -851,13 +862,14 @@ nm_status nm_dose_create(nm_dose** out, const nm_grid* g, const nm_materials* mt
   if ((e = dalloc(&h->vox, V)) || (e = dalloc(&h->density, V)) || (e = dalloc(&h->tb, V)) ||
       (e = dalloc(&h->tsum, V)) || (e = dalloc(&h->s2, V)) || (e = dalloc(&h->kn, kKnTable)) ||
       (e = dalloc(&h->minv, kKnTable)) || (e = dalloc(&h->minv_out, kKnTable)) ||
-      (e = dalloc(&h->counters, kCtrCount)) || (e = dalloc(&h->work, 1)) ||
+      (e = dalloc(&h->counters, kCtrCount + 1)) || (e = dalloc(&h->kept, kCtrCount + 1)) ||
       (e = dalloc(&h->status, 1)) || (e = dalloc(&h->rho_max_bits, NM_MAX_MATERIALS)) ||
       (e = dalloc(&h->org_s1, kLabelSlots)) || (e = dalloc(&h->org_s2, kLabelSlots)) ||
       (e = dalloc(&h->organ_count, kLabelSlots)) ||
       (e = dalloc(&h->organ_partial, (size_t)organ_tiles(V) * 2 * kLabelSlots)) ||
       (e = dalloc(&h->organ_out, 4 * kLabelSlots)))
     return bail(cuda_fail(e, "device allocation"));
+  h->work = reinterpret_cast<unsigned*>(h->kept + kCtrCount);
   if (labels && ((e = dalloc(&h->labels, V)) || (e = dalloc(&h->label_bad, 1))))
     return bail(cuda_fail(e, "device allocation"));
   {
@@ -963,7 +975,7 @@ nm_status nm_dose_create(nm_dose** out, const nm_grid* g, const nm_materials* mt
   e = cudaMemsetAsync(h->tb, 0, V * sizeof(ull), s);
   if (!e) e = cudaMemsetAsync(h->tsum, 0, V * sizeof(ull), s);
   if (!e) e = cudaMemsetAsync(h->s2, 0, V * sizeof(double), s);
-  if (!e) e = cudaMemsetAsync(h->counters, 0, kCtrCount * sizeof(ull), s);
+  if (!e) e = cudaMemsetAsync(h->counters, 0, (kCtrCount + 1) * sizeof(ull), s);
   if (!e) e = cudaMemsetAsync(h->org_s1, 0, kLabelSlots * sizeof(double), s);
   if (!e) e = cudaMemsetAsync(h->org_s2, 0, kLabelSlots * sizeof(double), s);
   if (!e) e = cudaMemsetAsync(h->organ_count, 0, kLabelSlots * sizeof(long long), s);
@@ -1023,15 +1035,30 @@ static nm_status ensure_slots(nm_dose* h, int want) {
   return NM_OK;
 }
 
-// Clears what a run that failed half-way left in the batch tallies and the
-// launch's sums of squares.
-static cudaError_t clear_dirty(nm_dose* h) {
-  if (!h->dirty) return cudaSuccess;
+// Clears the batch tallies and the launch's sums of squares.
+static cudaError_t clear_tallies(nm_dose* h, cudaStream_t s) {
   const size_t V8 = 8 * (size_t)h->V;
-  cudaError_t e = cudaMemsetAsync(h->tb, 0, V8 * h->slots, h->stream);
-  if (!e && h->q_lo) e = cudaMemsetAsync(h->q_lo, 0, V8, h->stream);
-  if (!e && h->q_hi) e = cudaMemsetAsync(h->q_hi, 0, V8, h->stream);
+  cudaError_t e = cudaMemsetAsync(h->tb, 0, V8 * h->slots, s);
+  if (!e && h->q_lo) e = cudaMemsetAsync(h->q_lo, 0, V8, s);
+  if (!e && h->q_hi) e = cudaMemsetAsync(h->q_hi, 0, V8, s);
   return e;
+}
+
+// Takes back a group of batches whose launch is on stream s and whose fold is not.
+static cudaError_t undo_launch(nm_dose* h, cudaStream_t s) {
+  uint32_t st = 0;
+  cudaError_t e = cudaMemcpyAsync(h->counters, h->kept, kCtrCount * sizeof(ull), cudaMemcpyDeviceToDevice, s);
+  if (!e) e = clear_tallies(h, s);
+  if (!e) e = cudaMemcpyAsync(&st, h->status, 4, cudaMemcpyDeviceToHost, s);
+  if (!e) e = cudaStreamSynchronize(s);
+  if (!e) e = cudaMemsetAsync(h->status, 0, 4, s);
+  h->status_seen |= st;
+  return e;
+}
+
+static nm_status check_whole(const nm_dose* h) {
+  return h->broken ? fail(NM_ERR_STATE, "a run of this handle ended half-way: nm_dose_reset or nm_dose_restore first")
+                   : NM_OK;
 }
 
 static FoldParams fold_params(const nm_dose* h) {
@@ -1062,14 +1089,19 @@ static int launch_batches(uint64_t n, int B, int b0, int slots) {
 
 // Enqueues n histories of h in B batches on stream s with the launch shape of
 // `like`: per group of batches one launch that tallies each batch in its own
-// slot, then one fold of the slots in batch order.  minv: the majorants
-// [2][kKnTable] to fly with, NULL = the handle's.  mark() is called before a
-// launch, after it and after its fold.
+// slot, then one fold of the slots in batch order, after which the group counts
+// among the handle's histories.  minv: the majorants [2][kKnTable] to fly with,
+// NULL = the handle's.  mark() is called before a launch, after it and after
+// its fold.  On an error the groups before the one at hand stay, and that one's
+// launch is taken back; where that fails, or its fold had begun, the handle is
+// `broken`.
 static cudaError_t enqueue_run(nm_dose* h, uint64_t n, int B, uint64_t seed, const nm_dose* like, const float* minv,
                                cudaStream_t s, const std::function<cudaError_t()>& mark) {
   const uint64_t q = n / B, r = n % B;
-  uint64_t id = h->id_next;
   cudaError_t e = cudaSuccess;
+  auto step = [&e](auto&& f) {
+    if (!e) e = fail_now(g_fail_enqueue) ? cudaErrorUnknown : f();
+  };
   for (int b0 = 0; b0 < B && !e;) {
     NvtxRange batch_range("batches");
     const int k = launch_batches(n, B, b0, h->slots);
@@ -1078,10 +1110,16 @@ static cudaError_t enqueue_run(nm_dose* h, uint64_t n, int B, uint64_t seed, con
     FoldParams fp = fold_params(h);
     fp.n_slots = k;
     for (int b = 0; b < k; ++b) fp.set_batch(b, q + ((uint32_t)b < big ? 1 : 0));
-    e = mark();
+    bool launched = false, folding = false;
+    // a launch's squares fit their two sums; of several launches they go first
+    auto fold_squares = [&] {
+      folding = true;
+      return launch_fold_history(h->q_lo, h->q_hi, h->s2h_lo, h->s2h_hi, h->V, s);
+    };
+    step(mark);
     for (uint64_t done = 0; done < total && !e;) {
       const uint64_t part = std::min<uint64_t>(total - done, 1ull << 31);
-      TransportParams p = h->params(id + done, part, seed);
+      TransportParams p = h->params(h->id_next + done, part, seed);
       if (k > 1) p.g.split = batch_split((uint32_t)k, big, (uint32_t)q);
       if (minv) {
         p.minv = minv;
@@ -1092,17 +1130,34 @@ static cudaError_t enqueue_run(nm_dose* h, uint64_t n, int B, uint64_t seed, con
       p.regroup_compton = p.regroup_refill = like->regroup_lanes;
       // no more CTAs than have a chunk to take
       const uint64_t want = (part + (uint64_t)p.chunk * warps - 1) / ((uint64_t)p.chunk * warps);
-      e = cudaMemsetAsync(h->work, 0, sizeof(unsigned), s);
-      if (!e)
-        e = launch_transport(p, (int)std::min<uint64_t>((uint64_t)like->grid, want), like->block, like->warp_agg,
-                             h->rayleigh, like->regroup, s, h->opt.history_sigma != 0);
-      if (!e && h->q_lo) e = launch_fold_history(h->q_lo, h->q_hi, h->s2h_lo, h->s2h_hi, h->V, s);
+      if (done == 0)
+        step([&] {
+          return cudaMemcpyAsync(h->kept, h->counters, (kCtrCount + 1) * sizeof(ull), cudaMemcpyDeviceToDevice, s);
+        });
+      else
+        step([&] { return cudaMemsetAsync(h->work, 0, sizeof(unsigned), s); });
+      launched |= !e;
+      step([&] {
+        return launch_transport(p, (int)std::min<uint64_t>((uint64_t)like->grid, want), like->block, like->warp_agg,
+                                h->rayleigh, like->regroup, s, h->opt.history_sigma != 0);
+      });
+      if (h->q_lo && part < total) step(fold_squares);
       done += part;
     }
-    if (!e) e = mark();
-    if (!e) e = launch_fold(fp, s);
-    if (!e) e = mark();
-    id += total;
+    step(mark);
+    step([&] {
+      folding = true;
+      return launch_fold(fp, s);
+    });
+    if (h->q_lo && total <= (1ull << 31)) step(fold_squares);
+    if (e) {
+      h->broken = folding || (launched && undo_launch(h, s) != cudaSuccess);
+      break;
+    }
+    h->hist_next += total;
+    h->id_next += total;
+    h->n_batches += (uint64_t)k;
+    step(mark);
     b0 += k;
   }
   return e;
@@ -1112,6 +1167,8 @@ nm_status nm_dose_run(nm_dose* h, uint64_t n, uint64_t seed) {
   NvtxRange range("nm_dose_run");
   if (!h) return fail(NM_ERR_ARG, "handle is NULL");
   if (n == 0) return NM_OK;
+  nm_status ws = check_whole(h);
+  if (ws != NM_OK) return ws;
   const uint64_t per = h->units_per_history();
   const uint64_t lim = (uint64_t)INT64_MAX / (per ? per : 1);
   if (h->hist_next > lim || n > lim - h->hist_next)
@@ -1121,10 +1178,7 @@ nm_status nm_dose_run(nm_dose* h, uint64_t n, uint64_t seed) {
     return fail(NM_ERR_OVERFLOW, "history ids exhausted");
   const int B = (uint64_t)h->opt.batches < n ? h->opt.batches : (int)n;
   cudaStream_t s = h->stream;
-  const nm_status es = ensure_slots(h, B);
-  if (es != NM_OK) return es;
-  const bool was_dirty = h->dirty;      // a run before this one failed half-way
-  h->dirty = true;
+  if ((ws = ensure_slots(h, B)) != NM_OK) return ws;
   // per launch: transport start and end, fold end
   size_t used = 0;
   const cudaError_t e = enqueue_run(h, n, B, seed, h, nullptr, s, [&]() -> cudaError_t {
@@ -1135,14 +1189,15 @@ nm_status nm_dose_run(nm_dose* h, uint64_t n, uint64_t seed) {
     }
     return cudaEventRecord(h->ev[used++], s);
   });
-  NM_CUDA(e, "nm_dose_run");
-  h->hist_next += n;
-  h->id_next += n;
-  h->n_batches += (uint64_t)B;
+  if (e) {
+    if (cudaStreamSynchronize(s) != cudaSuccess) h->broken = true;
+    return cuda_fail(e, "nm_dose_run");
+  }
   uint32_t st = 0;
+  h->broken = true;                     // unless the device gets to the end of it
   NM_CUDA(cudaMemcpyAsync(&st, h->status, 4, cudaMemcpyDeviceToHost, s), "status read");
   NM_CUDA(cudaStreamSynchronize(s), "nm_dose_run");
-  h->dirty = was_dirty;
+  h->broken = false;
   for (size_t g = 0; g < used; g += 3) {
     float ms = 0;
     if (cudaEventElapsedTime(&ms, h->ev[g], h->ev[g + 1]) == cudaSuccess) h->transport_ms += ms;
@@ -1187,6 +1242,8 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
     return fail(NM_ERR_ARG, "need 1..%d handles and their decay counts", kMaxBatchPatients);
   for (int i = 0; i < n; ++i) {
     if (!hs[i]) return fail(NM_ERR_ARG, "handle %d is NULL", i);
+    const nm_status ws = check_whole(hs[i]);
+    if (ws != NM_OK) return ws;
     for (int j = 0; j < i; ++j)
       if (hs[j] == hs[i]) return fail(NM_ERR_ARG, "handle %d appears twice", i);
     if (hs[i]->opt.history_sigma || hs[i]->nuclide)
@@ -1250,16 +1307,16 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
     e = cudaStreamCreateWithFlags(&st[j], cudaStreamNonBlocking);
     if (!e) e = cudaStreamWaitEvent(st[j], e0, 0);
   }
-  std::vector<char> was_dirty(n);
-  for (int i = 0; i < n; ++i) {
-    was_dirty[i] = hs[i]->dirty;
-    hs[i]->dirty = true;
-  }
   // the launch shape is the first handle's
   for (int i = 0; i < n && !e; ++i)
     if (n_decays[i])
       e = enqueue_run(hs[i], n_decays[i], (int)std::min<uint64_t>(B, n_decays[i]), seed, h0, d_minv,
                       st[i % n_streams], [] { return cudaSuccess; });
+  if (e) {
+    cleanup();                          // the patients and batches before the failed one stay
+    return cuda_fail(e, "nm_dose_run_batch");
+  }
+  for (int i = 0; i < n; ++i) hs[i]->broken = n_decays[i] != 0;   // unless the device gets to the end of it
   for (int j = 0; j < n_streams && !e; ++j) {
     e = cudaEventRecord(join, st[j]);
     if (!e) e = cudaStreamWaitEvent(s, join, 0);
@@ -1280,12 +1337,9 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
     cleanup();
     return cuda_fail(e, "nm_dose_run_batch");
   }
-  for (int i = 0; i < n; ++i) hs[i]->dirty = was_dirty[i];
   for (int i = 0; i < n; ++i) {
     if (n_decays[i] == 0) continue;
-    hs[i]->hist_next += n_decays[i];
-    hs[i]->id_next += n_decays[i];
-    hs[i]->n_batches += (uint64_t)std::min<uint64_t>(B, n_decays[i]);
+    hs[i]->broken = false;
     hs[i]->transport_ms += ms * (double)n_decays[i] / (double)total;  // the call's device time, shared by decays
     hs[i]->status_seen |= flags;
   }
@@ -1295,6 +1349,8 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
 }
 
 static nm_status finalize(nm_dose* h, float* dose, float* sigma, bool organs) {
+  const nm_status ws = check_whole(h);
+  if (ws != NM_OK) return ws;
   if (h->hist_next == 0) return fail(NM_ERR_STATE, "no histories simulated yet");
   if (h->n_batches < 2) return fail(NM_ERR_STATE, "need at least 2 batches for the uncertainty");
   cudaStream_t s = h->stream;
@@ -1317,6 +1373,8 @@ static nm_status finalize(nm_dose* h, float* dose, float* sigma, bool organs) {
 nm_status nm_dose_get(nm_dose* h, float* dose, float* sigma, double* organ_dose) {
   NvtxRange range("nm_dose_get");
   if (!h) return fail(NM_ERR_ARG, "handle is NULL");
+  const nm_status ws = check_whole(h);
+  if (ws != NM_OK) return ws;
   cudaStream_t s = h->stream;
   const bool dd = is_device_ptr(dose), ds = is_device_ptr(sigma);
   if ((dose && !dd) || (sigma && !ds)) {
@@ -1350,6 +1408,8 @@ nm_status nm_dose_get_organs(nm_dose* h, double* mean, double* eps_rms, double* 
                              int64_t* voxels) {
   NvtxRange range("nm_dose_get_organs");
   if (!h) return fail(NM_ERR_ARG, "handle is NULL");
+  const nm_status ws = check_whole(h);
+  if (ws != NM_OK) return ws;
   if (!eps_rms && h->labels) {
     // Eq. 2 and the batch sigma from the per-organ batch sums of the fold, no
     // pass over the voxels: mean = A sum_b O_b / (N cnt) with O_b the batch's
@@ -1399,6 +1459,8 @@ nm_status nm_dose_get_organs(nm_dose* h, double* mean, double* eps_rms, double* 
 
 nm_status nm_dose_get_history_sigma(nm_dose* h, float* sigma) {
   if (!h || !sigma) return fail(NM_ERR_ARG, "bad arguments");
+  const nm_status ws = check_whole(h);
+  if (ws != NM_OK) return ws;
   if (!h->s2h_lo) return fail(NM_ERR_STATE, "the handle was created without history_sigma");
   if (h->hist_next < 2) return fail(NM_ERR_STATE, "need at least 2 histories");
   cudaStream_t s = h->stream;
@@ -1502,6 +1564,8 @@ nm_status nm_time_integrated_activity(const float* const* act, const double* t_h
 
 nm_status nm_dose_get_tally(nm_dose* h, int64_t* tally) {
   if (!h || !tally) return fail(NM_ERR_ARG, "bad arguments");
+  const nm_status ws = check_whole(h);
+  if (ws != NM_OK) return ws;
   NM_CUDA(cudaMemcpyAsync(tally, h->tsum, h->V * sizeof(int64_t), cudaMemcpyDefault, h->stream), "tally copy");
   NM_CUDA(cudaStreamSynchronize(h->stream), "nm_dose_get_tally");
   return NM_OK;
@@ -1578,6 +1642,8 @@ nm_status nm_dose_checkpoint_size(const nm_dose* h, uint64_t* bytes) {
 nm_status nm_dose_checkpoint(nm_dose* h, void* buf, uint64_t bytes) {
   if (!h || !buf) return fail(NM_ERR_ARG, "bad arguments");
   if (bytes < ckpt_bytes(h)) return fail(NM_ERR_ARG, "checkpoint buffer too small");
+  const nm_status ws = check_whole(h);
+  if (ws != NM_OK) return ws;
   CkptHeader hd;
   memset(&hd, 0, sizeof hd);
   memcpy(hd.magic, kCkptMagic, 8);
@@ -1621,9 +1687,10 @@ nm_status nm_dose_restore(nm_dose* h, const void* buf, uint64_t bytes) {
     NM_CUDA(cudaMemcpyAsync(h->s2h_lo, b + o.lo, V8, cudaMemcpyDefault, s), "restore");
     NM_CUDA(cudaMemcpyAsync(h->s2h_hi, b + o.hi, V8, cudaMemcpyDefault, s), "restore");
   }
-  NM_CUDA(clear_dirty(h), "restore");
+  if (h->broken) NM_CUDA(clear_tallies(h, s), "restore");
+  if (h->broken) NM_CUDA(cudaMemsetAsync(h->status, 0, 4, s), "restore");
   NM_CUDA(cudaStreamSynchronize(s), "nm_dose_restore");
-  h->dirty = false;
+  h->broken = false;
   h->hist_next = hd.hist_next;
   h->id_next = hd.id_next;
   h->n_batches = hd.n_batches;
@@ -1636,6 +1703,7 @@ nm_status nm_dose_merge(nm_dose* h, const void* buf, uint64_t bytes) {
   if (!h) return fail(NM_ERR_ARG, "handle is NULL");
   CkptHeader hd;
   nm_status st = ckpt_read_header(h, buf, bytes, &hd);
+  if (st == NM_OK) st = check_whole(h);
   if (st != NM_OK) return st;
   const uint64_t per = h->units_per_history();
   const uint64_t lim = (uint64_t)INT64_MAX / (per ? per : 1);
@@ -1711,7 +1779,8 @@ nm_status nm_dose_counters(nm_dose* h, nm_counters* c) {
 nm_status nm_dose_reset(nm_dose* h) {
   if (!h) return fail(NM_ERR_ARG, "handle is NULL");
   cudaStream_t s = h->stream;
-  NM_CUDA(clear_dirty(h), "reset");
+  if (h->broken) NM_CUDA(clear_tallies(h, s), "reset");
+  if (h->broken) NM_CUDA(cudaMemsetAsync(h->status, 0, 4, s), "reset");
   NM_CUDA(cudaMemsetAsync(h->tsum, 0, h->V * sizeof(ull), s), "reset");
   NM_CUDA(cudaMemsetAsync(h->s2, 0, h->V * sizeof(double), s), "reset");
   NM_CUDA(cudaMemsetAsync(h->counters, 0, kCtrCount * sizeof(ull), s), "reset");
@@ -1722,7 +1791,7 @@ nm_status nm_dose_reset(nm_dose* h) {
     NM_CUDA(cudaMemsetAsync(h->s2h_hi, 0, h->V * sizeof(ull), s), "reset");
   }
   NM_CUDA(cudaStreamSynchronize(s), "reset");
-  h->dirty = false;
+  h->broken = false;
   h->hist_next = 0;
   h->id_next = 0;
   h->n_batches = 0;
@@ -1772,6 +1841,7 @@ nm_status nm_check_kahn(double e_mev, int64_t n, uint64_t seed, float* cos_out) 
 }
 
 void nm_debug_fail_alloc(int32_t n) { g_fail_alloc.store(n > 0 ? n : 0); }
+void nm_debug_fail_enqueue(int32_t n) { g_fail_enqueue.store(n > 0 ? n : 0); }
 
 void nm_release_cached_memory(void) {
   {
