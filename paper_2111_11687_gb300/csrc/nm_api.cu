@@ -380,8 +380,6 @@ struct nm_dose {
   double transport_ms = 0, fold_ms = 0;
   int block = 256, chunk = 256, warp_agg = 0, regroup = 0, regroup_lanes = 12, grid = 0;
   std::vector<cudaEvent_t> ev;
-  std::vector<float> minv_host;   // host copy of the majorant table
-  std::vector<float> minv_out_host;  // ... and of the one outside the tracking box
   float blo[3] = {0, 0, 0}, bhi[3] = {0, 0, 0};  // tracking box, voxel units
   bool tuned = false;             // launch shape chosen by the autotuner
 
@@ -948,8 +946,6 @@ nm_status nm_dose_create(nm_dose** out, const nm_grid* g, const nm_materials* mt
   if ((e = cudaMemcpy(h->minv, minv.data(), kKnTable * sizeof(float), cudaMemcpyHostToDevice)) ||
       (e = cudaMemcpy(h->minv_out, minv_out.data(), kKnTable * sizeof(float), cudaMemcpyHostToDevice)))
     return bail(cuda_fail(e, "majorant table"));
-  h->minv_host = minv;
-  h->minv_out_host = minv_out;
 
   // Decay sampler: alias table over the active voxels, FP64 on the device.
   if (o.source_mode == NM_SOURCE_DECAY) {
@@ -1090,13 +1086,12 @@ static int launch_batches(uint64_t n, int B, int b0, int slots) {
 // Enqueues n histories of h in B batches on stream s with the launch shape of
 // `like`: per group of batches one launch that tallies each batch in its own
 // slot, then one fold of the slots in batch order, after which the group counts
-// among the handle's histories.  minv: the majorants [2][kKnTable] to fly with,
-// NULL = the handle's.  mark() is called before a launch, after it and after
-// its fold.  On an error the groups before the one at hand stay, and that one's
+// among the handle's histories.  mark() is called before a launch, after it
+// and after its fold.  On an error the groups before the one at hand stay, and that one's
 // launch is taken back; where that fails, or its fold had begun, the handle is
 // `broken`.
-static cudaError_t enqueue_run(nm_dose* h, uint64_t n, int B, uint64_t seed, const nm_dose* like, const float* minv,
-                               cudaStream_t s, const std::function<cudaError_t()>& mark) {
+static cudaError_t enqueue_run(nm_dose* h, uint64_t n, int B, uint64_t seed, const nm_dose* like, cudaStream_t s,
+                               const std::function<cudaError_t()>& mark) {
   const uint64_t q = n / B, r = n % B;
   cudaError_t e = cudaSuccess;
   auto step = [&e](auto&& f) {
@@ -1121,10 +1116,6 @@ static cudaError_t enqueue_run(nm_dose* h, uint64_t n, int B, uint64_t seed, con
       const uint64_t part = std::min<uint64_t>(total - done, 1ull << 31);
       TransportParams p = h->params(h->id_next + done, part, seed);
       if (k > 1) p.g.split = batch_split((uint32_t)k, big, (uint32_t)q);
-      if (minv) {
-        p.minv = minv;
-        p.minv_out = minv + kKnTable;
-      }
       const int warps = like->block / 32;
       p.chunk = like->opt.chunk > 0 ? like->chunk : launch_chunk(like->chunk, (uint64_t)like->grid * warps, part);
       p.regroup_compton = p.regroup_refill = like->regroup_lanes;
@@ -1181,7 +1172,7 @@ nm_status nm_dose_run(nm_dose* h, uint64_t n, uint64_t seed) {
   if ((ws = ensure_slots(h, B)) != NM_OK) return ws;
   // per launch: transport start and end, fold end
   size_t used = 0;
-  const cudaError_t e = enqueue_run(h, n, B, seed, h, nullptr, s, [&]() -> cudaError_t {
+  const cudaError_t e = enqueue_run(h, n, B, seed, h, s, [&]() -> cudaError_t {
     if (used == h->ev.size()) {
       cudaEvent_t ev;
       if (cudaError_t c = cudaEventCreate(&ev)) return c;
@@ -1264,17 +1255,6 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
   for (int i = 0; i < n; ++i) total += n_decays[i];
   if (total == 0) return NM_OK;
 
-  // Shared physics: the batch majorant is the largest of the patients'.
-  std::vector<float> minv(2 * kKnTable);   // inside the tracking boxes, then outside
-  for (int k = 0; k < kKnTable; ++k) {
-    float m = h0->minv_host[k], mo = h0->minv_out_host[k];
-    for (int i = 1; i < n; ++i) {
-      m = std::min(m, hs[i]->minv_host[k]);
-      mo = std::min(mo, hs[i]->minv_out_host[k]);
-    }
-    minv[k] = m;
-    minv[kKnTable + k] = mo;
-  }
   for (int i = 0; i < n; ++i)
     if (n_decays[i] / B + (n_decays[i] % B ? 1 : 0) >= (1ull << 31))
       return fail(NM_ERR_ARG, "handle %d: batches above 2^31 histories", i);
@@ -1282,7 +1262,6 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
     const nm_status es = ensure_slots(hs[i], (int)std::min<uint64_t>(B, n_decays[i]));
     if (es != NM_OK) return es;
   }
-  float* d_minv = nullptr;
   cudaStream_t st[kBatchStreams] = {};
   cudaEvent_t e0 = nullptr, e1 = nullptr, join = nullptr;
   auto cleanup = [&]() {
@@ -1291,14 +1270,11 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
         cudaStreamSynchronize(c);
         cudaStreamDestroy(c);
       }
-    cudaStreamSynchronize(s);           // nothing on the device may still use the buffer
+    cudaStreamSynchronize(s);
     for (cudaEvent_t c : {e0, e1, join})
       if (c) cudaEventDestroy(c);
-    dfree(d_minv);
   };
-  cudaError_t e = dalloc(&d_minv, 2 * kKnTable);
-  if (!e) e = cudaMemcpyAsync(d_minv, minv.data(), 2 * kKnTable * sizeof(float), cudaMemcpyHostToDevice, s);
-  if (!e) e = cudaEventCreate(&e0);
+  cudaError_t e = cudaEventCreate(&e0);
   if (!e) e = cudaEventCreate(&e1);
   if (!e) e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
   const int n_streams = std::min(n, kBatchStreams);
@@ -1307,11 +1283,11 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
     e = cudaStreamCreateWithFlags(&st[j], cudaStreamNonBlocking);
     if (!e) e = cudaStreamWaitEvent(st[j], e0, 0);
   }
-  // the launch shape is the first handle's
+  // the launch shape is the first handle's, the majorants each its own
   for (int i = 0; i < n && !e; ++i)
     if (n_decays[i])
-      e = enqueue_run(hs[i], n_decays[i], (int)std::min<uint64_t>(B, n_decays[i]), seed, h0, d_minv,
-                      st[i % n_streams], [] { return cudaSuccess; });
+      e = enqueue_run(hs[i], n_decays[i], (int)std::min<uint64_t>(B, n_decays[i]), seed, h0, st[i % n_streams],
+                      [] { return cudaSuccess; });
   if (e) {
     cleanup();                          // the patients and batches before the failed one stay
     return cuda_fail(e, "nm_dose_run_batch");
