@@ -1304,9 +1304,11 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
   if (!e) e = cudaStreamSynchronize(s);
   if (!e) e = cudaEventElapsedTime(&ms, e0, e1);
   uint32_t flags = 0;
+  std::string flagged;                  // handles whose own checks fired
   for (int i = 0; i < n && !e; ++i)
     if (flag[i]) {
       flags |= flag[i];
+      flagged += " " + std::to_string(i);
       e = cudaMemsetAsync(hs[i]->status, 0, 4, s);
     }
   if (e) {
@@ -1317,10 +1319,10 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
     if (n_decays[i] == 0) continue;
     hs[i]->broken = false;
     hs[i]->transport_ms += ms * (double)n_decays[i] / (double)total;  // the call's device time, shared by decays
-    hs[i]->status_seen |= flags;
+    hs[i]->status_seen |= flag[i];
   }
   cleanup();
-  if (flags) return fail(NM_ERR_DEVICE, "device check fired (flags 0x%x)", flags);
+  if (flags) return fail(NM_ERR_DEVICE, "device check fired (flags 0x%x, handles%s)", flags, flagged.c_str());
   return NM_OK;
 }
 
