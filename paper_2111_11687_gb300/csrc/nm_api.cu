@@ -652,8 +652,8 @@ static std::mutex g_tune_mu;
 static std::map<TuneKey, Shape> g_tune_cache;
 
 static int grid_for_shape(const nm_dose* h, const Shape& sh) {
-  return h->sms * transport_max_blocks_per_sm(sh.block, sh.warp_agg, h->rayleigh, sh.regroup,
-                                              h->opt.history_sigma != 0, h->kind());
+  return h->sms * transport_max_blocks_per_sm(sh.block, sh.warp_agg, h->rayleigh, h->opt.kn_sampler != 0,
+                                              sh.regroup, h->opt.history_sigma != 0, h->kind());
 }
 
 // Histories per work grab of a launch of n: the handle's chunk, but where it is
@@ -680,7 +680,7 @@ static nm_status autotune(nm_dose* h, Shape sh, bool free_block, bool free_chunk
   const TuneKey key{h->device, h->nx, h->ny, h->nz, h->opt.source_mode, h->rayleigh,
                     (free_block ? 1 : 0) | (free_chunk ? 2 : 0) | (free_agg ? 4 : 0) |
                         (free_regroup ? 8 : 0) | (free_lanes ? 16 : 0) | (h->opt.history_sigma ? 32 : 0) |
-                        ((h->kind() + 1) << 6),
+                        ((h->kind() + 1) << 6) | (h->opt.kn_sampler ? 256 : 0),
                     free_block ? 0 : sh.block, free_chunk ? 0 : sh.chunk, free_agg ? 0 : sh.warp_agg,
                     free_regroup ? 0 : sh.regroup, free_lanes ? 0 : sh.lanes};
   {

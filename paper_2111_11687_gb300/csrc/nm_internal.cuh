@@ -207,7 +207,9 @@ int nuclide_kind(bool decay, bool beta_track, bool annihilate, int n_gamma);
 // uptake before the first, physical decay after the last), FP64 per voxel.
 cudaError_t launch_time_integral(const float* const* act, const double* t_s, int n, int64_t V, double tail_s,
                                  float* out, double* block_sums, int blocks, cudaStream_t s);
-int transport_max_blocks_per_sm(int block, bool warp_agg, bool rayleigh, bool regroup,
+// CTAs per SM of the kernel that launch_transport takes for the same choices
+// (kahn: no Klein-Nishina table, p.kn_inv NULL).
+int transport_max_blocks_per_sm(int block, bool warp_agg, bool rayleigh, bool kahn, bool regroup,
                                 bool history = false, int nuclide = 0);
 cudaError_t launch_check_philox(const uint4* ctr, const uint2* key, int64_t n, uint4* out,
                                 cudaStream_t s);

@@ -259,7 +259,7 @@ extern "C" nm_status nm_dose_tally_noalloc(const nm_grid* g, const nm_materials*
   int dev = 0, sms = 0;
   if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)))
     return cuda_fail(e, "device query");
-  const int per_sm = transport_max_blocks_per_sm(block, warp_agg, rayleigh, regroup);
+  const int per_sm = transport_max_blocks_per_sm(block, warp_agg, rayleigh, !p.kn_inv, regroup);
   if (per_sm <= 0) return fail(NM_ERR_CUDA, "transport kernel cannot be launched");
 
   if ((e = cudaMemsetAsync(tally, 0, 8 * V, s))) return cuda_fail(e, "tally clear");

@@ -1618,12 +1618,13 @@ cudaError_t launch_transport(const TransportParams& p, int grid, int block, bool
   return e;
 }
 
-int transport_max_blocks_per_sm(int block, bool warp_agg, bool rayleigh, bool regroup, bool history, int nuc) {
+int transport_max_blocks_per_sm(int block, bool warp_agg, bool rayleigh, bool kahn, bool regroup, bool history,
+                                int nuc) {
   int n = 0;
   if (nuc != kPair && warp_agg) return 0;
-  const bool ring = use_ring(regroup, history, nuc);
-  void* fn = ring ? pick_ring(warp_agg, rayleigh, nuc) : pick(warp_agg, rayleigh, regroup, history, nuc != kPair);
-  const size_t smem = ring ? ring_smem(block, rayleigh, nuc) : transport_smem(block, history, nuc != kPair);
+  const bool ring = use_ring(regroup, history, nuc), general = rayleigh || kahn;
+  void* fn = ring ? pick_ring(warp_agg, general, nuc) : pick(warp_agg, rayleigh, regroup, history, nuc != kPair);
+  const size_t smem = ring ? ring_smem(block, general, nuc) : transport_smem(block, history, nuc != kPair);
   if (!fn || cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, block, smem) != cudaSuccess) {
     cudaGetLastError();
