@@ -196,8 +196,10 @@ nm_status nm_dose_create(nm_dose** out, const nm_grid* grid, const nm_materials*
 /* Simulates n_decays more histories (§2.1-2.2) in opts.batches batches of
  * near-equal size, folding each batch into the statistics.  Up to 16 batches
  * share a launch, each with a tally of its own: the first run of more than one
- * batch adds 8 bytes per voxel and further batch to the handle, up to 16 GiB
- * (fewer batches share a launch where memory is short).  History ids
+ * batch (of 64 decays or more) adds 8 bytes per voxel and further batch to the
+ * handle, up to 16 GiB, a quarter of the device memory that is free then, and
+ * with the other handles' an eighth of all of it (fewer batches share a launch
+ * where memory is short).  History ids
  * continue across calls and every history's random numbers depend only on
  * (seed, history id) (Philox4x32-10), so the tally after run(a) + run(b) is
  * bit-identical to run(a + b); the batch uncertainty depends on the split.
@@ -358,6 +360,12 @@ void nm_debug_fail_alloc(int32_t n);
  * the device from now on fails on the host instead (NM_ERR_CUDA); 0 switches it
  * off. */
 void nm_debug_fail_enqueue(int32_t n);
+
+/* Batch tallies that a handle of so many voxels takes for a run: the rule of
+ * nm_dose_run, on made-up memory (free and total of the device, and what other
+ * handles hold in tallies beyond their first). */
+int32_t nm_debug_batch_slots(int64_t voxels, uint64_t n_decays, int32_t batches, uint64_t free_bytes,
+                             uint64_t total_bytes, uint64_t held_bytes);
 
 /* Runs one bounded device wait on an mbarrier that nothing completes (the
  * wait of the tensor-core kernels) with a limit of max_cycles SM clocks:

@@ -223,6 +223,23 @@ StreamPools& stream_pools() {
   return *p;
 }
 
+// Whether dalloc would take such a buffer from the cache.
+bool dalloc_cached(int dev, size_t bytes) {
+  BufferCache& c = buffer_cache();
+  std::lock_guard<std::mutex> lock(c.mu);
+  return c.free.count(std::make_pair(dev, bytes)) != 0;
+}
+
+// Bytes of all handles' batch tallies beyond the first, per device.
+struct SlotMemory {
+  std::mutex mu;
+  std::map<int, uint64_t> held, total;   // total: of the device, once asked
+};
+SlotMemory& slot_memory() {
+  static SlotMemory* m = new SlotMemory();     // never destroyed, as the buffer cache
+  return *m;
+}
+
 // Returns a dalloc'd buffer; the caller guarantees that no device work still
 // uses it (its stream was synchronised).  Other pointers are cudaFree'd.
 void dfree(void* p) {
@@ -360,6 +377,7 @@ struct nm_dose {
   // Batch tallies [slots][V], all zero between runs unless `broken`: one from
   // the start, as many as a run can use at once from the first run that does.
   int slots = 1;
+  uint64_t slot_bytes = 0;     // of the tallies beyond the first, counted in slot_memory()
   // A run ended in the middle of a fold: the statistics are not those of the
   // histories counted, and runs and read-outs are refused until reset or restore.
   bool broken = false;
@@ -391,6 +409,10 @@ struct nm_dose {
                     out_dose, out_sigma};
     for (void* p : ptrs) dfree(p);
     for (auto e : ev) cudaEventDestroy(e);
+    if (slot_bytes) {
+      std::lock_guard<std::mutex> lock(slot_memory().mu);
+      slot_memory().held[device] -= slot_bytes;
+    }
   }
 
   int kind() const {
@@ -995,18 +1017,42 @@ nm_status nm_dose_create(nm_dose** out, const nm_grid* g, const nm_materials* mt
   return NM_OK;
 }
 
-// Memory of one handle's batch tallies beyond the first, at most.
+// Memory of one handle's batch tallies, at most; of all handles' beyond their
+// first, at most this part of the device's, and of what is free when a handle
+// takes its own, which leaves the rest to other handles and programs.
 static constexpr uint64_t kSlotBytes = 16ull << 30;
+static constexpr uint64_t kSlotShare = 8, kFreeShare = 4;
 
-// Batch tallies for `want` batches per launch, as far as kSlotBytes and the
-// device's memory go: at least the one the handle was made with.
-static nm_status ensure_slots(nm_dose* h, int want) {
+// Batch tallies for n histories in B batches on V voxels: as many as a launch
+// can use (launch_batches; slot x voxel stays below 2^32) and memory allows, in
+// near-equal launches; at least the one a handle is made with.
+static int batch_slots(int64_t V, uint64_t n, int B, uint64_t free, uint64_t total, uint64_t held) {
+  if (n / B < kMinSplit) return 1;
+  const uint64_t each = (uint64_t)V * sizeof(ull), big = n / B + (n % B ? 1 : 0);
+  const uint64_t share = total / kSlotShare > held ? total / kSlotShare - held : 0;
+  const int most = (int)std::max<uint64_t>(
+      1, std::min<uint64_t>({(uint64_t)kMaxSlots, (1ull << 31) / big, kSlotBytes / each,
+                             ((1ull << 32) - 1) / (uint64_t)V, 1 + std::min(share, free / kFreeShare) / each}));
+  const int launches = (B + most - 1) / most;
+  return (B + launches - 1) / launches;
+}
+
+// Batch tallies for a run of n histories in B batches.
+static nm_status ensure_slots(nm_dose* h, uint64_t n, int B) {
   const uint64_t each = (uint64_t)h->V * sizeof(ull);
-  // ... below 2^32 voxels in all
-  const int most = (int)std::min<uint64_t>({(uint64_t)kMaxSlots, std::max<uint64_t>(kSlotBytes / each, 1),
-                                            std::max<uint64_t>(((1ull << 32) - 1) / (uint64_t)h->V, 1)});
-  const int launches = (want + most - 1) / most;
-  want = (want + launches - 1) / launches;     // near-equal launches
+  if (batch_slots(h->V, n, B, UINT64_MAX, UINT64_MAX, 0) <= h->slots) return NM_OK;
+  SlotMemory& m = slot_memory();
+  std::lock_guard<std::mutex> lock(m.mu);
+  uint64_t &held = m.held[h->device], &total = m.total[h->device];
+  size_t free = 0, all = total;
+  if (!total) NM_CUDA(cudaMemGetInfo(&free, &all), "batch tallies");
+  total = all;
+  const uint64_t others = held - h->slot_bytes;
+  int want = batch_slots(h->V, n, B, UINT64_MAX, total, others);
+  if (!dalloc_cached(h->device, each * want)) {
+    NM_CUDA(cudaMemGetInfo(&free, &all), "batch tallies");
+    want = batch_slots(h->V, n, B, free, total, others);
+  }
   if (want <= h->slots) return NM_OK;
   ull* tb = nullptr;
   double* part = nullptr;
@@ -1028,6 +1074,8 @@ static nm_status ensure_slots(nm_dose* h, int want) {
     h->organ_partial = part;
   }
   h->slots = want;
+  held += each * (want - 1) - h->slot_bytes;
+  h->slot_bytes = each * (want - 1);
   return NM_OK;
 }
 
@@ -1169,7 +1217,7 @@ nm_status nm_dose_run(nm_dose* h, uint64_t n, uint64_t seed) {
     return fail(NM_ERR_OVERFLOW, "history ids exhausted");
   const int B = (uint64_t)h->opt.batches < n ? h->opt.batches : (int)n;
   cudaStream_t s = h->stream;
-  if ((ws = ensure_slots(h, B)) != NM_OK) return ws;
+  if ((ws = ensure_slots(h, n, B)) != NM_OK) return ws;
   // per launch: transport start and end, fold end
   size_t used = 0;
   const cudaError_t e = enqueue_run(h, n, B, seed, h, s, [&]() -> cudaError_t {
@@ -1259,7 +1307,8 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
     if (n_decays[i] / B + (n_decays[i] % B ? 1 : 0) >= (1ull << 31))
       return fail(NM_ERR_ARG, "handle %d: batches above 2^31 histories", i);
   for (int i = 0; i < n; ++i) {
-    const nm_status es = ensure_slots(hs[i], (int)std::min<uint64_t>(B, n_decays[i]));
+    if (n_decays[i] == 0) continue;
+    const nm_status es = ensure_slots(hs[i], n_decays[i], (int)std::min<uint64_t>(B, n_decays[i]));
     if (es != NM_OK) return es;
   }
   cudaStream_t st[kBatchStreams] = {};
@@ -1819,6 +1868,11 @@ nm_status nm_check_kahn(double e_mev, int64_t n, uint64_t seed, float* cos_out) 
 }
 
 void nm_debug_fail_alloc(int32_t n) { g_fail_alloc.store(n > 0 ? n : 0); }
+int32_t nm_debug_batch_slots(int64_t voxels, uint64_t n_decays, int32_t batches, uint64_t free_bytes,
+                             uint64_t total_bytes, uint64_t held_bytes) {
+  if (voxels < 1 || batches < 1) return 0;
+  return batch_slots(voxels, n_decays, batches, free_bytes, total_bytes, held_bytes);
+}
 void nm_debug_fail_enqueue(int32_t n) { g_fail_enqueue.store(n > 0 ? n : 0); }
 
 void nm_release_cached_memory(void) {

@@ -110,6 +110,7 @@ _SIGS = {
     "nm_check_beta": (C.c_int, [C.c_double, C.c_int32, C.c_int64, C.c_uint64, C.c_void_p]),
     "nm_debug_fail_alloc": (None, [C.c_int32]),
     "nm_debug_fail_enqueue": (None, [C.c_int32]),
+    "nm_debug_batch_slots": (C.c_int32, [C.c_int64, C.c_uint64, C.c_int32, C.c_uint64, C.c_uint64, C.c_uint64]),
     "nm_release_cached_memory": (None, []),
     "nm_check_kn_table": (C.c_int, [C.c_double, C.c_double, C.c_double, C.c_int64, C.c_uint64, C.c_void_p]),
     "nm_check_wait_timeout": (C.c_int, [C.c_int64]),
