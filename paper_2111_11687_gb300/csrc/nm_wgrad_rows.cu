@@ -64,7 +64,7 @@ constexpr uint32_t kPad = 256;                   // zero rows before and after d
 constexpr uint32_t kYBytes = kSteps * kRow + 2 * kPad;
 constexpr int kThreads = 192;
 constexpr long long kWaitCycles = 4ll << 30;
-constexpr int kChain = 10;                       // tiles summed in TMEM before they are added to the partial
+constexpr int kChain = 10;                       // tiles summed in TMEM before they are added to the partial, at most
 
 template <int COUT, int G, int ND>
 struct RLayout {
@@ -82,7 +82,7 @@ struct RLayout {
 };
 
 struct RGrid {
-  int n, d, h, w, tiles_x, tiles_y, tiles_z, cin, kpad;
+  int n, d, h, w, tiles_x, tiles_y, tiles_z, cin, kpad, chain;
   long long tiles;
   __device__ void coords(long long t, int& b, int& x0, int& y0, int& z0) const {
     x0 = (int)(t % tiles_x) * TX; t /= tiles_x;
@@ -112,8 +112,8 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_rows_kernel(const __grid_co
   const int nchunks = (g.cin + 15) / 16;
   const long long my_tiles = g.tiles > blockIdx.x ? (g.tiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
   const int passes = (nchunks + G - 1) / G * kDz;
-  // tiles per read-out of the accumulators: equal shares of at most kChain
-  const long long seg = my_tiles > 0 ? (my_tiles + (my_tiles + kChain - 1) / kChain - 1) / ((my_tiles + kChain - 1) / kChain) : 1;
+  // tiles per read-out of the accumulators: equal shares of at most `chain`
+  const long long reads = (my_tiles + g.chain - 1) / g.chain, seg = reads > 0 ? (my_tiles + reads - 1) / reads : 1;
 
   if (warp == 0) tc::tmem_alloc(&s_tmem, 512);
   // the rows before and after each dY atom stay zero
@@ -372,6 +372,19 @@ dim3 row_grid(const nm_conv3d_desc& d) {
   return dim3(gx, std::max(gy, std::min(passes, sms / gx)));
 }
 
+// Tiles summed in tensor memory at a time.  With 64 and 128 outputs no more
+// steps of 16 voxels than in the gather kernel's sums, which the row kernel takes
+// the place of there, so that its error is no larger: 4 x 16^3 voxels, 64 -> 64
+// channels 3.4e-7 in sums of three tiles (48 steps), 2.4e-7 in the gather
+// kernel's of 24.
+int row_chain(const nm_conv3d_desc& d) {
+  if (d.cout <= 32) return kChain;
+  const long long m = (long long)d.n * d.d * d.h * d.w, splits = conv_wgrad_splits(d);
+  const long long theirs = ((m + splits - 1) / splits + 63) / 64 * 4;
+  const long long rows = (long long)d.n * d.d * d.h * ((d.w + TX - 1) / TX);   // steps in all, without empty ones
+  return (int)std::min<long long>(kChain, theirs * row_tiles(d) / std::max(rows, 1ll));
+}
+
 bool encode_tensor(CUtensorMap* map, const void* t, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
                    const cuuint32_t* box) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
@@ -405,6 +418,7 @@ cudaError_t launch_rows(const nm_conv3d_desc& d, const void* x, const void* dy, 
   g.tiles = row_tiles(d);
   g.cin = d.c0;
   g.kpad = conv_kpad(d.c0);
+  g.chain = row_chain(d);
   const dim3 grid = row_grid(d);
   const cudaError_t e = cudaFuncSetAttribute(wgrad_rows_kernel<COUT, G, ND>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::kSmem);
@@ -430,16 +444,16 @@ bool conv_wgrad_rows_ok(const nm_conv3d_desc& d) {
   // as well (4 x 64^3 voxels, 16 -> 16 channels: 116 us a call there, 125 here).
   // Two chunks: 636 there, 240 here (32 -> 32); three: 283 and 150 (48 -> 16).
   if (d.cout == 16 || d.cout == 32) return d.c0 > 16;
-  // 64 and 128 outputs: a small layer is launches, and the gather kernel has
-  // fewer; its cost grows with voxels x inputs, this one's has a read-out of 27 x
-  // inputs x outputs in it.  Microseconds a call with the gather and here, below
-  // and above each line.  64 outputs: 800 voxels of 64 inputs 42, 46; 4096 of 64
-  // 60, 53; 32,000 of 32 73, 78; 65,340 of 32 104, 83; 288,000 of 128 1318, 440.
-  // 128 outputs: 16,384 of 128 128, 178; 54,000 of 64 182, 214; 55,296 of 128 332,
-  // 312; 81,120 of 128 565, 462.
+  // 64 and 128 outputs: where the gather kernel's sums are short, this kernel's
+  // would be longer than they (row_chain), and a layer that small gains little
+  // here: from two tiles a sum on.  With 128 outputs the read-out of 27 x inputs
+  // x outputs counts too.  Microseconds a call with the gather and here, below
+  // and above each line.  64 outputs: 4 x 16^3 voxels of 64 inputs 77, 84; 2 x 20
+  // x 33 x 33 of 32 89, 81; 2 x 40 x 60 x 60 of 128 1307, 443.  128 outputs: 4 x
+  // 24^3 of 64 178, 202; 4 x 30 x 26 x 26 of 64 298, 260, of 128 567, 464.
+  if (row_chain(d) < 2) return false;
   const long long work = (long long)d.n * d.d * d.h * d.w * d.c0;
-  if (d.cout == 64) return work >= (d.c0 >= 64 ? 1 << 17 : 1 << 20);
-  return d.cout == 128 && work >= 1 << 22;
+  return d.cout == 64 || (d.cout == 128 && work >= 1 << 22);
 }
 
 size_t conv_wgrad_rows_workspace(const nm_conv3d_desc& d) {
