@@ -134,12 +134,19 @@ std::vector<float> beta_inverse_cdf(const double* t_maxs, const double* inten, i
   std::vector<double> key{(double)z, (double)sign};
   key.insert(key.end(), t_maxs, t_maxs + n);
   key.insert(key.end(), inten, inten + n);
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    for (auto& k : kept)
+      if (k.first == key) return k.second;
+  }
+  // integrated outside the lock: other threads' handles do not wait for it
+  std::vector<float> tab = build_beta_inverse_cdf(t_maxs, inten, n, z, sign);
   std::lock_guard<std::mutex> lock(mu);
   for (auto& k : kept)
-    if (k.first == key) return k.second;
+    if (k.first == key) return tab;
   if (kept.size() == kKept) kept.pop_front();
-  kept.emplace_back(key, build_beta_inverse_cdf(t_maxs, inten, n, z, sign));
-  return kept.back().second;
+  kept.emplace_back(std::move(key), tab);
+  return tab;
 }
 
 std::vector<float> beta_inverse_cdf(double t_max, int z) {
