@@ -22,6 +22,8 @@ FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", 
          "--expt-relaxed-constexpr", "-I", INCLUDE, "-I", CSRC]
 # The transport flushes FP32 denormals: its logarithms, divisions and
 # reciprocal roots then need no scaling of denormal operands.
+# Densities below FP32's normal range, which handles accept, then count as
+# vacuum there; with either an interaction has a probability of 1e-27 or less.
 FILE_FLAGS = {"nm_transport.cu": ["-ftz=true"]}
 
 
