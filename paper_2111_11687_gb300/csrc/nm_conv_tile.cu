@@ -65,10 +65,11 @@ constexpr int kEpiThreads = 128 * kEpiParts;               // warps 2 .. 1 + 4 k
 constexpr int kThreads = 64 + kEpiThreads;
 constexpr long long kWaitCycles = 4ll << 30;
 
-// Tile geometry and resources for COUT outputs and tiles TZ voxels deep.
-// Every 128-row M-tile accumulates its 27 taps in order, so the M-tiles are
-// the independent MMA chains in flight: 16-output layers, whose small MMAs
-// are bound by that chain latency, take deeper tiles (more M-tiles).
+// Tile geometry and resources for COUT outputs and tiles of TZ x TY rows.
+// Every 128-row M-tile accumulates its taps in order, so the M-tiles are the
+// independent MMA chains in flight: 16 outputs with one tap per MMA, whose small
+// MMAs are bound by that chain latency, take deeper tiles (more M-tiles); with
+// three taps per MMA (PACK), and with more outputs, launch_fitting chooses.
 template <int COUT, int TZ, int TY, bool PACK = false>
 struct TileLayout {
   static constexpr int PX = TX + 2, PY = TY + 2, PZ = TZ + 2;

@@ -5,10 +5,12 @@
 //
 // One persistent launch for all batches of a run, each with a tally of its own
 // (a launch's last photons then leave SMs idle once, not once per batch), in
-// two kernels.  In transport_ring_kernel
-// (annihilation photons or a point source: the default) a warp's
-// lanes hand photons on to each other through a ring in shared memory.  In
-// transport_kernel (history statistics, other decays, or `regroup` off) each lane owns one photon; a lane whose photon ends takes the
+// two kernels.  In transport_ring_kernel (the default: a point source, and
+// decays with annihilation photons, from the decay site or the end of a
+// positron's track, or with gamma lines) a warp's lanes hand photons on to each
+// other through a ring in shared memory.  In transport_kernel (history
+// statistics, decays with both annihilation photons and gamma lines, or
+// `regroup` off) each lane owns one photon; a lane whose photon ends takes the
 // decay's second photon or, with the rest of its warp, refills from a
 // warp-private pool of history ids that one lane grabs from a global counter
 // in chunks.  Every iteration of the loop is one flight step for every live
@@ -357,7 +359,7 @@ __device__ __forceinline__ bool positron_track(const PatientGeom& G, const Philo
 }
 
 // Adds dq units to *cell.  With WARP_AGG the lanes that hit the same cell
-// (same address, so lanes of different patients never merge) add their
+// (same address, so lanes of different batches never merge) add their
 // deposits with one warp reduction and one atomic.
 template <bool WARP_AGG>
 __device__ __forceinline__ void tally_flush(ull* cell, bool has, uint32_t dq, uint32_t lane) {
@@ -589,7 +591,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
           idx = fresh + (rank - avail);
         } else {
           got = false;
-          if (fresh_end == 0) done = true;   // every queue is drained
+          if (fresh_end == 0) done = true;   // every history has been handed out
         }
         if (got) {
           if (HIST && hn) hist_flush(hl, hn, tal, p.s2h_lo, p.s2h_hi);   // the previous history ends
@@ -835,13 +837,14 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const TransportParams
 // photons of a launch do not wait in the ring (5e6 decays 1.15 -> 1.10 ms, 1e6
 // point-source histories in ten launches 0.76 -> 0.50 ms).
 //
-// Benchmark phantom, 1e9 decays: 234.6 -> 137.3 ms; per decay 238.8 -> 127.2
-// warp instructions at 16.2 -> 24.4 active lanes.  Of that, the ring itself
+// Benchmark phantom, 1e9 decays: 234.6 -> 136 ms; per decay 238.8 -> 128.7
+// warp instructions at 16.2 -> 25 active lanes.  Of that, the ring itself
 // with one word per access 234.6 -> 197.7; slots as 16-byte words, the uniform
 // variates without a conversion and no denormals -> 171.7; branches folded into
 // predicates, both regions' majorants kept with the photon, escapes counted
 // from what is left over -> 150.5; a loop of its own for the end, the region
-// and photon B as signs -> 137.8; shared-memory addresses formed once -> 135.9; the lanes' own scatters at the end -> 137.3.
+// and photon B as signs -> 137.8; shared-memory addresses formed once -> 135.9;
+// the lanes' own scatters at the end -> 137.3; all batches in one launch -> 136.
 // A FIFO that pushes to and pops from different slots (fewer register moves,
 // more bookkeeping) measured 148-160.
 // ---------------------------------------------------------------------------
