@@ -195,11 +195,12 @@ nm_status nm_dose_create(nm_dose** out, const nm_grid* grid, const nm_materials*
 
 /* Simulates n_decays more histories (§2.1-2.2) in opts.batches batches of
  * near-equal size, folding each batch into the statistics.  Up to 16 batches
- * share a launch, each with a tally of its own: the first run of more than one
- * batch (of 64 decays or more) adds 8 bytes per voxel and further batch to the
- * handle, up to 16 GiB, a quarter of the device memory that is free then, and
- * with the other handles' an eighth of all of it (fewer batches share a launch
- * where memory is short).  History ids
+ * share a launch, each with a tally of its own: for as long as it lasts a run
+ * of more than one batch (of 64 decays or more) takes 8 bytes per voxel and
+ * batch, up to 16 GiB, which the library keeps for all handles' runs; a new
+ * such buffer is at most a quarter of the device memory that is free then, and
+ * all of them an eighth of the device's (fewer batches share a launch where
+ * memory is short).  History ids
  * continue across calls and every history's random numbers depend only on
  * (seed, history id) (Philox4x32-10), so the tally after run(a) + run(b) is
  * bit-identical to run(a + b); the batch uncertainty depends on the split.
@@ -339,11 +340,11 @@ nm_status nm_check_kn_table(double e_mev, double cut_mev, double e0_mev, int64_t
 /* Device memory released by destroyed handles and by the library's per-call
  * temporaries is kept (up to 8 GiB, per device and buffer size) and handed to
  * the next allocation of the same size on the same device, so that a handle
- * created after one of the same grid maps no new memory; scratch of the
- * denoiser and its convolutions comes from a memory pool that keeps up to
- * 512 MiB per device.  This call returns
- * all of it to the device; buffers of live handles are not
- * affected.  A failed allocation releases them by itself before it retries.
+ * created after one of the same grid maps no new memory; so are the batch
+ * tallies of runs (up to 8 GiB, or what the live handles' runs ask for);
+ * scratch of the denoiser and its convolutions comes from a memory pool that
+ * keeps up to 512 MiB per device.  This call returns all of it to the device;
+ * buffers of live handles and of runs under way are not affected.  A failed allocation releases them by itself before it retries.
  * Safe to call at any time from any thread.  Kept buffers belong to the
  * device's context: destroy the handles and call this before cudaDeviceReset
  * or anything else that ends the primary context, whose memory (kept buffers

@@ -184,10 +184,50 @@ BufferCache& buffer_cache() {
   return *c;
 }
 
+// Memory for the batch tallies of runs under way, beyond the one that a handle
+// keeps: all zero, since a fold leaves its tallies so, and taken by a run for as
+// long as it lasts, so that handles share it however many they are and a new
+// handle's first run finds it cleared.  Idle buffers are kept up to kIdleTallies,
+// or what the live handles' runs ask for (`wants`) in a share of the device, and given back to the
+// device by a failed allocation and nm_release_cached_memory.
+constexpr uint64_t kIdleTallies = 8ull << 30;
+constexpr uint64_t kSlotShare = 8;             // part of a device's memory for tallies beyond a handle's own
+struct TallyPool {
+  std::mutex mu;                                         // taken after BufferCache::mu, never before
+  struct Dev {
+    uint64_t total = 0;                                  // bytes of the device, once asked
+    uint64_t busy = 0, idle = 0, wants = 0;
+    uint64_t keep() const { return std::max(kIdleTallies, std::min(wants, total / kSlotShare)); }
+    std::deque<std::pair<ull*, uint64_t>> free;          // idle buffers and their bytes, latest first
+    // Takes the oldest idle buffers out until `most` bytes stay; to be freed after mu.
+    void trim(uint64_t most, std::vector<ull*>& out) {
+      while (idle > most) {
+        out.push_back(free.back().first);
+        idle -= free.back().second;
+        free.pop_back();
+      }
+    }
+  };
+  std::map<int, Dev> dev;
+};
+TallyPool& tally_pool() {
+  static TallyPool* p = new TallyPool();       // never destroyed, as the buffer cache
+  return *p;
+}
+
 void release_cache_locked(BufferCache& c) {
   for (auto& kv : c.free) cudaFree(kv.second);
   c.free.clear();
   c.cached = 0;
+  std::vector<ull*> out;
+  {
+    std::lock_guard<std::mutex> lock(tally_pool().mu);
+    for (auto& kv : tally_pool().dev) kv.second.trim(0, out);
+  }
+  for (ull* p : out) {
+    c.live.erase(p);
+    cudaFree(p);
+  }
 }
 
 template <class T>
@@ -209,7 +249,7 @@ cudaError_t dalloc(T** p, size_t n) {
     c.cached -= bytes;
   } else {
     e = cudaMalloc((void**)p, bytes);
-    if (e == cudaErrorMemoryAllocation && c.cached) {
+    if (e == cudaErrorMemoryAllocation) {
       cudaGetLastError();
       release_cache_locked(c);
       e = cudaMalloc((void**)p, bytes);
@@ -228,23 +268,6 @@ struct StreamPools {
 StreamPools& stream_pools() {
   static StreamPools* p = new StreamPools();   // never destroyed, as the buffer cache
   return *p;
-}
-
-// Whether dalloc would take such a buffer from the cache.
-bool dalloc_cached(int dev, size_t bytes) {
-  BufferCache& c = buffer_cache();
-  std::lock_guard<std::mutex> lock(c.mu);
-  return c.free.count(std::make_pair(dev, bytes)) != 0;
-}
-
-// Bytes of all handles' batch tallies beyond the first, per device.
-struct SlotMemory {
-  std::mutex mu;
-  std::map<int, uint64_t> held, total;   // total: of the device, once asked
-};
-SlotMemory& slot_memory() {
-  static SlotMemory* m = new SlotMemory();     // never destroyed, as the buffer cache
-  return *m;
 }
 
 // Returns a dalloc'd buffer; the caller guarantees that no device work still
@@ -381,10 +404,10 @@ struct nm_dose {
   ull* counters = nullptr;
   ull* kept = nullptr;
   unsigned* work = nullptr;    // in kept
-  // Batch tallies [slots][V], all zero between runs unless `broken`: one from
-  // the start, as many as a run can use at once from the first run that does.
-  int slots = 1;
-  uint64_t slot_bytes = 0;     // of the tallies beyond the first, counted in slot_memory()
+  // tb: a batch tally [V], all zero between runs unless `broken`, for runs that
+  // take no others (take_tallies).
+  uint64_t want_bytes = 0;     // of the tallies that this handle's last run asked for, in TallyPool's `wants`
+  int part_slots = 2;          // batches that organ_partial holds
   // A run ended in the middle of a fold: the statistics are not those of the
   // histories counted, and runs and read-outs are refused until reset or restore.
   bool broken = false;
@@ -416,9 +439,15 @@ struct nm_dose {
                     out_dose, out_sigma};
     for (void* p : ptrs) dfree(p);
     for (auto e : ev) cudaEventDestroy(e);
-    if (slot_bytes) {
-      std::lock_guard<std::mutex> lock(slot_memory().mu);
-      slot_memory().held[device] -= slot_bytes;
+    if (want_bytes) {
+      std::vector<ull*> out;
+      {
+        std::lock_guard<std::mutex> lock(tally_pool().mu);
+        TallyPool::Dev& d = tally_pool().dev[device];
+        d.wants -= want_bytes;
+        d.trim(d.keep(), out);
+      }
+      for (ull* p : out) dfree_now(p);
     }
   }
 
@@ -1024,11 +1053,11 @@ nm_status nm_dose_create(nm_dose** out, const nm_grid* g, const nm_materials* mt
   return NM_OK;
 }
 
-// Memory of one handle's batch tallies, at most; of all handles' beyond their
-// first, at most this part of the device's, and of what is free when a handle
-// takes its own, which leaves the rest to other handles and programs.
+// Memory of one run's batch tallies, at most; of all runs' under way beyond the
+// first of each, at most this part of the device's, and of what is free when it
+// is allocated, which leaves the rest to other handles and programs.
 static constexpr uint64_t kSlotBytes = 16ull << 30;
-static constexpr uint64_t kSlotShare = 8, kFreeShare = 4;
+static constexpr uint64_t kFreeShare = 4;
 
 // Batch tallies for n histories in B batches on V voxels: as many as a launch
 // can use (launch_batches; slot x voxel stays below 2^32) and memory allows, in
@@ -1044,62 +1073,163 @@ static int batch_slots(int64_t V, uint64_t n, int B, uint64_t free, uint64_t tot
   return (B + launches - 1) / launches;
 }
 
-// Batch tallies for a run of n histories in B batches.
-static nm_status ensure_slots(nm_dose* h, uint64_t n, int B) {
-  const uint64_t each = (uint64_t)h->V * sizeof(ull);
-  if (batch_slots(h->V, n, B, UINT64_MAX, UINT64_MAX, 0) <= h->slots) return NM_OK;
-  SlotMemory& m = slot_memory();
-  std::lock_guard<std::mutex> lock(m.mu);
-  uint64_t &held = m.held[h->device], &total = m.total[h->device];
-  size_t free = 0, all = total;
-  if (!total) NM_CUDA(cudaMemGetInfo(&free, &all), "batch tallies");
-  total = all;
-  const uint64_t others = held - h->slot_bytes;
-  int want = batch_slots(h->V, n, B, UINT64_MAX, total, others);
-  if (!dalloc_cached(h->device, each * want)) {
-    NM_CUDA(cudaMemGetInfo(&free, &all), "batch tallies");
-    want = batch_slots(h->V, n, B, free, total, others);
+// One handle's part of a run or batched run, and the tallies it runs with:
+// `slots` of them at `tb`, the handle's own one or more in a buffer of the pool.
+struct RunPart {
+  nm_dose* h;
+  uint64_t n;
+  int B;
+  ull* tb;
+  int slots;
+};
+
+// A buffer of the pool that parts in one stream share, one after the other.
+struct TallyLoan {
+  int device = 0;
+  ull* p = nullptr;
+  uint64_t bytes = 0;
+};
+
+// Ends a loan, after the device has: `zero` if the tallies are.
+static void return_tallies(TallyLoan* loan, bool zero) {
+  if (!loan->p) return;
+  std::vector<ull*> out;
+  {
+    TallyPool& pool = tally_pool();
+    std::lock_guard<std::mutex> lock(pool.mu);
+    TallyPool::Dev& d = pool.dev[loan->device];
+    d.busy -= loan->bytes;
+    if (zero) {
+      d.free.emplace_front(loan->p, loan->bytes);
+      d.idle += loan->bytes;
+      d.trim(d.keep(), out);
+    } else {
+      out.push_back(loan->p);
+    }
   }
-  if (want <= h->slots) return NM_OK;
-  ull* tb = nullptr;
-  double* part = nullptr;
-  cudaError_t e = dalloc(&tb, (size_t)h->V * want);
-  if (!e && want > 2) e = dalloc(&part, (size_t)organ_tiles(h->V) * want * kLabelSlots);
-  if (!e) e = cudaMemsetAsync(tb, 0, each * want, h->stream);
-  if (!e) e = cudaStreamSynchronize(h->stream);
-  if (e) {
-    dfree(tb);
-    dfree(part);
-    if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "batch tallies");
-    cudaGetLastError();                 // one batch per launch then
-    return NM_OK;
+  for (ull* p : out) dfree_now(p);
+  loan->p = nullptr;
+}
+
+// Tallies for parts that run one after the other on one stream, cleared on
+// stream s if they are new; on one device.  Parts that get no more than one
+// tally keep their handle's.
+static nm_status take_tallies(RunPart* part, int n_parts, cudaStream_t s, TallyLoan* loan) {
+  TallyPool& pool = tally_pool();
+  loan->device = part[0].h->device;
+  uint64_t need = 0;
+  std::vector<ull*> out;
+  auto most_bytes = [&](uint64_t free, uint64_t total, uint64_t held) {
+    uint64_t bytes = 0;
+    for (int i = 0; i < n_parts; ++i) {
+      const RunPart& r = part[i];
+      const int k = batch_slots(r.h->V, r.n, r.B, free, total, held);
+      if (k > 1) bytes = std::max(bytes, (uint64_t)r.h->V * sizeof(ull) * k);
+    }
+    return bytes;
+  };
+  for (int i = 0; i < n_parts; ++i) {
+    part[i].tb = part[i].h->tb;
+    part[i].slots = 1;
   }
-  dfree(h->tb);
-  h->tb = tb;
-  if (part) {
-    dfree(h->organ_partial);
-    h->organ_partial = part;
+  if (most_bytes(UINT64_MAX, UINT64_MAX, 0) == 0) return NM_OK;
+  size_t free = 0, total = 0;
+  uint64_t busy = 0;
+  {
+    std::lock_guard<std::mutex> lock(pool.mu);
+    TallyPool::Dev& d = pool.dev[loan->device];
+    if (!d.total) {
+      NM_CUDA(cudaMemGetInfo(&free, &total), "batch tallies");
+      d.total = total;
+    }
+    total = d.total;
+    busy = d.busy;
+    need = most_bytes(UINT64_MAX, total, busy);
+    for (int i = 0; i < n_parts; ++i) {
+      nm_dose* h = part[i].h;
+      const int k = batch_slots(h->V, part[i].n, part[i].B, UINT64_MAX, total, busy);
+      const uint64_t want = k > 1 ? (uint64_t)h->V * sizeof(ull) * k : 0;
+      d.wants += want - h->want_bytes;
+      h->want_bytes = want;
+    }
+    if (need == 0) return NM_OK;
+    auto best = d.free.end();                            // the smallest that holds it
+    for (auto it = d.free.begin(); it != d.free.end(); ++it)
+      if (it->second >= need && (best == d.free.end() || it->second < best->second)) best = it;
+    if (best != d.free.end()) {
+      loan->p = best->first;
+      loan->bytes = best->second;
+      d.idle -= loan->bytes;
+      d.busy += loan->bytes;
+      d.free.erase(best);
+    } else {
+      // a new one in the place of idle ones, where all are too many
+      const uint64_t room = total / kSlotShare > busy + need ? total / kSlotShare - busy - need : 0;
+      d.trim(room, out);
+    }
   }
-  h->slots = want;
-  held += each * (want - 1) - h->slot_bytes;
-  h->slot_bytes = each * (want - 1);
+  for (ull* p : out) dfree_now(p);
+  if (!loan->p) {
+    NM_CUDA(cudaMemGetInfo(&free, &total), "batch tallies");
+    if ((need = most_bytes(free, total, busy)) == 0) return NM_OK;
+    const cudaError_t e = dalloc(&loan->p, need / sizeof(ull));
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();               // one batch per launch then
+      return NM_OK;
+    }
+    if (e) return cuda_fail(e, "batch tallies");
+    loan->bytes = need;
+    {
+      std::lock_guard<std::mutex> lock(pool.mu);
+      pool.dev[loan->device].busy += need;
+    }
+    if (cudaError_t m = cudaMemsetAsync(loan->p, 0, need, s)) {
+      return_tallies(loan, false);
+      return cuda_fail(m, "batch tallies");
+    }
+  }
+  for (int i = 0; i < n_parts; ++i) {
+    RunPart& r = part[i];
+    const uint64_t each = (uint64_t)r.h->V * sizeof(ull);
+    int k = std::min<int>(batch_slots(r.h->V, r.n, r.B, UINT64_MAX, UINT64_MAX, 0),
+                          (int)std::min<uint64_t>(loan->bytes / each, kMaxSlots));
+    if (k < 2) continue;
+    const int launches = (r.B + k - 1) / k;
+    k = (r.B + launches - 1) / launches;                 // near-equal ones
+    if (k < 2) continue;
+    if (k > r.h->part_slots) {
+      double* p = nullptr;
+      const cudaError_t e = dalloc(&p, (size_t)organ_tiles(r.h->V) * k * kLabelSlots);
+      if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        continue;
+      }
+      if (e) return cuda_fail(e, "organ partial sums");
+      dfree(r.h->organ_partial);
+      r.h->organ_partial = p;
+      r.h->part_slots = k;
+    }
+    r.tb = loan->p;
+    r.slots = k;
+  }
   return NM_OK;
 }
 
-// Clears the batch tallies and the launch's sums of squares.
-static cudaError_t clear_tallies(nm_dose* h, cudaStream_t s) {
+// Clears batch tallies and the launch's sums of squares.
+static cudaError_t clear_tallies(nm_dose* h, ull* tb, int slots, cudaStream_t s) {
   const size_t V8 = 8 * (size_t)h->V;
-  cudaError_t e = cudaMemsetAsync(h->tb, 0, V8 * h->slots, s);
+  cudaError_t e = cudaMemsetAsync(tb, 0, V8 * slots, s);
   if (!e && h->q_lo) e = cudaMemsetAsync(h->q_lo, 0, V8, s);
   if (!e && h->q_hi) e = cudaMemsetAsync(h->q_hi, 0, V8, s);
   return e;
 }
 
 // Takes back a group of batches whose launch is on stream s and whose fold is not.
-static cudaError_t undo_launch(nm_dose* h, cudaStream_t s) {
+static cudaError_t undo_launch(const RunPart& r, cudaStream_t s) {
+  nm_dose* h = r.h;
   uint32_t st = 0;
   cudaError_t e = cudaMemcpyAsync(h->counters, h->kept, kCtrCount * sizeof(ull), cudaMemcpyDeviceToDevice, s);
-  if (!e) e = clear_tallies(h, s);
+  if (!e) e = clear_tallies(h, r.tb, r.slots, s);
   if (!e) e = cudaMemcpyAsync(&st, h->status, 4, cudaMemcpyDeviceToHost, s);
   if (!e) e = cudaStreamSynchronize(s);
   if (!e) e = cudaMemsetAsync(h->status, 0, 4, s);
@@ -1112,10 +1242,11 @@ static nm_status check_whole(const nm_dose* h) {
                    : NM_OK;
 }
 
-static FoldParams fold_params(const nm_dose* h) {
+static FoldParams fold_params(const RunPart& r) {
+  const nm_dose* h = r.h;
   FoldParams fp;
   memset(&fp, 0, sizeof fp);
-  fp.tb = h->tb; fp.tsum = h->tsum; fp.s2 = h->s2; fp.density = h->density;
+  fp.tb = r.tb; fp.tsum = h->tsum; fp.s2 = h->s2; fp.density = h->density;
   fp.labels = h->labels; fp.V = h->V; fp.sms = h->sms; fp.gy_per_unit_vol = h->gy_per_unit_vol();
   fp.organ_partial = h->organ_partial; fp.org_s1 = h->org_s1; fp.org_s2 = h->org_s2;
   fp.deposited = h->counters + kCtrDepositedUnits;
@@ -1138,15 +1269,18 @@ static int launch_batches(uint64_t n, int B, int b0, int slots) {
   return std::max(k, 1);
 }
 
-// Enqueues n histories of h in B batches on stream s with the launch shape of
+// Enqueues a part's histories in its batches on stream s with the launch shape of
 // `like`: per group of batches one launch that tallies each batch in its own
 // slot, then one fold of the slots in batch order, after which the group counts
 // among the handle's histories.  mark() is called before a launch, after it
 // and after its fold.  On an error the groups before the one at hand stay, and that one's
 // launch is taken back; where that fails, or its fold had begun, the handle is
 // `broken`.
-static cudaError_t enqueue_run(nm_dose* h, uint64_t n, int B, uint64_t seed, const nm_dose* like, cudaStream_t s,
+static cudaError_t enqueue_run(const RunPart& run, uint64_t seed, const nm_dose* like, cudaStream_t s,
                                const std::function<cudaError_t()>& mark) {
+  nm_dose* const h = run.h;
+  const uint64_t n = run.n;
+  const int B = run.B;
   const uint64_t q = n / B, r = n % B;
   cudaError_t e = cudaSuccess;
   auto step = [&e](auto&& f) {
@@ -1154,10 +1288,10 @@ static cudaError_t enqueue_run(nm_dose* h, uint64_t n, int B, uint64_t seed, con
   };
   for (int b0 = 0; b0 < B && !e;) {
     NvtxRange batch_range("batches");
-    const int k = launch_batches(n, B, b0, h->slots);
+    const int k = launch_batches(n, B, b0, run.slots);
     const uint32_t big = (uint32_t)std::min<uint64_t>(r > (uint64_t)b0 ? r - b0 : 0, (uint64_t)k);
     const uint64_t total = q * k + big;
-    FoldParams fp = fold_params(h);
+    FoldParams fp = fold_params(run);
     fp.n_slots = k;
     for (int b = 0; b < k; ++b) fp.set_batch(b, q + ((uint32_t)b < big ? 1 : 0));
     bool launched = false, folding = false;
@@ -1170,6 +1304,7 @@ static cudaError_t enqueue_run(nm_dose* h, uint64_t n, int B, uint64_t seed, con
     for (uint64_t done = 0; done < total && !e;) {
       const uint64_t part = std::min<uint64_t>(total - done, 1ull << 31);
       TransportParams p = h->params(h->id_next + done, part, seed);
+      p.g.tally = run.tb;
       if (k > 1) p.g.split = batch_split((uint32_t)k, big, (uint32_t)q);
       const int warps = like->block / 32;
       p.chunk = like->opt.chunk > 0 ? like->chunk : launch_chunk(like->chunk, (uint64_t)like->grid * warps, part);
@@ -1197,7 +1332,7 @@ static cudaError_t enqueue_run(nm_dose* h, uint64_t n, int B, uint64_t seed, con
     });
     if (h->q_lo && total <= (1ull << 31)) step(fold_squares);
     if (e) {
-      h->broken = folding || (launched && undo_launch(h, s) != cudaSuccess);
+      h->broken = folding || (launched && undo_launch(run, s) != cudaSuccess);
       break;
     }
     h->hist_next += total;
@@ -1224,10 +1359,15 @@ nm_status nm_dose_run(nm_dose* h, uint64_t n, uint64_t seed) {
     return fail(NM_ERR_OVERFLOW, "history ids exhausted");
   const int B = (uint64_t)h->opt.batches < n ? h->opt.batches : (int)n;
   cudaStream_t s = h->stream;
-  if ((ws = ensure_slots(h, n, B)) != NM_OK) return ws;
+  RunPart part{h, n, B, nullptr, 0};
+  TallyLoan loan;
+  if ((ws = take_tallies(&part, 1, s, &loan)) != NM_OK) {
+    return_tallies(&loan, cudaStreamSynchronize(s) == cudaSuccess);
+    return ws;
+  }
   // per launch: transport start and end, fold end
   size_t used = 0;
-  const cudaError_t e = enqueue_run(h, n, B, seed, h, s, [&]() -> cudaError_t {
+  const cudaError_t e = enqueue_run(part, seed, h, s, [&]() -> cudaError_t {
     if (used == h->ev.size()) {
       cudaEvent_t ev;
       if (cudaError_t c = cudaEventCreate(&ev)) return c;
@@ -1235,15 +1375,12 @@ nm_status nm_dose_run(nm_dose* h, uint64_t n, uint64_t seed) {
     }
     return cudaEventRecord(h->ev[used++], s);
   });
-  if (e) {
-    if (cudaStreamSynchronize(s) != cudaSuccess) h->broken = true;
-    return cuda_fail(e, "nm_dose_run");
-  }
   uint32_t st = 0;
-  h->broken = true;                     // unless the device gets to the end of it
-  NM_CUDA(cudaMemcpyAsync(&st, h->status, 4, cudaMemcpyDeviceToHost, s), "status read");
-  NM_CUDA(cudaStreamSynchronize(s), "nm_dose_run");
-  h->broken = false;
+  cudaError_t end = e ? cudaSuccess : cudaMemcpyAsync(&st, h->status, 4, cudaMemcpyDeviceToHost, s);
+  if (!end) end = cudaStreamSynchronize(s);
+  if (end) h->broken = true;            // the device did not get to the end of it
+  return_tallies(&loan, !h->broken);
+  if (e || end) return cuda_fail(e ? e : end, "nm_dose_run");
   for (size_t g = 0; g < used; g += 3) {
     float ms = 0;
     if (cudaEventElapsedTime(&ms, h->ev[g], h->ev[g + 1]) == cudaSuccess) h->transport_ms += ms;
@@ -1313,10 +1450,28 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
   for (int i = 0; i < n; ++i)
     if (n_decays[i] / B + (n_decays[i] % B ? 1 : 0) >= (1ull << 31))
       return fail(NM_ERR_ARG, "handle %d: batches above 2^31 histories", i);
-  for (int i = 0; i < n; ++i) {
-    if (n_decays[i] == 0) continue;
-    const nm_status es = ensure_slots(hs[i], n_decays[i], (int)std::min<uint64_t>(B, n_decays[i]));
-    if (es != NM_OK) return es;
+  // parts by stream, which share the stream's tallies
+  const int n_streams = std::min(n, kBatchStreams);
+  std::vector<RunPart> parts[kBatchStreams];
+  TallyLoan loans[kBatchStreams];
+  for (int i = 0; i < n; ++i)
+    if (n_decays[i])
+      parts[i % n_streams].push_back({hs[i], n_decays[i], (int)std::min<uint64_t>(B, n_decays[i]), nullptr, 0});
+  auto return_loans = [&] {
+    for (int j = 0; j < n_streams; ++j) {
+      bool zero = true;
+      for (const RunPart& r : parts[j]) zero = zero && !r.h->broken;
+      return_tallies(&loans[j], zero);
+    }
+  };
+  for (int j = 0; j < n_streams; ++j) {
+    if (parts[j].empty()) continue;
+    const nm_status ts = take_tallies(parts[j].data(), (int)parts[j].size(), s, &loans[j]);
+    if (ts != NM_OK) {
+      cudaStreamSynchronize(s);
+      return_loans();
+      return ts;
+    }
   }
   cudaStream_t st[kBatchStreams] = {};
   cudaEvent_t e0 = nullptr, e1 = nullptr, join = nullptr;
@@ -1329,21 +1484,22 @@ extern "C" nm_status nm_dose_run_batch(nm_dose* const* hs, int32_t n, const uint
     cudaStreamSynchronize(s);
     for (cudaEvent_t c : {e0, e1, join})
       if (c) cudaEventDestroy(c);
+    return_loans();
   };
   cudaError_t e = cudaEventCreate(&e0);
   if (!e) e = cudaEventCreate(&e1);
   if (!e) e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
-  const int n_streams = std::min(n, kBatchStreams);
   if (!e) e = cudaEventRecord(e0, s);
   for (int j = 0; j < n_streams && !e; ++j) {
     e = cudaStreamCreateWithFlags(&st[j], cudaStreamNonBlocking);
     if (!e) e = cudaStreamWaitEvent(st[j], e0, 0);
   }
   // the launch shape is the first handle's, the majorants each its own
-  for (int i = 0; i < n && !e; ++i)
-    if (n_decays[i])
-      e = enqueue_run(hs[i], n_decays[i], (int)std::min<uint64_t>(B, n_decays[i]), seed, h0, st[i % n_streams],
-                      [] { return cudaSuccess; });
+  for (int i = 0; i < n && !e; ++i) {
+    const std::vector<RunPart>& mine = parts[i % n_streams];
+    for (size_t k = 0; k < mine.size() && !e; ++k)
+      if (mine[k].h == hs[i]) e = enqueue_run(mine[k], seed, h0, st[i % n_streams], [] { return cudaSuccess; });
+  }
   if (e) {
     cleanup();                          // the patients and batches before the failed one stay
     return cuda_fail(e, "nm_dose_run_batch");
@@ -1721,7 +1877,7 @@ nm_status nm_dose_restore(nm_dose* h, const void* buf, uint64_t bytes) {
     NM_CUDA(cudaMemcpyAsync(h->s2h_lo, b + o.lo, V8, cudaMemcpyDefault, s), "restore");
     NM_CUDA(cudaMemcpyAsync(h->s2h_hi, b + o.hi, V8, cudaMemcpyDefault, s), "restore");
   }
-  if (h->broken) NM_CUDA(clear_tallies(h, s), "restore");
+  if (h->broken) NM_CUDA(clear_tallies(h, h->tb, 1, s), "restore");
   if (h->broken) NM_CUDA(cudaMemsetAsync(h->status, 0, 4, s), "restore");
   NM_CUDA(cudaStreamSynchronize(s), "nm_dose_restore");
   h->broken = false;
@@ -1813,7 +1969,7 @@ nm_status nm_dose_counters(nm_dose* h, nm_counters* c) {
 nm_status nm_dose_reset(nm_dose* h) {
   if (!h) return fail(NM_ERR_ARG, "handle is NULL");
   cudaStream_t s = h->stream;
-  if (h->broken) NM_CUDA(clear_tallies(h, s), "reset");
+  if (h->broken) NM_CUDA(clear_tallies(h, h->tb, 1, s), "reset");
   if (h->broken) NM_CUDA(cudaMemsetAsync(h->status, 0, 4, s), "reset");
   NM_CUDA(cudaMemsetAsync(h->tsum, 0, h->V * sizeof(ull), s), "reset");
   NM_CUDA(cudaMemsetAsync(h->s2, 0, h->V * sizeof(double), s), "reset");
