@@ -1402,7 +1402,7 @@ nm_status nm_dose_run(nm_dose* h, uint64_t n, uint64_t seed) {
 // few streams, so that a patient's transport fills the SMs that others' last
 // photons and folds leave, and small patients run side by side.  (One launch
 // over all patients' queues, whose lanes carried their patient, took 23.3 ms
-// for eight patients of 1e7; the patients' own launches take 14.4 ms, folds included.)
+// for eight patients of 1e7; the patients' own launches take 14.5 ms, folds included.)
 // ---------------------------------------------------------------------------
 static bool same_physics(const nm_dose* a, const nm_dose* b) {
   if (a->n_mat != b->n_mat || a->rayleigh != b->rayleigh || a->e0 != b->e0 || a->cut != b->cut ||
